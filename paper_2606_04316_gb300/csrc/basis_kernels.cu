@@ -166,23 +166,11 @@ __device__ inline void pair_fp_decode(const PairDev &pr, int nfb, int fp, int &f
     }
 }
 
-__device__ inline void htrip(int h, int &t, int &u, int &v) {
-    int s = 0;
-    while (nherm(s) <= h) ++s;
-    int rem = h - (s ? nherm(s - 1) : 0);
-    int uv = 0;
-    while ((uv + 1) * (uv + 2) / 2 <= rem) ++uv;
-    v = rem - uv * (uv + 1) / 2;
-    u = uv - v;
-    t = s - uv;
-}
-
-// One CTA per primitive pair: 1D tables in shared memory, then the E matrix
-// E[h][fp] over the pair's Hermite functions h of order <= Lab and its
-// function pairs fp (function pairs contiguous, for coalesced reads).
+// One CTA per primitive pair: 1D tables in shared memory, then the E entries of
+// its function pairs, each over its box of Hermite functions (FuncPair).
 __global__ void prim_pair_kernel(const ShellDev *shells, const PairDev *pairs, const int *pp_pair,
                                  const double *exps, const double *coefs, const double *norms,
-                                 PrimPairDev *pp, double *E) {
+                                 const FuncPair *fptab, PrimPairDev *pp, double *E) {
     __shared__ double Ex[3][kE1][kE1][kEt];
     int ipp = blockIdx.x;
     int ip = pp_pair[ipp];
@@ -221,43 +209,53 @@ __global__ void prim_pair_kernel(const ShellDev *shells, const PairDev *pairs, c
             o.p = p;
             o.inv_p = 1.0 / p;
             for (int d = 0; d < 3; ++d) o.P[d] = (a * A.A[d] + b * B.A[d]) / p;
-            o.eoff = pp[ipp].eoff;
             o.ia = ia;
             o.ib = ib;
             pp[ipp] = o;
         }
     }
     __syncthreads();
-    int nh = nherm(pr.Lab);
-    double *Eo = E + pp[ipp].eoff;
-    for (int fp = threadIdx.x; fp < pr.nfp; fp += blockDim.x) {
+    const int kl = ipp - pr.ppoff;
+    double *Eo = E + 2 * (pr.eoff + (kl >> 1)) + (kl & 1);
+    for (int k = threadIdx.x; k < pr.nfp; k += blockDim.x) {
+        const FuncPair info = fptab[pr.fpoff + k];
         int fa, fb;
-        pair_fp_decode(pr, B.nfunc, fp, fa, fb);
+        pair_fp_decode(pr, B.nfunc, info.fp & 0xffff, fa, fb);
         FuncTerms ta, tb;
         func_terms(A, fa, a, da, norms, ta);
         func_terms(B, fb, b, db, norms, tb);
-        for (int h = 0; h < nh; ++h) {
-            int t, u, v;
-            htrip(h, t, u, v);
-            double s = 0.0;
-            for (int x = 0; x < ta.n; ++x)
-                for (int y = 0; y < tb.n; ++y) {
-                    const int *pa = ta.pw[x], *pb = tb.pw[y];
-                    if (t > pa[0] + pb[0] || u > pa[1] + pb[1] || v > pa[2] + pb[2]) continue;
-                    s += ta.w[x] * tb.w[y] * Ex[0][pa[0]][pb[0]][t] * Ex[1][pa[1]][pb[1]][u] *
-                         Ex[2][pa[2]][pb[2]][v];
+        int nx = 0, ny = 0, nz = 0;                   // the box: the largest powers of the terms
+        for (int x = 0; x < ta.n; ++x)
+            for (int y = 0; y < tb.n; ++y) {
+                nx = max(nx, ta.pw[x][0] + tb.pw[y][0]);
+                ny = max(ny, ta.pw[x][1] + tb.pw[y][1]);
+                nz = max(nz, ta.pw[x][2] + tb.pw[y][2]);
+            }
+        double *o = Eo + 2 * (long long)info.off * pr.nk2;
+        for (int t = 0; t <= nx; ++t)
+            for (int u = 0; u <= ny; ++u)
+                for (int v = 0; v <= nz; ++v) {
+                    double s = 0.0;
+                    for (int x = 0; x < ta.n; ++x)
+                        for (int y = 0; y < tb.n; ++y) {
+                            const int *pa = ta.pw[x], *pb = tb.pw[y];
+                            if (t > pa[0] + pb[0] || u > pa[1] + pb[1] || v > pa[2] + pb[2]) continue;
+                            s += ta.w[x] * tb.w[y] * Ex[0][pa[0]][pb[0]][t] * Ex[1][pa[1]][pb[1]][u] *
+                                 Ex[2][pa[2]][pb[2]][v];
+                        }
+                    *o = s;
+                    o += 2 * pr.nk2;
                 }
-            Eo[(size_t)h * pr.nfp + fp] = s;          // [h][fp]: function pairs contiguous
-        }
     }
 }
 
 // Launcher (pp_pair maps every primitive pair to its shell pair).
 void launch_prim_pairs_map(const ShellDev *shells, const PairDev *pairs, const int *pp_pair,
                            long long npp, const double *exps, const double *coefs,
-                           const double *norms, PrimPairDev *pp, double *E, cudaStream_t s) {
+                           const double *norms, const FuncPair *fptab, PrimPairDev *pp, double2 *E,
+                           cudaStream_t s) {
     if (npp <= 0) return;
-    prim_pair_kernel<<<(unsigned)npp, 64, 0, s>>>(shells, pairs, pp_pair, exps, coefs, norms, pp, E);
+    prim_pair_kernel<<<(unsigned)npp, 64, 0, s>>>(shells, pairs, pp_pair, exps, coefs, norms, fptab, pp, (double *)E);
     QDT_CHECK_LAUNCH();
 }
 

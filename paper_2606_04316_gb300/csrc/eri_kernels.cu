@@ -1,5 +1,5 @@
 // eri_kernels.cu -- AO two-electron integral tiles on the GPU (stage (i) of
-// the paper's Sec. 3.3.1 decomposition), McMurchie-Davidson in FP64:
+// the paper's Sec. 3.3.1 decomposition), McMurchie-Davidson:
 //
 //   (xy|K|zw) = sum_{ij in X, kl in Y} sum_{h, h'} E^{ij}_{xy,h} (-1)^{|h'|}
 //               E^{kl}_{zw,h'} R^K_{h+h'}(rho, P - Q)
@@ -11,25 +11,39 @@
 //                  the last term shifting the Hermite index of the r12 tensor by e_I + e_J,
 //   R^n_{t+1,u,v} = t R^{n+1}_{t-1,u,v} + X_PQ R^{n+1}_{t,u,v}  (same in u, v).
 //
+// The signs (-1)^{|h'|} are carried by the tensor: R~_g = (-1)^{|g|} R_g is the
+// tensor of Q - P, and (-1)^{|h'|} R_{h+h'} = (-1)^{|h|} R~_{h+h'}.
+//
 // Work layout: a CTA owns one bra shell pair and a run of ket shell pairs.
-// For every shell quartet the cheaper orientation is contracted (the pair with
-// more function pairs takes the outer role X).  The primitive quartets of a
-// quartet are processed in groups -- several outer primitive pairs times all
-// inner ones when they fit in shared memory -- so that every phase (Boys
-// values, one recursion level, the ket contraction T = sum R E', the bra
-// contraction G += E T) keeps the CTA's lanes busy between two barriers.
+// For every shell quartet the cheaper orientation is contracted: X outer, Y
+// inner.  Per outer primitive pair ij (several at once when the quartet is
+// small): the Hermite tensors of all inner primitive pairs by the recursion,
+// the ket pass T[h][y] = sum_kl sum_h' R~ E', and the bra pass G += E T.  The
+// headers (Boys values, prefactors) of the quartet's primitive quartets run
+// before that in one pass, because a header is one long dependent chain.
 //
-// FP64 issue rate is the limit of this kernel, so the FP64 pipe does only
-// arithmetic of the method: no pow, one exp, two divisions and one sqrt per
-// primitive quartet; recursion sources and coefficients come from tables; the
-// sign (-1)^{|h'|} is a negated FMA operand (even and odd Hermite orders run in
-// separate loops) instead of a multiplication.
+// What bounds it: the multiply-adds of the two passes and the recursion, on the
+// FP32 pipe in the split form (12 operations per compensated multiply-add) and
+// on the FP64 pipe in the FP64 form.  Two things keep their number down and the
+// pipe busy:
+//  * Boxes.  The expansion of a function pair is a product of one-dimensional
+//    ones, so only the Hermite functions of its box (FuncPair) contribute, 27 to
+//    37 % of all for the pairs of p functions and derivatives.  Both passes
+//    run over the box's list only (the other terms are exact zeros).
+//  * Twos of primitive pairs.  R and E hold the inner primitive pairs in twos
+//    (hi0, hi1, lo0, lo1), so one 16-byte load feeds one packed FP32
+//    instruction (fma.rn.f32x2) per operation: half the issue slots of the
+//    scalar form, and the two halves are independent chains.  The bra pass
+//    packs two function pairs y instead.
 //
-// Split form (DF): Boys values, prefactors and the Hermite recursion stay in
-// FP64; the two contraction passes run in compensated FP32 pairs (x = hi + lo,
-// ~48-bit significands): products by the exact-product FMA, sums by the
-// error-free two-sum, so each multiply-add costs about twelve FP32
-// operations, which issue 64 times faster than FP64 on this part.
+// Measured against all Hermite functions and scalar instructions (integral phase,
+// before -> after): 24-centre s+p chain, all blocks, split 477 -> 262 ms; 12-centre
+// s/p/d cluster 671 -> 121 ms; 7-centre chain, FP64 form 39 -> 17 ms.
+//
+// Split form (DF): recursion and both passes in compensated FP32 pairs (x = hi +
+// lo, ~48-bit significands): products by the exact-product FMA, sums by the
+// error-free two-sum.  FP32 issues 64 times faster than FP64 on this part.
+// Tiles the host admitted to the FP32 error budget run in plain FP32.
 #include <math.h>
 
 #include <algorithm>
@@ -55,6 +69,7 @@ __constant__ double c_inv_odd[16] = {1.0,      1.0 / 3,  1.0 / 5,  1.0 / 7,  1.0
                                      1.0 / 13, 1.0 / 15, 1.0 / 17, 1.0 / 19, 1.0 / 21, 1.0 / 23,
                                      1.0 / 25, 1.0 / 27, 1.0 / 29, 1.0 / 31};
 
+
 __device__ inline void htrip_d(int h, int &t, int &u, int &v) {
     int s = 0;
     while (nherm(s) <= h) ++s;
@@ -66,11 +81,28 @@ __device__ inline void htrip_d(int h, int &t, int &u, int &v) {
     t = s - uv;
 }
 
-// F_0..F_nmax at T into F[0..nmax]; returns exp(-T).  Inside the table: Taylor
+// A primitive quartet's header in shared memory: entry j (Q - P, then R^n_000) of one
+// half of a two of primitive quartets; `st` scalars between entries.
+struct HeadF64 {
+    double *p;
+    int st;
+    __device__ double get(int j) const { return p[j * st]; }
+    __device__ void set(int j, double v) const { p[j * st] = v; }
+    __device__ void zero(int j) const { p[j * st] = 0.0; }
+};
+struct HeadPair {                       // (hi0, hi1, lo0, lo1)
+    float *p;
+    int st;
+    __device__ float2 get(int j) const { return make_float2(p[j * st], p[j * st + 2]); }
+    __device__ void set(int j, float2 v) const { p[j * st] = v.x; p[j * st + 2] = v.y; }
+    __device__ void zero(int j) const { set(j, make_float2(0.f, 0.f)); }
+};
+
+// F_0..F_nmax at T into entries j0..j0+nmax; returns exp(-T).  Inside the table: Taylor
 // expansion of the top order about the nearest grid point (Horner form), then
 // the downward recursion.  Beyond it erf(sqrt T) = 1 to double precision, so
 // F_0 = sqrt(pi / T) / 2, then the upward recursion.
-__device__ __forceinline__ double boys_eval(const double *tab, double T, int nmax, double *F) {
+__device__ __forceinline__ double boys_eval(const double *tab, double T, int nmax, const HeadF64 &H, int j0) {
     const double e = exp(-T);
     if (T < kBoysTMax) {
         const double ti = rint(T * kBoysInvDelta);
@@ -80,19 +112,19 @@ __device__ __forceinline__ double boys_eval(const double *tab, double T, int nma
         double f = __ldg(row + kBoysTaylor - 1);
 #pragma unroll
         for (int k = kBoysTaylor - 1; k > 0; --k) f = fma(f, md * c_inv_int[k], __ldg(row + k - 1));
-        F[nmax] = f;
+        H.set(j0 + nmax, f);
         const double t2 = T + T;
         for (int n = nmax - 1; n >= 0; --n) {
             f = fma(t2, f, e) * c_inv_odd[n];
-            F[n] = f;
+            H.set(j0 + n, f);
         }
     } else {
         double f = kHalfSqrtPi * rsqrt(T);
         const double inv2t = 0.5 / T;
-        F[0] = f;
+        H.set(j0, f);
         for (int n = 0; n < nmax; ++n) {
             f = fma(c_odd[n], f, -e) * inv2t;
-            F[n + 1] = f;
+            H.set(j0 + n + 1, f);
         }
     }
     return e;
@@ -121,102 +153,56 @@ __device__ __forceinline__ float2 df_split_bits(double x) {
     return make_float2(h, __uint_as_float(__float_as_uint(l) | sign));
 }
 
-// (ah, al) += sign * a * b: exact product error of the high parts plus the
-// cross terms, then the two-sum of the high parts.
-template <bool NEG>
-__device__ __forceinline__ void df_madd(float2 a, float2 b, float &ah, float &al) {
-    float p = __fmul_rn(a.x, b.x);
-    float pe = __fmaf_rn(a.x, b.x, -p);
-    pe = __fmaf_rn(a.x, b.y, pe);
-    pe = __fmaf_rn(a.y, b.x, pe);
-    if (NEG) { p = -p; pe = -pe; }
-    const float t = __fadd_rn(ah, p);
-    const float bv = __fsub_rn(t, ah);
-    const float err = __fadd_rn(__fsub_rn(ah, __fsub_rn(t, bv)), __fsub_rn(p, bv));
-    ah = t;
-    al = __fadd_rn(al, __fadd_rn(err, pe));
-}
-
-// x a + cf c in compensated FP32 pairs, renormalised (one Hermite recursion step).
-__device__ __forceinline__ float2 df_rec(float2 x, float2 a, float cf, float2 c) {
-    const float p1 = __fmul_rn(x.x, a.x);
-    float e1 = __fmaf_rn(x.x, a.x, -p1);
-    e1 = __fmaf_rn(x.x, a.y, e1);
-    e1 = __fmaf_rn(x.y, a.x, e1);
-    const float p2 = __fmul_rn(cf, c.x);
-    float e2 = __fmaf_rn(cf, c.x, -p2);
-    e2 = __fmaf_rn(cf, c.y, e2);
-    const float t = __fadd_rn(p1, p2);
-    const float bv = __fsub_rn(t, p1);
-    const float err = __fadd_rn(__fsub_rn(p1, __fsub_rn(t, bv)), __fsub_rn(p2, bv));
-    const float lo = __fadd_rn(err, __fadd_rn(e1, e2));
-    const float hi = __fadd_rn(t, lo);
-    return make_float2(hi, __fsub_rn(lo, __fsub_rn(hi, t)));
-}
-
-__global__ void split_pairs_kernel(const double *E, long long n, float2 *E2, float *E1) {
+__global__ void split_pairs_kernel(const double2 *E, long long n, float4 *E2, float2 *E1) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
-        const float2 v = df_split(E[i]);
-        E2[i] = v;
-        E1[i] = v.x;
+        const double2 e = E[i];
+        const float2 a = df_split(e.x), b = df_split(e.y);
+        E2[i] = make_float4(a.x, b.x, a.y, b.y);
+        E1[i] = make_float2(a.x, b.x);
     }
 }
 
-// Doubles of one primitive quartet's header: X_PQ (3), R^n_000 of the Coulomb
-// tensor (n = 0..L) and, for the gauge kernel, of the r12 tensor (n = 0..L+2).
+// Header of a primitive quartet in FP64: Q - P, then R^n_000 of the Coulomb tensor
+// (n = 0..L) and, for the gauge kernel, of the r12 tensor (n = 0..L+2).
 __host__ __device__ inline int header_len(int L, bool gauge) { return gauge ? 2 * L + 7 : L + 4; }
-// Doubles per primitive quartet: header, then the recursion's two buffers per
-// tensor -- even auxiliary orders (order 0 ends there: nherm(L) entries) and
-// odd orders (the largest is order 1: nherm(L - 1) entries); the r12 tensor of
-// the gauge kernel has top order L + 2.
-__host__ __device__ inline int odd_len(int Ltop) { return Ltop >= 1 ? nherm(Ltop - 1) : 0; }
-__host__ __device__ inline int quartet_len(int L, bool gauge) {
-    return header_len(L, gauge) + nherm(L) + odd_len(L) + (gauge ? nherm(L + 2) + odd_len(L + 2) : 0);
-}
 
-template <bool GAUGE, bool DF>
+template <bool GAUGE>
 __device__ __forceinline__ void quartet_header(const double *boys, const PrimPairDev *pa, const PrimPairDev *pc,
-                                               int L, double *hd) {
+                                               int L, const HeadF64 &H) {
     const double p = pa->p, q = pc->p, s = p + q;
-    const double X = pa->P[0] - pc->P[0], Y = pa->P[1] - pc->P[1], Z = pa->P[2] - pc->P[2];
+    const double X = pc->P[0] - pa->P[0], Y = pc->P[1] - pa->P[1], Z = pc->P[2] - pa->P[2];
     const double inv_s = 1.0 / s;
     const double rho = p * q * inv_s;
     const double T = rho * fma(X, X, fma(Y, Y, Z * Z));
-    hd[0] = X;
-    hd[1] = Y;
-    hd[2] = Z;
+    H.set(0, X);
+    H.set(1, Y);
+    H.set(2, Z);
     const double sq = sqrt(s);
     const double d = pa->inv_p * pc->inv_p * inv_s * sq;      // 1 / (p q sqrt(p + q))
     const double m2r = -2.0 * rho;
     double fC = kTwoPi52 * d;
     if (!GAUGE) {
-        double *F = hd + 3;
-        boys_eval(boys, T, L, F);
+        boys_eval(boys, T, L, H, 3);
         for (int n = 0; n <= L; ++n) {
-            F[n] *= fC;
+            H.set(3 + n, H.get(3 + n) * fC);
             fC *= m2r;
         }
     } else {
-        double *RC = hd + 3, *RR = hd + 4 + L;
-        const double e = boys_eval(boys, T, L + 2, RR);
+        const int jR = 4 + L;
+        const double e = boys_eval(boys, T, L + 2, H, jR);
         double fR = kPi52 * s * sq * d * d;
-        double prev = -fma(T + T, RR[0], e);            // F_{-1}
+        double prev = -fma(T + T, H.get(jR), e);            // F_{-1}
         for (int n = 0; n <= L + 2; ++n) {
-            const double cur = RR[n];
+            const double cur = H.get(jR + n);
             if (n <= L) {
-                RC[n] = cur * fC;
+                H.set(3 + n, cur * fC);
                 fC *= m2r;
             }
-            RR[n] = (cur - prev) * fR;
+            H.set(jR + n, (cur - prev) * fR);
             fR *= m2r;
             prev = cur;
         }
-    }
-    if (DF) {       // the recursion runs in compensated FP32 pairs: X_PQ and R^n_000 as (hi, lo)
-        float2 *h2 = reinterpret_cast<float2 *>(hd);
-        const int len = header_len(L, GAUGE);
-        for (int i = 0; i < len; ++i) h2[i] = df_split_bits(hd[i]);
     }
 }
 
@@ -266,12 +252,12 @@ __constant__ float2 c_inv_odd_p[16] = {
     pair_const(1.0 / 17), pair_const(1.0 / 19), pair_const(1.0 / 21), pair_const(1.0 / 23),
     pair_const(1.0 / 25), pair_const(1.0 / 27), pair_const(1.0 / 29), pair_const(1.0 / 31)};
 
-// F_0..F_nmax at T (a pair) into F[0..nmax] as pairs; returns exp(-T).  Inside
+// F_0..F_nmax at T (a pair) into entries j0..j0+nmax as pairs; returns exp(-T).  Inside
 // the table: Taylor expansion of the top order about the nearest grid point
 // T_i, exp(-T) = exp(-T_i) exp(T_i - T) (|T_i - T| <= 0.025, eight terms), then
 // the downward recursion; beyond it F_0 = sqrt(pi / T) / 2 and the upward
 // recursion (exp(-T) < 3e-16 F_0 there, so its FP32 value suffices).
-__device__ __forceinline__ float2 boys_eval_pairs(const BoysTables &bt, float2 T, int nmax, float2 *F) {
+__device__ __forceinline__ float2 boys_eval_pairs(const BoysTables &bt, float2 T, int nmax, const HeadPair &H, int j0) {
     if (T.x < (float)kBoysTMax) {
         const int i = min((int)rintf(T.x * (float)kBoysInvDelta), kBoysGrid - 1);
         const float2 md = pr_add(bt.t_pair[i], pr_neg(T));        // T_i - T
@@ -279,7 +265,7 @@ __device__ __forceinline__ float2 boys_eval_pairs(const BoysTables &bt, float2 T
         float2 f = row[kBoysTaylor - 1];
 #pragma unroll
         for (int k = kBoysTaylor - 1; k > 0; --k) f = pr_add(pr_mul(f, pr_mul(md, c_inv_int_p[k])), row[k - 1]);
-        F[nmax] = f;
+        H.set(j0 + nmax, f);
         float2 em = make_float2(1.f, 0.f);
 #pragma unroll
         for (int k = 7; k > 0; --k) em = pr_add(make_float2(1.f, 0.f), pr_mul(em, pr_mul(md, c_inv_int_p[k])));
@@ -287,63 +273,61 @@ __device__ __forceinline__ float2 boys_eval_pairs(const BoysTables &bt, float2 T
         const float2 t2 = pr_pow2(T, 2.f);
         for (int n = nmax - 1; n >= 0; --n) {
             f = pr_mul(pr_add(pr_mul(t2, f), e), c_inv_odd_p[n]);
-            F[n] = f;
+            H.set(j0 + n, f);
         }
         return e;
     }
     const float2 e = make_float2(expf(-T.x), 0.f);
     float2 f = pr_mul(pair_const(kHalfSqrtPi), pr_rcp(pr_sqrt(T)));
     const float2 inv2t = pr_pow2(pr_rcp(T), 0.5f);
-    F[0] = f;
+    H.set(j0, f);
     for (int n = 0; n < nmax; ++n) {
         f = pr_mul(pr_add(pr_mul(f, make_float2((float)(2 * n + 1), 0.f)), pr_neg(e)), inv2t);
-        F[n + 1] = f;
+        H.set(j0 + n + 1, f);
     }
     return e;
 }
 
 // Header of a primitive quartet whose integrals run in compensated FP32 pairs:
-// the same quantities as quartet_header<GAUGE, true> computed in FP32 pairs
+// the same quantities as quartet_header computed in FP32 pairs
 // (X_PQ and p + q from FP64 sums, the rest in pairs), so the FP64 pipe does four
 // additions per quartet instead of the whole header.  Layout as quartet_header.
 template <bool GAUGE>
 __device__ __forceinline__ void quartet_header_pairs(const double *boys, const PrimPairDev *pa, const PrimPairDev *pc,
-                                                     int L, double *hd) {
-    float2 *h2 = reinterpret_cast<float2 *>(hd);
+                                                     int L, const HeadPair &H) {
     const BoysTables bt = boys_tables(boys);
     const float2 p = df_split_bits(pa->p), q = df_split_bits(pc->p);
     const float2 s = df_split_bits(pa->p + pc->p);
-    const float2 X = df_split_bits(pa->P[0] - pc->P[0]), Y = df_split_bits(pa->P[1] - pc->P[1]),
-                 Z = df_split_bits(pa->P[2] - pc->P[2]);
+    const float2 X = df_split_bits(pc->P[0] - pa->P[0]), Y = df_split_bits(pc->P[1] - pa->P[1]),
+                 Z = df_split_bits(pc->P[2] - pa->P[2]);
     const float2 inv_s = pr_rcp(s);
     const float2 rho = pr_mul(pr_mul(p, q), inv_s);
     const float2 T = pr_mul(rho, pr_add(pr_add(pr_mul(X, X), pr_mul(Y, Y)), pr_mul(Z, Z)));
-    h2[0] = X;
-    h2[1] = Y;
-    h2[2] = Z;
+    H.set(0, X);
+    H.set(1, Y);
+    H.set(2, Z);
     const float2 sq = pr_sqrt(s);
     const float2 d = pr_mul(pr_mul(pr_mul(df_split_bits(pa->inv_p), df_split_bits(pc->inv_p)), inv_s), sq);
     const float2 m2r = pr_pow2(rho, -2.f);
     float2 fC = pr_mul(pair_const(kTwoPi52), d);
     if (!GAUGE) {
-        float2 *F = h2 + 3;
-        boys_eval_pairs(bt, T, L, F);
+        boys_eval_pairs(bt, T, L, H, 3);
         for (int n = 0; n <= L; ++n) {
-            F[n] = pr_mul(F[n], fC);
+            H.set(3 + n, pr_mul(H.get(3 + n), fC));
             fC = pr_mul(fC, m2r);
         }
     } else {
-        float2 *RC = h2 + 3, *RR = h2 + 4 + L;
-        const float2 e = boys_eval_pairs(bt, T, L + 2, RR);
+        const int jR = 4 + L;
+        const float2 e = boys_eval_pairs(bt, T, L + 2, H, jR);
         float2 fR = pr_mul(pr_mul(pr_mul(pair_const(kPi52), s), sq), pr_mul(d, d));
-        float2 prev = pr_neg(pr_add(pr_mul(pr_pow2(T, 2.f), RR[0]), e));     // F_{-1}
+        float2 prev = pr_neg(pr_add(pr_mul(pr_pow2(T, 2.f), H.get(jR)), e));     // F_{-1}
         for (int n = 0; n <= L + 2; ++n) {
-            const float2 cur = RR[n];
+            const float2 cur = H.get(jR + n);
             if (n <= L) {
-                RC[n] = pr_mul(cur, fC);
+                H.set(3 + n, pr_mul(cur, fC));
                 fC = pr_mul(fC, m2r);
             }
-            RR[n] = pr_mul(pr_add(cur, pr_neg(prev)), fR);
+            H.set(jR + n, pr_mul(pr_add(cur, pr_neg(prev)), fR));
             fR = pr_mul(fR, m2r);
             prev = cur;
         }
@@ -362,9 +346,8 @@ __constant__ float c_inv_odd_f[16] = {1.f,      1.f / 3,  1.f / 5,  1.f / 7,  1.
                                       1.f / 13, 1.f / 15, 1.f / 17, 1.f / 19, 1.f / 21, 1.f / 23,
                                       1.f / 25, 1.f / 27, 1.f / 29, 1.f / 31};
 
-// F_0..F_nmax at T into F[0..nmax].x (FP32; Taylor offset from the FP64 T);
-// returns exp(-T).
-__device__ __forceinline__ float boys_eval_f32(const float *tab, double T, int nmax, float2 *F) {
+// F_0..F_nmax at T into entries j0..j0+nmax (FP32; Taylor offset from the FP64 T).
+__device__ __forceinline__ void boys_eval_f32(const float *tab, double T, int nmax, const HeadPair &H, int j0) {
     const float Tf = (float)T;
     const float e = expf(-Tf);
     if (T < kBoysTMax) {
@@ -374,107 +357,172 @@ __device__ __forceinline__ float boys_eval_f32(const float *tab, double T, int n
         float f = __ldg(row + kBoysTaylor - 1);
 #pragma unroll
         for (int k = kBoysTaylor - 1; k > 0; --k) f = fmaf(f, md * c_inv_int_f[k], __ldg(row + k - 1));
-        F[nmax] = make_float2(f, 0.f);
+        H.set(j0 + nmax, make_float2(f, 0.f));
         const float t2 = Tf + Tf;
         for (int n = nmax - 1; n >= 0; --n) {
             f = fmaf(t2, f, e) * c_inv_odd_f[n];
-            F[n] = make_float2(f, 0.f);
+            H.set(j0 + n, make_float2(f, 0.f));
         }
     } else {
         float f = (float)kHalfSqrtPi * rsqrtf(Tf);
         const float inv2t = 0.5f / Tf;
-        F[0] = make_float2(f, 0.f);
+        H.set(j0, make_float2(f, 0.f));
         for (int n = 0; n < nmax; ++n) {
             f = fmaf(c_odd_f[n], f, -e) * inv2t;
-            F[n + 1] = make_float2(f, 0.f);
+            H.set(j0 + n + 1, make_float2(f, 0.f));
         }
     }
-    return e;
 }
 
-template <bool GAUGE>
+// Coulomb kernel only (the r12 tensor of the gauge kernel takes differences
+// F_n - F_{n-1} that lose digits in FP32, measured 13 times the Coulomb kernel's
+// error ratio: its plain-FP32 tiles take the high parts of the FP32-pair header).
 __device__ __forceinline__ void quartet_header_f32(const double *boys, const PrimPairDev *pa, const PrimPairDev *pc,
-                                                   int L, double *hd) {
-    float2 *h2 = reinterpret_cast<float2 *>(hd);
-    const float *boysf = boys_tables(boys).f32;
+                                                   int L, const HeadPair &H) {
     const double p = pa->p, q = pc->p, s = p + q;
-    const double X = pa->P[0] - pc->P[0], Y = pa->P[1] - pc->P[1], Z = pa->P[2] - pc->P[2];
+    const double X = pc->P[0] - pa->P[0], Y = pc->P[1] - pa->P[1], Z = pc->P[2] - pa->P[2];
     const double inv_s = 1.0 / s;
     const double rho = p * q * inv_s;
     const double T = rho * fma(X, X, fma(Y, Y, Z * Z));
-    h2[0] = make_float2((float)X, 0.f);
-    h2[1] = make_float2((float)Y, 0.f);
-    h2[2] = make_float2((float)Z, 0.f);
-    const float sf = (float)s;
-    const float d = (float)pa->inv_p * (float)pc->inv_p * (float)inv_s * sqrtf(sf);    // 1 / (p q sqrt(p + q))
+    H.set(0, make_float2((float)X, 0.f));
+    H.set(1, make_float2((float)Y, 0.f));
+    H.set(2, make_float2((float)Z, 0.f));
+    const float d = (float)pa->inv_p * (float)pc->inv_p * (float)inv_s * sqrtf((float)s);    // 1 / (p q sqrt(p + q))
     const float m2r = (float)(-2.0 * rho);
     float fC = (float)kTwoPi52 * d;
-    if (!GAUGE) {
-        float2 *F = h2 + 3;
-        boys_eval_f32(boysf, T, L, F);
-        for (int n = 0; n <= L; ++n) {
-            F[n].x *= fC;
-            fC *= m2r;
-        }
-    } else {
-        float2 *RC = h2 + 3, *RR = h2 + 4 + L;
-        const float e = boys_eval_f32(boysf, T, L + 2, RR);
-        const float Tf = (float)T;
-        float fR = (float)kPi52 * sf * sqrtf(sf) * d * d;
-        float prev = -fmaf(Tf + Tf, RR[0].x, e);                 // F_{-1}
-        for (int n = 0; n <= L + 2; ++n) {
-            const float cur = RR[n].x;
-            if (n <= L) {
-                RC[n] = make_float2(cur * fC, 0.f);
-                fC *= m2r;
-            }
-            RR[n] = make_float2((cur - prev) * fR, 0.f);
-            fR *= m2r;
-            prev = cur;
-        }
+    boys_eval_f32(boys_tables(boys).f32, T, L, H, 3);
+    for (int n = 0; n <= L; ++n) {
+        H.set(3 + n, make_float2(H.get(3 + n).x * fC, 0.f));
+        fC *= m2r;
     }
 }
 
+// ---------------------------------------------------------------------------
+// Packed FP32: one instruction works on two floats, (lower, upper) in 64 bits.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// a - b (one rounding: -1 * b is exact)
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, 0xBF800000BF800000ull, a); }
+__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+    return (f32x2)__float_as_uint(x) | ((f32x2)__float_as_uint(y) << 32);
+}
+__device__ __forceinline__ float lower2(f32x2 a) { return __uint_as_float((unsigned)a); }
+__device__ __forceinline__ float upper2(f32x2 a) { return __uint_as_float((unsigned)(a >> 32)); }
+
+// (ah, al) += a * b in compensated FP32 pairs, two at once: exact product error of
+// the high parts plus the cross terms, then the two-sum of the high parts.
+// na = (-a.x, -a.y): the error is formed as p - a b, so no packed sum needs a
+// negated operand.
+__device__ __forceinline__ void df_madd2(ulonglong2 a, ulonglong2 na, ulonglong2 b, f32x2 &ah, f32x2 &al) {
+    const f32x2 p = mul2(a.x, b.x);
+    f32x2 pe = fma2(na.x, b.x, p);                    // -(product error)
+    pe = fma2(na.x, b.y, pe);
+    pe = fma2(na.y, b.x, pe);
+    const f32x2 t = add2(ah, p);
+    const f32x2 bv = sub2(t, ah);
+    const f32x2 err = add2(sub2(ah, sub2(t, bv)), sub2(p, bv));
+    ah = t;
+    al = add2(al, sub2(err, pe));
+}
+
+// x a + cf c in compensated FP32 pairs, renormalised, two at once (one Hermite
+// recursion step).
+__device__ __forceinline__ ulonglong2 df_rec2(ulonglong2 x, ulonglong2 a, f32x2 cf, ulonglong2 c) {
+    const f32x2 nxh = neg2(x.x), nxl = neg2(x.y), ncf = neg2(cf);
+    const f32x2 p1 = mul2(x.x, a.x);
+    f32x2 e1 = fma2(nxh, a.x, p1);
+    e1 = fma2(nxh, a.y, e1);
+    e1 = fma2(nxl, a.x, e1);
+    const f32x2 p2 = mul2(cf, c.x);
+    f32x2 e2 = fma2(ncf, c.x, p2);
+    e2 = fma2(ncf, c.y, e2);
+    const f32x2 t = add2(p1, p2);
+    const f32x2 bv = sub2(t, p1);
+    const f32x2 err = add2(sub2(p1, sub2(t, bv)), sub2(p2, bv));
+    const f32x2 lo = sub2(err, add2(e1, e2));
+    const f32x2 hi = add2(t, lo);
+    return make_ulonglong2(hi, sub2(lo, sub2(hi, t)));
+}
+
+// Arithmetic of a tile: FP64, compensated FP32 pairs, plain FP32.  Vec holds one
+// two of primitive pairs.
+enum { kF64 = 0, kDF = 1, kF32 = 2 };
+template <int A> struct Arith;
+template <> struct Arith<kF64> { typedef double2 Vec; };
+template <> struct Arith<kDF> { typedef ulonglong2 Vec; };
+template <> struct Arith<kF32> { typedef f32x2 Vec; };
+
 }  // namespace
 
-// Shared-memory plan (class maxima); plan_smem() gives its size.
+// ---------------------------------------------------------------- shared plan
+// Sizes from the class maxima.  Tables (built once per CTA) and a pool that
+// every quartet divides for itself (partition()).
 struct Plan {
-    int NC;          // 1 Coulomb, 7 gauge
-    int ach, cch;    // chunk of outer / inner function pairs
-    int nhMax;       // nherm(max Lab)
-    int LtC, LtR;    // top Hermite orders of the Coulomb and r12 tensors (LtR < 0: none)
-    int nTab;        // Hermite triples tabulated: nherm(top order)
-    int maxnpp;      // primitive pairs of a shell pair
+    int maxLab;
+    int nTab;        // Hermite triples tabulated: nherm of the top order
+    int nhm;         // nherm(maxLab)
+    int nG;          // T row triples tabulated: nherm(maxLab), gauge nherm(maxLab + 2)
+    int nLst;        // box entries of all boxes of order <= maxLab: C(maxLab + 6, 6)
     int threads;
-    long long pool;  // doubles shared by T, quartet headers and the R tensors
+    int pool;        // bytes
 };
 
 struct BlockSmem {
-    double *G, *P, *cf;
-    long long *eX, *eY;
-    int *trip, *src;
+    char *pool;
+    int2 *src;                  // recursion sources of R_h
+    int *trip;                  // Hermite triple h -> t | u << 8 | v << 16
+    int *box;                   // per box: first list entry | count << 16
+    unsigned short *hs;         // [nG][nhm]: Hermite index of the sum of two triples
+    unsigned short *r12row;     // [6][nhm]: Hermite index of h + e_I + e_J
+    unsigned char *lst;         // Hermite indices of the boxes' entries
+    int *slot;
 };
 
-size_t plan_smem(const Plan &p) {
-    return ((size_t)p.NC * p.ach * p.cch + p.pool + p.nTab + 2 * (size_t)p.maxnpp) * sizeof(double) +
-           2 * (size_t)p.nTab * sizeof(int) + 16;
+__host__ __device__ inline int up16(int n) { return (n + 15) & ~15; }
+size_t plan_tables(const Plan &p) {
+    return (size_t)up16(p.nTab * 8) + up16(p.nTab * 4) + up16(p.nhm * 4) + up16(p.nG * p.nhm * 2) +
+           up16(6 * p.nhm * 2) + up16(p.nLst) + 16;
 }
+size_t plan_smem(const Plan &p) { return plan_tables(p) + (size_t)p.pool; }
 
-__device__ inline BlockSmem carve(double *sm, const Plan &p) {
+__device__ inline BlockSmem carve(char *sm, const Plan &p) {
     BlockSmem b;
-    b.G = sm; sm += (size_t)p.NC * p.ach * p.cch;
-    b.P = sm; sm += p.pool;
-    b.cf = sm; sm += p.nTab;
-    b.eX = (long long *)sm; sm += p.maxnpp;
-    b.eY = (long long *)sm; sm += p.maxnpp;
-    b.trip = (int *)sm;
-    b.src = b.trip + p.nTab;
+    b.pool = sm; sm += p.pool;
+    b.src = (int2 *)sm; sm += up16(p.nTab * 8);
+    b.trip = (int *)sm; sm += up16(p.nTab * 4);
+    b.box = (int *)sm; sm += up16(p.nhm * 4);
+    b.hs = (unsigned short *)sm; sm += up16(p.nG * p.nhm * 2);
+    b.r12row = (unsigned short *)sm; sm += up16(6 * p.nhm * 2);
+    b.lst = (unsigned char *)sm; sm += up16(p.nLst);
+    b.slot = (int *)sm;
     return b;
 }
 
-// Hermite triple h -> packed (t, u, v); recursion sources of R_h: direction,
-// h - e_dir, h - 2 e_dir and the coefficient (component - 1) of the latter
-// (also packed into bits 22..25 of the source word for the FP32-pair path).
+// Box entries of all boxes of order < n: C(n + 5, 6).
+__host__ __device__ constexpr int box_entries_below(int n) {
+    return n * (n + 1) * (n + 2) / 6 * ((n + 3) * (n + 4) / 2) / 2 * (n + 5) / 30;
+}
+static_assert(box_entries_below(1) == 1 && box_entries_below(2) == 7 && box_entries_below(3) == 28 &&
+              box_entries_below(4) == 84 && box_entries_below(5) == 210 && box_entries_below(6) == 462 &&
+              box_entries_below(7) == 924, "C(n + 5, 6)");
+
+// Recursion source of R_h: direction, h - e_dir, h - 2 e_dir (packed) and the
+// coefficient (component - 1) of the latter as a float.
 __device__ void build_tables(const Plan &p, BlockSmem &b) {
     for (int h = threadIdx.x; h < p.nTab; h += blockDim.x) {
         int t, u, v;
@@ -490,598 +538,450 @@ __device__ void build_tables(const Plan &p, BlockSmem &b) {
             i1 = hidx(t - dt, u - du, v - dv);
             if (c >= 2) i2 = hidx(t - 2 * dt, u - 2 * du, v - 2 * dv);
         }
-        b.src[h] = dir | (i1 << 2) | (i2 << 12) | ((c >= 2 ? c - 1 : 0) << 22);
-        b.cf[h] = c >= 2 ? (double)(c - 1) : 0.0;
+        b.src[h] = make_int2(dir | (i1 << 2) | (i2 << 12), __float_as_int(c >= 2 ? (float)(c - 1) : 0.f));
+        if (h < p.nhm) {
+            // this box's list: the boxes before it, of lower order and of its own
+            int at = box_entries_below(t + u + v);
+            for (int q = nherm(t + u + v - 1); q < h; ++q) {
+                int a, bb, c2;
+                htrip_d(q, a, bb, c2);
+                at += box_count(a, bb, c2);
+            }
+            b.box[h] = at | (box_count(t, u, v) << 16);
+            for (int x = 0; x <= t; ++x)
+                for (int y = 0; y <= u; ++y)
+                    for (int z = 0; z <= v; ++z) b.lst[at++] = (unsigned char)hidx(x, y, z);
+            b.r12row[h] = (unsigned short)hidx(t + 2, u, v);
+            b.r12row[p.nhm + h] = (unsigned short)hidx(t + 1, u + 1, v);
+            b.r12row[2 * p.nhm + h] = (unsigned short)hidx(t + 1, u, v + 1);
+            b.r12row[3 * p.nhm + h] = (unsigned short)hidx(t, u + 2, v);
+            b.r12row[4 * p.nhm + h] = (unsigned short)hidx(t, u + 1, v + 1);
+            b.r12row[5 * p.nhm + h] = (unsigned short)hidx(t, u, v + 2);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < p.nG * p.nhm; i += blockDim.x) {
+        const int g = b.trip[i / p.nhm], h = b.trip[i % p.nhm];
+        b.hs[i] = (unsigned short)hidx((g & 255) + (h & 255), ((g >> 8) & 255) + ((h >> 8) & 255),
+                                       (g >> 16) + (h >> 16));
     }
     __syncthreads();
 }
 
-// Rows of T per outer primitive pair: the Hermite triples h of X for the
-// Coulomb tensor and, for the gauge kernel, the triples g with 2 <= |g| <= Lx+2
-// of the r12 tensor (g = h + e_I + e_J covers all six second derivatives).
-__host__ __device__ inline int t_rows(int Lx, bool gauge) { return nherm(Lx) + (gauge ? nherm(Lx + 2) - 4 : 0); }
-
-// FP64 multiply-adds of the contraction of a shell quartet with X outer: the
-// ket pass (T rows x inner function pairs x inner Hermite terms per primitive
-// quartet) plus the bra pass (components x function pairs x outer Hermite
-// terms per outer primitive pair).
-__host__ __device__ inline double orient_cost(const PairDev &X, const PairDev &Y, bool gauge) {
-    const double nhx = nherm(X.Lab), nhy = nherm(Y.Lab);
-    return (double)X.npp * Y.npp * t_rows(X.Lab, gauge) * Y.nfp * nhy +
-           (double)X.npp * X.nfp * Y.nfp * nhx * (gauge ? 7 : 1);
+// Sizes of a quartet (X outer, Y inner).  Order-0 and even-order tensors need
+// nherm(L) entries each, odd orders nherm(L - 1); the r12 tensor has top order L + 2.
+__host__ __device__ inline int odd_len(int Ltop) { return Ltop >= 1 ? nherm(Ltop - 1) : 0; }
+struct Shape {
+    int nE, nO, hs, nT, NC;
+};
+__host__ __device__ inline Shape quartet_shape(int Lx, int Ly, bool gauge) {
+    const int L = Lx + Ly;
+    return {nherm(L) + (gauge ? nherm(L + 2) : 0), odd_len(L) + (gauge ? odd_len(L + 2) : 0), header_len(L, gauge),
+            t_rows(Lx, gauge), gauge ? 7 : 1};
 }
 
-// acc += sign * sum_{h' of orders n0, n0+2, ...} sum_kl R_{kl}[h + h'] E^{kl}[h'][y],
-// sign = -1 (NEG) for the odd orders.
-template <bool NEG>
-__device__ __forceinline__ void ket_orders(int n0, int Ly, int tx, int ux, int vx, const int *trip,
-                                           const double *Rq, int nr, const double *ey, int nfpY,
-                                           const long long *eoff, int nk, double &acc) {
-    for (int n = n0; n <= Ly; n += 2) {
-        const int hb = n ? nherm(n - 1) : 0, he = nherm(n);
-        for (int hp = hb; hp < he; ++hp) {
-            const int tq = trip[hp];
-            const int T0 = tx + (tq & 255), U0 = ux + ((tq >> 8) & 255), V0 = vx + (tq >> 16);
-            const int s = T0 + U0 + V0, w = U0 + V0;
-            const int i0 = s * (s + 1) * (s + 2) / 6 + w * (w + 1) / 2 + V0;
-            const double *e = ey + (size_t)hp * nfpY;
-            double a = acc;
-            for (int kl = 0; kl < nk; ++kl) {
-                const double r = Rq[kl * nr + i0];
-                const double ev = __ldg(e + eoff[kl]);
-                a = NEG ? fma(-r, ev, a) : fma(r, ev, a);
-            }
-            acc = a;
-        }
+// How a quartet is cut to fit the pool: [headers][even tensors][T | odd tensors][G].
+// T of a group is written after the group's recursion has read the odd tensors
+// and read before the next group writes them, so the two share their bytes
+// unless T has to last over several runs of inner primitive pairs (nkc < nk2).
+struct Cut {
+    int xch, ych;        // function pairs of X, Y at a time
+    int nkc;             // twos of inner primitive pairs at a time
+    int nij, nijH;       // outer primitive pairs per group, per header pass
+};
+__host__ __device__ inline int cut_bytes(const Shape &s, int nk2, int xch, int ych, int nkc, int nij, int nijH) {
+    const int yp = (ych + 1) & ~1;
+    const int t = nij * s.nT * yp * 8, o = s.nO * nij * nkc * 16;
+    return s.hs * nijH * nkc * 16 + s.nE * nij * nkc * 16 + (nkc < nk2 ? t + o : (t > o ? t : o)) +
+           s.NC * xch * yp * 8;
+}
+// The cut depends on the quartet and the pool only; it decides no rounding
+// unless the inner primitive pairs are cut (contractions of dozens of
+// primitives), which a larger pool of another class's maxima does not change as
+// long as the tensors of one outer primitive pair take half the pool at most.
+__host__ __device__ inline Cut partition(const Shape &s, int nppx, int nfpx, int nk2y, int nfpy, int nchy, int pool,
+                                         int threads) {
+    Cut c;
+    c.xch = nfpx;
+    c.ych = nfpy;
+    c.nkc = nk2y > 1 ? nk2y : 1;
+    const int nk2 = c.nkc;
+    while (c.nkc > 1 && (s.hs + s.nE + s.nO) * 16 > pool / 2 / c.nkc) c.nkc = (c.nkc + 1) / 2;
+    while (cut_bytes(s, nk2, c.xch, c.ych, c.nkc, 1, 1) > pool) {
+        if (c.ych > 4) c.ych = (c.ych + 1) / 2;
+        else if (c.xch > 4) c.xch = (c.xch + 1) / 2;
+        else if (c.nkc > 1) c.nkc = (c.nkc + 1) / 2;
+        else if (c.ych > 2) c.ych = 2;
+        else if (c.xch > 1) c.xch = (c.xch + 1) / 2;
+        else break;
     }
-}
-
-// The same in compensated FP32 pairs (R, E and the accumulator as hi + lo).
-template <bool NEG>
-__device__ __forceinline__ void ket_orders_df(int n0, int Ly, int tx, int ux, int vx, const int *trip,
-                                              const float2 *Rq, int nr, const float2 *ey, int nfpY,
-                                              long long sE, int nk, float &ah, float &al) {
-    for (int n = n0; n <= Ly; n += 2) {
-        const int hb = n ? nherm(n - 1) : 0, he = nherm(n);
-        for (int hp = hb; hp < he; ++hp) {
-            const int tq = trip[hp];
-            const int T0 = tx + (tq & 255), U0 = ux + ((tq >> 8) & 255), V0 = vx + (tq >> 16);
-            const int s = T0 + U0 + V0, w = U0 + V0;
-            const int i0 = s * (s + 1) * (s + 2) / 6 + w * (w + 1) / 2 + V0;
-            const float2 *e = ey + (size_t)hp * nfpY;
-            const float2 *rk = Rq + i0;
-#pragma unroll 4
-            for (int kl = 0; kl < nk; ++kl) {
-                df_madd<NEG>(*rk, __ldg(e), ah, al);
-                rk += nr;
-                e += sE;
-            }
-        }
+    // outer primitive pairs per group: enough ket-pass items for four rounds of the CTA
+    int nij = (4 * threads + s.nT * nchy - 1) / (s.nT * nchy);
+    if (nij > nppx) nij = nppx;
+    if (nij < 1) nij = 1;
+    while (nij > 1 && cut_bytes(s, nk2, c.xch, c.ych, c.nkc, nij, nij) > pool) --nij;
+    const int groups = nppx > 0 ? (nppx + nij - 1) / nij : 1;
+    c.nij = nppx > 0 ? (nppx + groups - 1) / groups : 1;
+    c.nijH = c.nij;
+    if (c.nkc == nk2) {
+        const int rest = pool - cut_bytes(s, nk2, c.xch, c.ych, c.nkc, c.nij, 0);
+        int h = rest / (s.hs * c.nkc * 16);
+        if (h > nppx) h = nppx;
+        if (h < nppx) h = h / c.nij * c.nij;
+        if (h > c.nij) c.nijH = h;
     }
+    return c;
 }
 
-// The same in plain FP32 (the high parts of R and E): quartets whose error
-// bound the host has admitted to the FP32 budget.
-template <bool NEG>
-__device__ __forceinline__ void ket_orders_f32(int n0, int Ly, int tx, int ux, int vx, const int *trip,
-                                               const float2 *Rq, int nr, const float *ey, int nfpY,
-                                               long long sE, int nk, float &acc) {
-    for (int n = n0; n <= Ly; n += 2) {
-        const int hb = n ? nherm(n - 1) : 0, he = nherm(n);
-        for (int hp = hb; hp < he; ++hp) {
-            const int tq = trip[hp];
-            const int T0 = tx + (tq & 255), U0 = ux + ((tq >> 8) & 255), V0 = vx + (tq >> 16);
-            const int s = T0 + U0 + V0, w = U0 + V0;
-            const int i0 = s * (s + 1) * (s + 2) / 6 + w * (w + 1) / 2 + V0;
-            const float *e = ey + (size_t)hp * nfpY;
-            const float *rk = reinterpret_cast<const float *>(Rq + i0);
-            float a = acc;
-#pragma unroll 4
-            for (int kl = 0; kl < nk; ++kl) {
-                a = NEG ? fmaf(-*rk, __ldg(e), a) : fmaf(*rk, __ldg(e), a);
-                rk += 2 * nr;
-                e += sE;
-            }
-            acc = a;
-        }
-    }
-}
-
-// The same for two T rows (Hermite indices a, b) of one inner function pair:
-// each E value is loaded once for both rows (the FP32 tiles wait on these loads).
-template <bool NEG>
-__device__ __forceinline__ void ket_orders_f32x2(int n0, int Ly, int txa, int uxa, int vxa, int txb, int uxb,
-                                                 int vxb, const int *trip, const float2 *Rq, int nr,
-                                                 const float *ey, int nfpY, long long sE, int nk, float &acca,
-                                                 float &accb) {
-    for (int n = n0; n <= Ly; n += 2) {
-        const int hb = n ? nherm(n - 1) : 0, he = nherm(n);
-        for (int hp = hb; hp < he; ++hp) {
-            const int tq = trip[hp];
-            const int tp = tq & 255, up = (tq >> 8) & 255, vp = tq >> 16;
-            const int Ta = txa + tp, Ua = uxa + up, Va = vxa + vp, sa = Ta + Ua + Va, wa = Ua + Va;
-            const int Tb = txb + tp, Ub = uxb + up, Vb = vxb + vp, sb = Tb + Ub + Vb, wb = Ub + Vb;
-            const int ia = sa * (sa + 1) * (sa + 2) / 6 + wa * (wa + 1) / 2 + Va;
-            const int ib = sb * (sb + 1) * (sb + 2) / 6 + wb * (wb + 1) / 2 + Vb;
-            const float *e = ey + (size_t)hp * nfpY;
-            const float *ra = reinterpret_cast<const float *>(Rq + ia);
-            const float *rb = reinterpret_cast<const float *>(Rq + ib);
-            float a = acca, b2 = accb;
-#pragma unroll 4
-            for (int kl = 0; kl < nk; ++kl) {
-                const float ev = __ldg(e);
-                a = NEG ? fmaf(-*ra, ev, a) : fmaf(*ra, ev, a);
-                b2 = NEG ? fmaf(-*rb, ev, b2) : fmaf(*rb, ev, b2);
-                ra += 2 * nr;
-                rb += 2 * nr;
-                e += sE;
-            }
-            acca = a;
-            accb = b2;
-        }
-    }
-}
-
-// The same for two adjacent inner function pairs y, y + 1 at once (the second
-// when has1): R and the primitive-pair offsets are loaded once for both, and
-// the two accumulator chains are independent (gauge kernel, whose larger
-// plan leaves registers for the second chain).
-template <bool NEG>
-__device__ __forceinline__ void ket_orders_df2(int n0, int Ly, int tx, int ux, int vx, const int *trip,
-                                               const float2 *Rq, int nr, const float2 *ey, int nfpY,
-                                               long long sE, int nk, bool has1, float &ah0, float &al0,
-                                               float &ah1, float &al1) {
-    for (int n = n0; n <= Ly; n += 2) {
-        const int hb = n ? nherm(n - 1) : 0, he = nherm(n);
-        for (int hp = hb; hp < he; ++hp) {
-            const int tq = trip[hp];
-            const int T0 = tx + (tq & 255), U0 = ux + ((tq >> 8) & 255), V0 = vx + (tq >> 16);
-            const int s = T0 + U0 + V0, w = U0 + V0;
-            const int i0 = s * (s + 1) * (s + 2) / 6 + w * (w + 1) / 2 + V0;
-            const float2 *e = ey + (size_t)hp * nfpY;
-            const float2 *rk = Rq + i0;
-            if (has1) {
-#pragma unroll 2
-                for (int kl = 0; kl < nk; ++kl) {
-                    const float2 r = *rk;
-                    const float2 e0 = __ldg(e), e1 = __ldg(e + 1);
-                    df_madd<NEG>(r, e0, ah0, al0);
-                    df_madd<NEG>(r, e1, ah1, al1);
-                    rk += nr;
-                    e += sE;
-                }
-            } else {
-                for (int kl = 0; kl < nk; ++kl) {
-                    df_madd<NEG>(*rk, __ldg(e), ah0, al0);
-                    rk += nr;
-                    e += sE;
-                }
-            }
-        }
-    }
-}
-
-// Register tile of the ket pass: TH rows of T (Hermite rows of the outer pair,
-// each with its own R tensor base and stride: the Coulomb tensor, or for the
-// gauge kernel the r12 tensor) times TY adjacent inner function pairs, for one
-// outer primitive pair:
-//   acc[r][c] += sum_{kl} sum_{h'} (-1)^{|h'|} R_kl[h_r + h'] E^kl[h'][y_c].
-// Each E value is loaded once for the TH rows and each R value once for the TY
-// columns, and the TH x TY accumulators are independent chains.  DF: compensated
-// FP32 pairs (R, E and the accumulators as hi + lo); else plain FP32 (the high
-// parts).  Rows and columns past the chunk are clamped by the caller (their sums
-// are discarded).
-template <int TH, int TY, bool DF>
-struct KetTile {
-    float ah[TH][TY], al[TH][TY];
+// Device tables of the shell pairs.
+struct PairTables {
+    const PrimPairDev *pp;
+    const double2 *E;
+    const float4 *E2;
+    const float2 *E1;
+    const FuncPair *fp;
+    const PairChunk *ch;
+    const double *boys;
 };
 
-template <int TH, int TY, bool DF, bool NEG>
-__device__ __forceinline__ void ket_tile_orders(int n0, int Ly, const int (&rs)[TH], const int (&rw)[TH],
-                                                const int (&rv)[TH], const float2 *const (&Rb)[TH],
-                                                const int (&nr)[TH], const int *trip, const void *eyv, int nfpY,
-                                                long long sE, int nk, const int (&yo)[TY], KetTile<TH, TY, DF> &t) {
-    for (int n = n0; n <= Ly; n += 2) {
-        const int hb = n ? nherm(n - 1) : 0, he = nherm(n);
-        for (int hp = hb; hp < he; ++hp) {
-            const int tq = trip[hp];
-            const int up = (tq >> 8) & 255, vp = tq >> 16, wp = up + vp, sp = (tq & 255) + wp;
-            const float2 *rp[TH];
+template <int A> __device__ __forceinline__ const typename Arith<A>::Vec *e_entries(const PairTables &t);
+template <> __device__ __forceinline__ const double2 *e_entries<kF64>(const PairTables &t) { return t.E; }
+template <> __device__ __forceinline__ const ulonglong2 *e_entries<kDF>(const PairTables &t) {
+    return reinterpret_cast<const ulonglong2 *>(t.E2);
+}
+template <> __device__ __forceinline__ const f32x2 *e_entries<kF32>(const PairTables &t) {
+    return reinterpret_cast<const f32x2 *>(t.E1);
+}
+
+// One item of the ket pass: T rows are spread over the lanes, a thread sums one
+// row for M function pairs of one box,
+//   acc[m] = sum_{j in box} sum_kl R~_kl[h + h_j] E^kl_m[j].
+// Each R vector loaded serves the M function pairs; the E vectors are the same
+// for all lanes on the same chunk.  NK > 0: that many twos of primitive pairs,
+// unrolled (5 = two contractions of three primitives), else nk of them.
+template <int A, int M, int NK>
+__device__ __forceinline__ void ket_item(const typename Arith<A>::Vec *R, int Q2, const unsigned short *hs,
+                                         const unsigned char *lst, int cnt, const typename Arith<A>::Vec *E,
+                                         long long estride, int nk2, int nk, bool odd, float2 (&out)[M],
+                                         double (&outd)[M]) {
+    typedef typename Arith<A>::Vec Vec;
+    const int n = NK > 0 ? NK : nk;
+    int o = (int)hs[lst[0]] * Q2;
+    if constexpr (A == kF64) {
+        double a0[M], a1[M];
 #pragma unroll
-            for (int r = 0; r < TH; ++r) {
-                const int s = rs[r] + sp, w = rw[r] + wp;
-                rp[r] = Rb[r] + (s * (s + 1) * (s + 2) / 6 + w * (w + 1) / 2 + rv[r] + vp);
-            }
-            if constexpr (DF) {
-                const float2 *e = reinterpret_cast<const float2 *>(eyv) + (size_t)hp * nfpY;
-#pragma unroll 2
-                for (int kl = 0; kl < nk; ++kl) {
-                    float2 ev[TY];
+        for (int m = 0; m < M; ++m) a0[m] = a1[m] = 0.0;
+        const int full = odd ? n - 1 : n;               // the last two holds one primitive pair
+        for (int j = 0; j < cnt; ++j) {
+            const Vec *r = R + o;
+            if (j + 1 < cnt) o = (int)hs[lst[j + 1]] * Q2;
+#pragma unroll 4
+            for (int p = 0; p < full; ++p) {
+                const Vec rv = r[p];
 #pragma unroll
-                    for (int c = 0; c < TY; ++c) ev[c] = __ldg(e + yo[c]);
-#pragma unroll
-                    for (int r = 0; r < TH; ++r) {
-                        const float2 rvv = *rp[r];
-                        rp[r] += nr[r];
-#pragma unroll
-                        for (int c = 0; c < TY; ++c) df_madd<NEG>(rvv, ev[c], t.ah[r][c], t.al[r][c]);
-                    }
-                    e += sE;
-                }
-            } else {
-                const float *e = reinterpret_cast<const float *>(eyv) + (size_t)hp * nfpY;
-#pragma unroll 3
-                for (int kl = 0; kl < nk; ++kl) {
-                    float ev[TY];
-#pragma unroll
-                    for (int c = 0; c < TY; ++c) ev[c] = __ldg(e + yo[c]);
-#pragma unroll
-                    for (int r = 0; r < TH; ++r) {
-                        const float rvv = rp[r]->x;
-                        rp[r] += nr[r];
-#pragma unroll
-                        for (int c = 0; c < TY; ++c)
-                            t.ah[r][c] = NEG ? fmaf(-rvv, ev[c], t.ah[r][c]) : fmaf(rvv, ev[c], t.ah[r][c]);
-                    }
-                    e += sE;
+                for (int m = 0; m < M; ++m) {
+                    const Vec ev = __ldg(E + m * estride + p);
+                    a0[m] = fma(rv.x, ev.x, a0[m]);
+                    a1[m] = fma(rv.y, ev.y, a1[m]);
                 }
             }
+            if (odd) {
+                const double rv = r[full].x;
+#pragma unroll
+                for (int m = 0; m < M; ++m)
+                    a0[m] = fma(rv, __ldg(reinterpret_cast<const double *>(E + m * estride + full)), a0[m]);
+            }
+            E += nk2;
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m) outd[m] = a0[m] + a1[m];
+    } else if constexpr (A == kDF) {
+        f32x2 ah[M], al[M];
+#pragma unroll
+        for (int m = 0; m < M; ++m) ah[m] = al[m] = 0;
+        for (int j = 0; j < cnt; ++j) {
+            const Vec *r = R + o;
+            if (j + 1 < cnt) o = (int)hs[lst[j + 1]] * Q2;
+#pragma unroll
+            for (int p = 0; p < (NK > 0 ? NK : 1); ++p) {
+                for (int q = p; q < n; q += (NK > 0 ? n : 1)) {
+                    const Vec rv = r[q];
+                    const Vec nr = make_ulonglong2(neg2(rv.x), neg2(rv.y));
+#pragma unroll
+                    for (int m = 0; m < M; ++m) df_madd2(rv, nr, __ldg(E + m * estride + q), ah[m], al[m]);
+                }
+            }
+            E += nk2;
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+            out[m] = pr_add(make_float2(lower2(ah[m]), lower2(al[m])), make_float2(upper2(ah[m]), upper2(al[m])));
+    } else {
+        f32x2 a[M];
+#pragma unroll
+        for (int m = 0; m < M; ++m) a[m] = 0;
+        for (int j = 0; j < cnt; ++j) {
+            const Vec *r = R + o;
+            if (j + 1 < cnt) o = (int)hs[lst[j + 1]] * Q2;
+#pragma unroll
+            for (int p = 0; p < (NK > 0 ? NK : 1); ++p) {
+                for (int q = p; q < n; q += (NK > 0 ? n : 1)) {
+                    const Vec rv = r[q];
+#pragma unroll
+                    for (int m = 0; m < M; ++m) a[m] = fma2(rv, __ldg(E + m * estride + q), a[m]);
+                }
+            }
+            E += nk2;
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m) out[m] = make_float2(lower2(a[m]) + upper2(a[m]), 0.f);
+    }
+}
+
+template <int A, int M>
+__device__ __forceinline__ void ket_store(const typename Arith<A>::Vec *R, int Q2, const unsigned short *hs,
+                                          const unsigned char *lst, int cnt, const typename Arith<A>::Vec *E,
+                                          long long estride, int nk2, int nk, bool odd, bool neg, bool add, char *T,
+                                          int at, int plane) {
+    float2 s[M];
+    double sd[M];
+    if (A != kF64 && nk == 5) ket_item<A, M, 5>(R, Q2, hs, lst, cnt, E, estride, nk2, nk, odd, s, sd);
+    else ket_item<A, M, 0>(R, Q2, hs, lst, cnt, E, estride, nk2, nk, odd, s, sd);
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        if constexpr (A == kF64) {
+            double *t = reinterpret_cast<double *>(T) + at + m;
+            const double v = neg ? -sd[m] : sd[m];
+            *t = add ? *t + v : v;
+        } else {
+            float *t = reinterpret_cast<float *>(T) + at + m;
+            float2 v = neg ? pr_neg(s[m]) : s[m];
+            if (add) v = pr_add(make_float2(t[0], A == kDF ? t[plane] : 0.f), v);
+            t[0] = v.x;
+            if (A == kDF) t[plane] = v.y;
         }
     }
 }
 
-// The tiled ket pass over every (outer primitive pair, row block, column
-// block) of a chunk: T[ij][hh][y] (float2 slots) += the sums above.  Rows hh <
-// nhx use the Coulomb tensor RC (Hermite index hh); for the gauge kernel rows
-// hh >= nhx use the r12 tensor RR (Hermite index hh - nhx + 4).
-template <int TH, int TY, bool DF, bool GAUGE>
-__device__ __forceinline__ void ket_pass_tiled(int nij, int nT, int nhx, int ych, int Ly, const int *trip,
-                                               float2 *T, int tsz, const float2 *RC, int nrC, const float2 *RR,
-                                               int nrR, int nk, const void *ey0, int nfpY, long long sE) {
-    const int nHB = (nT + TH - 1) / TH, nYB = (ych + TY - 1) / TY;
-    for (int it = threadIdx.x; it < nij * nHB * nYB; it += blockDim.x) {
-        const int ijl = it / (nHB * nYB);
-        const int rem = it - ijl * nHB * nYB;
-        const int hb = rem / nYB, yb = rem - hb * nYB;
-        const int h0 = hb * TH, y0 = yb * TY;
-        int rs[TH], rw[TH], rv[TH], nr[TH], hh[TH];
-        const float2 *Rb[TH];
-#pragma unroll
-        for (int r = 0; r < TH; ++r) {
-            hh[r] = min(h0 + r, nT - 1);
-            const bool r12 = GAUGE && hh[r] >= nhx;
-            const int tr = trip[r12 ? hh[r] - nhx + 4 : hh[r]];
-            const int u = (tr >> 8) & 255, v = tr >> 16;
-            rv[r] = v;
-            rw[r] = u + v;
-            rs[r] = (tr & 255) + u + v;
-            nr[r] = r12 ? nrR : nrC;
-            Rb[r] = r12 ? RR + (size_t)ijl * nk * nrR : RC + (size_t)ijl * nk * nrC;
-        }
-        int yo[TY];
-#pragma unroll
-        for (int c = 0; c < TY; ++c) yo[c] = min(y0 + c, ych - 1) - y0;
-        KetTile<TH, TY, DF> t;
-        float2 *Tq = T + (size_t)ijl * tsz + y0;
-#pragma unroll
-        for (int r = 0; r < TH; ++r)
-#pragma unroll
-            for (int c = 0; c < TY; ++c) {
-                const float2 v = Tq[(size_t)hh[r] * ych + yo[c]];
-                t.ah[r][c] = v.x;
-                t.al[r][c] = DF ? v.y : 0.f;
-            }
-        const void *ey = DF ? (const void *)(reinterpret_cast<const float2 *>(ey0) + y0)
-                            : (const void *)(reinterpret_cast<const float *>(ey0) + y0);
-        ket_tile_orders<TH, TY, DF, false>(0, Ly, rs, rw, rv, Rb, nr, trip, ey, nfpY, sE, nk, yo, t);
-        ket_tile_orders<TH, TY, DF, true>(1, Ly, rs, rw, rv, Rb, nr, trip, ey, nfpY, sE, nk, yo, t);
-#pragma unroll
-        for (int r = 0; r < TH; ++r)
-#pragma unroll
-            for (int c = 0; c < TY; ++c)
-                if (h0 + r < nT && y0 + c < ych) Tq[(size_t)(h0 + r) * ych + c] = make_float2(t.ah[r][c], DF ? t.al[r][c] : 0.f);
-    }
-}
-
-// One chunk (x in [x0,x1) of X, y in [y0,y1) of Y) of the block (X|Y);
-// results in b.G[comp][x][y].  NC = 1 (Coulomb) or 7 (gauge: [0] Coulomb,
-// [1..6] (xy|d_I d_J r|zw) for IJ = xx,xy,xz,yy,yz,zz).
-template <bool GAUGE, bool DF, bool F32 = false>
-__device__ void block_chunk(const PrimPairDev *pp, const double *E, const float2 *E2, const float *E1,
-                            const double *boys,
-                            const PairDev &X, const PairDev &Y, int x0, int x1, int y0, int y1, const Plan &pl,
-                            BlockSmem &b) {
+// The block (X|Y), chunk by chunk; emit(x0, xch, y0, ych, value) is called by all
+// threads once the chunk's results stand in shared memory, value(c, x, y) being
+// component c of function pairs x, y (sorted order, relative to the chunk).
+// Components: 0 Coulomb; gauge kernel 1..6: (xy|d_I d_J r|zw), IJ = xx, xy, xz, yy, yz, zz.
+template <bool GAUGE, int A, class Emit>
+__device__ void quartet_block(const PairTables &tb, const PairDev &X, const PairDev &Y, const Plan &pl, BlockSmem &b,
+                              Emit emit) {
+    typedef typename Arith<A>::Vec Vec;
+    typedef typename Arith<A == kF64 ? kF64 : kDF>::Vec HVec;      // headers: FP64 or pairs
     constexpr int NC = GAUGE ? 7 : 1;
     const int tid = threadIdx.x, nt = blockDim.x;
-    const int Lx = X.Lab, Ly = Y.Lab;
+    const int Lx = X.Lab, Ly = Y.Lab, L = Lx + Ly, Lr = L + 2, Ltop = GAUGE ? Lr : L;
     const int nhx = nherm(Lx);
-    const int L = Lx + Ly, Lr = L + 2, Ltop = GAUGE ? Lr : L;
-    const int nrC = nherm(L), nrR = GAUGE ? nherm(Lr) : 0;
-    const int hs = header_len(L, GAUGE), perq = quartet_len(L, GAUGE);
-    const int xch = x1 - x0, ych = y1 - y0;
-    const int nT = t_rows(Lx, GAUGE);                   // T rows per outer primitive pair
-    // the E matrices of a pair's primitive pairs are stored back to back,
-    // nherm(L) x nfp each: inner primitive kl starts kl sE past the first (the
-    // compensated-FP32 ket pass walks them by this stride)
-    const long long sE = (long long)Y.nfp * nherm(Ly);
-    const int tsz = nT * ych;                           // T doubles per outer primitive pair
+    const Shape sh = quartet_shape(Lx, Ly, GAUGE);
+    const Cut c = partition(sh, X.npp, X.nfp, Y.nk2, Y.nfp, Y.nch, pl.pool, nt);
+    const int nE_C = nherm(L), nO_C = odd_len(L);       // entries before the r12 tensor
+    const FuncPair *fx = tb.fp + X.fpoff;
+    const PairChunk *cy = tb.ch + Y.choff;
+    const Vec *EX = e_entries<A>(tb) + X.eoff, *EY = e_entries<A>(tb) + Y.eoff;
+    const bool lastodd = Y.npp & 1;
 
-    // primitive grouping: nij outer pairs x nkl inner pairs at a time
-    int nijMax, nkl;
-    if ((long long)Y.npp * perq + tsz <= pl.pool) {
-        nkl = Y.npp;
-        nijMax = (int)min((long long)X.npp, pl.pool / ((long long)Y.npp * perq + tsz));
-    } else {
-        nkl = (int)((pl.pool - tsz) / perq);
-        nijMax = 1;
-    }
-    nijMax = max(nijMax, 1);
-    nkl = max(nkl, 1);
-    double *T = b.P;
-    double *H = T + (size_t)nijMax * tsz;
-    const int nqMax = nijMax * nkl;
-    // order-0 (and even-order) buffers RC, RR [nqMax][nrC | nrR]; odd-order buffers RC1, RR1
-    const int nrC1 = odd_len(L), nrR1 = GAUGE ? odd_len(Lr) : 0;
-    double *RC = H + (size_t)nqMax * hs;
-    double *RC1 = RC + (size_t)nqMax * nrC;
-    double *RR = RC1 + (size_t)nqMax * nrC1;
-    double *RR1 = RR + (size_t)nqMax * nrR;
+    HVec *H = reinterpret_cast<HVec *>(b.pool);
+    Vec *Re = reinterpret_cast<Vec *>(b.pool + (size_t)sh.hs * c.nijH * c.nkc * 16);
+    char *U = reinterpret_cast<char *>(Re) + (size_t)sh.nE * c.nij * c.nkc * 16;
+    const bool runs = c.nkc < Y.nk2;
+    Vec *Ro = reinterpret_cast<Vec *>(U);
+    const int ypmax = (c.ych + 1) & ~1;
+    const int tbytes = c.nij * sh.nT * ypmax * 8, obytes = sh.nO * c.nij * c.nkc * 16;
+    char *T = runs ? U + obytes : U;
+    char *G = U + (runs ? tbytes + obytes : max(tbytes, obytes));
 
-    for (int i = tid; i < X.npp; i += nt) b.eX[i] = pp[X.ppoff + i].eoff;
-    for (int i = tid; i < Y.npp; i += nt) b.eY[i] = pp[Y.ppoff + i].eoff;
-    for (int i = tid; i < NC * xch * ych; i += nt) b.G[i] = 0.0;
-    __syncthreads();
-
-    for (int i0 = 0; i0 < X.npp; i0 += nijMax) {
-        const int nij = min(nijMax, X.npp - i0);
-        for (int i = tid; i < nij * tsz; i += nt) T[i] = 0.0;
-        for (int k0 = 0; k0 < Y.npp; k0 += nkl) {
-            const int nk = min(nkl, Y.npp - k0);
-            const int nq = nij * nk;
-            // Boys values, prefactors and X_PQ of every primitive quartet of the group
-            for (int q = tid; q < nq; q += nt) {
-                const int ijl = q / nk, kl = q - ijl * nk;
-                // plain-FP32 quartets of the Coulomb kernel: FP32 header; those of
-                // the gauge kernel take the FP32-pair header (its r12 tensor takes
-                // differences F_n - F_{n-1} that lose digits in FP32: measured 13x
-                // the Coulomb kernel's error ratio with an FP32 header), of which
-                // the FP32 recursion reads the high parts
-                if constexpr (DF && F32 && !GAUGE)
-                    quartet_header_f32<GAUGE>(boys, pp + X.ppoff + i0 + ijl, pp + Y.ppoff + k0 + kl, L, H + (size_t)q * hs);
-                else if constexpr (DF)
-                    quartet_header_pairs<GAUGE>(boys, pp + X.ppoff + i0 + ijl, pp + Y.ppoff + k0 + kl, L,
-                                                H + (size_t)q * hs);
-                else
-                    quartet_header<GAUGE, false>(boys, pp + X.ppoff + i0 + ijl, pp + Y.ppoff + k0 + kl, L,
-                                                 H + (size_t)q * hs);
+    for (int c0 = 0; c0 < Y.nch;) {
+        const int y0 = cy[c0].k0;
+        int c1 = c0;
+        while (c1 < Y.nch && cy[c1].k0 + cy[c1].m - y0 <= c.ych) ++c1;
+        const int ych = cy[c1 - 1].k0 + cy[c1 - 1].m - y0, yp = (ych + 1) & ~1, nyp = yp >> 1;
+        for (int x0 = 0; x0 < X.nfp; x0 += c.xch) {
+            const int xch = min(c.xch, X.nfp - x0);
+            const int gplane = NC * xch * yp;               // FP32 pairs: high parts, then low parts
+            for (int i = tid; i < gplane; i += nt) {
+                if (A == kF64) reinterpret_cast<double *>(G)[i] = 0.0;
+                else reinterpret_cast<float2 *>(G)[i] = make_float2(0.f, 0.f);
+            }
+            for (int ih = 0; ih < X.npp; ih += c.nijH) {
+                const int nijH = min(c.nijH, X.npp - ih);
+                for (int k0 = 0; k0 < Y.nk2; k0 += c.nkc) {
+                    const int nk = min(c.nkc, Y.nk2 - k0);
+                    const bool odd = lastodd && k0 + nk == Y.nk2;
+                    const int QH = nijH * nk;
+                    // Q - P, Boys values and prefactors of the primitive quartets
+                    __syncthreads();                        // the last recursion has read the headers
+                    for (int q = tid; q < 2 * QH; q += nt) {
+                        const int ij = q / (2 * nk), r = q - ij * 2 * nk, kl = 2 * k0 + r;
+                        const int at = ij * nk + (r >> 1);
+                        if constexpr (A == kF64) {
+                            const HeadF64 h{reinterpret_cast<double *>(H + at) + (r & 1), 2 * QH};
+                            if (kl < Y.npp) {
+                                quartet_header<GAUGE>(tb.boys, tb.pp + X.ppoff + ih + ij, tb.pp + Y.ppoff + kl, L, h);
+                            } else {
+                                for (int j = 0; j < sh.hs; ++j) h.zero(j);
+                            }
+                        } else {
+                            const HeadPair h{reinterpret_cast<float *>(H + at) + (r & 1), 4 * QH};
+                            if (kl < Y.npp) {
+                                if constexpr (A == kF32 && !GAUGE)
+                                    quartet_header_f32(tb.boys, tb.pp + X.ppoff + ih + ij, tb.pp + Y.ppoff + kl, L, h);
+                                else
+                                    quartet_header_pairs<GAUGE>(tb.boys, tb.pp + X.ppoff + ih + ij,
+                                                                tb.pp + Y.ppoff + kl, L, h);
+                            } else {
+                                for (int j = 0; j < sh.hs; ++j) h.zero(j);
+                            }
+                        }
+                    }
+                    __syncthreads();
+                    for (int i0 = 0; i0 < nijH; i0 += c.nij) {
+                        const int nij = min(c.nij, nijH - i0);
+                        const int Q2 = nij * nk, hoff = i0 * nk;
+                        // Hermite recursion, one auxiliary order per pass; order 0 ends in Re.
+                        // Items (entry, two of primitive quartets) are the addresses of the
+                        // results, so the stores are contiguous.
+                        if (Ltop & 1) __syncthreads();      // T, which the odd tensors overwrite, has been read
+                        const unsigned magic = Q2 > 1 ? 0xFFFFFFFFu / (unsigned)Q2 + 1u : 0u;
+                        for (int m = Ltop; m >= 0; --m) {
+                            const int cC = m <= L ? nherm(L - m) : 0;
+                            const int cR = GAUGE ? nherm(Lr - m) : 0;
+                            Vec *dst = (m & 1) ? Ro : Re;
+                            const Vec *src = (m & 1) ? Re : Ro;
+                            const int dR = ((m & 1) ? nO_C : nE_C), sR = ((m & 1) ? nE_C : nO_C);
+                            for (int it = tid; it < (cC + cR) * Q2; it += nt) {
+                                // it / Q2 by a multiply-high (exact: it Q2 < 2^32)
+                                const int e = Q2 > 1 ? (int)__umulhi((unsigned)it, magic) : it;
+                                const int q = it - e * Q2;
+                                const bool r12 = GAUGE && e >= cC;
+                                const int h = r12 ? e - cC : e;
+                                const int db = r12 ? dR : 0, sb = r12 ? sR : 0;
+                                Vec r;
+                                if (h == 0) {
+                                    const HVec v = H[(r12 ? 4 + L + m : 3 + m) * QH + hoff + q];
+                                    if constexpr (A == kF32) r = v.x;
+                                    else r = v;
+                                } else {
+                                    const int2 sw = b.src[h];
+                                    const HVec xv = H[(sw.x & 3) * QH + hoff + q];
+                                    const Vec a = src[(sb + ((sw.x >> 2) & 1023)) * Q2 + q];
+                                    const Vec cc = src[(sb + (sw.x >> 12)) * Q2 + q];
+                                    const float cf = __int_as_float(sw.y);
+                                    if constexpr (A == kF64) {
+                                        const double cd = (double)cf;
+                                        r = make_double2(fma(cd, cc.x, xv.x * a.x), fma(cd, cc.y, xv.y * a.y));
+                                    } else if constexpr (A == kDF) {
+                                        r = df_rec2(xv, a, pack2(cf, cf), cc);
+                                    } else {
+                                        r = fma2(xv.x, a, mul2(pack2(cf, cf), cc));
+                                    }
+                                }
+                                dst[(db + h) * Q2 + q] = r;
+                            }
+                            __syncthreads();
+                        }
+                        // ket pass: T rows h < nhx from the Coulomb tensor, then (gauge) rows
+                        // g = 4.. from the r12 tensor
+                        const int nrows = nij * sh.nT;
+                        const int tplane = nrows * yp;
+                        for (int it = tid; it < nrows * (c1 - c0); it += nt) {
+                            const int ci = it / nrows, row = it - ci * nrows;
+                            const int ij = row / sh.nT, hh = row - ij * sh.nT;
+                            const PairChunk k = cy[c0 + ci];
+                            const bool r12 = GAUGE && hh >= nhx;
+                            const int g = r12 ? hh - nhx + 4 : hh;
+                            const int tr = b.trip[g];
+                            const bool neg = ((tr ^ (tr >> 8) ^ (tr >> 16)) & 1) != 0;      // |g| odd
+                            const int bx = b.box[k.box], cnt = bx >> 16;
+                            const Vec *R = Re + (r12 ? nE_C : 0) * Q2 + ij * nk;
+                            const Vec *E = EY + (long long)k.off * Y.nk2 + k0;
+                            const int at = row * yp + k.k0 - y0;
+                            if (k.m == 2)
+                                ket_store<A, 2>(R, Q2, b.hs + g * pl.nhm, b.lst + (bx & 0xffff), cnt, E,
+                                                (long long)cnt * Y.nk2, Y.nk2, nk, odd, neg, k0 > 0, T, at, tplane);
+                            else
+                                ket_store<A, 1>(R, Q2, b.hs + g * pl.nhm, b.lst + (bx & 0xffff), cnt, E, 0, Y.nk2, nk,
+                                                odd, neg, k0 > 0, T, at, tplane);
+                        }
+                        __syncthreads();
+                        if (k0 + nk < Y.nk2) continue;      // T is not complete yet (then nijH == nij)
+                        // bra pass, outer primitive pairs in order (the group size changes no rounding):
+                        // G[c][x][y] += sum_ij sum_{j in box x} E^{ij}_x[j] T[ij][row(c, h_j)][y]
+                        if constexpr (A == kF64) {
+                            for (int it = tid; it < NC * xch * ych; it += nt) {
+                                const int cx = it / ych, y = it - cx * ych, cc = cx / xch, x = cx - cc * xch;
+                                const FuncPair f = fx[x0 + x];
+                                const int bx = b.box[f.fp >> 16], cnt = bx >> 16;
+                                const unsigned char *lst = b.lst + (bx & 0xffff);
+                                double *g = reinterpret_cast<double *>(G) + (size_t)cx * yp + y;
+                                double s = *g;
+                                for (int i = 0; i < nij; ++i) {
+                                    const int ij = ih + i0 + i;
+                                    const double *e = reinterpret_cast<const double *>(
+                                        EX + (long long)f.off * X.nk2 + (ij >> 1)) + (ij & 1);
+                                    const double *t = reinterpret_cast<const double *>(T) + (size_t)i * sh.nT * yp + y;
+                                    for (int j = 0; j < cnt; ++j) {
+                                        const int h = lst[j];
+                                        const int row = (GAUGE && cc) ? nhx - 4 + b.r12row[(cc - 1) * pl.nhm + h] : h;
+                                        s = fma(__ldg(e), t[row * yp], s);
+                                        e += 2 * X.nk2;
+                                    }
+                                }
+                                *g = s;
+                            }
+                        } else {
+                            for (int it = tid; it < NC * xch * nyp; it += nt) {
+                                const int cx = it / nyp, y = 2 * (it - cx * nyp), cc = cx / xch, x = cx - cc * xch;
+                                const FuncPair f = fx[x0 + x];
+                                const int bx = b.box[f.fp >> 16], cnt = bx >> 16;
+                                const unsigned char *lst = b.lst + (bx & 0xffff);
+                                float *g = reinterpret_cast<float *>(G) + (size_t)cx * yp + y;
+                                f32x2 sh_ = *reinterpret_cast<const f32x2 *>(g), sl_ = 0;
+                                if (A == kDF) sl_ = *reinterpret_cast<const f32x2 *>(g + gplane);
+                                for (int i = 0; i < nij; ++i) {
+                                    const int ij = ih + i0 + i;
+                                    const float *e = reinterpret_cast<const float *>(
+                                        EX + (long long)f.off * X.nk2 + (ij >> 1)) + (ij & 1);
+                                    const float *t = reinterpret_cast<const float *>(T) + (size_t)i * sh.nT * yp + y;
+                                    for (int j = 0; j < cnt; ++j) {
+                                        const int h = lst[j];
+                                        const int row = (GAUGE && cc) ? nhx - 4 + b.r12row[(cc - 1) * pl.nhm + h] : h;
+                                        const float *tr = t + row * yp;
+                                        if constexpr (A == kDF) {
+                                            const float eh = __ldg(e), el = __ldg(e + 2);
+                                            const ulonglong2 ev = make_ulonglong2(pack2(eh, eh), pack2(el, el));
+                                            const ulonglong2 tv =
+                                                make_ulonglong2(*reinterpret_cast<const f32x2 *>(tr),
+                                                                *reinterpret_cast<const f32x2 *>(tr + tplane));
+                                            df_madd2(ev, make_ulonglong2(neg2(ev.x), neg2(ev.y)), tv, sh_, sl_);
+                                            e += 4 * X.nk2;
+                                        } else {
+                                            const float eh = __ldg(e);
+                                            sh_ = fma2(pack2(eh, eh), *reinterpret_cast<const f32x2 *>(tr), sh_);
+                                            e += 2 * X.nk2;
+                                        }
+                                    }
+                                }
+                                *reinterpret_cast<f32x2 *>(g) = sh_;
+                                if (A == kDF) *reinterpret_cast<f32x2 *>(g + gplane) = sl_;
+                            }
+                        }
+                    }
+                }
             }
             __syncthreads();
-            // Hermite recursion, one auxiliary order per pass; order 0 ends in buffer 0.
-            // Each warp runs all orders of its own primitive quartets (q = warp,
-            // warp + nwarps, ...), so consecutive orders need only a warp barrier;
-            // one CTA barrier after the last order.
-            const int nw = nt >> 5, wq = tid >> 5, lane = tid & 31;
-            const int nqw = wq < nq ? (nq - wq + nw - 1) / nw : 0;
-            for (int m = Ltop; m >= 0; --m) {
-                const int cC = m <= L ? nherm(L - m) : 0;
-                const int cR = GAUGE ? nherm(Lr - m) : 0;
-                const int cnt = cC + cR;
-                const int cur = m & 1, prv = cur ^ 1;
-                // items (quartet of this warp, Hermite entry) of the order; for cnt >= 2
-                // the quotient it / cnt by a multiply-high with ceil(2^32 / cnt) =
-                // floor((2^32 - 1) / cnt) + 1 (exact while it * cnt < 2^32; here
-                // it * cnt < 2^16 * 2^8); cnt == 1 (the top order) has quotient it
-                const unsigned magic = cnt > 1 ? 0xFFFFFFFFu / (unsigned)cnt + 1u : 0u;
-                for (int it = lane; it < nqw * cnt; it += 32) {
-                    const int qi = cnt > 1 ? (int)__umulhi((unsigned)it, magic) : it;
-                    const int q = wq + qi * nw;
-                    const int hh = it - qi * cnt;
-                    const double *hd = H + (size_t)q * hs;
-                    const bool cpart = !GAUGE || hh < cC;
-                    const int h = cpart ? hh : hh - cC;
-                    double *dst = cpart ? (cur ? RC1 + (size_t)q * nrC1 : RC + (size_t)q * nrC)
-                                        : (cur ? RR1 + (size_t)q * nrR1 : RR + (size_t)q * nrR);
-                    const double *src = cpart ? (prv ? RC1 + (size_t)q * nrC1 : RC + (size_t)q * nrC)
-                                              : (prv ? RR1 + (size_t)q * nrR1 : RR + (size_t)q * nrR);
-                    const int i0h = cpart ? 3 + m : 4 + L + m;
-                    if constexpr (DF && F32) {
-                        const float2 *hd2 = reinterpret_cast<const float2 *>(hd);
-                        const float2 *src2 = reinterpret_cast<const float2 *>(src);
-                        float r = hd2[i0h].x;
-                        if (h > 0) {
-                            const int sw = b.src[h];
-                            r = fmaf(hd2[sw & 3].x, src2[(sw >> 2) & 1023].x,
-                                     (float)((sw >> 22) & 15) * src2[(sw >> 12) & 1023].x);
-                        }
-                        reinterpret_cast<float2 *>(dst)[h] = make_float2(r, 0.f);
-                    } else if constexpr (DF) {
-                        const float2 *hd2 = reinterpret_cast<const float2 *>(hd);
-                        const float2 *src2 = reinterpret_cast<const float2 *>(src);
-                        float2 r = hd2[i0h];
-                        if (h > 0) {
-                            const int sw = b.src[h];
-                            r = df_rec(hd2[sw & 3], src2[(sw >> 2) & 1023], (float)((sw >> 22) & 15),
-                                       src2[(sw >> 12) & 1023]);
-                        }
-                        reinterpret_cast<float2 *>(dst)[h] = r;
-                    } else {
-                        double r = hd[i0h];
-                        if (h > 0) {
-                            const int sw = b.src[h];
-                            r = fma(b.cf[h], src[(sw >> 12) & 1023], hd[sw & 3] * src[(sw >> 2) & 1023]);
-                        }
-                        dst[h] = r;
-                    }
-                }
-                __syncwarp();
-            }
+            emit(x0, xch, y0, ych, [&](int cc, int x, int y) -> double {
+                const int i = (cc * xch + x) * yp + y;
+                if constexpr (A == kF64) return reinterpret_cast<const double *>(G)[i];
+                const float *g = reinterpret_cast<const float *>(G);
+                return (double)g[i] + (double)g[gplane + i];
+            });
             __syncthreads();
-            // T[ij][h][y] += sum_kl sum_h' (-1)^{|h'|} R[h+h'] E^{kl}[h'][y]: rows h < nhx
-            // with the Coulomb tensor, then (gauge) rows g = 4.. with the r12 tensor
-            if (DF && nT >= 4 && ych >= 2) {
-                // register tiles: 4 T rows x 2 inner function pairs per thread
-                if constexpr (DF) {
-                    float2 *T2 = reinterpret_cast<float2 *>(T);
-                    const float2 *RC2 = reinterpret_cast<const float2 *>(RC), *RR2 = reinterpret_cast<const float2 *>(RR);
-                    const void *ey = F32 ? (const void *)(E1 + b.eY[k0] + y0) : (const void *)(E2 + b.eY[k0] + y0);
-                    // plain FP32 waits on the loads: 3 inner function pairs per thread when the
-                    // chunk comes in threes (the derivative functions do), so 7 loads serve 12 FMAs
-                    if (F32 && ych % 3 == 0)
-                        ket_pass_tiled<4, 3, false, GAUGE>(nij, nT, nhx, ych, Ly, b.trip, T2, tsz, RC2, nrC, RR2, nrR,
-                                                           nk, ey, Y.nfp, sE);
-                    else
-                        ket_pass_tiled<4, 2, !F32, GAUGE>(nij, nT, nhx, ych, Ly, b.trip, T2, tsz, RC2, nrC, RR2, nrR,
-                                                          nk, ey, Y.nfp, sE);
-                }
-            } else if constexpr (DF && F32 && !GAUGE) {
-                // two T rows per thread sharing the E loads
-                const int nT2 = (nT + 1) / 2;
-                for (int it = tid; it < nij * nT2 * ych; it += nt) {
-                    const int ijl = it / (nT2 * ych);
-                    const int rem = it - ijl * nT2 * ych;
-                    const int h0 = 2 * (rem / ych), yy = rem - (rem / ych) * ych;
-                    const bool has1 = h0 + 1 < nT;
-                    const int h1 = has1 ? h0 + 1 : h0;
-                    const int tra = b.trip[h0], trb = b.trip[h1];
-                    float2 *T2 = reinterpret_cast<float2 *>(T + (size_t)ijl * tsz + (size_t)h0 * ych + yy);
-                    float acca = T2[0].x, accb = has1 ? T2[ych].x : 0.f;
-                    const float2 *R2 = reinterpret_cast<const float2 *>(RC + (size_t)ijl * nk * nrC);
-                    const float *ey = E1 + b.eY[k0] + (y0 + yy);
-                    ket_orders_f32x2<false>(0, Ly, tra & 255, (tra >> 8) & 255, tra >> 16, trb & 255, (trb >> 8) & 255,
-                                            trb >> 16, b.trip, R2, nrC, ey, Y.nfp, sE, nk, acca, accb);
-                    ket_orders_f32x2<true>(1, Ly, tra & 255, (tra >> 8) & 255, tra >> 16, trb & 255, (trb >> 8) & 255,
-                                           trb >> 16, b.trip, R2, nrC, ey, Y.nfp, sE, nk, acca, accb);
-                    T2[0] = make_float2(acca, 0.f);
-                    if (has1) T2[ych] = make_float2(accb, 0.f);
-                }
-            } else if constexpr (DF && F32) {
-                for (int it = tid; it < nij * nT * ych; it += nt) {
-                    const int ijl = it / (nT * ych);
-                    const int rem = it - ijl * nT * ych;
-                    const int hh = rem / ych, yy = rem - hh * ych;
-                    const bool r12 = GAUGE && hh >= nhx;
-                    const int h = r12 ? hh - nhx + 4 : hh;
-                    const int tr = b.trip[h];
-                    const int tx = tr & 255, ux = (tr >> 8) & 255, vx = tr >> 16;
-                    float2 *T2 = reinterpret_cast<float2 *>(T + (size_t)ijl * tsz + (size_t)hh * ych + yy);
-                    float acc = T2[0].x;
-                    const float2 *R2 = reinterpret_cast<const float2 *>(r12 ? RR + (size_t)ijl * nk * nrR
-                                                                            : RC + (size_t)ijl * nk * nrC);
-                    const int nr = r12 ? nrR : nrC;
-                    const float *ey = E1 + b.eY[k0] + (y0 + yy);
-                    ket_orders_f32<false>(0, Ly, tx, ux, vx, b.trip, R2, nr, ey, Y.nfp, sE, nk, acc);
-                    ket_orders_f32<true>(1, Ly, tx, ux, vx, b.trip, R2, nr, ey, Y.nfp, sE, nk, acc);
-                    T2[0] = make_float2(acc, 0.f);
-                }
-            } else if constexpr (DF) {
-                // gauge kernel: pairs of adjacent y per thread when the chunk has enough
-                // of them to keep the lanes busy; single y otherwise (same sums either way)
-                const int yb = (GAUGE && ych >= 8) ? 2 : 1;
-                const int ych2 = (ych + yb - 1) / yb;
-                for (int it = tid; it < nij * nT * ych2; it += nt) {
-                    const int ijl = it / (nT * ych2);
-                    const int rem = it - ijl * nT * ych2;
-                    const int hh = rem / ych2, yy = yb * (rem - hh * ych2);
-                    const bool has1 = yb == 2 && yy + 1 < ych;
-                    const bool r12 = GAUGE && hh >= nhx;
-                    const int h = r12 ? hh - nhx + 4 : hh;
-                    const int tr = b.trip[h];
-                    const int tx = tr & 255, ux = (tr >> 8) & 255, vx = tr >> 16;
-                    float2 *T2 = reinterpret_cast<float2 *>(T + (size_t)ijl * tsz + (size_t)hh * ych + yy);
-                    float ah0 = T2[0].x, al0 = T2[0].y, ah1 = 0.f, al1 = 0.f;
-                    if (has1) { ah1 = T2[1].x; al1 = T2[1].y; }
-                    const float2 *R2 = reinterpret_cast<const float2 *>(r12 ? RR + (size_t)ijl * nk * nrR
-                                                                            : RC + (size_t)ijl * nk * nrC);
-                    const int nr = r12 ? nrR : nrC;
-                    const float2 *ey = E2 + b.eY[k0] + (y0 + yy);
-                    if constexpr (GAUGE) {
-                        ket_orders_df2<false>(0, Ly, tx, ux, vx, b.trip, R2, nr, ey, Y.nfp, sE, nk, has1, ah0,
-                                              al0, ah1, al1);
-                        ket_orders_df2<true>(1, Ly, tx, ux, vx, b.trip, R2, nr, ey, Y.nfp, sE, nk, has1, ah0,
-                                             al0, ah1, al1);
-                    } else {
-                        ket_orders_df<false>(0, Ly, tx, ux, vx, b.trip, R2, nr, ey, Y.nfp, sE, nk, ah0, al0);
-                        ket_orders_df<true>(1, Ly, tx, ux, vx, b.trip, R2, nr, ey, Y.nfp, sE, nk, ah0, al0);
-                    }
-                    T2[0] = make_float2(ah0, al0);
-                    if (has1) T2[1] = make_float2(ah1, al1);
-                }
-            } else
-            for (int it = tid; it < nij * nT * ych; it += nt) {
-                const int ijl = it / (nT * ych);
-                const int rem = it - ijl * nT * ych;
-                const int hh = rem / ych, yy = rem - hh * ych;
-                const bool r12 = GAUGE && hh >= nhx;
-                const int h = r12 ? hh - nhx + 4 : hh;
-                const int tr = b.trip[h];
-                const int tx = tr & 255, ux = (tr >> 8) & 255, vx = tr >> 16;
-                double *Tq = T + (size_t)ijl * tsz + (size_t)hh * ych + yy;
-                const double *Rq = r12 ? RR + (size_t)ijl * nk * nrR : RC + (size_t)ijl * nk * nrC;
-                const int nr = r12 ? nrR : nrC;
-                double acc = *Tq;
-                const double *ey = E + (y0 + yy);
-                ket_orders<false>(0, Ly, tx, ux, vx, b.trip, Rq, nr, ey, Y.nfp, b.eY + k0, nk, acc);
-                ket_orders<true>(1, Ly, tx, ux, vx, b.trip, Rq, nr, ey, Y.nfp, b.eY + k0, nk, acc);
-                *Tq = acc;
-            }
-            // the next group's header pass touches neither T nor R, and its
-            // barrier orders this pass before the recursion overwrites R
-            if (k0 + nkl >= Y.npp) __syncthreads();
         }
-        // G[0][x][y] += sum_{ij} sum_h E^{ij}[h][x] T[ij][h][y]; gauge: G[1+IJ] from
-        // the r12 rows h + e_I + e_J (order |h| + 2) for IJ = xx, xy, xz, yy, yz, zz
-        for (int it = tid; it < xch * ych; it += nt) {
-            const int xx = it / ych, yy = it - xx * ych;
-            double s[NC];
-            float sh[NC], sl[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) { s[c] = 0.0; sh[c] = 0.f; sl[c] = 0.f; }
-            for (int ijl = 0; ijl < nij; ++ijl) {
-                const size_t off = (size_t)ijl * tsz + yy;
-#pragma unroll 4
-                for (int h = 0; h < nhx; ++h) {
-                    int g[6] = {0, 0, 0, 0, 0, 0};               // r12 rows, offset by nhx - 4
-                    if (GAUGE) {
-                        const int tr = b.trip[h];
-                        const int u = (tr >> 8) & 255, v = tr >> 16;
-                        const int o = (tr & 255) + u + v, w = u + v;
-                        const int b2 = (o + 2) * (o + 3) * (o + 4) / 6 + nhx - 4;
-                        g[0] = b2 + w * (w + 1) / 2 + v;
-                        g[1] = b2 + (w + 1) * (w + 2) / 2 + v;
-                        g[2] = g[1] + 1;
-                        g[3] = b2 + (w + 2) * (w + 3) / 2 + v;
-                        g[4] = g[3] + 1;
-                        g[5] = g[3] + 2;
-                    }
-                    if constexpr (DF && F32) {
-                        const float *T1 = reinterpret_cast<const float *>(reinterpret_cast<const float2 *>(T) + off);
-                        const float ev = __ldg(E1 + b.eX[i0 + ijl] + (x0 + xx) + (size_t)h * X.nfp);
-                        sh[0] = fmaf(ev, T1[2 * (size_t)h * ych], sh[0]);
-                        if (GAUGE)
-#pragma unroll
-                            for (int c = 1; c < NC; ++c) sh[c] = fmaf(ev, T1[2 * (size_t)g[c - 1] * ych], sh[c]);
-                    } else if constexpr (DF) {
-                        const float2 *T2 = reinterpret_cast<const float2 *>(T) + off;
-                        const float2 ev = __ldg(E2 + b.eX[i0 + ijl] + (x0 + xx) + (size_t)h * X.nfp);
-                        df_madd<false>(ev, T2[(size_t)h * ych], sh[0], sl[0]);
-                        if (GAUGE)
-#pragma unroll
-                            for (int c = 1; c < NC; ++c) df_madd<false>(ev, T2[(size_t)g[c - 1] * ych], sh[c], sl[c]);
-                    } else {
-                        const double *Tq = T + off;
-                        const double ev = __ldg(E + b.eX[i0 + ijl] + (x0 + xx) + (size_t)h * X.nfp);
-                        s[0] = fma(ev, Tq[(size_t)h * ych], s[0]);
-                        if (GAUGE)
-#pragma unroll
-                            for (int c = 1; c < NC; ++c) s[c] = fma(ev, Tq[(size_t)g[c - 1] * ych], s[c]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < NC; ++c)
-                b.G[((size_t)c * xch + xx) * ych + yy] += DF ? (double)sh[c] + (double)sl[c] : s[c];
-        }
-        __syncthreads();
+        c0 = c1;
     }
 }
 
@@ -1092,20 +992,20 @@ __device__ void block_chunk(const PrimPairDev *pp, const double *E, const float2
 template <bool GAUGE, bool DF>
 __global__ void __launch_bounds__(256, 2) eri_rows_kernel(const EriParams *prms, const EriTask *tasks, int ntasks,
                                                           int *next, Plan pl) {
-    extern __shared__ double sm[];
+    extern __shared__ __align__(16) char sm[];
     BlockSmem b = carve(sm, pl);
-    int *slot = b.src + pl.nTab;                     // in the plan's 16 spare bytes
     build_tables(pl, b);
     const int ij_of[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
     for (;;) {
-        if (threadIdx.x == 0) *slot = atomicAdd(next, 1);
+        if (threadIdx.x == 0) *b.slot = atomicAdd(next, 1);
         __syncthreads();
-        const int t = *slot;
+        const int t = *b.slot;
         __syncthreads();
         if (t >= ntasks) break;
         const EriTask tk = tasks[t];
         const EriParams &prm = prms[tk.req];
         const PairDev AB = prm.pairs[tk.bra_sp];
+        const PairTables tb{prm.pp, prm.E, prm.E2, prm.E1, prm.fp, prm.ch, prm.boys};
         for (int kp = tk.k0; kp < tk.k1; ++kp) {
             const int cd_id = prm.ket_sp[kp];
             const PairDev CD = prm.pairs[cd_id];
@@ -1122,96 +1022,80 @@ __global__ void __launch_bounds__(256, 2) eri_rows_kernel(const EriParams *prms,
             }
             if (rev && cd_id < tk.bra_sp) continue;
             const long long col_rev = rev ? prm.ket_col[prm.ket_pos[tk.bra_sp]] : 0;
-            // contract the orientation with the smaller cost; swapped -> G is (CD|AB)
-            const bool swap = orient_cost(CD, AB, GAUGE) < orient_cost(AB, CD, GAUGE);
+            // contract the orientation with fewer multiply-adds; swapped -> the block is (CD|AB)
+            const bool swap = orient_madds(CD, AB, GAUGE) < orient_madds(AB, CD, GAUGE);
             const PairDev &X = swap ? CD : AB, &Y = swap ? AB : CD;
             double *W = prm.W, *Wc = prm.Wc;
             const long long ldw = prm.ldw, ldwc = prm.ldwc, row0 = prm.row0;
             const bool wc = prm.with_coulomb != 0;
-            for (int x0 = 0; x0 < X.nfp; x0 += pl.ach) {
-                const int x1 = min(X.nfp, x0 + pl.ach);
-                for (int y0 = 0; y0 < Y.nfp; y0 += pl.cch) {
-                    const int y1 = min(Y.nfp, y0 + pl.cch);
-                    if constexpr (DF) {
-                        if (tk.f32)
-                            block_chunk<GAUGE, true, true>(prm.pp, prm.E, prm.E2, prm.E1, prm.boys, X, Y, x0, x1, y0, y1,
-                                                           pl, b);
-                        else
-                            block_chunk<GAUGE, true, false>(prm.pp, prm.E, prm.E2, prm.E1, prm.boys, X, Y, x0, x1, y0,
-                                                            y1, pl, b);
-                    } else {
-                        block_chunk<GAUGE, false>(prm.pp, prm.E, prm.E2, prm.E1, prm.boys, X, Y, x0, x1, y0, y1, pl, b);
-                    }
-                    const int xch = x1 - x0, ych = y1 - y0;
-                    for (int idx = threadIdx.x; idx < xch * ych; idx += blockDim.x) {
-                        const int xx = idx / ych, yy = idx - xx * ych;
-                        const int a = swap ? y0 + yy : x0 + xx;      // bra function pair
-                        const int c = swap ? x0 + xx : y0 + yy;      // ket function pair
-                        // the block's entry into row `r`, column `k` of an output
-                        // (gauge: rows (r, I), columns (k, J); K_IJ is symmetric, so the
-                        // transposed entry needs no index change)
-                        auto put = [&](double *Wo, long long ldo, double *Wco, long long ldco, long long r,
-                                       long long k) {
-                            if (!GAUGE) {
-                                Wo[r * ldo + k] = b.G[idx];
-                            } else {
-                                const double C = b.G[idx];
-                                const double *Hh = b.G + (size_t)xch * ych;
-                                for (int I = 0; I < 3; ++I)
-                                    for (int J = 0; J < 3; ++J) {
-                                        const double h = Hh[(size_t)ij_of[I][J] * xch * ych + idx];
-                                        Wo[(r * 3 + I) * ldo + k * 3 + J] = (I == J ? C : 0.0) - h;
-                                    }
-                                if (wc) Wco[r * ldco + k] = C;
-                            }
-                        };
-                        put(W, ldw, Wc, ldwc, AB.rowoff + a - row0, col + c);
-                        // the same integrals at (cd, ab): rows of CD, columns of AB
-                        if (rev) put(W, ldw, Wc, ldwc, CD.rowoff + c - row0, col_rev + a);
-                        if (mir) put(prm.W2, prm.ldw2, prm.Wc2, prm.ldwc2, CD.rowoff + c - prm.row2,
-                                     prm.col2[tk.bra_sp] + a);
-                    }
-                    __syncthreads();
+            auto emit = [&](int x0, int xch, int y0, int ych, auto value) {
+                for (int idx = threadIdx.x; idx < xch * ych; idx += blockDim.x) {
+                    const int xx = idx / ych, yy = idx - xx * ych;
+                    const int fx = prm.fp[X.fpoff + x0 + xx].fp & 0xffff, fy = prm.fp[Y.fpoff + y0 + yy].fp & 0xffff;
+                    const int a = swap ? fy : fx;                // bra function pair
+                    const int c = swap ? fx : fy;                // ket function pair
+                    const double C = value(0, xx, yy);
+                    double hc[6];
+                    if (GAUGE)
+#pragma unroll
+                        for (int j = 0; j < 6; ++j) hc[j] = value(j + 1, xx, yy);
+                    // the block's entry into row `r`, column `k` of an output
+                    // (gauge: rows (r, I), columns (k, J); K_IJ is symmetric, so the
+                    // transposed entry needs no index change)
+                    auto put = [&](double *Wo, long long ldo, double *Wco, long long ldco, long long r, long long k) {
+                        if (!GAUGE) {
+                            Wo[r * ldo + k] = C;
+                        } else {
+#pragma unroll
+                            for (int I = 0; I < 3; ++I)
+#pragma unroll
+                                for (int J = 0; J < 3; ++J)
+                                    Wo[(r * 3 + I) * ldo + k * 3 + J] = (I == J ? C : 0.0) - hc[ij_of[I][J]];
+                            if (wc) Wco[r * ldco + k] = C;
+                        }
+                    };
+                    put(W, ldw, Wc, ldwc, AB.rowoff + a - row0, col + c);
+                    // the same integrals at (cd, ab): rows of CD, columns of AB
+                    if (rev) put(W, ldw, Wc, ldwc, CD.rowoff + c - row0, col_rev + a);
+                    if (mir) put(prm.W2, prm.ldw2, prm.Wc2, prm.ldwc2, CD.rowoff + c - prm.row2,
+                                 prm.col2[tk.bra_sp] + a);
                 }
+            };
+            if constexpr (DF) {
+                if (tk.f32) quartet_block<GAUGE, kF32>(tb, X, Y, pl, b, emit);
+                else quartet_block<GAUGE, kDF>(tb, X, Y, pl, b, emit);
+            } else {
+                quartet_block<GAUGE, kF64>(tb, X, Y, pl, b, emit);
             }
         }
     }
 }
 
-// Plan for a class: the largest function-pair chunk (halved while needed) such
-// that the pool holds the T of one outer primitive pair plus at least eight
-// primitive quartets of the highest order.  Small classes run as 128-thread
-// CTAs in 56 KB, four per SM, so that a CTA waiting at a barrier leaves the
-// FP64 pipe to the others; classes that do not fit take 112 KB or 200 KB.
+// Plan for a class: the smallest shared-memory tier (so the most CTAs per SM)
+// that holds the class's largest quartet uncut, one outer primitive pair at a
+// time with the headers of all; at most what its small quartets can use.
 Plan eri_plan(int maxnfp, int maxLab, int maxnpp, bool gauge) {
     struct Tier { int kb, threads; };
-    const Tier tiers[3] = {{56, 128}, {112, 256}, {200, 256}};
+    const Tier tiers[4] = {{56, 128}, {75, 128}, {112, 256}, {224, 256}};
     Plan p{};
-    for (int ti = gauge ? 1 : 0; ti < 3; ++ti) {
-        p.NC = gauge ? 7 : 1;
-        p.nhMax = nherm(maxLab);
-        p.LtC = 2 * maxLab;
-        p.LtR = gauge ? p.LtC + 2 : -1;
-        p.nTab = nherm(gauge ? p.LtR : p.LtC);
-        p.maxnpp = maxnpp > 0 ? maxnpp : 1;
+    p.maxLab = maxLab;
+    p.nTab = nherm(2 * maxLab + (gauge ? 2 : 0));
+    p.nhm = nherm(maxLab);
+    p.nG = nherm(maxLab + (gauge ? 2 : 0));
+    p.nLst = box_entries_below(maxLab + 1);
+    const int npp = std::max(maxnpp, 1), nk2 = (npp + 1) / 2, nfp = std::max(maxnfp, 1);
+    const Shape s = quartet_shape(maxLab, maxLab, gauge);
+    const long long tables = (long long)plan_tables(p);
+    auto bytes = [&](long long nij, long long nijH) {        // cut_bytes in 64 bits
+        const long long yp = (nfp + 1) / 2 * 2, t = nij * s.nT * yp * 8, o = s.nO * nij * nk2 * 16;
+        return s.hs * nijH * nk2 * 16 + s.nE * nij * nk2 * 16 + std::max(t, o) + s.NC * nfp * yp * 8;
+    };
+    const long long least = bytes(1, npp), most = bytes(npp, npp);
+    for (int ti = 0; ti < 4; ++ti) {
+        const long long room = (long long)tiers[ti].kb * 1024 - tables;
         p.threads = tiers[ti].threads;
-        p.ach = p.cch = maxnfp > 0 ? maxnfp : 1;
-        const long long perq = quartet_len(p.LtC, gauge);
-        const long long budget = (long long)tiers[ti].kb * 1024;
-        long long tsz = 0;
-        for (;;) {
-            p.pool = 0;
-            const long long fixed = (long long)plan_smem(p);
-            tsz = (long long)t_rows(maxLab, gauge) * p.cch;
-            const long long pool = (budget - fixed) / (long long)sizeof(double);
-            if (pool >= tsz + 8 * perq || p.ach <= 8) {
-                p.pool = pool > tsz + perq ? pool : tsz + perq;
-                break;
-            }
-            p.ach = p.cch = (p.ach + 1) / 2;
-        }
-        const int want = maxnfp < 32 ? maxnfp : 32;
-        if ((p.ach >= want && p.pool >= tsz + 8 * perq) || ti == 2) break;
+        p.pool = (int)(std::min(std::max(most, 4096LL), room) / 16 * 16);
+        if (least <= room) break;
     }
     return p;
 }
@@ -1285,40 +1169,43 @@ void launch_ratio(const double *A, const double *B, long long rows, long long ld
     QDT_CHECK_LAUNCH();
 }
 
-void launch_split_pairs(const double *E, long long n, float2 *E2, float *E1, cudaStream_t s) {
+void launch_split_pairs(const double2 *E, long long n, float4 *E2, float2 *E1, cudaStream_t s) {
     if (n <= 0) return;
     split_pairs_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(E, n, E2, E1);
     QDT_CHECK_KERNEL("split_pairs_kernel");
 }
 
 // Schwarz diagonals: Q[AB] = max over ab of sqrt(|(ab|ab)|), Coulomb kernel.
-__global__ void __launch_bounds__(256, 2) schwarz_kernel(const PrimPairDev *pp, const PairDev *pairs, const double *E,
-                                                         const double *boys, Plan pl, double *Q) {
-    extern __shared__ double sm[];
+__global__ void __launch_bounds__(256, 2) schwarz_kernel(PairTables tb, const PairDev *pairs, Plan pl, double *Q) {
+    extern __shared__ __align__(16) char sm[];
     const PairDev AB = pairs[blockIdx.x];
     BlockSmem b = carve(sm, pl);
     build_tables(pl, b);
     double qmax = 0.0;
-    for (int a0 = 0; a0 < AB.nfp; a0 += pl.ach) {
-        const int a1 = min(AB.nfp, a0 + pl.ach);
-        block_chunk<false, false>(pp, E, nullptr, nullptr, boys, AB, AB, a0, a1, a0, a1, pl, b);
-        const int ach = a1 - a0;
-        if (threadIdx.x == 0)
-            for (int a = 0; a < ach; ++a) qmax = fmax(qmax, sqrt(fabs(b.G[(size_t)a * ach + a])));
-        __syncthreads();
+    quartet_block<false, kF64>(tb, AB, AB, pl, b, [&](int x0, int xch, int y0, int ych, auto value) {
+        for (int x = threadIdx.x; x < xch; x += blockDim.x) {
+            const int y = x0 + x - y0;
+            if (y >= 0 && y < ych) qmax = fmax(qmax, sqrt(fabs(value(0, x, y))));
+        }
+    });
+    double *red = reinterpret_cast<double *>(b.pool);       // the block's last use of the pool is over
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) qmax = fmax(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = qmax;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) qmax = fmax(qmax, red[w]);
+        Q[blockIdx.x] = qmax;
     }
-    if (threadIdx.x == 0) Q[blockIdx.x] = qmax;
 }
 
-void launch_schwarz(const ShellDev *shells, const PairDev *pairs, const PrimPairDev *pp, const double *E,
-                    const double *boys, int npairs, int maxnfp, int maxLab, int maxnpp, double *Q,
-                    cudaStream_t s) {
-    (void)shells;
-    if (npairs <= 0) return;
-    const Plan pl = eri_plan(maxnfp, maxLab, maxnpp, false);
+void launch_schwarz(const PairClass &pc, const double *boys, double *Q, cudaStream_t s) {
+    if (pc.nsp <= 0) return;
+    const Plan pl = eri_plan(pc.maxnfp, pc.maxLab, pc.maxnpp, false);
     const size_t smem = plan_smem(pl);
     QDT_CUDA_TRY(cudaFuncSetAttribute(schwarz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    schwarz_kernel<<<npairs, pl.threads, smem, s>>>(pp, pairs, E, boys, pl, Q);
+    const PairTables tb{pc.d_pp, pc.d_E, nullptr, nullptr, pc.d_fp, pc.d_ch, boys};
+    schwarz_kernel<<<pc.nsp, pl.threads, smem, s>>>(tb, pc.d_pairs, pl, Q);
     QDT_CHECK_LAUNCH();
 }
 

@@ -29,7 +29,8 @@
 namespace qdt {
 void launch_prim_pairs_map(const ShellDev *shells, const PairDev *pairs, const int *pp_pair,
                            long long npp, const double *exps, const double *coefs,
-                           const double *norms, PrimPairDev *pp, double *E, cudaStream_t s);
+                           const double *norms, const FuncPair *fptab, PrimPairDev *pp, double2 *E,
+                           cudaStream_t s);
 void launch_density(bool gaunt, bool ku, bool pairs_arith, const PairDev *pairs, const int *bra_order, int nsp,
                     const ShellDev *shells, int maxnf, int maxnfp, const double *Cq, int nK, int k0, const int *rsR,
                     const int *rsS, int nRS, double *D, double *Dmax, cudaStream_t s);
@@ -127,7 +128,7 @@ T *dcopy_pinned(PinnedArena &a, DBuf &b, const std::vector<T> &v, cudaStream_t s
 }
 
 struct ClassBufs {
-    DBuf pairs, pp, E, E2, E1, Q, bra, brapos, pp_pair;
+    DBuf pairs, pp, E, E2, E1, fp, ch, Q, bra, brapos, pp_pair;
 };
 
 // Instantiated graph of a batch round and the signature it was captured for.
@@ -219,19 +220,59 @@ constexpr size_t kSliceBudget = (size_t)8 << 30;
 // FP64 intermediates of one row chunk of the quarter route
 constexpr size_t kQuarterBudget = (size_t)4 << 30;
 
-// FP64 multiply-adds of the E R E contraction of one shell quartet with X as
-// the outer (per primitive pair) side: the ket pass over T rows (X's Hermite
-// triples; gauge: also the r12 rows 2 <= |g| <= Lx + 2) and the bra pass per
-// component (1 Coulomb, 7 gauge).
-double orient_cost_h(const PairDev &X, const PairDev &Y, bool gauge) {
-    const double nhx = nherm(X.Lab), nhy = nherm(Y.Lab);
-    const double trows = nherm(X.Lab) + (gauge ? nherm(X.Lab + 2) - 4 : 0);
-    return (double)X.npp * Y.npp * trows * Y.nfp * nhy + (double)X.npp * X.nfp * Y.nfp * nhx * (gauge ? 7 : 1);
+// Cost proxy of the tiles of a bra pair: primitive pairs x Hermite terms.
+double bra_cost(const PairDev &p) { return (double)p.npp * nherm(p.Lab) * p.nbox; }
+
+// Powers (x, y, z) of function f of a shell: the Cartesian component, one
+// higher along the derivative's axis; the reduced derivative shell of a p shell
+// holds the six functions of order 2 (func_terms in basis_kernels.cu).
+void func_powers(const ShellDev &sh, int f, int pw[3]) {
+    auto cart = [&](int l, int c) {
+        for (int i = l, n = 0; i >= 0; --i)
+            for (int j = l - i; j >= 0; --j, ++n)
+                if (n == c) { pw[0] = i; pw[1] = j; pw[2] = l - i - j; return; }
+    };
+    if (!sh.isS) cart(sh.l, f);
+    else if (sh.red) cart(2, f);
+    else { cart(sh.l, f / 3); ++pw[f % 3]; }
 }
 
-// Cost proxy of the tiles of a bra pair: primitive pairs x Hermite terms x
-// function pairs.
-double bra_cost(const PairDev &p) { return (double)p.npp * nherm(p.Lab) * p.nfp; }
+// Tables of one kind of shell pair: its function pairs sorted by box (largest
+// first, so that the last round of a ket or bra pass is its cheapest), and the
+// chunks of at most two function pairs of one box that share the Hermite
+// integrals a thread of the ket pass loads.
+struct PairKind {
+    int nfp = 0, nbox = 0, fpoff = 0, choff = 0, nch = 0;
+};
+PairKind make_kind(const ShellDev &A, const ShellDev &B, bool same, std::vector<FuncPair> &fp,
+                   std::vector<PairChunk> &ch) {
+    struct Item { int fp, box, cnt; };
+    std::vector<Item> v;
+    for (int fa = 0; fa < A.nfunc; ++fa)
+        for (int fb = same ? fa : 0; fb < B.nfunc; ++fb) {
+            int a[3], b[3];
+            func_powers(A, fa, a);
+            func_powers(B, fb, b);
+            for (int d = 0; d < 3; ++d) a[d] += b[d];
+            v.push_back({(int)v.size(), hidx(a[0], a[1], a[2]), box_count(a[0], a[1], a[2])});
+        }
+    std::stable_sort(v.begin(), v.end(), [](const Item &x, const Item &y) {
+        return x.cnt != y.cnt ? x.cnt > y.cnt : x.box < y.box;
+    });
+    PairKind k;
+    k.nfp = (int)v.size();
+    k.fpoff = (int)fp.size();
+    k.choff = (int)ch.size();
+    for (int i = 0; i < k.nfp; ++i) {
+        const bool join = i > 0 && v[i].box == v[i - 1].box && ch.back().m == 1 && (int)ch.size() > k.choff;
+        if (join) ch.back().m = 2;
+        else ch.push_back({i, 1, v[i].box, k.nbox});
+        fp.push_back({v[i].fp | (v[i].box << 16), k.nbox});
+        k.nbox += v[i].cnt;
+    }
+    k.nch = (int)ch.size() - k.choff;
+    return k;
+}
 
 // Bra pairs of a list in tile order: as given (the bra order, Schwarz Q
 // descending) or most expensive first, so that the tile queue ends on cheap
@@ -427,13 +468,23 @@ void build_class(qdt_ctx *ctx, int c) {
     pc.nsp = (int)sp.size();
     std::vector<PrimPairDev> hpp;
     std::vector<int> pp_pair;
+    std::vector<FuncPair> fptab;
+    std::vector<PairChunk> chtab;
+    std::map<std::tuple<int, int, int, int, bool>, PairKind> kinds;
     long long eoff = 0, M = 0;
     for (int i = 0; i < pc.nsp; ++i) {
         const ShellDev &A = ctx->h_shells[sp[i].first], &B = ctx->h_shells[sp[i].second];
         PairDev pr;
         pr.sa = sp[i].first;
         pr.sb = sp[i].second;
-        pr.nfp = (pr.sa == pr.sb) ? A.nfunc * (A.nfunc + 1) / 2 : A.nfunc * B.nfunc;
+        const auto key = std::make_tuple(A.l, A.isS, B.l, B.isS, pr.sa == pr.sb);
+        auto kd = kinds.find(key);
+        if (kd == kinds.end()) kd = kinds.emplace(key, make_kind(A, B, pr.sa == pr.sb, fptab, chtab)).first;
+        pr.nfp = kd->second.nfp;
+        pr.nbox = kd->second.nbox;
+        pr.fpoff = kd->second.fpoff;
+        pr.choff = kd->second.choff;
+        pr.nch = kd->second.nch;
         pr.Lab = (A.l + A.isS) + (B.l + B.isS);
         pr.ppoff = (int)hpp.size();
         pr.rowoff = 0;
@@ -444,14 +495,15 @@ void build_class(qdt_ctx *ctx, int c) {
                 double a = ctx->h_exps[A.poff + ia], bb = ctx->h_exps[B.poff + ib];
                 if (std::exp(-a * bb / (a + bb) * r2) < kPrimPairTol) continue;
                 PrimPairDev q{};
-                q.eoff = eoff;
                 q.ia = ia;
                 q.ib = ib;
-                eoff += (long long)pr.nfp * nherm(pr.Lab);
                 hpp.push_back(q);
                 pp_pair.push_back(i);
             }
         pr.npp = (int)hpp.size() - pr.ppoff;
+        pr.nk2 = (pr.npp + 1) / 2;
+        pr.eoff = eoff;
+        eoff += (long long)pr.nbox * pr.nk2;
         pc.maxnpp = std::max(pc.maxnpp, pr.npp);
         M += pr.nfp;
         pc.maxnfp = std::max(pc.maxnfp, pr.nfp);
@@ -466,18 +518,20 @@ void build_class(qdt_ctx *ctx, int c) {
     pc.d_pairs = dcopy(b.pairs, pc.h_pairs, s);
     pc.d_pp = dcopy(b.pp, hpp, s);
     int *d_ppp = dcopy(b.pp_pair, pp_pair, s);
-    pc.d_E = (double *)b.E.get(std::max<long long>(1, eoff) * sizeof(double));
+    pc.d_fp = dcopy(b.fp, fptab, s);
+    pc.d_ch = dcopy(b.ch, chtab, s);
+    pc.d_E = (double2 *)b.E.get(std::max<long long>(1, eoff) * sizeof(double2));
+    QDT_CUDA_TRY(cudaMemsetAsync(pc.d_E, 0, std::max<long long>(1, eoff) * sizeof(double2), s));   // odd counts: zero
     launch_prim_pairs_map(ctx->shells.p ? (const ShellDev *)ctx->shells.p : nullptr, pc.d_pairs, d_ppp,
                           pc.npp_total, (const double *)ctx->exps.p, (const double *)ctx->coefs.p,
-                          (const double *)ctx->norms.p, pc.d_pp, pc.d_E, s);
-    pc.d_E2 = (float2 *)b.E2.get(std::max<long long>(1, eoff) * sizeof(float2));
-    pc.d_E1 = (float *)b.E1.get(std::max<long long>(1, eoff) * sizeof(float));
+                          (const double *)ctx->norms.p, pc.d_fp, pc.d_pp, pc.d_E, s);
+    pc.d_E2 = (float4 *)b.E2.get(std::max<long long>(1, eoff) * sizeof(float4));
+    pc.d_E1 = (float2 *)b.E1.get(std::max<long long>(1, eoff) * sizeof(float2));
     launch_split_pairs(pc.d_E, eoff, pc.d_E2, pc.d_E1, s);
     ctx->launches += 2;
     // Schwarz diagonals, then the bra order (Q descending, ties by id)
     pc.d_Q = (double *)b.Q.get(std::max(1, pc.nsp) * sizeof(double));
-    launch_schwarz((const ShellDev *)ctx->shells.p, pc.d_pairs, pc.d_pp, pc.d_E,
-                   (const double *)ctx->boys.p, pc.nsp, pc.maxnfp, pc.maxLab, pc.maxnpp, pc.d_Q, s);
+    launch_schwarz(pc, (const double *)ctx->boys.p, pc.d_Q, s);
     ctx->launches++;
     pc.h_Q.resize(pc.nsp);
     QDT_CUDA_TRY(cudaMemcpyAsync(pc.h_Q.data(), pc.d_Q, pc.nsp * sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -930,6 +984,8 @@ void batch_prepare(qdt_ctx *ctx, const ClassPlan &P, int b0, RowBatch &B) {
     prm.E = pc.d_E;
     prm.E2 = P.precision == QDT_SPLIT ? pc.d_E2 : nullptr;
     prm.E1 = P.precision == QDT_SPLIT ? pc.d_E1 : nullptr;
+    prm.fp = pc.d_fp;
+    prm.ch = pc.d_ch;
     prm.boys = (const double *)ctx->boys.p;
     prm.ket_sp = P.mirror ? B.d_list : P.ketsp;
     prm.ket_col = P.mirror ? B.d_col1 : P.ketcol;
@@ -993,7 +1049,7 @@ void batch_stats(qdt_ctx *ctx, const ClassPlan &P, const RowBatch &B, long long 
                 const int bp = pc.bra_pos[cid];
                 if (bp < B.b0 || (bp < B.b1 && cid < sp)) continue;
             }
-            const double f = 2.0 * std::min(orient_cost_h(ab, cd, gauge), orient_cost_h(cd, ab, gauge));
+            const double f = 2.0 * (double)std::min(orient_madds(ab, cd, gauge), orient_madds(cd, ab, gauge));
             fl += f;
             if (B.prm.E2 && q >= P.h_split[sp]) fl32 += f;
         }
@@ -1691,7 +1747,7 @@ void qdt_destroy(qdt_ctx *c) {
                     &c->kpre1, &c->ksplit1};
     for (DBuf *b : bufs) b->release();
     for (int k = 0; k < 2; ++k) {
-        c->cb[k].pairs.release(); c->cb[k].pp.release(); c->cb[k].E.release(); c->cb[k].E2.release(); c->cb[k].E1.release();
+        c->cb[k].pairs.release(); c->cb[k].pp.release(); c->cb[k].E.release(); c->cb[k].E2.release(); c->cb[k].E1.release(); c->cb[k].fp.release(); c->cb[k].ch.release();
         c->cb[k].Q.release(); c->cb[k].bra.release(); c->cb[k].brapos.release(); c->cb[k].pp_pair.release();
     }
     split_release(c->split);

@@ -114,14 +114,37 @@ struct PairDev {
     int Lab;        // Hermite order of the pair
     int npp;        // primitive pairs
     int ppoff;      // first primitive pair
+    int nk2;        // primitive pairs in twos: (npp + 1) / 2
+    int nbox;       // Hermite terms of all function pairs together (see FuncPair)
+    int fpoff;      // first entry of its kind in the class's FuncPair table
+    int choff, nch; // its kind's entries in the class's PairChunk table
+    long long eoff; // first E entry, in twos of primitive pairs
     long long rowoff;   // first row in the bra (Q-sorted) order
 };
+
+// The Hermite expansion of a function pair is a product of one-dimensional
+// expansions, so of the nherm(Lab) Hermite functions of its shell pair only the
+// box t <= Nx, u <= Ny, v <= Nz carries a non-zero coefficient, N being the
+// summed powers of the two functions (Nx + Ny + Nz = Lab).  A box is named by
+// the Hermite index of (Nx, Ny, Nz).  The function pairs of a shell pair are
+// sorted by box (largest first); tables per kind of shell pair (shell orders,
+// large or derivative, same shell or not), shared by all pairs of the kind.
+struct FuncPair {               // one per function pair, in sorted order
+    int fp;                     // function pair (natural order) | box << 16
+    int off;                    // E entries of the pair's function pairs before it
+};
+struct PairChunk {              // one or two neighbouring function pairs of the same box
+    int k0, m;                  // first (sorted), count
+    int box;
+    int off;                    // E entries before k0
+};
+// Entries of box (Nx, Ny, Nz) in order: t slowest, v fastest.
+__host__ __device__ constexpr int box_count(int nx, int ny, int nz) { return (nx + 1) * (ny + 1) * (nz + 1); }
 
 struct PrimPairDev {
     double p;
     double inv_p;   // 1 / p
     double P[3];
-    long long eoff; // offset of this primitive pair's E matrix [nherm(Lab)][nfp]
     int ia, ib;     // primitives of the two shells
 };
 
@@ -138,9 +161,14 @@ struct PairClass {
     std::vector<double> h_Q;
     PairDev *d_pairs = nullptr;
     PrimPairDev *d_pp = nullptr;
-    double *d_E = nullptr;
-    float2 *d_E2 = nullptr;     // E split into FP32 pairs (hi, lo) for the split form's integrals
-    float *d_E1 = nullptr;      // the high parts alone, for the quartets run in plain FP32
+    // Hermite coefficients E of a shell pair: [function pair (sorted)][box entry]
+    // [primitive pairs in twos], zero past the last primitive pair, so that one
+    // vector load brings two primitive pairs
+    double2 *d_E = nullptr;
+    float4 *d_E2 = nullptr;     // E as FP32 pairs (hi0, hi1, lo0, lo1) for the split form's integrals
+    float2 *d_E1 = nullptr;     // the high parts alone, for the quartets run in plain FP32
+    FuncPair *d_fp = nullptr;
+    PairChunk *d_ch = nullptr;
     double *d_Q = nullptr;
     int *d_bra_order = nullptr;
     std::vector<int> bra_pos;   // bra position of every shell pair (inverse of bra_order)
@@ -154,9 +182,11 @@ struct EriParams {
     const ShellDev *shells;
     const PairDev *pairs;
     const PrimPairDev *pp;
-    const double *E;
-    const float2 *E2;           // E as FP32 pairs: non-null selects the compensated FP32 contraction
-    const float *E1;            // fl32(E), read by the tiles run in plain FP32
+    const double2 *E;
+    const float4 *E2;           // E as FP32 pairs: non-null selects the compensated FP32 contraction
+    const float2 *E1;           // fl32(E), read by the tiles run in plain FP32
+    const FuncPair *fp;
+    const PairChunk *ch;
     const double *boys;         // [kBoysGrid][kBoysCols], followed by the same as floats
     // the ket list the tiles index: the w-sorted ket order of the class, or in
     // row batches with bra-ket symmetry the batch's own list (plan.h
@@ -226,15 +256,26 @@ void launch_shell_norms(const ShellDev *shells, int nL_shells, const double *exp
 // FP32 pairs (the split form); otherwise in FP64.
 void launch_eri(const EriParams *prms, const EriTask *tasks, int ntasks, int *next, const EriShape &shape,
                 bool gauge, bool df, const EriLaunch &how, cudaStream_t s);
-// E2[i] = (hi, lo) with hi = fl32(E[i]), lo = fl32(E[i] - hi).
 // max |A - B| / (Q_row Q_col) over integral rows (FP32 error model check).
 void launch_ratio(const double *A, const double *B, long long rows, long long ldw, int mult, const int *row_pair,
                   const int *col_pair, long long ncols, const double *Q, double *out, cudaStream_t s);
-void launch_split_pairs(const double *E, long long n, float2 *E2, float *E1, cudaStream_t s);
+// E2[i] = (hi, lo) of the two entries of E[i], hi = fl32(x), lo = fl32(x - hi); E1[i] the hi parts.
+void launch_split_pairs(const double2 *E, long long n, float4 *E2, float2 *E1, cudaStream_t s);
 int eri_default_threads(const EriShape &shape, bool gauge);
-void launch_schwarz(const ShellDev *shells, const PairDev *pairs, const PrimPairDev *pp,
-                    const double *E, const double *boys, int npairs, int maxnfp, int maxLab,
-                    int maxnpp, double *Q, cudaStream_t s);
+void launch_schwarz(const PairClass &pc, const double *boys, double *Q, cudaStream_t s);
+
+// T rows per outer primitive pair: the Hermite triples h of X for the Coulomb
+// tensor and, for the gauge kernel, the triples g with 2 <= |g| <= Lx + 2 of the
+// r12 tensor (g = h + e_I + e_J covers all six second derivatives).
+__host__ __device__ inline int t_rows(int Lx, bool gauge) { return nherm(Lx) + (gauge ? nherm(Lx + 2) - 4 : 0); }
+// Multiply-adds of the contraction of a shell quartet with X outer: the ket
+// pass (T rows x the inner pair's box entries per primitive quartet) plus the
+// bra pass (components x the outer pair's box entries x inner function pairs
+// per outer primitive pair).
+__host__ __device__ inline long long orient_madds(const PairDev &X, const PairDev &Y, bool gauge) {
+    return (long long)X.npp * ((long long)Y.npp * t_rows(X.Lab, gauge) * Y.nbox +
+                               (long long)X.nbox * Y.nfp * (gauge ? 7 : 1));
+}
 
 void launch_ket_order(const double *Q, const double *Dmax, int nsp, double *w, int *ket_sp,
                       cudaStream_t s);
