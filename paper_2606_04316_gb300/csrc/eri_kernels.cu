@@ -36,10 +36,6 @@
 //    scalar form, and the two halves are independent chains.  The bra pass
 //    packs two function pairs y instead.
 //
-// Measured against all Hermite functions and scalar instructions (integral phase,
-// before -> after): 24-centre s+p chain, all blocks, split 477 -> 262 ms; 12-centre
-// s/p/d cluster 671 -> 121 ms; 7-centre chain, FP64 form 39 -> 17 ms.
-//
 // Split form (DF): recursion and both passes in compensated FP32 pairs (x = hi +
 // lo, ~48-bit significands): products by the exact-product FMA, sums by the
 // error-free two-sum.  FP32 issues 64 times faster than FP64 on this part.
@@ -417,44 +413,46 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
 }
 // a - b (one rounding: -1 * b is exact)
 __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, 0xBF800000BF800000ull, a); }
-__device__ __forceinline__ f32x2 neg2(f32x2 a) { return a ^ 0x8000000080000000ull; }
 __device__ __forceinline__ f32x2 pack2(float x, float y) {
     return (f32x2)__float_as_uint(x) | ((f32x2)__float_as_uint(y) << 32);
 }
 __device__ __forceinline__ float lower2(f32x2 a) { return __uint_as_float((unsigned)a); }
 __device__ __forceinline__ float upper2(f32x2 a) { return __uint_as_float((unsigned)(a >> 32)); }
 
+// a b - p for p = fl(a b), exact, two at once: scalar FMAs, which negate an operand
+// for free (a packed one would need the negated operand formed first).
+__device__ __forceinline__ f32x2 prod_err2(f32x2 a, f32x2 b, f32x2 p) {
+    return pack2(__fmaf_rn(lower2(a), lower2(b), -lower2(p)), __fmaf_rn(upper2(a), upper2(b), -upper2(p)));
+}
+
 // (ah, al) += a * b in compensated FP32 pairs, two at once: exact product error of
 // the high parts plus the cross terms, then the two-sum of the high parts.
-// na = (-a.x, -a.y): the error is formed as p - a b, so no packed sum needs a
-// negated operand.
-__device__ __forceinline__ void df_madd2(ulonglong2 a, ulonglong2 na, ulonglong2 b, f32x2 &ah, f32x2 &al) {
+__device__ __forceinline__ void df_madd2(ulonglong2 a, ulonglong2 b, f32x2 &ah, f32x2 &al) {
     const f32x2 p = mul2(a.x, b.x);
-    f32x2 pe = fma2(na.x, b.x, p);                    // -(product error)
-    pe = fma2(na.x, b.y, pe);
-    pe = fma2(na.y, b.x, pe);
+    f32x2 pe = prod_err2(a.x, b.x, p);
+    pe = fma2(a.x, b.y, pe);
+    pe = fma2(a.y, b.x, pe);
     const f32x2 t = add2(ah, p);
     const f32x2 bv = sub2(t, ah);
     const f32x2 err = add2(sub2(ah, sub2(t, bv)), sub2(p, bv));
     ah = t;
-    al = add2(al, sub2(err, pe));
+    al = add2(al, add2(err, pe));
 }
 
 // x a + cf c in compensated FP32 pairs, renormalised, two at once (one Hermite
 // recursion step).
 __device__ __forceinline__ ulonglong2 df_rec2(ulonglong2 x, ulonglong2 a, f32x2 cf, ulonglong2 c) {
-    const f32x2 nxh = neg2(x.x), nxl = neg2(x.y), ncf = neg2(cf);
     const f32x2 p1 = mul2(x.x, a.x);
-    f32x2 e1 = fma2(nxh, a.x, p1);
-    e1 = fma2(nxh, a.y, e1);
-    e1 = fma2(nxl, a.x, e1);
+    f32x2 e1 = prod_err2(x.x, a.x, p1);
+    e1 = fma2(x.x, a.y, e1);
+    e1 = fma2(x.y, a.x, e1);
     const f32x2 p2 = mul2(cf, c.x);
-    f32x2 e2 = fma2(ncf, c.x, p2);
-    e2 = fma2(ncf, c.y, e2);
+    f32x2 e2 = prod_err2(cf, c.x, p2);
+    e2 = fma2(cf, c.y, e2);
     const f32x2 t = add2(p1, p2);
     const f32x2 bv = sub2(t, p1);
     const f32x2 err = add2(sub2(p1, sub2(t, bv)), sub2(p2, bv));
-    const f32x2 lo = sub2(err, add2(e1, e2));
+    const f32x2 lo = add2(err, add2(e1, e2));
     const f32x2 hi = add2(t, lo);
     return make_ulonglong2(hi, sub2(lo, sub2(hi, t)));
 }
@@ -488,15 +486,23 @@ struct BlockSmem {
     int *trip;                  // Hermite triple h -> t | u << 8 | v << 16
     int *box;                   // per box: first list entry | count << 16
     unsigned short *hs;         // [nG][nhm]: Hermite index of the sum of two triples
-    unsigned short *r12row;     // [6][nhm]: Hermite index of h + e_I + e_J
+    uint4 *r12row;              // [nhm]: Hermite indices of h + e_I + e_J, 16 bits each
     unsigned char *lst;         // Hermite indices of the boxes' entries
-    int *slot;
+    struct KetRef *ket;         // [kMaxKets]: the tile's kets to compute
+    int *slot;                  // [2]: tile index, kets to compute
 };
+
+// A ket shell pair of the current tile.
+struct KetRef {
+    long long eoff, rowoff, col, col_rev;    // col_rev: its column for the transposed block, < 0: none
+    int ppoff, id, mir, pad;                 // mir: transposed block into W2
+};
+constexpr int kMaxKets = kMaxTileKets;
 
 __host__ __device__ inline int up16(int n) { return (n + 15) & ~15; }
 size_t plan_tables(const Plan &p) {
     return (size_t)up16(p.nTab * 8) + up16(p.nTab * 4) + up16(p.nhm * 4) + up16(p.nG * p.nhm * 2) +
-           up16(6 * p.nhm * 2) + up16(p.nLst) + 16;
+           p.nhm * 16 + up16(p.nLst) + kMaxKets * (int)sizeof(KetRef) + 16;
 }
 size_t plan_smem(const Plan &p) { return plan_tables(p) + (size_t)p.pool; }
 
@@ -507,8 +513,9 @@ __device__ inline BlockSmem carve(char *sm, const Plan &p) {
     b.trip = (int *)sm; sm += up16(p.nTab * 4);
     b.box = (int *)sm; sm += up16(p.nhm * 4);
     b.hs = (unsigned short *)sm; sm += up16(p.nG * p.nhm * 2);
-    b.r12row = (unsigned short *)sm; sm += up16(6 * p.nhm * 2);
+    b.r12row = (uint4 *)sm; sm += p.nhm * 16;
     b.lst = (unsigned char *)sm; sm += up16(p.nLst);
+    b.ket = (KetRef *)sm; sm += kMaxKets * sizeof(KetRef);
     b.slot = (int *)sm;
     return b;
 }
@@ -551,12 +558,9 @@ __device__ void build_tables(const Plan &p, BlockSmem &b) {
             for (int x = 0; x <= t; ++x)
                 for (int y = 0; y <= u; ++y)
                     for (int z = 0; z <= v; ++z) b.lst[at++] = (unsigned char)hidx(x, y, z);
-            b.r12row[h] = (unsigned short)hidx(t + 2, u, v);
-            b.r12row[p.nhm + h] = (unsigned short)hidx(t + 1, u + 1, v);
-            b.r12row[2 * p.nhm + h] = (unsigned short)hidx(t + 1, u, v + 1);
-            b.r12row[3 * p.nhm + h] = (unsigned short)hidx(t, u + 2, v);
-            b.r12row[4 * p.nhm + h] = (unsigned short)hidx(t, u + 1, v + 1);
-            b.r12row[5 * p.nhm + h] = (unsigned short)hidx(t, u, v + 2);
+            b.r12row[h] = make_uint4(hidx(t + 2, u, v) | (hidx(t + 1, u + 1, v) << 16),
+                                     hidx(t + 1, u, v + 1) | (hidx(t, u + 2, v) << 16),
+                                     hidx(t, u + 1, v + 1) | (hidx(t, u, v + 2) << 16), 0u);
         }
     }
     __syncthreads();
@@ -580,58 +584,82 @@ __host__ __device__ inline Shape quartet_shape(int Lx, int Ly, bool gauge) {
             t_rows(Lx, gauge), gauge ? 7 : 1};
 }
 
-// How a quartet is cut to fit the pool: [headers][even tensors][T | odd tensors][G].
-// T of a group is written after the group's recursion has read the odd tensors
-// and read before the next group writes them, so the two share their bytes
-// unless T has to last over several runs of inner primitive pairs (nkc < nk2).
+// How the quartets of a tile (one bra pair, kets of one kind) are cut to fit the
+// pool: [headers][even tensors][T | odd tensors][G].  T of a group is written after
+// the group's recursion has read the odd tensors and read before the next group
+// writes them, so the two share their bytes unless T has to last over several runs
+// of inner primitive pairs (nkc < nk2).
 struct Cut {
     int xch, ych;        // function pairs of X, Y at a time
     int nkc;             // twos of inner primitive pairs at a time
+    int nb;              // kets at a time
     int nij, nijH;       // outer primitive pairs per group, per header pass
 };
+constexpr int kTensorBytes = 112 * 1024;
 __host__ __device__ inline int cut_bytes(const Shape &s, int nk2, int xch, int ych, int nkc, int nij, int nijH) {
     const int yp = (ych + 1) & ~1;
     const int t = nij * s.nT * yp * 8, o = s.nO * nij * nkc * 16;
     return s.hs * nijH * nkc * 16 + s.nE * nij * nkc * 16 + (nkc < nk2 ? t + o : (t > o ? t : o)) +
            s.NC * xch * yp * 8;
 }
-// The cut depends on the quartet and the pool only; it decides no rounding
-// unless the inner primitive pairs are cut (contractions of dozens of
-// primitives), which a larger pool of another class's maxima does not change as
-// long as the tensors of one outer primitive pair take half the pool at most.
-__host__ __device__ inline Cut partition(const Shape &s, int nppx, int nfpx, int nk2y, int nfpy, int nchy, int pool,
-                                         int threads) {
+// The cut decides no rounding except where the inner primitive pairs are cut (nkc,
+// contractions of dozens of primitives), and that depends on the quartet alone:
+// headers and tensors of one outer primitive pair take at most kTensorBytes, half
+// of the largest pool.  Several kets, then several outer primitive pairs are taken at a time until
+// the ket pass has work for four rounds of the CTA: a small quartet alone leaves
+// most lanes of every phase idle and pays each phase's latency for itself.
+__host__ __device__ inline Cut partition(const Shape &s, int nppx, int nfpx, int nppy, int nfpy, int nchy, int nkets,
+                                         int pool, int threads) {
     Cut c;
+    const int nk2y = (nppy + 1) / 2;
     c.xch = nfpx;
     c.ych = nfpy;
     c.nkc = nk2y > 1 ? nk2y : 1;
+    c.nb = 1;
     const int nk2 = c.nkc;
-    while (c.nkc > 1 && (s.hs + s.nE + s.nO) * 16 > pool / 2 / c.nkc) c.nkc = (c.nkc + 1) / 2;
+    while (c.nkc > 1 && (s.hs + s.nE + s.nO) * 16 > kTensorBytes / c.nkc) c.nkc = (c.nkc + 1) / 2;
     while (cut_bytes(s, nk2, c.xch, c.ych, c.nkc, 1, 1) > pool) {
         if (c.ych > 4) c.ych = (c.ych + 1) / 2;
         else if (c.xch > 4) c.xch = (c.xch + 1) / 2;
-        else if (c.nkc > 1) c.nkc = (c.nkc + 1) / 2;
         else if (c.ych > 2) c.ych = 2;
         else if (c.xch > 1) c.xch = (c.xch + 1) / 2;
         else break;
     }
-    // outer primitive pairs per group: enough ket-pass items for four rounds of the CTA
-    int nij = (4 * threads + s.nT * nchy - 1) / (s.nT * nchy);
-    if (nij > nppx) nij = nppx;
-    if (nij < 1) nij = 1;
-    while (nij > 1 && cut_bytes(s, nk2, c.xch, c.ych, c.nkc, nij, nij) > pool) --nij;
-    const int groups = nppx > 0 ? (nppx + nij - 1) / nij : 1;
-    c.nij = nppx > 0 ? (nppx + groups - 1) / groups : 1;
-    c.nijH = c.nij;
-    if (c.nkc == nk2) {
+    const int np = nppx > 1 ? nppx : 1, items = s.nT * nchy, want = 4 * threads;
+    if (c.nkc == nk2 && c.xch == nfpx && c.ych == nfpy) {
+        const int one = cut_bytes(s, nk2, c.xch, c.ych, c.nkc, 1, np);
+        int nb = (want + items - 1) / items;
+        const int nbh = (2 * threads + np * nppy - 1) / (np * (nppy > 1 ? nppy : 1));   // two header rounds
+        if (nb < nbh) nb = nbh;
+        if (nb > nkets) nb = nkets;
+        if (nb > pool / one) nb = pool / one;
+        if (nb > 1) {
+            const int groups = (nkets + nb - 1) / nb;
+            c.nb = (nkets + groups - 1) / groups;
+        }
+    }
+    int nij = (want + items * c.nb - 1) / (items * c.nb);
+    if (nij > np) nij = np;
+    while (nij > 1 && c.nb * cut_bytes(s, nk2, c.xch, c.ych, c.nkc, nij, c.nb > 1 ? np : nij) > pool) --nij;
+    const int groups = (np + nij - 1) / nij;
+    c.nij = (np + groups - 1) / groups;
+    c.nijH = c.nb > 1 ? np : c.nij;
+    if (c.nb == 1 && c.nkc == nk2) {
         const int rest = pool - cut_bytes(s, nk2, c.xch, c.ych, c.nkc, c.nij, 0);
         int h = rest / (s.hs * c.nkc * 16);
-        if (h > nppx) h = nppx;
-        if (h < nppx) h = h / c.nij * c.nij;
+        if (h > np) h = np;
+        if (h < np) h = h / c.nij * c.nij;
         if (h > c.nij) c.nijH = h;
     }
     return c;
 }
+
+// it / d for it d < 2^32 by a multiply-high with ceil(2^32 / d) (d = 1: the identity).
+struct FastDiv {
+    unsigned d, magic;
+    __device__ explicit FastDiv(int n) : d((unsigned)n), magic(n > 1 ? 0xFFFFFFFFu / (unsigned)n + 1u : 0u) {}
+    __device__ int div(int it) const { return magic ? (int)__umulhi((unsigned)it, magic) : it; }
+};
 
 // Device tables of the shell pairs.
 struct PairTables {
@@ -662,7 +690,7 @@ template <> __device__ __forceinline__ const f32x2 *e_entries<kF32>(const PairTa
 template <int A, int M, int NK>
 __device__ __forceinline__ void ket_item(const typename Arith<A>::Vec *R, int Q2, const unsigned short *hs,
                                          const unsigned char *lst, int cnt, const typename Arith<A>::Vec *E,
-                                         long long estride, int nk2, int nk, bool odd, float2 (&out)[M],
+                                         int estride, int nk2, int nk, bool odd, float2 (&out)[M],
                                          double (&outd)[M]) {
     typedef typename Arith<A>::Vec Vec;
     const int n = NK > 0 ? NK : nk;
@@ -706,9 +734,8 @@ __device__ __forceinline__ void ket_item(const typename Arith<A>::Vec *R, int Q2
             for (int p = 0; p < (NK > 0 ? NK : 1); ++p) {
                 for (int q = p; q < n; q += (NK > 0 ? n : 1)) {
                     const Vec rv = r[q];
-                    const Vec nr = make_ulonglong2(neg2(rv.x), neg2(rv.y));
 #pragma unroll
-                    for (int m = 0; m < M; ++m) df_madd2(rv, nr, __ldg(E + m * estride + q), ah[m], al[m]);
+                    for (int m = 0; m < M; ++m) df_madd2(rv, __ldg(E + m * estride + q), ah[m], al[m]);
                 }
             }
             E += nk2;
@@ -741,7 +768,7 @@ __device__ __forceinline__ void ket_item(const typename Arith<A>::Vec *R, int Q2
 template <int A, int M>
 __device__ __forceinline__ void ket_store(const typename Arith<A>::Vec *R, int Q2, const unsigned short *hs,
                                           const unsigned char *lst, int cnt, const typename Arith<A>::Vec *E,
-                                          long long estride, int nk2, int nk, bool odd, bool neg, bool add, char *T,
+                                          int estride, int nk2, int nk, bool odd, bool neg, bool add, char *T,
                                           int at, int plane) {
     float2 s[M];
     double sd[M];
@@ -763,112 +790,129 @@ __device__ __forceinline__ void ket_store(const typename Arith<A>::Vec *R, int Q
     }
 }
 
-// The block (X|Y), chunk by chunk; emit(x0, xch, y0, ych, value) is called by all
-// threads once the chunk's results stand in shared memory, value(c, x, y) being
-// component c of function pairs x, y (sorted order, relative to the chunk).
+// The blocks (X|Y) of one bra pair AB and `nkets` ket pairs b.ket[] of CD's kind (X =
+// CD when swap), some kets and chunks at a time; emit(ket0, nb, x0, xch, y0, ych,
+// value) is called by all threads once a group's results stand in shared memory,
+// value(ket, c, x, y) being component c of function pairs x, y (sorted order,
+// relative to the chunk).
 // Components: 0 Coulomb; gauge kernel 1..6: (xy|d_I d_J r|zw), IJ = xx, xy, xz, yy, yz, zz.
 template <bool GAUGE, int A, class Emit>
-__device__ void quartet_block(const PairTables &tb, const PairDev &X, const PairDev &Y, const Plan &pl, BlockSmem &b,
-                              Emit emit) {
+__device__ void quartet_blocks(const PairTables &tb, const PairDev &AB, const PairDev &CD, bool swap, int nkets,
+                               const Plan &pl, BlockSmem &b, Emit emit) {
     typedef typename Arith<A>::Vec Vec;
     typedef typename Arith<A == kF64 ? kF64 : kDF>::Vec HVec;      // headers: FP64 or pairs
     constexpr int NC = GAUGE ? 7 : 1;
     const int tid = threadIdx.x, nt = blockDim.x;
+    const PairDev &X = swap ? CD : AB, &Y = swap ? AB : CD;
     const int Lx = X.Lab, Ly = Y.Lab, L = Lx + Ly, Lr = L + 2, Ltop = GAUGE ? Lr : L;
+    const int nppx = X.npp, nppy = Y.npp, nk2x = X.nk2, nk2y = Y.nk2;
     const int nhx = nherm(Lx);
     const Shape sh = quartet_shape(Lx, Ly, GAUGE);
-    const Cut c = partition(sh, X.npp, X.nfp, Y.nk2, Y.nfp, Y.nch, pl.pool, nt);
+    const Cut c = partition(sh, nppx, X.nfp, nppy, Y.nfp, Y.nch, nkets, pl.pool, nt);
     const int nE_C = nherm(L), nO_C = odd_len(L);       // entries before the r12 tensor
     const FuncPair *fx = tb.fp + X.fpoff;
     const PairChunk *cy = tb.ch + Y.choff;
-    const Vec *EX = e_entries<A>(tb) + X.eoff, *EY = e_entries<A>(tb) + Y.eoff;
-    const bool lastodd = Y.npp & 1;
+    const Vec *E0 = e_entries<A>(tb);
+    const long long eAB = AB.eoff;
+    const int pAB = AB.ppoff, nfpx = X.nfp, nchy = Y.nch;
 
     HVec *H = reinterpret_cast<HVec *>(b.pool);
-    Vec *Re = reinterpret_cast<Vec *>(b.pool + (size_t)sh.hs * c.nijH * c.nkc * 16);
-    char *U = reinterpret_cast<char *>(Re) + (size_t)sh.nE * c.nij * c.nkc * 16;
-    const bool runs = c.nkc < Y.nk2;
+    Vec *Re = reinterpret_cast<Vec *>(b.pool + (size_t)sh.hs * c.nb * c.nijH * c.nkc * 16);
+    char *U = reinterpret_cast<char *>(Re) + (size_t)sh.nE * c.nb * c.nij * c.nkc * 16;
+    const bool runs = c.nkc < nk2y;
     Vec *Ro = reinterpret_cast<Vec *>(U);
     const int ypmax = (c.ych + 1) & ~1;
-    const int tbytes = c.nij * sh.nT * ypmax * 8, obytes = sh.nO * c.nij * c.nkc * 16;
+    const int tbytes = c.nb * c.nij * sh.nT * ypmax * 8, obytes = sh.nO * c.nb * c.nij * c.nkc * 16;
     char *T = runs ? U + obytes : U;
     char *G = U + (runs ? tbytes + obytes : max(tbytes, obytes));
 
-    for (int c0 = 0; c0 < Y.nch;) {
+    for (int ket0 = 0; ket0 < nkets; ket0 += c.nb) {
+    const int nb = min(c.nb, nkets - ket0);
+    const KetRef *kets = b.ket + ket0;
+    for (int c0 = 0; c0 < nchy;) {
         const int y0 = cy[c0].k0;
-        int c1 = c0;
-        while (c1 < Y.nch && cy[c1].k0 + cy[c1].m - y0 <= c.ych) ++c1;
-        const int ych = cy[c1 - 1].k0 + cy[c1 - 1].m - y0, yp = (ych + 1) & ~1, nyp = yp >> 1;
-        for (int x0 = 0; x0 < X.nfp; x0 += c.xch) {
-            const int xch = min(c.xch, X.nfp - x0);
-            const int gplane = NC * xch * yp;               // FP32 pairs: high parts, then low parts
+        int c1 = nchy, ych = Y.nfp - y0;
+        if (ych > c.ych) {
+            c1 = c0;
+            while (cy[c1].k0 + cy[c1].m - y0 <= c.ych) ++c1;
+            ych = cy[c1 - 1].k0 + cy[c1 - 1].m - y0;
+        }
+        const int yp = (ych + 1) & ~1;
+        for (int x0 = 0; x0 < nfpx; x0 += c.xch) {
+            const int xch = min(c.xch, nfpx - x0);
+            const int gket = NC * xch * yp, gplane = nb * gket;     // FP32 pairs: high parts, then low parts
             for (int i = tid; i < gplane; i += nt) {
                 if (A == kF64) reinterpret_cast<double *>(G)[i] = 0.0;
                 else reinterpret_cast<float2 *>(G)[i] = make_float2(0.f, 0.f);
             }
-            for (int ih = 0; ih < X.npp; ih += c.nijH) {
-                const int nijH = min(c.nijH, X.npp - ih);
-                for (int k0 = 0; k0 < Y.nk2; k0 += c.nkc) {
-                    const int nk = min(c.nkc, Y.nk2 - k0);
-                    const bool odd = lastodd && k0 + nk == Y.nk2;
-                    const int QH = nijH * nk;
-                    // Q - P, Boys values and prefactors of the primitive quartets
+            for (int ih = 0; ih < nppx; ih += c.nijH) {
+                const int nijH = min(c.nijH, nppx - ih);
+                for (int k0 = 0; k0 < nk2y; k0 += c.nkc) {
+                    const int nk = min(c.nkc, nk2y - k0);
+                    const bool odd = (nppy & 1) && k0 + nk == nk2y;
+                    const int QH = nb * nijH * nk;
                     __syncthreads();                        // the last recursion has read the headers
-                    for (int q = tid; q < 2 * QH; q += nt) {
-                        const int ij = q / (2 * nk), r = q - ij * 2 * nk, kl = 2 * k0 + r;
-                        const int at = ij * nk + (r >> 1);
-                        if constexpr (A == kF64) {
-                            const HeadF64 h{reinterpret_cast<double *>(H + at) + (r & 1), 2 * QH};
-                            if (kl < Y.npp) {
-                                quartet_header<GAUGE>(tb.boys, tb.pp + X.ppoff + ih + ij, tb.pp + Y.ppoff + kl, L, h);
+                    {
+                        // Q - P, Boys values and prefactors of the primitive quartets
+                        const FastDiv dk(2 * nk), dij(nijH);
+                        for (int q = tid; q < 2 * QH; q += nt) {
+                            const int o = dk.div(q), r = q - o * 2 * nk, kl = 2 * k0 + r;
+                            const int bk = dij.div(o), ij = ih + o - bk * nijH;
+                            const int pk = kets[bk].ppoff;
+                            const PrimPairDev *px = tb.pp + (swap ? pk : pAB) + ij, *py = tb.pp + (swap ? pAB : pk) + kl;
+                            const int at = o * nk + (r >> 1);
+                            if constexpr (A == kF64) {
+                                const HeadF64 h{reinterpret_cast<double *>(H + at) + (r & 1), 2 * QH};
+                                if (kl < nppy) {
+                                    quartet_header<GAUGE>(tb.boys, px, py, L, h);
+                                } else {
+                                    for (int j = 0; j < sh.hs; ++j) h.zero(j);
+                                }
                             } else {
-                                for (int j = 0; j < sh.hs; ++j) h.zero(j);
-                            }
-                        } else {
-                            const HeadPair h{reinterpret_cast<float *>(H + at) + (r & 1), 4 * QH};
-                            if (kl < Y.npp) {
-                                if constexpr (A == kF32 && !GAUGE)
-                                    quartet_header_f32(tb.boys, tb.pp + X.ppoff + ih + ij, tb.pp + Y.ppoff + kl, L, h);
-                                else
-                                    quartet_header_pairs<GAUGE>(tb.boys, tb.pp + X.ppoff + ih + ij,
-                                                                tb.pp + Y.ppoff + kl, L, h);
-                            } else {
-                                for (int j = 0; j < sh.hs; ++j) h.zero(j);
+                                const HeadPair h{reinterpret_cast<float *>(H + at) + (r & 1), 4 * QH};
+                                if (kl < nppy) {
+                                    if constexpr (A == kF32 && !GAUGE) quartet_header_f32(tb.boys, px, py, L, h);
+                                    else quartet_header_pairs<GAUGE>(tb.boys, px, py, L, h);
+                                } else {
+                                    for (int j = 0; j < sh.hs; ++j) h.zero(j);
+                                }
                             }
                         }
                     }
                     __syncthreads();
                     for (int i0 = 0; i0 < nijH; i0 += c.nij) {
                         const int nij = min(c.nij, nijH - i0);
-                        const int Q2 = nij * nk, hoff = i0 * nk;
+                        const int Q2 = nb * nij * nk;
                         // Hermite recursion, one auxiliary order per pass; order 0 ends in Re.
-                        // Items (entry, two of primitive quartets) are the addresses of the
-                        // results, so the stores are contiguous.
+                        // Items (entry, ket, outer primitive pair, two of inner ones) are the
+                        // addresses of the results, so the stores are contiguous.
                         if (Ltop & 1) __syncthreads();      // T, which the odd tensors overwrite, has been read
-                        const unsigned magic = Q2 > 1 ? 0xFFFFFFFFu / (unsigned)Q2 + 1u : 0u;
+                        const FastDiv dq(Q2), db1(nij * nk);
+                        const int hskip = (nijH - nij) * nk, hoff = i0 * nk;
                         for (int m = Ltop; m >= 0; --m) {
                             const int cC = m <= L ? nherm(L - m) : 0;
                             const int cR = GAUGE ? nherm(Lr - m) : 0;
                             Vec *dst = (m & 1) ? Ro : Re;
                             const Vec *src = (m & 1) ? Re : Ro;
-                            const int dR = ((m & 1) ? nO_C : nE_C), sR = ((m & 1) ? nE_C : nO_C);
+                            const int dR = ((m & 1) ? nO_C : nE_C) * Q2, sR = ((m & 1) ? nE_C : nO_C) * Q2;
+                            const int jC = (3 + m) * QH, jR = (4 + L + m) * QH;
                             for (int it = tid; it < (cC + cR) * Q2; it += nt) {
-                                // it / Q2 by a multiply-high (exact: it Q2 < 2^32)
-                                const int e = Q2 > 1 ? (int)__umulhi((unsigned)it, magic) : it;
+                                const int e = dq.div(it);
                                 const int q = it - e * Q2;
+                                const int hq = q + hoff + (nb > 1 ? db1.div(q) * hskip : 0);
                                 const bool r12 = GAUGE && e >= cC;
                                 const int h = r12 ? e - cC : e;
-                                const int db = r12 ? dR : 0, sb = r12 ? sR : 0;
                                 Vec r;
                                 if (h == 0) {
-                                    const HVec v = H[(r12 ? 4 + L + m : 3 + m) * QH + hoff + q];
+                                    const HVec v = H[(r12 ? jR : jC) + hq];
                                     if constexpr (A == kF32) r = v.x;
                                     else r = v;
                                 } else {
                                     const int2 sw = b.src[h];
-                                    const HVec xv = H[(sw.x & 3) * QH + hoff + q];
-                                    const Vec a = src[(sb + ((sw.x >> 2) & 1023)) * Q2 + q];
-                                    const Vec cc = src[(sb + (sw.x >> 12)) * Q2 + q];
+                                    const Vec *sp = src + (r12 ? sR : 0) + q;
+                                    const HVec xv = H[(sw.x & 3) * QH + hq];
+                                    const Vec a = sp[((sw.x >> 2) & 1023) * Q2];
+                                    const Vec cc = sp[(sw.x >> 12) * Q2];
                                     const float cf = __int_as_float(sw.y);
                                     if constexpr (A == kF64) {
                                         const double cd = (double)cf;
@@ -879,102 +923,135 @@ __device__ void quartet_block(const PairTables &tb, const PairDev &X, const Pair
                                         r = fma2(xv.x, a, mul2(pack2(cf, cf), cc));
                                     }
                                 }
-                                dst[(db + h) * Q2 + q] = r;
+                                dst[(r12 ? dR - cC * Q2 : 0) + it] = r;
                             }
                             __syncthreads();
                         }
                         // ket pass: T rows h < nhx from the Coulomb tensor, then (gauge) rows
                         // g = 4.. from the r12 tensor
-                        const int nrows = nij * sh.nT;
+                        const int nrows = nb * nij * sh.nT;
                         const int tplane = nrows * yp;
-                        for (int it = tid; it < nrows * (c1 - c0); it += nt) {
-                            const int ci = it / nrows, row = it - ci * nrows;
-                            const int ij = row / sh.nT, hh = row - ij * sh.nT;
-                            const PairChunk k = cy[c0 + ci];
-                            const bool r12 = GAUGE && hh >= nhx;
-                            const int g = r12 ? hh - nhx + 4 : hh;
-                            const int tr = b.trip[g];
-                            const bool neg = ((tr ^ (tr >> 8) ^ (tr >> 16)) & 1) != 0;      // |g| odd
-                            const int bx = b.box[k.box], cnt = bx >> 16;
-                            const Vec *R = Re + (r12 ? nE_C : 0) * Q2 + ij * nk;
-                            const Vec *E = EY + (long long)k.off * Y.nk2 + k0;
-                            const int at = row * yp + k.k0 - y0;
-                            if (k.m == 2)
-                                ket_store<A, 2>(R, Q2, b.hs + g * pl.nhm, b.lst + (bx & 0xffff), cnt, E,
-                                                (long long)cnt * Y.nk2, Y.nk2, nk, odd, neg, k0 > 0, T, at, tplane);
-                            else
-                                ket_store<A, 1>(R, Q2, b.hs + g * pl.nhm, b.lst + (bx & 0xffff), cnt, E, 0, Y.nk2, nk,
-                                                odd, neg, k0 > 0, T, at, tplane);
+                        {
+                            const FastDiv drow(nrows), dT(sh.nT), dnij(nij);
+                            for (int it = tid; it < nrows * (c1 - c0); it += nt) {
+                                const int ci = drow.div(it), row = it - ci * nrows;
+                                const int o = dT.div(row), hh = row - o * sh.nT;
+                                const PairChunk k = cy[c0 + ci];
+                                const bool r12 = GAUGE && hh >= nhx;
+                                const int g = r12 ? hh - nhx + 4 : hh;
+                                const int tr = b.trip[g];
+                                const bool neg = ((tr ^ (tr >> 8) ^ (tr >> 16)) & 1) != 0;      // |g| odd
+                                const int bx = b.box[k.box], cnt = bx >> 16;
+                                const Vec *R = Re + (r12 ? nE_C : 0) * Q2 + o * nk;
+                                const long long ey = swap ? eAB : kets[dnij.div(o)].eoff;
+                                const Vec *E = E0 + ey + (k.off * nk2y + k0);
+                                const int at = row * yp + k.k0 - y0;
+                                if (k.m == 2)
+                                    ket_store<A, 2>(R, Q2, b.hs + g * pl.nhm, b.lst + (bx & 0xffff), cnt, E,
+                                                    cnt * nk2y, nk2y, nk, odd, neg, k0 > 0, T, at, tplane);
+                                else
+                                    ket_store<A, 1>(R, Q2, b.hs + g * pl.nhm, b.lst + (bx & 0xffff), cnt, E, 0, nk2y,
+                                                    nk, odd, neg, k0 > 0, T, at, tplane);
+                            }
                         }
                         __syncthreads();
-                        if (k0 + nk < Y.nk2) continue;      // T is not complete yet (then nijH == nij)
+                        if (k0 + nk < nk2y) continue;       // T is not complete yet (then nijH == nij)
                         // bra pass, outer primitive pairs in order (the group size changes no rounding):
-                        // G[c][x][y] += sum_ij sum_{j in box x} E^{ij}_x[j] T[ij][row(c, h_j)][y]
-                        if constexpr (A == kF64) {
-                            for (int it = tid; it < NC * xch * ych; it += nt) {
-                                const int cx = it / ych, y = it - cx * ych, cc = cx / xch, x = cx - cc * xch;
-                                const FuncPair f = fx[x0 + x];
-                                const int bx = b.box[f.fp >> 16], cnt = bx >> 16;
-                                const unsigned char *lst = b.lst + (bx & 0xffff);
-                                double *g = reinterpret_cast<double *>(G) + (size_t)cx * yp + y;
-                                double s = *g;
+                        // G[c][x][y] += sum_ij sum_{j in box x} E^{ij}_x[j] T[ij][row(c, h_j)][y];
+                        // a thread sums all components of one x and one y (FP64) or two (packed)
+                        const int ny = A == kF64 ? ych : yp >> 1;
+                        const FastDiv dy(ny), dx(xch);
+                        for (int it = tid; it < nb * xch * ny; it += nt) {
+                            const int bx_ = dy.div(it), bk = dx.div(bx_), x = bx_ - bk * xch;
+                            const int y = (it - bx_ * ny) * (A == kF64 ? 1 : 2);
+                            const FuncPair f = fx[x0 + x];
+                            const int bx = b.box[f.fp >> 16], cnt = bx >> 16;
+                            const unsigned char *lst = b.lst + (bx & 0xffff);
+                            const Vec *ex = E0 + (swap ? kets[bk].eoff : eAB) + f.off * nk2x;
+                            const int gi = bk * gket + x * yp + y, gc = xch * yp;
+                            if constexpr (A == kF64) {
+                                double s[NC];
+                                double *g = reinterpret_cast<double *>(G) + gi;
+#pragma unroll
+                                for (int cc = 0; cc < NC; ++cc) s[cc] = g[cc * gc];
                                 for (int i = 0; i < nij; ++i) {
                                     const int ij = ih + i0 + i;
-                                    const double *e = reinterpret_cast<const double *>(
-                                        EX + (long long)f.off * X.nk2 + (ij >> 1)) + (ij & 1);
-                                    const double *t = reinterpret_cast<const double *>(T) + (size_t)i * sh.nT * yp + y;
+                                    const double *e = reinterpret_cast<const double *>(ex + (ij >> 1)) + (ij & 1);
+                                    const double *t = reinterpret_cast<const double *>(T) +
+                                                      (bk * nij + i) * sh.nT * yp + y;
+                                    const double *tr12 = t + (nhx - 4) * yp;
+#pragma unroll 2
                                     for (int j = 0; j < cnt; ++j) {
                                         const int h = lst[j];
-                                        const int row = (GAUGE && cc) ? nhx - 4 + b.r12row[(cc - 1) * pl.nhm + h] : h;
-                                        s = fma(__ldg(e), t[row * yp], s);
-                                        e += 2 * X.nk2;
-                                    }
-                                }
-                                *g = s;
-                            }
-                        } else {
-                            for (int it = tid; it < NC * xch * nyp; it += nt) {
-                                const int cx = it / nyp, y = 2 * (it - cx * nyp), cc = cx / xch, x = cx - cc * xch;
-                                const FuncPair f = fx[x0 + x];
-                                const int bx = b.box[f.fp >> 16], cnt = bx >> 16;
-                                const unsigned char *lst = b.lst + (bx & 0xffff);
-                                float *g = reinterpret_cast<float *>(G) + (size_t)cx * yp + y;
-                                f32x2 sh_ = *reinterpret_cast<const f32x2 *>(g), sl_ = 0;
-                                if (A == kDF) sl_ = *reinterpret_cast<const f32x2 *>(g + gplane);
-                                for (int i = 0; i < nij; ++i) {
-                                    const int ij = ih + i0 + i;
-                                    const float *e = reinterpret_cast<const float *>(
-                                        EX + (long long)f.off * X.nk2 + (ij >> 1)) + (ij & 1);
-                                    const float *t = reinterpret_cast<const float *>(T) + (size_t)i * sh.nT * yp + y;
-                                    for (int j = 0; j < cnt; ++j) {
-                                        const int h = lst[j];
-                                        const int row = (GAUGE && cc) ? nhx - 4 + b.r12row[(cc - 1) * pl.nhm + h] : h;
-                                        const float *tr = t + row * yp;
-                                        if constexpr (A == kDF) {
-                                            const float eh = __ldg(e), el = __ldg(e + 2);
-                                            const ulonglong2 ev = make_ulonglong2(pack2(eh, eh), pack2(el, el));
-                                            const ulonglong2 tv =
-                                                make_ulonglong2(*reinterpret_cast<const f32x2 *>(tr),
-                                                                *reinterpret_cast<const f32x2 *>(tr + tplane));
-                                            df_madd2(ev, make_ulonglong2(neg2(ev.x), neg2(ev.y)), tv, sh_, sl_);
-                                            e += 4 * X.nk2;
-                                        } else {
-                                            const float eh = __ldg(e);
-                                            sh_ = fma2(pack2(eh, eh), *reinterpret_cast<const f32x2 *>(tr), sh_);
-                                            e += 2 * X.nk2;
+                                        const double ev = __ldg(e + 2 * j * nk2x);
+                                        s[0] = fma(ev, t[h * yp], s[0]);
+                                        if constexpr (GAUGE) {
+                                            const uint4 w = b.r12row[h];
+                                            s[1] = fma(ev, tr12[(w.x & 0xffff) * yp], s[1]);
+                                            s[2] = fma(ev, tr12[(w.x >> 16) * yp], s[2]);
+                                            s[3] = fma(ev, tr12[(w.y & 0xffff) * yp], s[3]);
+                                            s[4] = fma(ev, tr12[(w.y >> 16) * yp], s[4]);
+                                            s[5] = fma(ev, tr12[(w.z & 0xffff) * yp], s[5]);
+                                            s[6] = fma(ev, tr12[(w.z >> 16) * yp], s[6]);
                                         }
                                     }
                                 }
-                                *reinterpret_cast<f32x2 *>(g) = sh_;
-                                if (A == kDF) *reinterpret_cast<f32x2 *>(g + gplane) = sl_;
+#pragma unroll
+                                for (int cc = 0; cc < NC; ++cc) g[cc * gc] = s[cc];
+                            } else {
+                                f32x2 ah[NC], al[NC];
+                                float *g = reinterpret_cast<float *>(G) + gi;
+#pragma unroll
+                                for (int cc = 0; cc < NC; ++cc) {
+                                    ah[cc] = *reinterpret_cast<const f32x2 *>(g + cc * gc);
+                                    al[cc] = A == kDF ? *reinterpret_cast<const f32x2 *>(g + gplane + cc * gc) : 0;
+                                }
+                                for (int i = 0; i < nij; ++i) {
+                                    const int ij = ih + i0 + i;
+                                    const float *e = reinterpret_cast<const float *>(ex + (ij >> 1)) + (ij & 1);
+                                    const float *t = reinterpret_cast<const float *>(T) +
+                                                     (bk * nij + i) * sh.nT * yp + y;
+                                    const float *tr12 = t + (nhx - 4) * yp;
+                                    constexpr int es = A == kDF ? 4 : 2;        // floats per two of primitive pairs
+#pragma unroll 2
+                                    for (int j = 0; j < cnt; ++j) {
+                                        const int h = lst[j];
+                                        const float eh = __ldg(e + es * j * nk2x);
+                                        const float el = A == kDF ? __ldg(e + es * j * nk2x + 2) : 0.f;
+                                        const ulonglong2 ev = make_ulonglong2(pack2(eh, eh), pack2(el, el));
+                                        auto term = [&](const float *tr, f32x2 &sh_, f32x2 &sl_) {
+                                            const f32x2 th = *reinterpret_cast<const f32x2 *>(tr);
+                                            if constexpr (A == kDF)
+                                                df_madd2(ev, make_ulonglong2(th, *reinterpret_cast<const f32x2 *>(tr + tplane)),
+                                                         sh_, sl_);
+                                            else
+                                                sh_ = fma2(ev.x, th, sh_);
+                                        };
+                                        term(t + h * yp, ah[0], al[0]);
+                                        if constexpr (GAUGE) {
+                                            const uint4 w = b.r12row[h];
+                                            term(tr12 + (w.x & 0xffff) * yp, ah[1], al[1]);
+                                            term(tr12 + (w.x >> 16) * yp, ah[2], al[2]);
+                                            term(tr12 + (w.y & 0xffff) * yp, ah[3], al[3]);
+                                            term(tr12 + (w.y >> 16) * yp, ah[4], al[4]);
+                                            term(tr12 + (w.z & 0xffff) * yp, ah[5], al[5]);
+                                            term(tr12 + (w.z >> 16) * yp, ah[6], al[6]);
+                                        }
+                                    }
+                                }
+#pragma unroll
+                                for (int cc = 0; cc < NC; ++cc) {
+                                    *reinterpret_cast<f32x2 *>(g + cc * gc) = ah[cc];
+                                    if (A == kDF) *reinterpret_cast<f32x2 *>(g + gplane + cc * gc) = al[cc];
+                                }
                             }
                         }
                     }
                 }
             }
             __syncthreads();
-            emit(x0, xch, y0, ych, [&](int cc, int x, int y) -> double {
-                const int i = (cc * xch + x) * yp + y;
+            emit(ket0, nb, x0, xch, y0, ych, [&](int bk, int cc, int x, int y) -> double {
+                const int i = bk * gket + (cc * xch + x) * yp + y;
                 if constexpr (A == kF64) return reinterpret_cast<const double *>(G)[i];
                 const float *g = reinterpret_cast<const float *>(G);
                 return (double)g[i] + (double)g[gplane + i];
@@ -983,91 +1060,113 @@ __device__ void quartet_block(const PairTables &tb, const PairDev &X, const Pair
         }
         c0 = c1;
     }
+    }
 }
 
 // Screened rows as a persistent kernel: every CTA builds its tables once, then
-// takes tiles (bra shell pair x range of sorted ket positions) from the shared
-// counter until none are left.  A tile's parameter set comes from prms[req],
+// takes tiles (bra shell pair x kets of one kind, from the bucket list) from the
+// shared counter until none are left.  A tile's parameter set comes from prms[req],
 // so one launch can mix the tiles of several transformations.
 template <bool GAUGE, bool DF>
-__global__ void __launch_bounds__(256, 2) eri_rows_kernel(const EriParams *prms, const EriTask *tasks, int ntasks,
-                                                          int *next, Plan pl) {
+__global__ void __launch_bounds__(256, 2) eri_rows_kernel(const EriParams *prms, const EriTask *tasks,
+                                                          int *queue, Plan pl) {
     extern __shared__ __align__(16) char sm[];
     BlockSmem b = carve(sm, pl);
     build_tables(pl, b);
+    const int nt = queue[1];
     const int ij_of[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
     for (;;) {
-        if (threadIdx.x == 0) *b.slot = atomicAdd(next, 1);
+        if (threadIdx.x == 0) *b.slot = atomicAdd(queue, 1);
         __syncthreads();
         const int t = *b.slot;
-        __syncthreads();
-        if (t >= ntasks) break;
+        if (t >= nt) break;
         const EriTask tk = tasks[t];
         const EriParams &prm = prms[tk.req];
-        const PairDev AB = prm.pairs[tk.bra_sp];
-        const PairTables tb{prm.pp, prm.E, prm.E2, prm.E1, prm.fp, prm.ch, prm.boys};
-        for (int kp = tk.k0; kp < tk.k1; ++kp) {
-            const int cd_id = prm.ket_sp[kp];
-            const PairDev CD = prm.pairs[cd_id];
-            const long long col = prm.ket_col[kp];
-            // (CD|AB) also kept?  Then one block serves both (EriParams::sym):
-            // rev writes it at (cd, ab) of W, mir into W2 for a later batch
-            const bool both = prm.sym && cd_id != tk.bra_sp && prm.ket_pos[tk.bra_sp] < prm.prefix[cd_id];
-            bool rev = both, mir = false;
-            if (both && prm.sym == 2) {
-                const int bp = prm.bra_pos[cd_id];
-                if (bp < prm.b0) continue;           // its transpose came from W2 of CD's batch
-                rev = bp < prm.b1;
-                mir = !rev;
+        // the tile's kets that are computed here, in list order (first warp)
+        if (threadIdx.x < 32) {
+            bool use = (int)threadIdx.x < tk.k1 - tk.k0;
+            KetRef k{};
+            if (use) {
+                const int kp = prm.bucket[tk.k0 + threadIdx.x];
+                const int cd = prm.ket_sp[kp];
+                const PairDev &p = prm.pairs[cd];
+                k.id = cd;
+                k.eoff = p.eoff;
+                k.rowoff = p.rowoff;
+                k.ppoff = p.ppoff;
+                k.col = prm.ket_col[kp];
+                // (CD|AB) also kept?  Then one block serves both (EriParams::sym):
+                // rev writes it at (cd, ab) of W, mir into W2 for a later batch
+                const bool both = prm.sym && cd != tk.bra_sp && prm.ket_pos[tk.bra_sp] < prm.prefix[cd];
+                bool rev = both;
+                if (both && prm.sym == 2) {
+                    const int bp = prm.bra_pos[cd];
+                    if (bp < prm.b0) use = false;        // its transpose came from W2 of CD's batch
+                    rev = bp < prm.b1;
+                    k.mir = !rev;
+                }
+                if (rev && cd < tk.bra_sp) use = false;
+                k.col_rev = rev ? prm.ket_col[prm.ket_pos[tk.bra_sp]] : -1;
             }
-            if (rev && cd_id < tk.bra_sp) continue;
-            const long long col_rev = rev ? prm.ket_col[prm.ket_pos[tk.bra_sp]] : 0;
+            const unsigned mask = __ballot_sync(0xffffffffu, use);
+            if (use) b.ket[__popc(mask & ((1u << threadIdx.x) - 1u))] = k;
+            if (threadIdx.x == 0) b.slot[1] = __popc(mask);
+        }
+        __syncthreads();
+        const int nkets = b.slot[1];
+        if (nkets > 0) {
+            const PairDev AB = prm.pairs[tk.bra_sp];
+            const PairDev CD = prm.pairs[b.ket[0].id];      // all kets of the tile are of its kind
+            const PairTables tb{prm.pp, prm.E, prm.E2, prm.E1, prm.fp, prm.ch, prm.boys};
             // contract the orientation with fewer multiply-adds; swapped -> the block is (CD|AB)
             const bool swap = orient_madds(CD, AB, GAUGE) < orient_madds(AB, CD, GAUGE);
-            const PairDev &X = swap ? CD : AB, &Y = swap ? AB : CD;
-            double *W = prm.W, *Wc = prm.Wc;
-            const long long ldw = prm.ldw, ldwc = prm.ldwc, row0 = prm.row0;
-            const bool wc = prm.with_coulomb != 0;
-            auto emit = [&](int x0, int xch, int y0, int ych, auto value) {
-                for (int idx = threadIdx.x; idx < xch * ych; idx += blockDim.x) {
-                    const int xx = idx / ych, yy = idx - xx * ych;
-                    const int fx = prm.fp[X.fpoff + x0 + xx].fp & 0xffff, fy = prm.fp[Y.fpoff + y0 + yy].fp & 0xffff;
+            auto emit = [&](int ket0, int nb, int x0, int xch, int y0, int ych, auto value) {
+                const FuncPair *fpx = prm.fp + (swap ? CD.fpoff : AB.fpoff) + x0;
+                const FuncPair *fpy = prm.fp + (swap ? AB.fpoff : CD.fpoff) + y0;
+                const long long ldw = prm.ldw, ldwc = prm.ldwc, row0 = prm.row0;
+                const bool wc = prm.with_coulomb != 0;
+                const FastDiv dy(ych), dx(xch);
+                for (int idx = threadIdx.x; idx < nb * xch * ych; idx += blockDim.x) {
+                    const int bx = dy.div(idx), yy = idx - bx * ych, bk = dx.div(bx), xx = bx - bk * xch;
+                    const int fx = fpx[xx].fp & 0xffff, fy = fpy[yy].fp & 0xffff;
                     const int a = swap ? fy : fx;                // bra function pair
                     const int c = swap ? fx : fy;                // ket function pair
-                    const double C = value(0, xx, yy);
+                    const KetRef &k = b.ket[ket0 + bk];
+                    const double C = value(bk, 0, xx, yy);
                     double hc[6];
                     if (GAUGE)
 #pragma unroll
-                        for (int j = 0; j < 6; ++j) hc[j] = value(j + 1, xx, yy);
+                        for (int j = 0; j < 6; ++j) hc[j] = value(bk, j + 1, xx, yy);
                     // the block's entry into row `r`, column `k` of an output
                     // (gauge: rows (r, I), columns (k, J); K_IJ is symmetric, so the
                     // transposed entry needs no index change)
-                    auto put = [&](double *Wo, long long ldo, double *Wco, long long ldco, long long r, long long k) {
+                    auto put = [&](double *Wo, long long ldo, double *Wco, long long ldco, long long r, long long kc) {
                         if (!GAUGE) {
-                            Wo[r * ldo + k] = C;
+                            Wo[r * ldo + kc] = C;
                         } else {
 #pragma unroll
                             for (int I = 0; I < 3; ++I)
 #pragma unroll
                                 for (int J = 0; J < 3; ++J)
-                                    Wo[(r * 3 + I) * ldo + k * 3 + J] = (I == J ? C : 0.0) - hc[ij_of[I][J]];
-                            if (wc) Wco[r * ldco + k] = C;
+                                    Wo[(r * 3 + I) * ldo + kc * 3 + J] = (I == J ? C : 0.0) - hc[ij_of[I][J]];
+                            if (wc) Wco[r * ldco + kc] = C;
                         }
                     };
-                    put(W, ldw, Wc, ldwc, AB.rowoff + a - row0, col + c);
+                    put(prm.W, ldw, prm.Wc, ldwc, AB.rowoff + a - row0, k.col + c);
                     // the same integrals at (cd, ab): rows of CD, columns of AB
-                    if (rev) put(W, ldw, Wc, ldwc, CD.rowoff + c - row0, col_rev + a);
-                    if (mir) put(prm.W2, prm.ldw2, prm.Wc2, prm.ldwc2, CD.rowoff + c - prm.row2,
-                                 prm.col2[tk.bra_sp] + a);
+                    if (k.col_rev >= 0) put(prm.W, ldw, prm.Wc, ldwc, k.rowoff + c - row0, k.col_rev + a);
+                    if (k.mir) put(prm.W2, prm.ldw2, prm.Wc2, prm.ldwc2, k.rowoff + c - prm.row2,
+                                   prm.col2[tk.bra_sp] + a);
                 }
             };
             if constexpr (DF) {
-                if (tk.f32) quartet_block<GAUGE, kF32>(tb, X, Y, pl, b, emit);
-                else quartet_block<GAUGE, kDF>(tb, X, Y, pl, b, emit);
+                if (tk.f32) quartet_blocks<GAUGE, kF32>(tb, AB, CD, swap, nkets, pl, b, emit);
+                else quartet_blocks<GAUGE, kDF>(tb, AB, CD, swap, nkets, pl, b, emit);
             } else {
-                quartet_block<GAUGE, kF64>(tb, X, Y, pl, b, emit);
+                quartet_blocks<GAUGE, kF64>(tb, AB, CD, swap, nkets, pl, b, emit);
             }
         }
+        __syncthreads();
     }
 }
 
@@ -1083,8 +1182,9 @@ Plan eri_plan(int maxnfp, int maxLab, int maxnpp, bool gauge) {
     p.nhm = nherm(maxLab);
     p.nG = nherm(maxLab + (gauge ? 2 : 0));
     p.nLst = box_entries_below(maxLab + 1);
-    const int npp = std::max(maxnpp, 1), nk2 = (npp + 1) / 2, nfp = std::max(maxnfp, 1);
+    const int npp = std::max(maxnpp, 1), nfp = std::max(maxnfp, 1);
     const Shape s = quartet_shape(maxLab, maxLab, gauge);
+    const int nk2 = std::max(1, std::min((npp + 1) / 2, kTensorBytes / ((s.hs + s.nE + s.nO) * 16)));
     const long long tables = (long long)plan_tables(p);
     auto bytes = [&](long long nij, long long nijH) {        // cut_bytes in 64 bits
         const long long yp = (nfp + 1) / 2 * 2, t = nij * s.nT * yp * 8, o = s.nO * nij * nk2 * 16;
@@ -1115,29 +1215,29 @@ int resident_ctas(int threads, size_t smem) {
 }
 
 template <bool GAUGE, bool DF>
-void launch_rows(const EriParams *prms, const EriTask *tasks, int ntasks, int *next, const Plan &pl, int threads,
+void launch_rows(const EriParams *prms, const EriTask *tasks, int maxtasks, int *queue, const Plan &pl, int threads,
                  size_t smem, cudaStream_t s) {
     QDT_CUDA_TRY(cudaFuncSetAttribute(eri_rows_kernel<GAUGE, DF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem));
-    const int grid = min(ntasks, resident_ctas<GAUGE, DF>(threads, smem));
-    QDT_CUDA_TRY(cudaMemsetAsync(next, 0, sizeof(int), s));
-    eri_rows_kernel<GAUGE, DF><<<grid, threads, smem, s>>>(prms, tasks, ntasks, next, pl);
+    const int grid = min(maxtasks, resident_ctas<GAUGE, DF>(threads, smem));
+    QDT_CUDA_TRY(cudaMemsetAsync(queue, 0, sizeof(int), s));
+    eri_rows_kernel<GAUGE, DF><<<grid, threads, smem, s>>>(prms, tasks, queue, pl);
 }
 }  // namespace
 
-void launch_eri(const EriParams *prms, const EriTask *tasks, int ntasks, int *next, const EriShape &shape,
+void launch_eri(const EriParams *prms, const EriTask *tasks, int maxtasks, int *queue, const EriShape &shape,
                 bool gauge, bool df, const EriLaunch &how, cudaStream_t s) {
-    if (ntasks <= 0) return;
+    if (maxtasks <= 0) return;
     const Plan pl = eri_plan(shape.maxnfp, shape.maxLab, shape.maxnpp, gauge);
     const size_t smem = plan_smem(pl);
     const int threads = how.threads > 0 ? how.threads : pl.threads;
     if (threads % 32 || threads > 256) throw Error{QDT_ERR_ARG, "integral kernel: threads must be 32..256, a multiple of 32"};
     if (gauge) {
-        if (df) launch_rows<true, true>(prms, tasks, ntasks, next, pl, threads, smem, s);
-        else launch_rows<true, false>(prms, tasks, ntasks, next, pl, threads, smem, s);
+        if (df) launch_rows<true, true>(prms, tasks, maxtasks, queue, pl, threads, smem, s);
+        else launch_rows<true, false>(prms, tasks, maxtasks, queue, pl, threads, smem, s);
     } else {
-        if (df) launch_rows<false, true>(prms, tasks, ntasks, next, pl, threads, smem, s);
-        else launch_rows<false, false>(prms, tasks, ntasks, next, pl, threads, smem, s);
+        if (df) launch_rows<false, true>(prms, tasks, maxtasks, queue, pl, threads, smem, s);
+        else launch_rows<false, false>(prms, tasks, maxtasks, queue, pl, threads, smem, s);
     }
     QDT_CHECK_KERNEL("eri_rows_kernel");
 }
@@ -1181,11 +1281,14 @@ __global__ void __launch_bounds__(256, 2) schwarz_kernel(PairTables tb, const Pa
     const PairDev AB = pairs[blockIdx.x];
     BlockSmem b = carve(sm, pl);
     build_tables(pl, b);
+    if (threadIdx.x == 0) b.ket[0] = KetRef{AB.eoff, 0, 0, -1, AB.ppoff, (int)blockIdx.x, 0, 0};
+    __syncthreads();
     double qmax = 0.0;
-    quartet_block<false, kF64>(tb, AB, AB, pl, b, [&](int x0, int xch, int y0, int ych, auto value) {
+    quartet_blocks<false, kF64>(tb, AB, AB, false, 1, pl, b,
+                                [&](int, int, int x0, int xch, int y0, int ych, auto value) {
         for (int x = threadIdx.x; x < xch; x += blockDim.x) {
             const int y = x0 + x - y0;
-            if (y >= 0 && y < ych) qmax = fmax(qmax, sqrt(fabs(value(0, x, y))));
+            if (y >= 0 && y < ych) qmax = fmax(qmax, sqrt(fabs(value(0, 0, x, y))));
         }
     });
     double *red = reinterpret_cast<double *>(b.pool);       // the block's last use of the pool is over

@@ -119,4 +119,43 @@ inline BatchKets batch_kets(const std::vector<int> &order, const std::vector<int
     return b;
 }
 
+// Ket positions of a list grouped by the bucket of their shell pair (pairs whose
+// quartets with one bra pair are alike), ascending within a bucket: the kets of a
+// bucket that a bra pair keeps, a prefix of the w-sorted list, are then a prefix
+// of the bucket.  Empty buckets are left out.
+struct KetBuckets {
+    std::vector<int> pos;       // ket positions, bucket by bucket
+    std::vector<int> first;     // first entry of each bucket in pos; one more at the end
+};
+
+inline KetBuckets ket_buckets(const std::vector<int> &list, const std::vector<int> &bucket_of, int nbucket) {
+    KetBuckets k;
+    std::vector<int> count(nbucket + 1, 0);
+    for (int sp : list) ++count[bucket_of[sp] + 1];
+    k.first.push_back(0);
+    for (int b = 0; b < nbucket; ++b) {
+        if (count[b + 1]) k.first.push_back(k.first.back() + count[b + 1]);
+        count[b + 1] += count[b];
+    }
+    k.pos.resize(list.size());
+    for (int p = 0; p < (int)list.size(); ++p) k.pos[count[bucket_of[list[p]]]++] = p;
+    return k;
+}
+
+// Entries of each bucket below every ket position, for the tiles cut on the host.
+struct BucketCounts {
+    int n = 0;
+    std::vector<int> below;     // [buckets][n + 1]
+    explicit BucketCounts(const KetBuckets &k) : n((int)k.pos.size()) {
+        const int nb = (int)k.first.size() - 1;
+        below.assign((size_t)nb * (n + 1), 0);
+        for (int b = 0; b < nb; ++b) {
+            int *c = &below[(size_t)b * (n + 1)];
+            for (int i = k.first[b]; i < k.first[b + 1]; ++i) c[k.pos[i] + 1] = 1;
+            for (int p = 0; p < n; ++p) c[p + 1] += c[p];
+        }
+    }
+    int operator()(int b, int pos) const { return below[(size_t)b * (n + 1) + pos]; }
+};
+
 }  // namespace qdt

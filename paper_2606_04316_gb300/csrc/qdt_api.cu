@@ -171,6 +171,8 @@ struct qdt_ctx {
     // ket list of a row batch with bra-ket symmetry: pairs, columns, list position,
     // kept prefix and FP32 split point per pair in list positions
     DBuf klist, kcol1, kpos1, kpre1, ksplit1;
+    // ket positions by bucket and the buckets' first entries (ket_buckets)
+    DBuf kbpos, kbfirst;
     PinnedArena pin;            // page-locked staging of a transformation's uploads
     SplitWorkspace split;
     // first-half route of the Coulomb block: density (Eq. firsthalf) or the
@@ -284,70 +286,128 @@ std::vector<int> tile_order(const PairClass &pc, std::vector<int> v, int order) 
     return v;
 }
 
-// Tiles: each bra pair's kept ket prefix cut into runs of `kets` positions.
-// Tiles of `kets` sorted ket positions per bra pair; with `split`, positions
+// Tiles of at most tile_kets() kets of one bucket per bra pair (list: shell pair at
+// each ket position); with `split`, positions
 // [0, split) and [split, prefix) are tiled apart, the second set in plain FP32.
-void build_tiles(const std::vector<int> &bras, const std::vector<int> &prefix, int kets, int req,
-                 std::vector<EriTask> &out, const std::vector<int> *split = nullptr) {
-    for (int sp : bras) {
-        const int mid = split ? (*split)[sp] : prefix[sp];
-        for (int q = 0; q < mid; q += kets) out.push_back({sp, q, std::min(mid, q + kets), req, 0});
-        for (int q = mid; q < prefix[sp]; q += kets) out.push_back({sp, q, std::min(prefix[sp], q + kets), req, 1});
-    }
+void build_tiles(const PairClass &pc, const std::vector<int> &bras, const std::vector<int> &prefix,
+                 const KetBuckets &kb, const BucketCounts &below, const std::vector<int> &list, bool gauge,
+                 const EriLaunch &how, int req, std::vector<EriTask> &out, const std::vector<int> *split = nullptr) {
+    for (int sp : bras)
+        for (int b = 0; b + 1 < (int)kb.first.size(); ++b) {
+            const PairDev &CD = pc.h_pairs[list[kb.pos[kb.first[b]]]];
+            const int kets = tile_kets(pc.h_pairs[sp], CD, gauge, how.budget, how.kets);
+            const int f = kb.first[b], pre = f + below(b, prefix[sp]), mid = split ? f + below(b, (*split)[sp]) : pre;
+            for (int q = f; q < mid; q += kets) out.push_back({sp, q, std::min(mid, q + kets), req, 0});
+            for (int q = mid; q < pre; q += kets) out.push_back({sp, q, std::min(pre, q + kets), req, 1});
+        }
 }
 
-// The same tiles written on the device, one warp per bra pair: bras[i] (tile
-// order) starts at tile off[i]; its kept prefix and FP32 split point come from
-// the device copies of the screening outcome (split null: no FP32 tiles).
-// Only the bra list and the offsets are uploaded, not the tiles.
-__global__ void build_tiles_kernel(const int *bras, const long long *off, const int *prefix, const int *split,
-                                   int n, int kets, int req, EriTask *out) {
-    const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// The same tiles written on the device, one warp per bra pair (tile order), lanes
+// over the buckets: the kets of a bucket below the kept prefix and the FP32 split
+// point are found by bisection (split null: no FP32 tiles).  First pass (out null):
+// tiles of each bra pair into count; their exclusive sums are the second pass's
+// offsets, so only the bra list is uploaded, not the tiles.
+__device__ inline int bucket_below(const int *pos, int lo, int hi, int p) {
+    while (lo < hi) {
+        const int m = (lo + hi) >> 1;
+        if (pos[m] < p) lo = m + 1; else hi = m;
+    }
+    return lo;
+}
+__global__ void tiles_kernel(const PairDev *pairs, const int *bras, const int *prefix, const int *split,
+                             const int *list, const int *pos, const int *first, int nbucket, int n, bool gauge,
+                             EriLaunch how, const int *off, int *count, EriTask *out) {
+    const int w = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (w >= n) return;
-    const int sp = bras[w];
-    const int pre = prefix[sp], mid = split ? split[sp] : pre;
-    const int n1 = (mid + kets - 1) / kets, n2 = (pre - mid + kets - 1) / kets;
-    EriTask *o = out + off[w];
-    for (int j = lane; j < n1 + n2; j += 32) {
-        EriTask t;
-        t.bra_sp = sp;
-        t.req = req;
-        if (j < n1) {
-            t.k0 = j * kets;
-            t.k1 = min(mid, t.k0 + kets);
-            t.f32 = 0;
-        } else {
-            t.k0 = mid + (j - n1) * kets;
-            t.k1 = min(pre, t.k0 + kets);
-            t.f32 = 1;
+    const int sp = bras[w], p_end = prefix[sp], p_mid = split ? split[sp] : p_end;
+    const PairDev AB = pairs[sp];
+    int done = out ? off[w] : 0;
+    for (int b0 = 0; b0 < nbucket; b0 += 32) {
+        const int b = b0 + lane;
+        int f = 0, mid = 0, pre = 0, kets = 1;
+        if (b < nbucket) {
+            f = first[b];
+            kets = tile_kets(AB, pairs[list[pos[f]]], gauge, how.budget, how.kets);
+            pre = bucket_below(pos, f, first[b + 1], p_end);
+            mid = split ? bucket_below(pos, f, pre, p_mid) : pre;
         }
-        o[j] = t;
+        const int n1 = (mid - f + kets - 1) / kets, n2 = (pre - mid + kets - 1) / kets;
+        int x = n1 + n2;                                    // inclusive scan over the lanes
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (out) {
+            EriTask *o = out + done + x - n1 - n2;
+            for (int q = f; q < mid; q += kets) *o++ = EriTask{sp, q, min(mid, q + kets), 0, 0};
+            for (int q = mid; q < pre; q += kets) *o++ = EriTask{sp, q, min(pre, q + kets), 0, 1};
+        }
+        done += __shfl_sync(0xffffffffu, x, 31);
     }
+    if (!out && lane == 0) count[w] = done;
 }
 
-// Host side of build_tiles_kernel: per-bra tile offsets (from the host copy of
-// the screening outcome), the uploads, the launch; returns the tile count.
-int launch_build_tiles(qdt_ctx *ctx, const std::vector<int> &bras, const std::vector<int> &prefix,
-                       const std::vector<int> *split, const int *d_prefix, const int *d_split, int kets,
-                       EriTask *&d_tiles, cudaStream_t s) {
-    std::vector<long long> off(bras.size() + 1, 0);
-    for (size_t i = 0; i < bras.size(); ++i) {
-        const int sp = bras[i], pre = prefix[sp], mid = split ? (*split)[sp] : pre;
-        off[i + 1] = off[i] + (mid + kets - 1) / kets + (pre - mid + kets - 1) / kets;
+// In place: count[i] -> sum of the counts before i; the total into *total.  One CTA.
+__global__ void __launch_bounds__(1024) tile_scan_kernel(int *count, int n, int *total) {
+    __shared__ int wsum[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int carry = 0;
+    for (int base = 0; base < n; base += 1024) {
+        const int i = base + threadIdx.x;
+        const int v = i < n ? count[i] : 0;
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[w] = x;
+        __syncthreads();
+        if (w == 0) {
+            int t = wsum[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, t, o);
+                if (lane >= o) t += y;
+            }
+            wsum[lane] = t;
+        }
+        __syncthreads();
+        if (i < n) count[i] = carry + (w > 0 ? wsum[w - 1] : 0) + x - v;
+        carry += wsum[31];
+        __syncthreads();
     }
-    const long long nt = off.back();
-    if (nt > 0x7fffffffLL) throw Error{QDT_ERR_ARG, "integral tiles: more than 2^31 tiles in one batch"};
-    d_tiles = (EriTask *)ctx->tasks.get((size_t)std::max<long long>(1, nt) * sizeof(EriTask));
-    if (nt == 0) return 0;
+    if (threadIdx.x == 0) *total = carry;
+}
+
+// Host side: the uploads and launches; tiles into ctx->tasks, their number into
+// queue[1].  Returns a bound on it: full tiles of the smallest size and, for every
+// bucket of a bra pair, at most two part tiles.
+int launch_build_tiles(qdt_ctx *ctx, const std::vector<int> &bras, const std::vector<int> &prefix, int nbucket,
+                       const PairDev *d_pairs, const int *d_prefix, const int *d_split, const int *d_list,
+                       const int *d_pos, const int *d_first, bool gauge, const EriLaunch &how, int *queue,
+                       EriTask *&d_tiles, cudaStream_t s) {
+    long long most = 0;
+    for (int sp : bras) most += prefix[sp] / how.least + std::min<long long>(2LL * nbucket, prefix[sp]);
+    if (most > 0x7fffffffLL) throw Error{QDT_ERR_ARG, "integral tiles: more than 2^31 tiles in one batch"};
+    d_tiles = (EriTask *)ctx->tasks.get((size_t)std::max<long long>(1, most) * sizeof(EriTask));
+    if (most == 0) return 0;
+    const int n = (int)bras.size();
     const int *d_bras = dcopy_pinned(ctx->pin, ctx->tbras, bras, s);
-    const long long *d_off = dcopy_pinned(ctx->pin, ctx->toff, off, s);
-    const long long threads = 32LL * (long long)bras.size();
-    build_tiles_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(d_bras, d_off, d_prefix, split ? d_split : nullptr,
-                                                                          (int)bras.size(), kets, 0, d_tiles);
-    QDT_CHECK_KERNEL("build_tiles_kernel");
-    ctx->launches++;
-    return (int)nt;
+    int *d_off = (int *)ctx->toff.get((size_t)n * sizeof(int));
+    const unsigned grid = (unsigned)((32LL * n + 255) / 256);
+    tiles_kernel<<<grid, 256, 0, s>>>(d_pairs, d_bras, d_prefix, d_split, d_list, d_pos, d_first, nbucket, n, gauge, how,
+                                      nullptr, d_off, nullptr);
+    QDT_CHECK_KERNEL("tiles_kernel");
+    tile_scan_kernel<<<1, 1024, 0, s>>>(d_off, n, queue + 1);
+    QDT_CHECK_KERNEL("tile_scan_kernel");
+    tiles_kernel<<<grid, 256, 0, s>>>(d_pairs, d_bras, d_prefix, d_split, d_list, d_pos, d_first, nbucket, n, gauge, how,
+                                      d_off, nullptr, d_tiles);
+    QDT_CHECK_KERNEL("tiles_kernel");
+    ctx->launches += 3;
+    return (int)most;
 }
 
 // ---------------------------------------------------------------- autotuner
@@ -355,8 +415,8 @@ int launch_build_tiles(qdt_ctx *ctx, const std::vector<int> &bras, const std::ve
 // class maxima), chosen by timing on a sample of the class: every 8th bra
 // pair of the bra order (an eighth of the work, so that every candidate runs
 // many tiles per CTA slot).  The search is coordinate-wise from (plan threads,
-// 8 kets, bra order), after one warm-up run: ket positions per tile
-// {2, 4, 8, 16}, then CTA threads {128, 256}, then the tile order; each
+// 32 kets, most expensive first), after one warm-up run: kets per tile at most
+// {8, 16, 32}, then CTA threads {128, 256}, then the tile order; each
 // candidate keeps the faster of two timings.  The candidates differ only in how the work is cut and scheduled,
 // never in the arithmetic of an integral, so the choice changes no result bit.
 // Process-wide cache; QDT_AUTOTUNE=0 keeps the start point, QDT_AUTOTUNE_VERBOSE=1
@@ -380,15 +440,37 @@ bool env_flag(const char *name, bool dflt) {
 
 EriLaunch eri_launch_for(qdt_ctx *ctx, const PairClass &pc, const EriShape &shape, bool gauge, bool df,
                          const EriParams *d_prm, const std::vector<int> &bras, const std::vector<int> &prefix,
-                         cudaStream_t s) {
+                         const KetBuckets &kb, const std::vector<int> &list, long long quartets, cudaStream_t s) {
+    int nsm = 0;
+    QDT_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
     EriLaunch def;
     def.threads = eri_default_threads(shape, gauge);
-    def.kets = 8;
-    def.order = 0;
+    // a tile may cost a 32nd of a CTA slot's share of the work (4 slots per SM; about
+    // half of the kept quartets are computed, the others are their transposes), so
+    // that the queue ends evenly
+    double mean = 0.0, weight = 0.0;
+    for (int i = 0; i + 1 < (int)kb.first.size(); ++i)
+        for (int j = 0; j + 1 < (int)kb.first.size(); ++j) {
+            const double w = (double)(kb.first[i + 1] - kb.first[i]) * (kb.first[j + 1] - kb.first[j]);
+            mean += w * (double)quartet_cost(pc.h_pairs[list[kb.pos[kb.first[i]]]], pc.h_pairs[list[kb.pos[kb.first[j]]]],
+                                             gauge);
+            weight += w;
+        }
+    if (weight > 0.0) {
+        def.budget = std::max<long long>(1, (long long)(mean / weight * 0.5 * (double)quartets / (4.0 * nsm * 32.0)));
+        def.least = def.kets;
+        for (int i : pc.bucket_rep)
+            for (int j : pc.bucket_rep)
+                def.least = std::min(def.least, tile_kets(pc.h_pairs[i], pc.h_pairs[j], gauge, def.budget, def.kets));
+    }
     if (const char *pin = std::getenv("QDT_ERI_LAUNCH")) {
         EriLaunch p = def;
         if (std::sscanf(pin, "%d,%d,%d", &p.threads, &p.kets, &p.order) == 3 && p.threads > 0 && p.kets > 0)
-            return p;
+            {
+                p.kets = std::min(p.kets, kMaxTileKets);
+                p.least = std::min(p.kets, p.least);
+                return p;
+            }
         throw Error{QDT_ERR_ARG, "QDT_ERI_LAUNCH must read threads,kets,order"};
     }
     if (!env_flag("QDT_AUTOTUNE", true)) return def;
@@ -397,10 +479,13 @@ EriLaunch eri_launch_for(qdt_ctx *ctx, const PairClass &pc, const EriShape &shap
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune.find(key);
-        if (it != g_tune.end()) return it->second;
+        if (it != g_tune.end()) {
+            EriLaunch how = it->second;
+            how.budget = def.budget;
+            how.least = std::min(how.kets, def.least);
+            return how;
+        }
     }
-    int nsm = 0;
-    QDT_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
     long long total = 0;
     for (int sp : bras) total += prefix[sp];
     // too little work to tell the candidates apart: fewer than ~64 tiles per CTA slot in the sample
@@ -410,17 +495,20 @@ EriLaunch eri_launch_for(qdt_ctx *ctx, const PairClass &pc, const EriShape &shap
     cudaEvent_t e0, e1;
     QDT_CUDA_TRY(cudaEventCreate(&e0));
     QDT_CUDA_TRY(cudaEventCreate(&e1));
-    int *next = (int *)ctx->next.get(sizeof(int));
+    int *queue = (int *)ctx->next.get(2 * sizeof(int));
+    const BucketCounts below(kb);
     // each candidate runs the sample twice and keeps the faster time: the
     // candidates differ by a few per cent, about the spread of one timing
     auto time_of = [&](const EriLaunch &how) {
         std::vector<EriTask> tk;
-        build_tiles(tile_order(pc, sample, how.order), prefix, how.kets, 0, tk);
+        build_tiles(pc, tile_order(pc, sample, how.order), prefix, kb, below, list, gauge, how, 0, tk);
         EriTask *d_tk = dcopy(ctx->tasks, tk, s);
+        const int n = (int)tk.size();
+        QDT_CUDA_TRY(cudaMemcpyAsync(queue + 1, &n, sizeof n, cudaMemcpyHostToDevice, s));
         float ms = 0.f;
         for (int rep = 0; rep < 2; ++rep) {
             QDT_CUDA_TRY(cudaEventRecord(e0, s));
-            launch_eri(d_prm, d_tk, (int)tk.size(), next, shape, gauge, df, how, s);
+            launch_eri(d_prm, d_tk, n, queue, shape, gauge, df, how, s);
             QDT_CUDA_TRY(cudaEventRecord(e1, s));
             QDT_CUDA_TRY(cudaEventSynchronize(e1));
             float t = 0.f;
@@ -440,9 +528,9 @@ EriLaunch eri_launch_for(qdt_ctx *ctx, const PairClass &pc, const EriShape &shap
         const float ms = time_of(c);
         if (ms < best_ms) { best_ms = ms; best = c; }
     };
-    for (int k : {2, 4, 16}) { EriLaunch c = best; c.kets = k; consider(c); }
+    for (int k : {8, 16}) { EriLaunch c = best; c.kets = k; consider(c); }
     { EriLaunch c = best; c.threads = best.threads == 128 ? 256 : 128; consider(c); }
-    { EriLaunch c = best; c.order = 1; consider(c); }
+    { EriLaunch c = best; c.order = 0; consider(c); }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -471,6 +559,7 @@ void build_class(qdt_ctx *ctx, int c) {
     std::vector<FuncPair> fptab;
     std::vector<PairChunk> chtab;
     std::map<std::tuple<int, int, int, int, bool>, PairKind> kinds;
+    std::map<std::pair<int, int>, int> buckets;         // (kind, primitive pairs)
     long long eoff = 0, M = 0;
     for (int i = 0; i < pc.nsp; ++i) {
         const ShellDev &A = ctx->h_shells[sp[i].first], &B = ctx->h_shells[sp[i].second];
@@ -502,6 +591,9 @@ void build_class(qdt_ctx *ctx, int c) {
             }
         pr.npp = (int)hpp.size() - pr.ppoff;
         pr.nk2 = (pr.npp + 1) / 2;
+        const auto bk = buckets.emplace(std::make_pair(pr.fpoff, pr.npp), (int)buckets.size());
+        if (bk.second) pc.bucket_rep.push_back(i);
+        pc.h_bucket.push_back(bk.first->second);
         pr.eoff = eoff;
         eoff += (long long)pr.nbox * pr.nk2;
         pc.maxnpp = std::max(pc.maxnpp, pr.npp);
@@ -600,6 +692,8 @@ struct ClassPlan {
     std::vector<double> h_Dmax;
     std::vector<long long> h_col, Krow;
     size_t wbudget = 0;
+    KetBuckets kb;                // the ket list's positions by bucket, and on the device
+    int *d_kbpos = nullptr, *d_kbfirst = nullptr;
 };
 
 // Steps 2-3 for the current P.Dmax: ket order and kept prefixes (copied to
@@ -805,6 +899,11 @@ void class_finish(qdt_ctx *ctx, ClassPlan &P, qdt_stats *st) {
     for (int q = 0; q < pc.nsp; ++q) P.h_kpos[P.h_ketsp[q]] = q;
     P.d_kpos = (P.one_batch || P.mirror) ? dcopy_pinned(ctx->pin, ctx->kpos, P.h_kpos, s) : nullptr;
     P.d_split = P.precision == QDT_SPLIT ? dcopy_pinned(ctx->pin, ctx->dsplit, P.h_split, s) : nullptr;
+    if (!P.mirror) {        // row batches with bra-ket symmetry have their own lists (batch_kets_prepare)
+        P.kb = ket_buckets(P.h_ketsp, pc.h_bucket, (int)pc.bucket_rep.size());
+        P.d_kbpos = dcopy_pinned(ctx->pin, ctx->kbpos, P.kb.pos, s);
+        P.d_kbfirst = dcopy_pinned(ctx->pin, ctx->kbfirst, P.kb.first, s);
+    }
 }
 
 // One batch of bra rows of a class.
@@ -829,6 +928,10 @@ struct RowBatch {
     std::vector<long long> krow1;
     int *d_list = nullptr, *d_pos1 = nullptr, *d_pre1 = nullptr, *d_split1 = nullptr;
     long long *d_col1 = nullptr;
+    KetBuckets kb;                          // the batch's ket list by bucket (ClassPlan's, or its own)
+    std::vector<int> own_list;              // its own list, with bra-ket symmetry across batches
+    const std::vector<int> &list(const ClassPlan &P) const { return P.mirror ? own_list : P.h_ketsp; }
+    int *d_kbpos = nullptr, *d_kbfirst = nullptr;
 };
 
 // The ket list of a row batch with bra-ket symmetry (plan.h batch_kets): the
@@ -854,6 +957,10 @@ void batch_kets_prepare(qdt_ctx *ctx, const ClassPlan &P, RowBatch &B) {
     }
     B.krow1.assign(pc.nsp, 0);
     for (int sp : B.bras) B.krow1[sp] = col1[B.pre1[sp]];
+    B.own_list = bk.list;
+    B.kb = ket_buckets(bk.list, pc.h_bucket, (int)pc.bucket_rep.size());
+    B.d_kbpos = dcopy_pinned(ctx->pin, ctx->kbpos, B.kb.pos, s);
+    B.d_kbfirst = dcopy_pinned(ctx->pin, ctx->kbfirst, B.kb.first, s);
     B.d_list = dcopy_pinned(ctx->pin, ctx->klist, bk.list, s);
     B.d_col1 = dcopy_pinned(ctx->pin, ctx->kcol1, col1, s);
     B.d_pos1 = dcopy_pinned(ctx->pin, ctx->kpos1, bk.pos, s);
@@ -972,6 +1079,11 @@ void batch_prepare(qdt_ctx *ctx, const ClassPlan &P, int b0, RowBatch &B) {
         kmax = 0;
         for (int sp : B.bras) kmax = std::max(kmax, B.krow1[sp]);
     }
+    if (!P.mirror) {
+        B.kb = P.kb;
+        B.d_kbpos = P.d_kbpos;
+        B.d_kbfirst = P.d_kbfirst;
+    }
     B.kmax = kmax;
     B.ldw = std::max<long long>(kmax, 1) * mult;
     B.W = (double *)ctx->W.get((size_t)std::max<long long>(rows, 1) * mult * B.ldw * sizeof(double));
@@ -989,6 +1101,7 @@ void batch_prepare(qdt_ctx *ctx, const ClassPlan &P, int b0, RowBatch &B) {
     prm.boys = (const double *)ctx->boys.p;
     prm.ket_sp = P.mirror ? B.d_list : P.ketsp;
     prm.ket_col = P.mirror ? B.d_col1 : P.ketcol;
+    prm.bucket = B.d_kbpos;
     prm.W = B.W;
     prm.ldw = B.ldw;
     prm.row0 = B.row0;
@@ -1305,12 +1418,16 @@ void run_batches(qdt_ctx *ctx, ClassPlan &P, long long c0, long long c1, qdt_sta
         const EriShape shape{pc.maxnfp, pc.maxLab, pc.maxnpp};
         const bool df = B.prm.E2 != nullptr;
         const std::vector<int> &pre = P.mirror ? B.pre1 : P.h_prefix;       // in the kernel's ket list
-        const EriLaunch how = eri_launch_for(ctx, pc, shape, B.prm.gauge != 0, df, d_prm, B.bras, pre, s);
+        long long quartets = 0;
+        for (int sp : B.bras) quartets += pre[sp];
+        const EriLaunch how =
+            eri_launch_for(ctx, pc, shape, B.prm.gauge != 0, df, d_prm, B.bras, pre, B.kb, B.list(P), quartets, s);
         EriTask *d_tk = nullptr;
-        const int ntiles = launch_build_tiles(ctx, tile_order(pc, B.bras, how.order), pre,
-                                              df ? (P.mirror ? &B.split1 : &P.h_split) : nullptr,
-                                              P.mirror ? B.d_pre1 : P.prefix, P.mirror ? B.d_split1 : P.d_split,
-                                              how.kets, d_tk, s);
+        int *queue = (int *)ctx->next.get(2 * sizeof(int));
+        const int ntiles = launch_build_tiles(ctx, tile_order(pc, B.bras, how.order), pre, (int)B.kb.first.size() - 1,
+                                              pc.d_pairs, P.mirror ? B.d_pre1 : P.prefix,
+                                              df ? (P.mirror ? B.d_split1 : P.d_split) : nullptr, B.prm.ket_sp, B.d_kbpos,
+                                              B.d_kbfirst, B.prm.gauge != 0, how, queue, d_tk, s);
         int te = tm.n; tm.mark();
         if (P.quarter) {    // the quarter route lays out whole rows
             launch_zero(B.W, B.rows * P.mult * B.ldw, s);
@@ -1320,7 +1437,7 @@ void run_batches(qdt_ctx *ctx, ClassPlan &P, long long c0, long long c1, qdt_sta
         }
         if (B.W2) launch_zero_rows(B.W2, B.ldw2, B.rows2 * P.mult, B.d_kt2, (long long)B.kt2.size(), s);
         if (B.Wc2) launch_zero_rows(B.Wc2, B.ld2, B.rows2, B.d_kg2, (long long)B.kg2.size(), s);
-        launch_eri(d_prm, d_tk, ntiles, (int *)ctx->next.get(sizeof(int)), shape, B.prm.gauge != 0, df, how, s);
+        launch_eri(d_prm, d_tk, ntiles, queue, shape, B.prm.gauge != 0, df, how, s);
         ctx->launches += 2 + (B.Wc ? 1 : 0);
         batch_stats(ctx, P, B, c1 - c0, st);
         int th = tm.n; tm.mark();
@@ -1566,12 +1683,17 @@ void batch_round(qdt_ctx *owner, std::vector<BatchReq> &R, int round, unsigned f
         for (int k = 0; k < kKinds; ++k) {
             if (prms[k].empty()) continue;
             d_prms[k] = dcopy_pinned(owner->pin, owner->bprms[k], prms[k], s0);
-            owner->bnext[k].get(sizeof(int));
+            owner->bnext[k].get(2 * sizeof(int));
             // the tuner samples the first request of this kind
             size_t first = 0;
             while (kind_of(fz[first]->B.prm) != k) ++first;
+            long long quartets = 0;
+            for (BatchReq *r : fz)
+                if (kind_of(r->B.prm) == k)
+                    for (int sp : r->B.bras) quartets += r->P.h_prefix[sp];
             how[k] = eri_launch_for(owner, fz[first]->c->cls[fz[first]->P.cr.c], shape[k], (k & 2) != 0,
-                                    (k & 1) != 0, d_prms[k], fz[first]->B.bras, fz[first]->P.h_prefix, s0);
+                                    (k & 1) != 0, d_prms[k], fz[first]->B.bras, fz[first]->P.h_prefix,
+                                    fz[first]->B.kb, fz[first]->P.h_ketsp, quartets, s0);
             // tile order across requests: request by request in bra order, or
             // all bra pairs most expensive first
             struct Key { double cost; int i; int sp; };
@@ -1584,16 +1706,25 @@ void batch_round(qdt_ctx *owner, std::vector<BatchReq> &R, int round, unsigned f
             }
             if (how[k].order == 1)
                 std::stable_sort(order.begin(), order.end(), [](const Key &a, const Key &b) { return a.cost > b.cost; });
+            std::vector<BucketCounts> below;
+            std::vector<int> at(fz.size(), -1);
+            for (size_t i = 0; i < fz.size(); ++i)
+                if (kind_of(fz[i]->B.prm) == k) {
+                    at[i] = (int)below.size();
+                    below.emplace_back(fz[i]->B.kb);
+                }
+            std::vector<int> one(1);
             for (const Key &o : order) {
-                const std::vector<int> &pre = fz[o.i]->P.h_prefix;
-                const int mid = (k & 1) ? fz[o.i]->P.h_split[o.sp] : pre[o.sp];    // FP32 tail (split form)
-                for (int q = 0; q < mid; q += how[k].kets)
-                    tiles[k].push_back({o.sp, q, std::min(mid, q + how[k].kets), req_of[o.i], 0});
-                for (int q = mid; q < pre[o.sp]; q += how[k].kets)
-                    tiles[k].push_back({o.sp, q, std::min(pre[o.sp], q + how[k].kets), req_of[o.i], 1});
+                const ClassPlan &P = fz[o.i]->P;
+                one[0] = o.sp;
+                build_tiles(fz[o.i]->c->cls[P.cr.c], one, P.h_prefix, fz[o.i]->B.kb, below[at[o.i]], P.h_ketsp, (k & 2) != 0,
+                            how[k], req_of[o.i], tiles[k], (k & 1) ? &P.h_split : nullptr);   // split form: FP32 tail
             }
             d_tiles[k] = dcopy_pinned(owner->pin, owner->btasks[k], tiles[k], s0);
             ntiles[k] = (int)tiles[k].size();
+            void *hn = owner->pin.take(sizeof(int));
+            std::memcpy(hn, &ntiles[k], sizeof(int));
+            QDT_CUDA_TRY(cudaMemcpyAsync((int *)owner->bnext[k].p + 1, hn, sizeof(int), cudaMemcpyHostToDevice, s0));
         }
         for (BatchReq *r : fz) r->c->split.deferred = true;
         QDT_CUDA_TRY(cudaStreamSynchronize(s0));          // uploads done before any capture
@@ -1686,7 +1817,7 @@ void release_workspace(qdt_ctx *c) {
                     &c->next, &c->ktile2, &c->qcols, &c->qWL, &c->qWS, &c->qT1, &c->qT, &c->qVf, &c->qkt[0],
                     &c->qkt[1], &c->qkt[2], &c->W2, &c->Wc2, &c->ktile3, &c->ktile4, &c->col2, &c->ketsp2,
                     &c->ketcol2, &c->Dbra2, &c->tbras, &c->toff, &c->dsplit, &c->klist, &c->kcol1, &c->kpos1,
-                    &c->kpre1, &c->ksplit1};
+                    &c->kpre1, &c->ksplit1, &c->kbpos, &c->kbfirst};
     for (DBuf *b : bufs) b->release();
     split_release(c->split);
     for (GraphEntry &g : c->graph) {
@@ -1744,7 +1875,7 @@ void qdt_destroy(qdt_ctx *c) {
                     &c->qWL, &c->qWS, &c->qT1, &c->qT, &c->qVf, &c->qCr1, &c->qCr2, &c->qkt[0],
                     &c->qkt[1], &c->qkt[2], &c->W2, &c->Wc2, &c->ktile3, &c->ktile4, &c->col2, &c->ketsp2,
                     &c->ketcol2, &c->Dbra2, &c->tbras, &c->toff, &c->dsplit, &c->klist, &c->kcol1, &c->kpos1,
-                    &c->kpre1, &c->ksplit1};
+                    &c->kpre1, &c->ksplit1, &c->kbpos, &c->kbfirst};
     for (DBuf *b : bufs) b->release();
     for (int k = 0; k < 2; ++k) {
         c->cb[k].pairs.release(); c->cb[k].pp.release(); c->cb[k].E.release(); c->cb[k].E2.release(); c->cb[k].E1.release(); c->cb[k].fp.release(); c->cb[k].ch.release();
@@ -1933,21 +2064,24 @@ int qdt_f32_error_ratio(qdt_ctx *c, unsigned blocks, int k_begin, int k_end, dou
             const EriShape shape{pc.maxnfp, pc.maxLab, pc.maxnpp};
             EriLaunch how;
             how.threads = eri_default_threads(shape, B.prm.gauge != 0);
-            const size_t n = (size_t)B.rows * P.mult * B.ldw;
+            const size_t nw = (size_t)B.rows * P.mult * B.ldw;
             struct Bufs {         // released on every exit path
                 DBuf ref, rp, cp, out;
                 ~Bufs() { ref.release(); rp.release(); cp.release(); out.release(); }
             } tmp;
-            double *W2 = (double *)tmp.ref.get(std::max<size_t>(1, n) * sizeof(double));
+            double *W2 = (double *)tmp.ref.get(std::max<size_t>(1, nw) * sizeof(double));
             std::vector<int> none(pc.nsp, 0);
             for (int pass = 0; pass < 2; ++pass) {      // compensated FP32, then plain FP32
                 std::vector<EriTask> tk;
-                build_tiles(B.bras, P.h_prefix, how.kets, 0, tk, pass ? &none : nullptr);
+                build_tiles(pc, B.bras, P.h_prefix, B.kb, BucketCounts(B.kb), P.h_ketsp, B.prm.gauge != 0, how, 0, tk,
+                            pass ? &none : nullptr);
                 EriTask *d_tk = dcopy(c->tasks, tk, s);
-                launch_zero(B.W, (long long)n, s);
-                launch_eri(d_prm, d_tk, (int)tk.size(), (int *)c->next.get(sizeof(int)), shape, B.prm.gauge != 0, true,
-                           how, s);
-                if (pass == 0) QDT_CUDA_TRY(cudaMemcpyAsync(W2, B.W, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
+                const int n = (int)tk.size();
+                int *queue = (int *)c->next.get(2 * sizeof(int));
+                QDT_CUDA_TRY(cudaMemcpyAsync(queue + 1, &n, sizeof n, cudaMemcpyHostToDevice, s));
+                launch_zero(B.W, (long long)nw, s);
+                launch_eri(d_prm, d_tk, n, queue, shape, B.prm.gauge != 0, true, how, s);
+                if (pass == 0) QDT_CUDA_TRY(cudaMemcpyAsync(W2, B.W, nw * sizeof(double), cudaMemcpyDeviceToDevice, s));
             }
             std::vector<int> rp(P.M), cp(P.M);
             for (int k = 0; k < pc.nsp; ++k) {

@@ -171,6 +171,10 @@ struct PairClass {
     PairChunk *d_ch = nullptr;
     double *d_Q = nullptr;
     int *d_bra_order = nullptr;
+    // bucket of every shell pair: pairs of one kind with the same number of primitive
+    // pairs, whose quartets with a bra pair are alike (ket_buckets in plan.h)
+    std::vector<int> h_bucket;
+    std::vector<int> bucket_rep;    // a shell pair of every bucket
     std::vector<int> bra_pos;   // bra position of every shell pair (inverse of bra_order)
     int *d_bra_pos = nullptr;
     long long npp_total = 0, e_total = 0;
@@ -193,6 +197,7 @@ struct EriParams {
     // batch_kets); positions, prefixes and columns below are in that list
     const int *ket_sp;          // shell pair id at each ket position
     const long long *ket_col;   // first column of each ket position
+    const int *bucket;          // ket positions grouped by bucket, ascending: the tiles' k0, k1 index this list
     double *W;                  // output rows
     long long ldw;
     long long row0;             // bra-order row of W's first row
@@ -221,12 +226,14 @@ struct EriParams {
     const long long *col2;      // sym 2: W2 column of every pair id of the batch
 };
 
-struct EriTask {                // one tile: bra shell pair x range of sorted ket positions
+struct EriTask {                // one tile: bra shell pair x kets of one bucket
     int bra_sp;
-    int k0, k1;
+    int k0, k1;                 // range of EriParams::bucket, at most kMaxTileKets
     int req;                    // index into the EriParams array of the launch
     int f32 = 0;                // compensated-FP32 kernels: 1 = these quartets in plain FP32
 };
+
+constexpr int kMaxTileKets = 32;    // one warp looks them over
 
 // Class maxima that fix the integral kernel's shared-memory plan.
 struct EriShape {
@@ -238,23 +245,25 @@ struct EriShape {
     }
 };
 
-// Launch shape of the integral kernel (the autotuned part): CTA threads and
-// ket positions per tile.  Neither changes the arithmetic of an integral.
+// Launch shape of the integral kernel (the autotuned part): CTA threads, kets per
+// tile at most, tile order.  None changes the arithmetic of an integral.
 struct EriLaunch {
     int threads = 0;            // 0: the plan's default
-    int kets = 8;
-    int order = 0;              // tile order: 0 bra pairs by Schwarz Q (bra order), 1 most expensive first
+    int kets = kMaxTileKets;
+    int order = 1;              // tile order: 0 bra pairs by Schwarz Q (bra order), 1 most expensive first
+    int least = 1;              // the smallest tile_kets() of the class under the budget
+    long long budget = 0;       // quartet cost a tile may reach with more than one ket (0: no limit)
 };
 
 void launch_boys_table(double *d_tab, cudaStream_t s);
 void launch_shell_norms(const ShellDev *shells, int nL_shells, const double *exps,
                         const double *coefs, double *norms, cudaStream_t s);
-// Persistent integral kernel over a shared tile queue: `next` (device int,
-// zeroed by this call) hands out the tiles in array order.  prms: device array
-// of the parameter sets the tiles' `req` index.
+// Persistent integral kernel over a shared tile queue: queue[0] (zeroed by this
+// call) hands out the queue[1] tiles in array order; maxtasks bounds queue[1].
+// prms: device array of the parameter sets the tiles' `req` index.
 // df: every parameter set carries E2 and the contractions run in compensated
 // FP32 pairs (the split form); otherwise in FP64.
-void launch_eri(const EriParams *prms, const EriTask *tasks, int ntasks, int *next, const EriShape &shape,
+void launch_eri(const EriParams *prms, const EriTask *tasks, int maxtasks, int *queue, const EriShape &shape,
                 bool gauge, bool df, const EriLaunch &how, cudaStream_t s);
 // max |A - B| / (Q_row Q_col) over integral rows (FP32 error model check).
 void launch_ratio(const double *A, const double *B, long long rows, long long ldw, int mult, const int *row_pair,
@@ -275,6 +284,21 @@ __host__ __device__ inline int t_rows(int Lx, bool gauge) { return nherm(Lx) + (
 __host__ __device__ inline long long orient_madds(const PairDev &X, const PairDev &Y, bool gauge) {
     return (long long)X.npp * ((long long)Y.npp * t_rows(X.Lab, gauge) * Y.nbox +
                                (long long)X.nbox * Y.nfp * (gauge ? 7 : 1));
+}
+// Cost of a shell quartet in multiply-adds: its contraction, and the Hermite
+// recursion as four per entry of its order-0 tensors.
+__host__ __device__ inline long long quartet_cost(const PairDev &A, const PairDev &C, bool gauge) {
+    const int L = A.Lab + C.Lab;
+    const long long a = orient_madds(A, C, gauge), c = orient_madds(C, A, gauge);
+    return (a < c ? a : c) + 4LL * A.npp * C.npp * (nherm(L) + (gauge ? nherm(L + 2) : 0));
+}
+// Kets per tile of a bra pair and a bucket: a tile's kets share its CTA one group
+// after another, so expensive quartets come in small tiles and cheap ones, which
+// run several at a time, in large ones.
+__host__ __device__ inline int tile_kets(const PairDev &A, const PairDev &C, bool gauge, long long budget, int most) {
+    if (budget <= 0) return most;
+    const long long k = budget / (quartet_cost(A, C, gauge) + 1);
+    return k < 1 ? 1 : (k < most ? (int)k : most);
 }
 
 void launch_ket_order(const double *Q, const double *Dmax, int nsp, double *w, int *ket_sp,
