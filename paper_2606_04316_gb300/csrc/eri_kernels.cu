@@ -480,18 +480,6 @@ struct Plan {
     int pool;        // bytes
 };
 
-struct BlockSmem {
-    char *pool;
-    int2 *src;                  // recursion sources of R_h
-    int *trip;                  // Hermite triple h -> t | u << 8 | v << 16
-    int *box;                   // per box: first list entry | count << 16
-    unsigned short *hs;         // [nG][nhm]: Hermite index of the sum of two triples
-    uint4 *r12row;              // [nhm]: Hermite indices of h + e_I + e_J, 16 bits each
-    unsigned char *lst;         // Hermite indices of the boxes' entries
-    struct KetRef *ket;         // [kMaxKets]: the tile's kets to compute
-    int *slot;                  // [2]: tile index, kets to compute
-};
-
 // A ket shell pair of the current tile.
 struct KetRef {
     long long eoff, rowoff, col, col_rev;    // col_rev: its column for the transposed block, < 0: none
@@ -499,91 +487,9 @@ struct KetRef {
 };
 constexpr int kMaxKets = kMaxTileKets;
 
-__host__ __device__ inline int up16(int n) { return (n + 15) & ~15; }
-size_t plan_tables(const Plan &p) {
-    return (size_t)up16(p.nTab * 8) + up16(p.nTab * 4) + up16(p.nhm * 4) + up16(p.nG * p.nhm * 2) +
-           p.nhm * 16 + up16(p.nLst) + kMaxKets * (int)sizeof(KetRef) + 16;
-}
-size_t plan_smem(const Plan &p) { return plan_tables(p) + (size_t)p.pool; }
-
-__device__ inline BlockSmem carve(char *sm, const Plan &p) {
-    BlockSmem b;
-    b.pool = sm; sm += p.pool;
-    b.src = (int2 *)sm; sm += up16(p.nTab * 8);
-    b.trip = (int *)sm; sm += up16(p.nTab * 4);
-    b.box = (int *)sm; sm += up16(p.nhm * 4);
-    b.hs = (unsigned short *)sm; sm += up16(p.nG * p.nhm * 2);
-    b.r12row = (uint4 *)sm; sm += p.nhm * 16;
-    b.lst = (unsigned char *)sm; sm += up16(p.nLst);
-    b.ket = (KetRef *)sm; sm += kMaxKets * sizeof(KetRef);
-    b.slot = (int *)sm;
-    return b;
-}
-
-// Box entries of all boxes of order < n: C(n + 5, 6).
-__host__ __device__ constexpr int box_entries_below(int n) {
-    return n * (n + 1) * (n + 2) / 6 * ((n + 3) * (n + 4) / 2) / 2 * (n + 5) / 30;
-}
-static_assert(box_entries_below(1) == 1 && box_entries_below(2) == 7 && box_entries_below(3) == 28 &&
-              box_entries_below(4) == 84 && box_entries_below(5) == 210 && box_entries_below(6) == 462 &&
-              box_entries_below(7) == 924, "C(n + 5, 6)");
-
-// Recursion source of R_h: direction, h - e_dir, h - 2 e_dir (packed) and the
-// coefficient (component - 1) of the latter as a float.
-__device__ void build_tables(const Plan &p, BlockSmem &b) {
-    for (int h = threadIdx.x; h < p.nTab; h += blockDim.x) {
-        int t, u, v;
-        htrip_d(h, t, u, v);
-        b.trip[h] = t | (u << 8) | (v << 16);
-        int dir, c;
-        if (t > 0) { dir = 0; c = t; }
-        else if (u > 0) { dir = 1; c = u; }
-        else { dir = 2; c = v; }
-        int i1 = 0, i2 = 0;
-        if (h > 0) {
-            const int dt = dir == 0, du = dir == 1, dv = dir == 2;
-            i1 = hidx(t - dt, u - du, v - dv);
-            if (c >= 2) i2 = hidx(t - 2 * dt, u - 2 * du, v - 2 * dv);
-        }
-        b.src[h] = make_int2(dir | (i1 << 2) | (i2 << 12), __float_as_int(c >= 2 ? (float)(c - 1) : 0.f));
-        if (h < p.nhm) {
-            // this box's list: the boxes before it, of lower order and of its own
-            int at = box_entries_below(t + u + v);
-            for (int q = nherm(t + u + v - 1); q < h; ++q) {
-                int a, bb, c2;
-                htrip_d(q, a, bb, c2);
-                at += box_count(a, bb, c2);
-            }
-            b.box[h] = at | (box_count(t, u, v) << 16);
-            for (int x = 0; x <= t; ++x)
-                for (int y = 0; y <= u; ++y)
-                    for (int z = 0; z <= v; ++z) b.lst[at++] = (unsigned char)hidx(x, y, z);
-            b.r12row[h] = make_uint4(hidx(t + 2, u, v) | (hidx(t + 1, u + 1, v) << 16),
-                                     hidx(t + 1, u, v + 1) | (hidx(t, u + 2, v) << 16),
-                                     hidx(t, u + 1, v + 1) | (hidx(t, u, v + 2) << 16), 0u);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < p.nG * p.nhm; i += blockDim.x) {
-        const int g = b.trip[i / p.nhm], h = b.trip[i % p.nhm];
-        b.hs[i] = (unsigned short)hidx((g & 255) + (h & 255), ((g >> 8) & 255) + ((h >> 8) & 255),
-                                       (g >> 16) + (h >> 16));
-    }
-    __syncthreads();
-}
-
-// Sizes of a quartet (X outer, Y inner).  Order-0 and even-order tensors need
-// nherm(L) entries each, odd orders nherm(L - 1); the r12 tensor has top order L + 2.
-__host__ __device__ inline int odd_len(int Ltop) { return Ltop >= 1 ? nherm(Ltop - 1) : 0; }
 struct Shape {
     int nE, nO, hs, nT, NC;
 };
-__host__ __device__ inline Shape quartet_shape(int Lx, int Ly, bool gauge) {
-    const int L = Lx + Ly;
-    return {nherm(L) + (gauge ? nherm(L + 2) : 0), odd_len(L) + (gauge ? odd_len(L + 2) : 0), header_len(L, gauge),
-            t_rows(Lx, gauge), gauge ? 7 : 1};
-}
-
 // How the quartets of a tile (one bra pair, kets of one kind) are cut to fit the
 // pool: [headers][even tensors][T | odd tensors][G].  T of a group is written after
 // the group's recursion has read the odd tensors and read before the next group
@@ -595,12 +501,170 @@ struct Cut {
     int nb;              // kets at a time
     int nij, nijH;       // outer primitive pairs per group, per header pass
 };
+// Device tables of the shell pairs.
+struct PairTables {
+    const PrimPairDev *pp;
+    const double2 *E;
+    const float4 *E2;
+    const float2 *E1;
+    const FuncPair *fp;
+    const PairChunk *ch;
+    const double *boys;
+};
+
+// What the phases of a tile need to know about it, written once per tile.  It lives
+// in shared memory and the phases are functions of their own, so that a phase's
+// loops have the registers to themselves (with everything in one function the
+// compensated kernel spilled in its inner loops: 201 ms for the integrals of the
+// 24-centre chain, 179 with 168 instead of 128 registers, and this way 179 with 128).
+struct TileState {
+    PairTables tb;
+    const FuncPair *fx;          // X's and Y's tables
+    const PairChunk *cy;
+    long long eAB;               // AB's first E entry
+    int pAB;                     // and primitive pair
+    int swap;                    // X is the ket pair, Y the bra pair AB
+    int nkets;
+    int L, Ltop;                 // Hermite order of the quartet; top order of its tensors
+    int nppx, nfpx, nk2x, nppy, nfpy, nk2y, nchy, nhx;
+    int nE_C, nO_C;              // entries of the even and odd tensors before the r12 tensor
+    Shape sh;
+    Cut c;
+    int Re, U, T, G;             // byte offsets in shared memory: even tensors, odd tensors, T, G
+    KetRef ket[kMaxKets];        // the tile's kets to compute
+    int slot, n_use;             // tile index, kets to compute
+    // byte offsets of the tables (built once per CTA) and the pool (headers first)
+    int o_src, o_trip, o_box, o_hs, o_r12, o_lst, o_pool;
+    int nG;
+};
+
+// Shared memory: TileState, tables, pool.  Every function takes its pointers from
+// the array itself, so that the compiler sees shared addresses.
+extern __shared__ __align__(16) char sm[];
+__device__ __forceinline__ TileState &tile_state() { return *reinterpret_cast<TileState *>(sm); }
+template <class T> __device__ __forceinline__ T *at_byte(int off) { return reinterpret_cast<T *>(sm + off); }
+// A group within the tile: `nb` kets from ket0, outer primitive pairs ih + i0 ..
+// + nij of the header pass's nijH from ih, nk twos of inner primitive pairs from k0,
+// function pairs x0 .. + xch, chunks c0 .. c1 of Y (y0 .. + ych, row stride yp).
+struct Group {
+    int ket0, nb, ih, nijH, i0, nij, k0, nk, x0, xch, c0, c1, y0, ych, yp;
+};
+
+__host__ __device__ inline int up16(int n) { return (n + 15) & ~15; }
+// Tables: recursion sources of R_h (int2[nTab]); Hermite triple h -> t | u << 8 | v <<
+// 16 (int[nTab]); per box its first list entry | count << 16 (int[nhm]); Hermite index
+// of the sum of two triples (unsigned short[nhm][nG]); Hermite indices of h + e_I + e_J,
+// 16 bits each (uint4[nhm]); Hermite indices of the boxes' entries (unsigned char[nLst]).
+__host__ __device__ inline int table_bytes(const Plan &p, int (&o)[7]) {
+    o[0] = up16((int)sizeof(TileState));
+    o[1] = o[0] + up16(p.nTab * 8);
+    o[2] = o[1] + up16(p.nTab * 4);
+    o[3] = o[2] + up16(p.nhm * 4);
+    o[4] = o[3] + up16(p.nG * p.nhm * 2);
+    o[5] = o[4] + p.nhm * 16;
+    o[6] = o[5] + up16(p.nLst);
+    return o[6];
+}
+size_t plan_tables(const Plan &p) {
+    int o[7];
+    return (size_t)table_bytes(p, o);
+}
+size_t plan_smem(const Plan &p) { return plan_tables(p) + (size_t)p.pool; }
+
+// Box entries of all boxes of order < n: C(n + 5, 6).
+__host__ __device__ constexpr int box_entries_below(int n) {
+    return n * (n + 1) * (n + 2) / 6 * ((n + 3) * (n + 4) / 2) / 2 * (n + 5) / 30;
+}
+static_assert(box_entries_below(1) == 1 && box_entries_below(2) == 7 && box_entries_below(3) == 28 &&
+              box_entries_below(4) == 84 && box_entries_below(5) == 210 && box_entries_below(6) == 462 &&
+              box_entries_below(7) == 924, "C(n + 5, 6)");
+
+// Recursion source of R_h: direction, h - e_dir, h - 2 e_dir (packed) and the
+// coefficient (component - 1) of the latter as a float.
+__device__ void build_tables(const Plan &p) {
+    int o[7];
+    table_bytes(p, o);
+    int2 *src = at_byte<int2>(o[0]);
+    int *trip = at_byte<int>(o[1]), *box = at_byte<int>(o[2]);
+    unsigned short *hs = at_byte<unsigned short>(o[3]);
+    uint4 *r12row = at_byte<uint4>(o[4]);
+    unsigned char *lst = at_byte<unsigned char>(o[5]);
+    if (threadIdx.x == 0) {
+        TileState &s = tile_state();
+        s.o_src = o[0];
+        s.o_trip = o[1];
+        s.o_box = o[2];
+        s.o_hs = o[3];
+        s.o_r12 = o[4];
+        s.o_lst = o[5];
+        s.o_pool = o[6];
+        s.nG = p.nG;
+    }
+    for (int h = threadIdx.x; h < p.nTab; h += blockDim.x) {
+        int t, u, v;
+        htrip_d(h, t, u, v);
+        trip[h] = t | (u << 8) | (v << 16);
+        int dir, c;
+        if (t > 0) { dir = 0; c = t; }
+        else if (u > 0) { dir = 1; c = u; }
+        else { dir = 2; c = v; }
+        int i1 = 0, i2 = 0;
+        if (h > 0) {
+            const int dt = dir == 0, du = dir == 1, dv = dir == 2;
+            i1 = hidx(t - dt, u - du, v - dv);
+            if (c >= 2) i2 = hidx(t - 2 * dt, u - 2 * du, v - 2 * dv);
+        }
+        src[h] = make_int2(dir | (i1 << 2) | (i2 << 12), __float_as_int(c >= 2 ? (float)(c - 1) : 0.f));
+        if (h < p.nhm) {
+            // this box's list: the boxes before it, of lower order and of its own
+            int at = box_entries_below(t + u + v);
+            for (int q = nherm(t + u + v - 1); q < h; ++q) {
+                int a, bb, c2;
+                htrip_d(q, a, bb, c2);
+                at += box_count(a, bb, c2);
+            }
+            box[h] = at | (box_count(t, u, v) << 16);
+            for (int x = 0; x <= t; ++x)
+                for (int y = 0; y <= u; ++y)
+                    for (int z = 0; z <= v; ++z) lst[at++] = (unsigned char)hidx(x, y, z);
+            r12row[h] = make_uint4(hidx(t + 2, u, v) | (hidx(t + 1, u + 1, v) << 16),
+                                     hidx(t + 1, u, v + 1) | (hidx(t, u + 2, v) << 16),
+                                     hidx(t, u + 1, v + 1) | (hidx(t, u, v + 2) << 16), 0u);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < p.nG * p.nhm; i += blockDim.x) {
+        const int g = trip[i % p.nG], h = trip[i / p.nG];
+        hs[i] = (unsigned short)hidx((g & 255) + (h & 255), ((g >> 8) & 255) + ((h >> 8) & 255),
+                                       (g >> 16) + (h >> 16));
+    }
+    __syncthreads();
+}
+
+// Sizes of a quartet (X outer, Y inner).  Order-0 and even-order tensors need
+// nherm(L) entries each, odd orders nherm(L - 1); the r12 tensor has top order L + 2.
+__host__ __device__ inline int odd_len(int Ltop) { return Ltop >= 1 ? nherm(Ltop - 1) : 0; }
+__host__ __device__ inline Shape quartet_shape(int Lx, int Ly, bool gauge) {
+    const int L = Lx + Ly;
+    return {nherm(L) + (gauge ? nherm(L + 2) : 0), odd_len(L) + (gauge ? odd_len(L + 2) : 0), header_len(L, gauge),
+            t_rows(Lx, gauge), gauge ? 7 : 1};
+}
+
 constexpr int kTensorBytes = 112 * 1024;
-__host__ __device__ inline int cut_bytes(const Shape &s, int nk2, int xch, int ych, int nkc, int nij, int nijH) {
+// Row stride of T and G: even (a packed load takes two y) but no multiple of 4, so
+// that lanes on consecutive T rows store to different banks.
+__host__ __device__ inline int y_stride(int ych) {
     const int yp = (ych + 1) & ~1;
-    const int t = nij * s.nT * yp * 8, o = s.nO * nij * nkc * 16;
-    return s.hs * nijH * nkc * 16 + s.nE * nij * nkc * 16 + (nkc < nk2 ? t + o : (t > o ? t : o)) +
-           s.NC * xch * yp * 8;
+    return yp & 3 ? yp : yp + 2;
+}
+// Entry stride of the tensors, in twos of primitive quartets: odd, so that 16-byte
+// loads of consecutive entries (the lanes of the ket pass) fall into different banks.
+__host__ __device__ inline int q_stride(int q) { return q | 1; }
+__host__ __device__ inline int cut_bytes(const Shape &s, int nk2, int nb, int xch, int ych, int nkc, int nij, int nijH) {
+    const int yp = y_stride(ych), qs = q_stride(nb * nij * nkc);
+    const int t = nb * nij * s.nT * yp * 8, o = s.nO * qs * 16;
+    return s.hs * nb * nijH * nkc * 16 + s.nE * qs * 16 + (nkc < nk2 ? t + o : (t > o ? t : o)) +
+           nb * s.NC * xch * yp * 8;
 }
 // The cut decides no rounding except where the inner primitive pairs are cut (nkc,
 // contractions of dozens of primitives), and that depends on the quartet alone:
@@ -618,7 +682,7 @@ __host__ __device__ inline Cut partition(const Shape &s, int nppx, int nfpx, int
     c.nb = 1;
     const int nk2 = c.nkc;
     while (c.nkc > 1 && (s.hs + s.nE + s.nO) * 16 > kTensorBytes / c.nkc) c.nkc = (c.nkc + 1) / 2;
-    while (cut_bytes(s, nk2, c.xch, c.ych, c.nkc, 1, 1) > pool) {
+    while (cut_bytes(s, nk2, 1, c.xch, c.ych, c.nkc, 1, 1) > pool) {
         if (c.ych > 4) c.ych = (c.ych + 1) / 2;
         else if (c.xch > 4) c.xch = (c.xch + 1) / 2;
         else if (c.ych > 2) c.ych = 2;
@@ -627,12 +691,11 @@ __host__ __device__ inline Cut partition(const Shape &s, int nppx, int nfpx, int
     }
     const int np = nppx > 1 ? nppx : 1, items = s.nT * nchy, want = 4 * threads;
     if (c.nkc == nk2 && c.xch == nfpx && c.ych == nfpy) {
-        const int one = cut_bytes(s, nk2, c.xch, c.ych, c.nkc, 1, np);
-        int nb = (want + items - 1) / items;
+                int nb = (want + items - 1) / items;
         const int nbh = (2 * threads + np * nppy - 1) / (np * (nppy > 1 ? nppy : 1));   // two header rounds
         if (nb < nbh) nb = nbh;
         if (nb > nkets) nb = nkets;
-        if (nb > pool / one) nb = pool / one;
+        while (nb > 1 && cut_bytes(s, nk2, nb, c.xch, c.ych, c.nkc, 1, np) > pool) --nb;
         if (nb > 1) {
             const int groups = (nkets + nb - 1) / nb;
             c.nb = (nkets + groups - 1) / groups;
@@ -640,12 +703,12 @@ __host__ __device__ inline Cut partition(const Shape &s, int nppx, int nfpx, int
     }
     int nij = (want + items * c.nb - 1) / (items * c.nb);
     if (nij > np) nij = np;
-    while (nij > 1 && c.nb * cut_bytes(s, nk2, c.xch, c.ych, c.nkc, nij, c.nb > 1 ? np : nij) > pool) --nij;
+    while (nij > 1 && cut_bytes(s, nk2, c.nb, c.xch, c.ych, c.nkc, nij, c.nb > 1 ? np : nij) > pool) --nij;
     const int groups = (np + nij - 1) / nij;
     c.nij = (np + groups - 1) / groups;
     c.nijH = c.nb > 1 ? np : c.nij;
     if (c.nb == 1 && c.nkc == nk2) {
-        const int rest = pool - cut_bytes(s, nk2, c.xch, c.ych, c.nkc, c.nij, 0);
+        const int rest = pool - cut_bytes(s, nk2, 1, c.xch, c.ych, c.nkc, c.nij, 0);
         int h = rest / (s.hs * c.nkc * 16);
         if (h > np) h = np;
         if (h < np) h = h / c.nij * c.nij;
@@ -659,17 +722,6 @@ struct FastDiv {
     unsigned d, magic;
     __device__ explicit FastDiv(int n) : d((unsigned)n), magic(n > 1 ? 0xFFFFFFFFu / (unsigned)n + 1u : 0u) {}
     __device__ int div(int it) const { return magic ? (int)__umulhi((unsigned)it, magic) : it; }
-};
-
-// Device tables of the shell pairs.
-struct PairTables {
-    const PrimPairDev *pp;
-    const double2 *E;
-    const float4 *E2;
-    const float2 *E1;
-    const FuncPair *fp;
-    const PairChunk *ch;
-    const double *boys;
 };
 
 template <int A> __device__ __forceinline__ const typename Arith<A>::Vec *e_entries(const PairTables &t);
@@ -688,13 +740,13 @@ template <> __device__ __forceinline__ const f32x2 *e_entries<kF32>(const PairTa
 // for all lanes on the same chunk.  NK > 0: that many twos of primitive pairs,
 // unrolled (5 = two contractions of three primitives), else nk of them.
 template <int A, int M, int NK>
-__device__ __forceinline__ void ket_item(const typename Arith<A>::Vec *R, int Q2, const unsigned short *hs,
+__device__ __forceinline__ void ket_item(const typename Arith<A>::Vec *R, int QS, const unsigned short *hs, int nG,
                                          const unsigned char *lst, int cnt, const typename Arith<A>::Vec *E,
                                          int estride, int nk2, int nk, bool odd, float2 (&out)[M],
                                          double (&outd)[M]) {
     typedef typename Arith<A>::Vec Vec;
     const int n = NK > 0 ? NK : nk;
-    int o = (int)hs[lst[0]] * Q2;
+    int o = (int)hs[lst[0] * nG] * QS;
     if constexpr (A == kF64) {
         double a0[M], a1[M];
 #pragma unroll
@@ -702,7 +754,7 @@ __device__ __forceinline__ void ket_item(const typename Arith<A>::Vec *R, int Q2
         const int full = odd ? n - 1 : n;               // the last two holds one primitive pair
         for (int j = 0; j < cnt; ++j) {
             const Vec *r = R + o;
-            if (j + 1 < cnt) o = (int)hs[lst[j + 1]] * Q2;
+            if (j + 1 < cnt) o = (int)hs[lst[j + 1] * nG] * QS;
 #pragma unroll 4
             for (int p = 0; p < full; ++p) {
                 const Vec rv = r[p];
@@ -729,7 +781,7 @@ __device__ __forceinline__ void ket_item(const typename Arith<A>::Vec *R, int Q2
         for (int m = 0; m < M; ++m) ah[m] = al[m] = 0;
         for (int j = 0; j < cnt; ++j) {
             const Vec *r = R + o;
-            if (j + 1 < cnt) o = (int)hs[lst[j + 1]] * Q2;
+            if (j + 1 < cnt) o = (int)hs[lst[j + 1] * nG] * QS;
 #pragma unroll
             for (int p = 0; p < (NK > 0 ? NK : 1); ++p) {
                 for (int q = p; q < n; q += (NK > 0 ? n : 1)) {
@@ -749,7 +801,7 @@ __device__ __forceinline__ void ket_item(const typename Arith<A>::Vec *R, int Q2
         for (int m = 0; m < M; ++m) a[m] = 0;
         for (int j = 0; j < cnt; ++j) {
             const Vec *r = R + o;
-            if (j + 1 < cnt) o = (int)hs[lst[j + 1]] * Q2;
+            if (j + 1 < cnt) o = (int)hs[lst[j + 1] * nG] * QS;
 #pragma unroll
             for (int p = 0; p < (NK > 0 ? NK : 1); ++p) {
                 for (int q = p; q < n; q += (NK > 0 ? n : 1)) {
@@ -766,14 +818,14 @@ __device__ __forceinline__ void ket_item(const typename Arith<A>::Vec *R, int Q2
 }
 
 template <int A, int M>
-__device__ __forceinline__ void ket_store(const typename Arith<A>::Vec *R, int Q2, const unsigned short *hs,
+__device__ __forceinline__ void ket_store(const typename Arith<A>::Vec *R, int QS, const unsigned short *hs, int nG,
                                           const unsigned char *lst, int cnt, const typename Arith<A>::Vec *E,
                                           int estride, int nk2, int nk, bool odd, bool neg, bool add, char *T,
                                           int at, int plane) {
     float2 s[M];
     double sd[M];
-    if (A != kF64 && nk == 5) ket_item<A, M, 5>(R, Q2, hs, lst, cnt, E, estride, nk2, nk, odd, s, sd);
-    else ket_item<A, M, 0>(R, Q2, hs, lst, cnt, E, estride, nk2, nk, odd, s, sd);
+    if (A != kF64 && nk == 5) ket_item<A, M, 5>(R, QS, hs, nG, lst, cnt, E, estride, nk2, nk, odd, s, sd);
+    else ket_item<A, M, 0>(R, QS, hs, nG, lst, cnt, E, estride, nk2, nk, odd, s, sd);
 #pragma unroll
     for (int m = 0; m < M; ++m) {
         if constexpr (A == kF64) {
@@ -790,276 +842,332 @@ __device__ __forceinline__ void ket_store(const typename Arith<A>::Vec *R, int Q
     }
 }
 
-// The blocks (X|Y) of one bra pair AB and `nkets` ket pairs b.ket[] of CD's kind (X =
-// CD when swap), some kets and chunks at a time; emit(ket0, nb, x0, xch, y0, ych,
-// value) is called by all threads once a group's results stand in shared memory,
-// value(ket, c, x, y) being component c of function pairs x, y (sorted order,
-// relative to the chunk).
-// Components: 0 Coulomb; gauge kernel 1..6: (xy|d_I d_J r|zw), IJ = xx, xy, xz, yy, yz, zz.
-template <bool GAUGE, int A, class Emit>
-__device__ void quartet_blocks(const PairTables &tb, const PairDev &AB, const PairDev &CD, bool swap, int nkets,
-                               const Plan &pl, BlockSmem &b, Emit emit) {
-    typedef typename Arith<A>::Vec Vec;
-    typedef typename Arith<A == kF64 ? kF64 : kDF>::Vec HVec;      // headers: FP64 or pairs
-    constexpr int NC = GAUGE ? 7 : 1;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const PairDev &X = swap ? CD : AB, &Y = swap ? AB : CD;
-    const int Lx = X.Lab, Ly = Y.Lab, L = Lx + Ly, Lr = L + 2, Ltop = GAUGE ? Lr : L;
-    const int nppx = X.npp, nppy = Y.npp, nk2x = X.nk2, nk2y = Y.nk2;
-    const int nhx = nherm(Lx);
-    const Shape sh = quartet_shape(Lx, Ly, GAUGE);
-    const Cut c = partition(sh, nppx, X.nfp, nppy, Y.nfp, Y.nch, nkets, pl.pool, nt);
-    const int nE_C = nherm(L), nO_C = odd_len(L);       // entries before the r12 tensor
-    const FuncPair *fx = tb.fp + X.fpoff;
-    const PairChunk *cy = tb.ch + Y.choff;
-    const Vec *E0 = e_entries<A>(tb);
-    const long long eAB = AB.eoff;
-    const int pAB = AB.ppoff, nfpx = X.nfp, nchy = Y.nch;
-
-    HVec *H = reinterpret_cast<HVec *>(b.pool);
-    Vec *Re = reinterpret_cast<Vec *>(b.pool + (size_t)sh.hs * c.nb * c.nijH * c.nkc * 16);
-    char *U = reinterpret_cast<char *>(Re) + (size_t)sh.nE * c.nb * c.nij * c.nkc * 16;
-    const bool runs = c.nkc < nk2y;
-    Vec *Ro = reinterpret_cast<Vec *>(U);
-    const int ypmax = (c.ych + 1) & ~1;
-    const int tbytes = c.nb * c.nij * sh.nT * ypmax * 8, obytes = sh.nO * c.nb * c.nij * c.nkc * 16;
-    char *T = runs ? U + obytes : U;
-    char *G = U + (runs ? tbytes + obytes : max(tbytes, obytes));
-
-    for (int ket0 = 0; ket0 < nkets; ket0 += c.nb) {
-    const int nb = min(c.nb, nkets - ket0);
-    const KetRef *kets = b.ket + ket0;
-    for (int c0 = 0; c0 < nchy;) {
-        const int y0 = cy[c0].k0;
-        int c1 = nchy, ych = Y.nfp - y0;
-        if (ych > c.ych) {
-            c1 = c0;
-            while (cy[c1].k0 + cy[c1].m - y0 <= c.ych) ++c1;
-            ych = cy[c1 - 1].k0 + cy[c1 - 1].m - y0;
-        }
-        const int yp = (ych + 1) & ~1;
-        for (int x0 = 0; x0 < nfpx; x0 += c.xch) {
-            const int xch = min(c.xch, nfpx - x0);
-            const int gket = NC * xch * yp, gplane = nb * gket;     // FP32 pairs: high parts, then low parts
-            for (int i = tid; i < gplane; i += nt) {
-                if (A == kF64) reinterpret_cast<double *>(G)[i] = 0.0;
-                else reinterpret_cast<float2 *>(G)[i] = make_float2(0.f, 0.f);
+// Headers of a group's primitive quartets: Q - P, Boys values and prefactors.
+template <bool GAUGE, int A>
+__device__ __noinline__ void header_pass(const Group g) {
+    typedef typename Arith<A == kF64 ? kF64 : kDF>::Vec HVec;      // FP64 or pairs
+    const TileState &s = tile_state();
+    HVec *H = at_byte<HVec>(s.o_pool);
+    const KetRef *kets = s.ket + g.ket0;
+    const int QH = g.nb * g.nijH * g.nk, hs = s.sh.hs;
+    const FastDiv dk(2 * g.nk), dij(g.nijH);
+    for (int q = threadIdx.x; q < 2 * QH; q += blockDim.x) {
+        const int o = dk.div(q), r = q - o * 2 * g.nk, kl = 2 * g.k0 + r;
+        const int bk = dij.div(o), ij = g.ih + o - bk * g.nijH;
+        const int pk = kets[bk].ppoff;
+        const PrimPairDev *px = s.tb.pp + (s.swap ? pk : s.pAB) + ij, *py = s.tb.pp + (s.swap ? s.pAB : pk) + kl;
+        const int at = o * g.nk + (r >> 1);
+        if constexpr (A == kF64) {
+            const HeadF64 h{reinterpret_cast<double *>(H + at) + (r & 1), 2 * QH};
+            if (kl < s.nppy) {
+                quartet_header<GAUGE>(s.tb.boys, px, py, s.L, h);
+            } else {
+                for (int j = 0; j < hs; ++j) h.zero(j);
             }
-            for (int ih = 0; ih < nppx; ih += c.nijH) {
-                const int nijH = min(c.nijH, nppx - ih);
-                for (int k0 = 0; k0 < nk2y; k0 += c.nkc) {
-                    const int nk = min(c.nkc, nk2y - k0);
-                    const bool odd = (nppy & 1) && k0 + nk == nk2y;
-                    const int QH = nb * nijH * nk;
-                    __syncthreads();                        // the last recursion has read the headers
-                    {
-                        // Q - P, Boys values and prefactors of the primitive quartets
-                        const FastDiv dk(2 * nk), dij(nijH);
-                        for (int q = tid; q < 2 * QH; q += nt) {
-                            const int o = dk.div(q), r = q - o * 2 * nk, kl = 2 * k0 + r;
-                            const int bk = dij.div(o), ij = ih + o - bk * nijH;
-                            const int pk = kets[bk].ppoff;
-                            const PrimPairDev *px = tb.pp + (swap ? pk : pAB) + ij, *py = tb.pp + (swap ? pAB : pk) + kl;
-                            const int at = o * nk + (r >> 1);
-                            if constexpr (A == kF64) {
-                                const HeadF64 h{reinterpret_cast<double *>(H + at) + (r & 1), 2 * QH};
-                                if (kl < nppy) {
-                                    quartet_header<GAUGE>(tb.boys, px, py, L, h);
-                                } else {
-                                    for (int j = 0; j < sh.hs; ++j) h.zero(j);
-                                }
-                            } else {
-                                const HeadPair h{reinterpret_cast<float *>(H + at) + (r & 1), 4 * QH};
-                                if (kl < nppy) {
-                                    if constexpr (A == kF32 && !GAUGE) quartet_header_f32(tb.boys, px, py, L, h);
-                                    else quartet_header_pairs<GAUGE>(tb.boys, px, py, L, h);
-                                } else {
-                                    for (int j = 0; j < sh.hs; ++j) h.zero(j);
-                                }
-                            }
-                        }
-                    }
-                    __syncthreads();
-                    for (int i0 = 0; i0 < nijH; i0 += c.nij) {
-                        const int nij = min(c.nij, nijH - i0);
-                        const int Q2 = nb * nij * nk;
-                        // Hermite recursion, one auxiliary order per pass; order 0 ends in Re.
-                        // Items (entry, ket, outer primitive pair, two of inner ones) are the
-                        // addresses of the results, so the stores are contiguous.
-                        if (Ltop & 1) __syncthreads();      // T, which the odd tensors overwrite, has been read
-                        const FastDiv dq(Q2), db1(nij * nk);
-                        const int hskip = (nijH - nij) * nk, hoff = i0 * nk;
-                        for (int m = Ltop; m >= 0; --m) {
-                            const int cC = m <= L ? nherm(L - m) : 0;
-                            const int cR = GAUGE ? nherm(Lr - m) : 0;
-                            Vec *dst = (m & 1) ? Ro : Re;
-                            const Vec *src = (m & 1) ? Re : Ro;
-                            const int dR = ((m & 1) ? nO_C : nE_C) * Q2, sR = ((m & 1) ? nE_C : nO_C) * Q2;
-                            const int jC = (3 + m) * QH, jR = (4 + L + m) * QH;
-                            for (int it = tid; it < (cC + cR) * Q2; it += nt) {
-                                const int e = dq.div(it);
-                                const int q = it - e * Q2;
-                                const int hq = q + hoff + (nb > 1 ? db1.div(q) * hskip : 0);
-                                const bool r12 = GAUGE && e >= cC;
-                                const int h = r12 ? e - cC : e;
-                                Vec r;
-                                if (h == 0) {
-                                    const HVec v = H[(r12 ? jR : jC) + hq];
-                                    if constexpr (A == kF32) r = v.x;
-                                    else r = v;
-                                } else {
-                                    const int2 sw = b.src[h];
-                                    const Vec *sp = src + (r12 ? sR : 0) + q;
-                                    const HVec xv = H[(sw.x & 3) * QH + hq];
-                                    const Vec a = sp[((sw.x >> 2) & 1023) * Q2];
-                                    const Vec cc = sp[(sw.x >> 12) * Q2];
-                                    const float cf = __int_as_float(sw.y);
-                                    if constexpr (A == kF64) {
-                                        const double cd = (double)cf;
-                                        r = make_double2(fma(cd, cc.x, xv.x * a.x), fma(cd, cc.y, xv.y * a.y));
-                                    } else if constexpr (A == kDF) {
-                                        r = df_rec2(xv, a, pack2(cf, cf), cc);
-                                    } else {
-                                        r = fma2(xv.x, a, mul2(pack2(cf, cf), cc));
-                                    }
-                                }
-                                dst[(r12 ? dR - cC * Q2 : 0) + it] = r;
-                            }
-                            __syncthreads();
-                        }
-                        // ket pass: T rows h < nhx from the Coulomb tensor, then (gauge) rows
-                        // g = 4.. from the r12 tensor
-                        const int nrows = nb * nij * sh.nT;
-                        const int tplane = nrows * yp;
-                        {
-                            const FastDiv drow(nrows), dT(sh.nT), dnij(nij);
-                            for (int it = tid; it < nrows * (c1 - c0); it += nt) {
-                                const int ci = drow.div(it), row = it - ci * nrows;
-                                const int o = dT.div(row), hh = row - o * sh.nT;
-                                const PairChunk k = cy[c0 + ci];
-                                const bool r12 = GAUGE && hh >= nhx;
-                                const int g = r12 ? hh - nhx + 4 : hh;
-                                const int tr = b.trip[g];
-                                const bool neg = ((tr ^ (tr >> 8) ^ (tr >> 16)) & 1) != 0;      // |g| odd
-                                const int bx = b.box[k.box], cnt = bx >> 16;
-                                const Vec *R = Re + (r12 ? nE_C : 0) * Q2 + o * nk;
-                                const long long ey = swap ? eAB : kets[dnij.div(o)].eoff;
-                                const Vec *E = E0 + ey + (k.off * nk2y + k0);
-                                const int at = row * yp + k.k0 - y0;
-                                if (k.m == 2)
-                                    ket_store<A, 2>(R, Q2, b.hs + g * pl.nhm, b.lst + (bx & 0xffff), cnt, E,
-                                                    cnt * nk2y, nk2y, nk, odd, neg, k0 > 0, T, at, tplane);
-                                else
-                                    ket_store<A, 1>(R, Q2, b.hs + g * pl.nhm, b.lst + (bx & 0xffff), cnt, E, 0, nk2y,
-                                                    nk, odd, neg, k0 > 0, T, at, tplane);
-                            }
-                        }
-                        __syncthreads();
-                        if (k0 + nk < nk2y) continue;       // T is not complete yet (then nijH == nij)
-                        // bra pass, outer primitive pairs in order (the group size changes no rounding):
-                        // G[c][x][y] += sum_ij sum_{j in box x} E^{ij}_x[j] T[ij][row(c, h_j)][y];
-                        // a thread sums all components of one x and one y (FP64) or two (packed)
-                        const int ny = A == kF64 ? ych : yp >> 1;
-                        const FastDiv dy(ny), dx(xch);
-                        for (int it = tid; it < nb * xch * ny; it += nt) {
-                            const int bx_ = dy.div(it), bk = dx.div(bx_), x = bx_ - bk * xch;
-                            const int y = (it - bx_ * ny) * (A == kF64 ? 1 : 2);
-                            const FuncPair f = fx[x0 + x];
-                            const int bx = b.box[f.fp >> 16], cnt = bx >> 16;
-                            const unsigned char *lst = b.lst + (bx & 0xffff);
-                            const Vec *ex = E0 + (swap ? kets[bk].eoff : eAB) + f.off * nk2x;
-                            const int gi = bk * gket + x * yp + y, gc = xch * yp;
-                            if constexpr (A == kF64) {
-                                double s[NC];
-                                double *g = reinterpret_cast<double *>(G) + gi;
+        } else {
+            const HeadPair h{reinterpret_cast<float *>(H + at) + (r & 1), 4 * QH};
+            if (kl < s.nppy) {
+                if constexpr (A == kF32 && !GAUGE) quartet_header_f32(s.tb.boys, px, py, s.L, h);
+                else quartet_header_pairs<GAUGE>(s.tb.boys, px, py, s.L, h);
+            } else {
+                for (int j = 0; j < hs; ++j) h.zero(j);
+            }
+        }
+    }
+}
+
+// Hermite recursion of a group, one auxiliary order per pass; order 0 ends in the
+// even tensors.  Items: (entry, ket, outer primitive pair, two of inner ones).
+template <bool GAUGE, int A>
+__device__ __noinline__ void recursion_pass(const Group g) {
+    typedef typename Arith<A>::Vec Vec;
+    typedef typename Arith<A == kF64 ? kF64 : kDF>::Vec HVec;
+    const TileState &s = tile_state();
+    const HVec *H = at_byte<HVec>(s.o_pool);
+    Vec *Re = at_byte<Vec>(s.Re), *Ro = at_byte<Vec>(s.U);
+    const int2 *stab = at_byte<int2>(s.o_src);
+    const int L = s.L, Ltop = s.Ltop, nE_C = s.nE_C, nO_C = s.nO_C;
+    const int Q2 = g.nb * g.nij * g.nk, QS = q_stride(Q2), QH = g.nb * g.nijH * g.nk;
+    const FastDiv dq(Q2), db1(g.nij * g.nk);
+    const int hskip = (g.nijH - g.nij) * g.nk, hoff = g.i0 * g.nk;
+    for (int m = Ltop; m >= 0; --m) {
+        const int cC = m <= L ? nherm(L - m) : 0;
+        const int cR = GAUGE ? nherm(Ltop - m) : 0;
+        Vec *dst = (m & 1) ? Ro : Re;
+        const Vec *src = (m & 1) ? Re : Ro;
+        const int dR = (m & 1) ? nO_C : nE_C, sR = ((m & 1) ? nE_C : nO_C) * QS;
+        const int jC = (3 + m) * QH, jR = (4 + L + m) * QH;
+        for (int it = threadIdx.x; it < (cC + cR) * Q2; it += blockDim.x) {
+            const int e = dq.div(it);
+            const int q = it - e * Q2;
+            const int hq = q + hoff + (g.nb > 1 ? db1.div(q) * hskip : 0);
+            const bool r12 = GAUGE && e >= cC;
+            const int h = r12 ? e - cC : e;
+            Vec r;
+            if (h == 0) {
+                const HVec v = H[(r12 ? jR : jC) + hq];
+                if constexpr (A == kF32) r = v.x;
+                else r = v;
+            } else {
+                const int2 sw = stab[h];
+                const Vec *sp = src + (r12 ? sR : 0) + q;
+                const HVec xv = H[(sw.x & 3) * QH + hq];
+                const Vec a = sp[((sw.x >> 2) & 1023) * QS];
+                const Vec cc = sp[(sw.x >> 12) * QS];
+                const float cf = __int_as_float(sw.y);
+                if constexpr (A == kF64) {
+                    const double cd = (double)cf;
+                    r = make_double2(fma(cd, cc.x, xv.x * a.x), fma(cd, cc.y, xv.y * a.y));
+                } else if constexpr (A == kDF) {
+                    r = df_rec2(xv, a, pack2(cf, cf), cc);
+                } else {
+                    r = fma2(xv.x, a, mul2(pack2(cf, cf), cc));
+                }
+            }
+            dst[((r12 ? dR : 0) + h) * QS + q] = r;
+        }
+        __syncthreads();
+    }
+}
+
+// Ket pass of a group: T rows h < nhx from the Coulomb tensor, then (gauge) rows
+// g = 4.. from the r12 tensor.
+template <bool GAUGE, int A>
+__device__ __noinline__ void ket_pass(const Group g) {
+    typedef typename Arith<A>::Vec Vec;
+    const TileState &s = tile_state();
+    const int nT = s.sh.nT, nhx = s.nhx, nk2y = s.nk2y;
+    const int nrows = g.nb * g.nij * nT, tplane = nrows * g.yp;
+    const int QS = q_stride(g.nb * g.nij * g.nk);
+    const bool odd = (s.nppy & 1) && g.k0 + g.nk == nk2y;
+    const Vec *Re = at_byte<Vec>(s.Re);
+    const Vec *E0 = e_entries<A>(s.tb);
+    char *T = at_byte<char>(s.T);
+    const int *trip = at_byte<int>(s.o_trip), *box = at_byte<int>(s.o_box);
+    const unsigned short *hs = at_byte<unsigned short>(s.o_hs);
+    const unsigned char *lst = at_byte<unsigned char>(s.o_lst);
+    const int nG = s.nG;
+    const FastDiv drow(nrows), dT(nT), dnij(g.nij);
+    for (int it = threadIdx.x; it < nrows * (g.c1 - g.c0); it += blockDim.x) {
+        const int ci = drow.div(it), row = it - ci * nrows;
+        const int o = dT.div(row), hh = row - o * nT;
+        const int4 kc = __ldg(reinterpret_cast<const int4 *>(s.cy + g.c0 + ci));
+        const PairChunk k{kc.x, kc.y, kc.z, kc.w};
+        const bool r12 = GAUGE && hh >= nhx;
+        const int gh = r12 ? hh - nhx + 4 : hh;
+        const int tr = trip[gh];
+        const bool neg = ((tr ^ (tr >> 8) ^ (tr >> 16)) & 1) != 0;      // |gh| odd
+        const int bx = box[k.box], cnt = bx >> 16;
+        const Vec *R = Re + (r12 ? s.nE_C : 0) * QS + o * g.nk;
+        const long long ey = s.swap ? s.eAB : s.ket[g.ket0 + dnij.div(o)].eoff;
+        const Vec *E = E0 + ey + (k.off * nk2y + g.k0);
+        const int at = row * g.yp + k.k0 - g.y0;
+        if (k.m == 2)
+            ket_store<A, 2>(R, QS, hs + gh, nG, lst + (bx & 0xffff), cnt, E, cnt * nk2y, nk2y, g.nk, odd, neg,
+                            g.k0 > 0, T, at, tplane);
+        else
+            ket_store<A, 1>(R, QS, hs + gh, nG, lst + (bx & 0xffff), cnt, E, 0, nk2y, g.nk, odd, neg, g.k0 > 0, T,
+                            at, tplane);
+    }
+}
+
+// Bra pass of a group, outer primitive pairs in order (the group size changes no rounding):
+// G[c][x][y] += sum_ij sum_{j in box x} E^{ij}_x[j] T[ij][row(c, h_j)][y];
+// a thread sums all components of one x and one y (FP64) or two (packed).
+template <bool GAUGE, int A>
+__device__ __noinline__ void bra_pass(const Group g) {
+    typedef typename Arith<A>::Vec Vec;
+    constexpr int NC = GAUGE ? 7 : 1;
+    const TileState &s = tile_state();
+    const int nT = s.sh.nT, nk2x = s.nk2x, nij = g.nij, yp = g.yp;
+    const int tplane = g.nb * nij * nT * yp, r12off = (s.nhx - 4) * yp;
+    const int gc = g.xch * yp, gket = NC * gc, gplane = g.nb * gket;
+    const int ny = A == kF64 ? g.ych : (g.ych + 1) >> 1;
+    const int *box = at_byte<int>(s.o_box);
+    const unsigned char *lst0 = at_byte<unsigned char>(s.o_lst);
+    const uint4 *r12row = at_byte<uint4>(s.o_r12);
+    const FastDiv dy(ny), dx(g.xch);
+    for (int it = threadIdx.x; it < g.nb * g.xch * ny; it += blockDim.x) {
+        const int bx_ = dy.div(it), bk = dx.div(bx_), x = bx_ - bk * g.xch;
+        const int y = (it - bx_ * ny) * (A == kF64 ? 1 : 2);
+        const int2 fc = __ldg(reinterpret_cast<const int2 *>(s.fx + g.x0 + x));
+        const FuncPair f{fc.x, fc.y};
+        const int bx = box[f.fp >> 16], cnt = bx >> 16;
+        const unsigned char *lst = lst0 + (bx & 0xffff);
+        const Vec *ex = e_entries<A>(s.tb) + (s.swap ? s.ket[g.ket0 + bk].eoff : s.eAB) + f.off * nk2x;
+        const int gi = bk * gket + x * yp + y;
+        if constexpr (A == kF64) {
+            double sum[NC];
+            double *go = at_byte<double>(s.G) + gi;
 #pragma unroll
-                                for (int cc = 0; cc < NC; ++cc) s[cc] = g[cc * gc];
-                                for (int i = 0; i < nij; ++i) {
-                                    const int ij = ih + i0 + i;
-                                    const double *e = reinterpret_cast<const double *>(ex + (ij >> 1)) + (ij & 1);
-                                    const double *t = reinterpret_cast<const double *>(T) +
-                                                      (bk * nij + i) * sh.nT * yp + y;
-                                    const double *tr12 = t + (nhx - 4) * yp;
+            for (int cc = 0; cc < NC; ++cc) sum[cc] = go[cc * gc];
+            for (int i = 0; i < nij; ++i) {
+                const int ij = g.ih + g.i0 + i;
+                const double *e = reinterpret_cast<const double *>(ex + (ij >> 1)) + (ij & 1);
+                const double *t = at_byte<const double>(s.T) + (bk * nij + i) * nT * yp + y;
+                const double *tr12 = t + r12off;
 #pragma unroll 2
-                                    for (int j = 0; j < cnt; ++j) {
-                                        const int h = lst[j];
-                                        const double ev = __ldg(e + 2 * j * nk2x);
-                                        s[0] = fma(ev, t[h * yp], s[0]);
-                                        if constexpr (GAUGE) {
-                                            const uint4 w = b.r12row[h];
-                                            s[1] = fma(ev, tr12[(w.x & 0xffff) * yp], s[1]);
-                                            s[2] = fma(ev, tr12[(w.x >> 16) * yp], s[2]);
-                                            s[3] = fma(ev, tr12[(w.y & 0xffff) * yp], s[3]);
-                                            s[4] = fma(ev, tr12[(w.y >> 16) * yp], s[4]);
-                                            s[5] = fma(ev, tr12[(w.z & 0xffff) * yp], s[5]);
-                                            s[6] = fma(ev, tr12[(w.z >> 16) * yp], s[6]);
-                                        }
-                                    }
-                                }
-#pragma unroll
-                                for (int cc = 0; cc < NC; ++cc) g[cc * gc] = s[cc];
-                            } else {
-                                f32x2 ah[NC], al[NC];
-                                float *g = reinterpret_cast<float *>(G) + gi;
-#pragma unroll
-                                for (int cc = 0; cc < NC; ++cc) {
-                                    ah[cc] = *reinterpret_cast<const f32x2 *>(g + cc * gc);
-                                    al[cc] = A == kDF ? *reinterpret_cast<const f32x2 *>(g + gplane + cc * gc) : 0;
-                                }
-                                for (int i = 0; i < nij; ++i) {
-                                    const int ij = ih + i0 + i;
-                                    const float *e = reinterpret_cast<const float *>(ex + (ij >> 1)) + (ij & 1);
-                                    const float *t = reinterpret_cast<const float *>(T) +
-                                                     (bk * nij + i) * sh.nT * yp + y;
-                                    const float *tr12 = t + (nhx - 4) * yp;
-                                    constexpr int es = A == kDF ? 4 : 2;        // floats per two of primitive pairs
-#pragma unroll 2
-                                    for (int j = 0; j < cnt; ++j) {
-                                        const int h = lst[j];
-                                        const float eh = __ldg(e + es * j * nk2x);
-                                        const float el = A == kDF ? __ldg(e + es * j * nk2x + 2) : 0.f;
-                                        const ulonglong2 ev = make_ulonglong2(pack2(eh, eh), pack2(el, el));
-                                        auto term = [&](const float *tr, f32x2 &sh_, f32x2 &sl_) {
-                                            const f32x2 th = *reinterpret_cast<const f32x2 *>(tr);
-                                            if constexpr (A == kDF)
-                                                df_madd2(ev, make_ulonglong2(th, *reinterpret_cast<const f32x2 *>(tr + tplane)),
-                                                         sh_, sl_);
-                                            else
-                                                sh_ = fma2(ev.x, th, sh_);
-                                        };
-                                        term(t + h * yp, ah[0], al[0]);
-                                        if constexpr (GAUGE) {
-                                            const uint4 w = b.r12row[h];
-                                            term(tr12 + (w.x & 0xffff) * yp, ah[1], al[1]);
-                                            term(tr12 + (w.x >> 16) * yp, ah[2], al[2]);
-                                            term(tr12 + (w.y & 0xffff) * yp, ah[3], al[3]);
-                                            term(tr12 + (w.y >> 16) * yp, ah[4], al[4]);
-                                            term(tr12 + (w.z & 0xffff) * yp, ah[5], al[5]);
-                                            term(tr12 + (w.z >> 16) * yp, ah[6], al[6]);
-                                        }
-                                    }
-                                }
-#pragma unroll
-                                for (int cc = 0; cc < NC; ++cc) {
-                                    *reinterpret_cast<f32x2 *>(g + cc * gc) = ah[cc];
-                                    if (A == kDF) *reinterpret_cast<f32x2 *>(g + gplane + cc * gc) = al[cc];
-                                }
-                            }
-                        }
+                for (int j = 0; j < cnt; ++j) {
+                    const int h = lst[j];
+                    const double ev = __ldg(e + 2 * j * nk2x);
+                    sum[0] = fma(ev, t[h * yp], sum[0]);
+                    if constexpr (GAUGE) {
+                        const uint4 w = r12row[h];
+                        sum[1] = fma(ev, tr12[(w.x & 0xffff) * yp], sum[1]);
+                        sum[2] = fma(ev, tr12[(w.x >> 16) * yp], sum[2]);
+                        sum[3] = fma(ev, tr12[(w.y & 0xffff) * yp], sum[3]);
+                        sum[4] = fma(ev, tr12[(w.y >> 16) * yp], sum[4]);
+                        sum[5] = fma(ev, tr12[(w.z & 0xffff) * yp], sum[5]);
+                        sum[6] = fma(ev, tr12[(w.z >> 16) * yp], sum[6]);
                     }
                 }
             }
-            __syncthreads();
-            emit(ket0, nb, x0, xch, y0, ych, [&](int bk, int cc, int x, int y) -> double {
-                const int i = bk * gket + (cc * xch + x) * yp + y;
-                if constexpr (A == kF64) return reinterpret_cast<const double *>(G)[i];
-                const float *g = reinterpret_cast<const float *>(G);
-                return (double)g[i] + (double)g[gplane + i];
-            });
-            __syncthreads();
+#pragma unroll
+            for (int cc = 0; cc < NC; ++cc) go[cc * gc] = sum[cc];
+        } else {
+            constexpr int es = A == kDF ? 4 : 2;        // floats per two of primitive pairs
+            f32x2 ah[NC], al[NC];
+            float *go = at_byte<float>(s.G) + gi;
+#pragma unroll
+            for (int cc = 0; cc < NC; ++cc) {
+                ah[cc] = *reinterpret_cast<const f32x2 *>(go + cc * gc);
+                al[cc] = A == kDF ? *reinterpret_cast<const f32x2 *>(go + gplane + cc * gc) : 0;
+            }
+            for (int i = 0; i < nij; ++i) {
+                const int ij = g.ih + g.i0 + i;
+                const float *e = reinterpret_cast<const float *>(ex + (ij >> 1)) + (ij & 1);
+                const float *t = at_byte<const float>(s.T) + (bk * nij + i) * nT * yp + y;
+                const float *tr12 = t + r12off;
+#pragma unroll 2
+                for (int j = 0; j < cnt; ++j) {
+                    const int h = lst[j];
+                    const float eh = __ldg(e + es * j * nk2x);
+                    const float el = A == kDF ? __ldg(e + es * j * nk2x + 2) : 0.f;
+                    const ulonglong2 ev = make_ulonglong2(pack2(eh, eh), pack2(el, el));
+                    auto term = [&](const float *tr, f32x2 &sh, f32x2 &sl) {
+                        const f32x2 th = *reinterpret_cast<const f32x2 *>(tr);
+                        if constexpr (A == kDF)
+                            df_madd2(ev, make_ulonglong2(th, *reinterpret_cast<const f32x2 *>(tr + tplane)), sh, sl);
+                        else
+                            sh = fma2(ev.x, th, sh);
+                    };
+                    term(t + h * yp, ah[0], al[0]);
+                    if constexpr (GAUGE) {
+                        const uint4 w = r12row[h];
+                        term(tr12 + (w.x & 0xffff) * yp, ah[1], al[1]);
+                        term(tr12 + (w.x >> 16) * yp, ah[2], al[2]);
+                        term(tr12 + (w.y & 0xffff) * yp, ah[3], al[3]);
+                        term(tr12 + (w.y >> 16) * yp, ah[4], al[4]);
+                        term(tr12 + (w.z & 0xffff) * yp, ah[5], al[5]);
+                        term(tr12 + (w.z >> 16) * yp, ah[6], al[6]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int cc = 0; cc < NC; ++cc) {
+                *reinterpret_cast<f32x2 *>(go + cc * gc) = ah[cc];
+                if (A == kDF) *reinterpret_cast<f32x2 *>(go + gplane + cc * gc) = al[cc];
+            }
         }
-        c0 = c1;
     }
+}
+
+// Describes the tile of bra pair AB and `nkets` ket pairs TileState::ket of CD's kind (X = CD
+// when swap) to the phases; ends with a barrier.
+__device__ __noinline__ void set_tile(const PairTables &tb, const PairDev &AB, const PairDev &CD, bool swap, bool gauge,
+                                      int nkets, int pool) {
+    const PairDev &X = swap ? CD : AB, &Y = swap ? AB : CD;
+    if (threadIdx.x == 0) {
+        TileState &s = tile_state();
+        s.tb = tb;
+        s.fx = tb.fp + X.fpoff;
+        s.cy = tb.ch + Y.choff;
+        s.eAB = AB.eoff;
+        s.pAB = AB.ppoff;
+        s.swap = swap;
+        s.nkets = nkets;
+        s.L = X.Lab + Y.Lab;
+        s.Ltop = s.L + (gauge ? 2 : 0);
+        s.nppx = X.npp;
+        s.nfpx = X.nfp;
+        s.nk2x = X.nk2;
+        s.nppy = Y.npp;
+        s.nfpy = Y.nfp;
+        s.nk2y = Y.nk2;
+        s.nchy = Y.nch;
+        s.nhx = nherm(X.Lab);
+        s.nE_C = nherm(s.L);
+        s.nO_C = odd_len(s.L);
+        const Shape sh = quartet_shape(X.Lab, Y.Lab, gauge);
+        const Cut c = partition(sh, X.npp, X.nfp, Y.npp, Y.nfp, Y.nch, nkets, pool, (int)blockDim.x);
+        s.sh = sh;
+        s.c = c;
+        const int qs = q_stride(c.nb * c.nij * c.nkc), tbytes = c.nb * c.nij * sh.nT * y_stride(c.ych) * 8;
+        const int obytes = sh.nO * qs * 16;
+        const bool runs = c.nkc < Y.nk2;
+        s.Re = s.o_pool + sh.hs * c.nb * c.nijH * c.nkc * 16;
+        s.U = s.Re + sh.nE * qs * 16;
+        s.T = runs ? s.U + obytes : s.U;
+        s.G = s.U + (runs ? tbytes + obytes : max(tbytes, obytes));
+    }
+    __syncthreads();
+}
+
+// The blocks (X|Y) of the tile, some kets and chunks at a time; emit(g, value) is
+// called by all threads once a group's results stand in shared memory, value(ket, c,
+// x, y) being component c of function pairs x, y (sorted order, relative to the
+// chunk).
+// Components: 0 Coulomb; gauge kernel 1..6: (xy|d_I d_J r|zw), IJ = xx, xy, xz, yy, yz, zz.
+template <bool GAUGE, int A, class Emit>
+__device__ __forceinline__ void quartet_blocks(Emit emit) {
+    constexpr int NC = GAUGE ? 7 : 1;
+    const TileState &s = tile_state();
+    Group g;
+    for (g.ket0 = 0; g.ket0 < s.nkets; g.ket0 += s.c.nb) {
+        g.nb = min(s.c.nb, s.nkets - g.ket0);
+        for (g.c0 = 0; g.c0 < s.nchy; g.c0 = g.c1) {
+            g.y0 = s.cy[g.c0].k0;
+            g.c1 = s.nchy;
+            g.ych = s.nfpy - g.y0;
+            if (g.ych > s.c.ych) {
+                g.c1 = g.c0;
+                while (s.cy[g.c1].k0 + s.cy[g.c1].m - g.y0 <= s.c.ych) ++g.c1;
+                g.ych = s.cy[g.c1 - 1].k0 + s.cy[g.c1 - 1].m - g.y0;
+            }
+            g.yp = y_stride(g.ych);
+            for (g.x0 = 0; g.x0 < s.nfpx; g.x0 += s.c.xch) {
+                g.xch = min(s.c.xch, s.nfpx - g.x0);
+                const int gplane = g.nb * NC * g.xch * g.yp;    // FP32 pairs: high parts, then low parts
+                double *G = at_byte<double>(s.G);
+                for (int i = threadIdx.x; i < gplane; i += blockDim.x) G[i] = 0.0;
+                for (g.ih = 0; g.ih < s.nppx; g.ih += s.c.nijH) {
+                    g.nijH = min(s.c.nijH, s.nppx - g.ih);
+                    for (g.k0 = 0; g.k0 < s.nk2y; g.k0 += s.c.nkc) {
+                        g.nk = min(s.c.nkc, s.nk2y - g.k0);
+                        __syncthreads();                    // the last recursion has read the headers
+                        header_pass<GAUGE, A>(g);
+                        __syncthreads();
+                        for (g.i0 = 0; g.i0 < g.nijH; g.i0 += s.c.nij) {
+                            g.nij = min(s.c.nij, g.nijH - g.i0);
+                            if (s.Ltop & 1) __syncthreads();    // T, which the odd tensors overwrite, has been read
+                            recursion_pass<GAUGE, A>(g);     // ends with a barrier
+                            ket_pass<GAUGE, A>(g);
+                            __syncthreads();
+                            // T is complete with the last run of inner primitive pairs (with several, nijH == nij)
+                            if (g.k0 + g.nk == s.nk2y) bra_pass<GAUGE, A>(g);
+                        }
+                    }
+                }
+                __syncthreads();
+                emit(g, [&](int bk, int cc, int x, int y) -> double {
+                    const int i = ((bk * NC + cc) * g.xch + x) * g.yp + y;
+                    if constexpr (A == kF64) return G[i];
+                    const float *f = reinterpret_cast<const float *>(G);
+                    return (double)f[i] + (double)f[gplane + i];
+                });
+                __syncthreads();
+            }
+        }
     }
 }
 
@@ -1070,15 +1178,14 @@ __device__ void quartet_blocks(const PairTables &tb, const PairDev &AB, const Pa
 template <bool GAUGE, bool DF>
 __global__ void __launch_bounds__(256, 2) eri_rows_kernel(const EriParams *prms, const EriTask *tasks,
                                                           int *queue, Plan pl) {
-    extern __shared__ __align__(16) char sm[];
-    BlockSmem b = carve(sm, pl);
-    build_tables(pl, b);
+    build_tables(pl);
+    TileState &s = tile_state();
     const int nt = queue[1];
     const int ij_of[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
     for (;;) {
-        if (threadIdx.x == 0) *b.slot = atomicAdd(queue, 1);
+        if (threadIdx.x == 0) s.slot = atomicAdd(queue, 1);
         __syncthreads();
-        const int t = *b.slot;
+        const int t = s.slot;
         if (t >= nt) break;
         const EriTask tk = tasks[t];
         const EriParams &prm = prms[tk.req];
@@ -1109,29 +1216,30 @@ __global__ void __launch_bounds__(256, 2) eri_rows_kernel(const EriParams *prms,
                 k.col_rev = rev ? prm.ket_col[prm.ket_pos[tk.bra_sp]] : -1;
             }
             const unsigned mask = __ballot_sync(0xffffffffu, use);
-            if (use) b.ket[__popc(mask & ((1u << threadIdx.x) - 1u))] = k;
-            if (threadIdx.x == 0) b.slot[1] = __popc(mask);
+            if (use) s.ket[__popc(mask & ((1u << threadIdx.x) - 1u))] = k;
+            if (threadIdx.x == 0) s.n_use = __popc(mask);
         }
         __syncthreads();
-        const int nkets = b.slot[1];
+        const int nkets = s.n_use;
         if (nkets > 0) {
-            const PairDev AB = prm.pairs[tk.bra_sp];
-            const PairDev CD = prm.pairs[b.ket[0].id];      // all kets of the tile are of its kind
-            const PairTables tb{prm.pp, prm.E, prm.E2, prm.E1, prm.fp, prm.ch, prm.boys};
+            const PairDev &AB = prm.pairs[tk.bra_sp];
+            const PairDev &CD = prm.pairs[s.ket[0].id];     // all kets of the tile are of its kind
             // contract the orientation with fewer multiply-adds; swapped -> the block is (CD|AB)
             const bool swap = orient_madds(CD, AB, GAUGE) < orient_madds(AB, CD, GAUGE);
-            auto emit = [&](int ket0, int nb, int x0, int xch, int y0, int ych, auto value) {
-                const FuncPair *fpx = prm.fp + (swap ? CD.fpoff : AB.fpoff) + x0;
-                const FuncPair *fpy = prm.fp + (swap ? AB.fpoff : CD.fpoff) + y0;
-                const long long ldw = prm.ldw, ldwc = prm.ldwc, row0 = prm.row0;
+            set_tile(PairTables{prm.pp, prm.E, prm.E2, prm.E1, prm.fp, prm.ch, prm.boys}, AB, CD, swap, GAUGE, nkets,
+                     pl.pool);
+            auto emit = [&](const Group &g, auto value) {
+                const FuncPair *fpx = s.fx + g.x0;
+                const FuncPair *fpy = prm.fp + (swap ? AB.fpoff : CD.fpoff) + g.y0;
+                const long long ldw = prm.ldw, ldwc = prm.ldwc, row0 = prm.row0, rowAB = AB.rowoff - row0;
                 const bool wc = prm.with_coulomb != 0;
-                const FastDiv dy(ych), dx(xch);
-                for (int idx = threadIdx.x; idx < nb * xch * ych; idx += blockDim.x) {
-                    const int bx = dy.div(idx), yy = idx - bx * ych, bk = dx.div(bx), xx = bx - bk * xch;
+                const FastDiv dy(g.ych), dx(g.xch);
+                for (int idx = threadIdx.x; idx < g.nb * g.xch * g.ych; idx += blockDim.x) {
+                    const int bx = dy.div(idx), yy = idx - bx * g.ych, bk = dx.div(bx), xx = bx - bk * g.xch;
                     const int fx = fpx[xx].fp & 0xffff, fy = fpy[yy].fp & 0xffff;
                     const int a = swap ? fy : fx;                // bra function pair
                     const int c = swap ? fx : fy;                // ket function pair
-                    const KetRef &k = b.ket[ket0 + bk];
+                    const KetRef &k = s.ket[g.ket0 + bk];
                     const double C = value(bk, 0, xx, yy);
                     double hc[6];
                     if (GAUGE)
@@ -1152,7 +1260,7 @@ __global__ void __launch_bounds__(256, 2) eri_rows_kernel(const EriParams *prms,
                             if (wc) Wco[r * ldco + kc] = C;
                         }
                     };
-                    put(prm.W, ldw, prm.Wc, ldwc, AB.rowoff + a - row0, k.col + c);
+                    put(prm.W, ldw, prm.Wc, ldwc, rowAB + a, k.col + c);
                     // the same integrals at (cd, ab): rows of CD, columns of AB
                     if (k.col_rev >= 0) put(prm.W, ldw, prm.Wc, ldwc, k.rowoff + c - row0, k.col_rev + a);
                     if (k.mir) put(prm.W2, prm.ldw2, prm.Wc2, prm.ldwc2, k.rowoff + c - prm.row2,
@@ -1160,10 +1268,10 @@ __global__ void __launch_bounds__(256, 2) eri_rows_kernel(const EriParams *prms,
                 }
             };
             if constexpr (DF) {
-                if (tk.f32) quartet_blocks<GAUGE, kF32>(tb, AB, CD, swap, nkets, pl, b, emit);
-                else quartet_blocks<GAUGE, kDF>(tb, AB, CD, swap, nkets, pl, b, emit);
+                if (tk.f32) quartet_blocks<GAUGE, kF32>(emit);
+                else quartet_blocks<GAUGE, kDF>(emit);
             } else {
-                quartet_blocks<GAUGE, kF64>(tb, AB, CD, swap, nkets, pl, b, emit);
+                quartet_blocks<GAUGE, kF64>(emit);
             }
         }
         __syncthreads();
@@ -1187,8 +1295,8 @@ Plan eri_plan(int maxnfp, int maxLab, int maxnpp, bool gauge) {
     const int nk2 = std::max(1, std::min((npp + 1) / 2, kTensorBytes / ((s.hs + s.nE + s.nO) * 16)));
     const long long tables = (long long)plan_tables(p);
     auto bytes = [&](long long nij, long long nijH) {        // cut_bytes in 64 bits
-        const long long yp = (nfp + 1) / 2 * 2, t = nij * s.nT * yp * 8, o = s.nO * nij * nk2 * 16;
-        return s.hs * nijH * nk2 * 16 + s.nE * nij * nk2 * 16 + std::max(t, o) + s.NC * nfp * yp * 8;
+        const long long yp = y_stride(nfp), qs = (nij * nk2) | 1, t = nij * s.nT * yp * 8, o = s.nO * qs * 16;
+        return s.hs * nijH * nk2 * 16 + s.nE * qs * 16 + std::max(t, o) + s.NC * nfp * yp * 8;
     };
     const long long least = bytes(1, npp), most = bytes(npp, npp);
     for (int ti = 0; ti < 4; ++ti) {
@@ -1277,21 +1385,19 @@ void launch_split_pairs(const double2 *E, long long n, float4 *E2, float2 *E1, c
 
 // Schwarz diagonals: Q[AB] = max over ab of sqrt(|(ab|ab)|), Coulomb kernel.
 __global__ void __launch_bounds__(256, 2) schwarz_kernel(PairTables tb, const PairDev *pairs, Plan pl, double *Q) {
-    extern __shared__ __align__(16) char sm[];
-    const PairDev AB = pairs[blockIdx.x];
-    BlockSmem b = carve(sm, pl);
-    build_tables(pl, b);
-    if (threadIdx.x == 0) b.ket[0] = KetRef{AB.eoff, 0, 0, -1, AB.ppoff, (int)blockIdx.x, 0, 0};
+    const PairDev &AB = pairs[blockIdx.x];
+    build_tables(pl);
+    if (threadIdx.x == 0) tile_state().ket[0] = KetRef{AB.eoff, 0, 0, -1, AB.ppoff, (int)blockIdx.x, 0, 0};
     __syncthreads();
+    set_tile(tb, AB, AB, false, false, 1, pl.pool);
     double qmax = 0.0;
-    quartet_blocks<false, kF64>(tb, AB, AB, false, 1, pl, b,
-                                [&](int, int, int x0, int xch, int y0, int ych, auto value) {
-        for (int x = threadIdx.x; x < xch; x += blockDim.x) {
-            const int y = x0 + x - y0;
-            if (y >= 0 && y < ych) qmax = fmax(qmax, sqrt(fabs(value(0, 0, x, y))));
+    quartet_blocks<false, kF64>([&](const Group &g, auto value) {
+        for (int x = threadIdx.x; x < g.xch; x += blockDim.x) {
+            const int y = g.x0 + x - g.y0;
+            if (y >= 0 && y < g.ych) qmax = fmax(qmax, sqrt(fabs(value(0, 0, x, y))));
         }
     });
-    double *red = reinterpret_cast<double *>(b.pool);       // the block's last use of the pool is over
+    double *red = at_byte<double>(tile_state().o_pool);       // the block's last use of the pool is over
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) qmax = fmax(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = qmax;
