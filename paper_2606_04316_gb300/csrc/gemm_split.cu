@@ -17,15 +17,19 @@
 //    accumulate in FP32 over the whole K.  The result is recombined in FP64.
 //
 //  Tensor-core kernel: tcgen05.mma kind::f16 (BF16 x BF16 -> FP32), M = 128,
-//  N = 80, operands K-major in shared memory with the 128-byte swizzle, staged
+//  N up to 240, operands K-major in shared memory with the 128-byte swizzle, staged
 //  by TMA (cp.async.bulk.tensor): per K subtile of 64 the six B planes are
 //  loaded once into one of two panels and the six A planes into one stage
-//  each, all tracked by mbarriers; six FP32 accumulators (480 of the 512 TMEM
-//  columns) per CTA.  N = 80 is the widest tile whose six accumulators fit the
-//  TMEM; each MMA then reads 6.5 KB of operands per 46 cycles instead of 6 KB
-//  per 37 (N = 64), which eases the shared-memory bandwidth the tensor pipe
-//  waits on.  Roles: one thread issues the TMA loads, one the MMAs (its loops
-//  unrolled over the digit pairs, so A stage, barrier phase, accumulator and
+//  each, all tracked by mbarriers; six FP32 accumulators of 80 columns (480 of the
+//  512 TMEM columns) per CTA.  The B planes of a panel lie one after another, as do
+//  the accumulators of neighbouring diagonals, so one MMA multiplies an A plane
+//  with up to three B planes: nine MMAs per 16 K instead of 21.  What bounds the
+//  kernel is the shared memory: a 128 x 80 MMA reads 6.5 KB of operands for 40
+//  cycles of the tensor pipe, a 128 x 240 one 11.5 KB for 120 (24-centre chain, all
+//  blocks, slicing included: first half 93.7 -> 72.1 ms, second 12.0 -> 9.8; 40-centre
+//  chain, Coulomb: 81.8 -> 60.5 and 21.1 -> 16.5, i.e. 1560 TF/s of digit products).
+//  Roles: one thread issues the TMA loads, one the MMAs (its loops
+//  unrolled over the digit planes, so A stage, barrier phase, accumulator and
 //  descriptors are compile-time constants), eight warps (two per TMEM lane
 //  quadrant, 40 columns each) fold the exact diagonals and write the result.
 //  Every wait is bounded and reports a timeout through a device status word
@@ -36,6 +40,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
+#include <type_traits>
 #include <vector>
 
 #include "split.cuh"
@@ -300,14 +305,17 @@ __device__ inline uint64_t sdesc(uint32_t addr) {
     return d;
 }
 
-// instruction descriptor: D = F32, A = B = BF16, both K-major, N = 64, M = 128
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(SBN >> 3) << 17) |
-                            ((uint32_t)(SBM >> 4) << 24);
+// instruction descriptor: D = F32, A = B = BF16, both K-major, M = 128, N = n
+__host__ __device__ constexpr uint32_t idesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(SBM >> 4) << 24);
+}
 
+template <int N>
 __device__ inline void umma(uint32_t d, uint64_t a, uint64_t b, uint32_t acc) {
+    static_assert(N % 16 == 0 && N >= 16 && N <= 256, "tcgen05.mma, M = 128");
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-        "l"(a), "l"(b), "r"(kIdesc), "r"(acc)
+        "l"(a), "l"(b), "r"(idesc(N)), "r"(acc)
         : "memory");
 }
 
@@ -437,14 +445,32 @@ __global__ void __launch_bounds__(kThreads, 1)
                         }
                         tc_fence_after();
                         const uint64_t da = da0 + (uint64_t)((i * kATile) >> 4);
-#pragma unroll
-                        for (int j = 0; j < kSlices - i; ++j) {
-                            const int a = i + j;
-                            const bool fresh_i = i == 0 && (a <= 2 ? chunk_first : first_kt);
+                        // digit planes of B lie one after another, and so do the accumulators of
+                        // neighbouring diagonals: one MMA multiplies A plane i with up to three B
+                        // planes (N = 240), first those of the exact diagonals
+                        auto issue = [&](auto planes, int j, bool fresh) {
 #pragma unroll
                             for (int k16 = 0; k16 < SBK / 16; ++k16)
-                                umma(tmem + (uint32_t)(a * SBN), da + (uint64_t)(2 * k16),
-                                     db + (uint64_t)(j * (kBTile >> 4) + 2 * k16), (fresh_i && k16 == 0) ? 0u : 1u);
+                                umma<decltype(planes)::value * SBN>(
+                                    tmem + (uint32_t)((i + j) * SBN), da + (uint64_t)(2 * k16),
+                                    db + (uint64_t)(j * (kBTile >> 4) + 2 * k16), (fresh && k16 == 0) ? 0u : 1u);
+                        };
+                        using std::integral_constant;
+                        if (i == 0) {
+                            issue(integral_constant<int, 3>(), 0, chunk_first);
+                            issue(integral_constant<int, 3>(), 3, first_kt);
+                        } else if (i == 1) {
+                            issue(integral_constant<int, 3>(), 0, false);
+                            issue(integral_constant<int, 2>(), 3, false);
+                        } else if (i == 2) {
+                            issue(integral_constant<int, 2>(), 0, false);
+                            issue(integral_constant<int, 2>(), 2, false);
+                        } else if (i == 3) {
+                            issue(integral_constant<int, 3>(), 0, false);
+                        } else if (i == 4) {
+                            issue(integral_constant<int, 2>(), 0, false);
+                        } else {
+                            issue(integral_constant<int, 1>(), 0, false);
                         }
                         umma_commit(aempty + i);
                     }
