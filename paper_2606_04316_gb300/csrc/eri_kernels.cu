@@ -159,6 +159,18 @@ __global__ void split_pairs_kernel(const double2 *E, long long n, float4 *E2, fl
     }
 }
 
+// EX of one shell pair per CTA: its entries as FP32 pairs (hi, lo), primitive pair by
+// primitive pair.
+__global__ void bra_entries_kernel(const PairDev *pairs, const double2 *E, float2 *EX) {
+    const PairDev p = pairs[blockIdx.x];
+    const double *e = reinterpret_cast<const double *>(E + p.eoff);
+    float2 *o = EX + 2 * p.eoff;
+    for (int i = threadIdx.x; i < p.nbox * p.npp; i += blockDim.x) {
+        const int ij = i / p.nbox, k = i - ij * p.nbox;
+        o[i] = df_split(e[2 * (k * p.nk2 + (ij >> 1)) + (ij & 1)]);
+    }
+}
+
 // Header of a primitive quartet in FP64: Q - P, then R^n_000 of the Coulomb tensor
 // (n = 0..L) and, for the gauge kernel, of the r12 tensor (n = 0..L+2).
 __host__ __device__ inline int header_len(int L, bool gauge) { return gauge ? 2 * L + 7 : L + 4; }
@@ -507,6 +519,7 @@ struct PairTables {
     const double2 *E;
     const float4 *E2;
     const float2 *E1;
+    const float2 *EX;
     const FuncPair *fp;
     const PairChunk *ch;
     const double *boys;
@@ -520,13 +533,13 @@ struct PairTables {
 struct TileState {
     PairTables tb;
     const FuncPair *fx;          // X's and Y's tables
-    const PairChunk *cy;
+    const PairChunk *cy, *cx;
     long long eAB;               // AB's first E entry
     int pAB;                     // and primitive pair
     int swap;                    // X is the ket pair, Y the bra pair AB
     int nkets;
     int L, Ltop;                 // Hermite order of the quartet; top order of its tensors
-    int nppx, nfpx, nk2x, nppy, nfpy, nk2y, nchy, nhx;
+    int nppx, nfpx, nk2x, nchx, nboxx, nppy, nfpy, nk2y, nchy, nhx;
     int nE_C, nO_C;              // entries of the even and odd tensors before the r12 tensor
     Shape sh;
     Cut c;
@@ -534,8 +547,8 @@ struct TileState {
     KetRef ket[kMaxKets];        // the tile's kets to compute
     int slot, n_use;             // tile index, kets to compute
     // byte offsets of the tables (built once per CTA) and the pool (headers first)
-    int o_src, o_trip, o_box, o_hs, o_r12, o_lst, o_pool;
-    int nG;
+    int o_src, o_trip, o_box, o_hs, o_rows, o_lst, o_pool;
+    int nG, nhm;
 };
 
 // Shared memory: TileState, tables, pool.  Every function takes its pointers from
@@ -553,15 +566,15 @@ struct Group {
 __host__ __device__ inline int up16(int n) { return (n + 15) & ~15; }
 // Tables: recursion sources of R_h (int2[nTab]); Hermite triple h -> t | u << 8 | v <<
 // 16 (int[nTab]); per box its first list entry | count << 16 (int[nhm]); Hermite index
-// of the sum of two triples (unsigned short[nhm][nG]); Hermite indices of h + e_I + e_J,
-// 16 bits each (uint4[nhm]); Hermite indices of the boxes' entries (unsigned char[nLst]).
+// of the sum of two triples (unsigned short[nhm][nG]); Hermite index that component c's T
+// row has for h: h, then h + e_I + e_J (unsigned short[7][nhm]); Hermite indices of the boxes' entries (unsigned char[nLst]).
 __host__ __device__ inline int table_bytes(const Plan &p, int (&o)[7]) {
     o[0] = up16((int)sizeof(TileState));
     o[1] = o[0] + up16(p.nTab * 8);
     o[2] = o[1] + up16(p.nTab * 4);
     o[3] = o[2] + up16(p.nhm * 4);
     o[4] = o[3] + up16(p.nG * p.nhm * 2);
-    o[5] = o[4] + p.nhm * 16;
+    o[5] = o[4] + up16(7 * p.nhm * 2);
     o[6] = o[5] + up16(p.nLst);
     return o[6];
 }
@@ -587,7 +600,7 @@ __device__ void build_tables(const Plan &p) {
     int2 *src = at_byte<int2>(o[0]);
     int *trip = at_byte<int>(o[1]), *box = at_byte<int>(o[2]);
     unsigned short *hs = at_byte<unsigned short>(o[3]);
-    uint4 *r12row = at_byte<uint4>(o[4]);
+    unsigned short *rows = at_byte<unsigned short>(o[4]);
     unsigned char *lst = at_byte<unsigned char>(o[5]);
     if (threadIdx.x == 0) {
         TileState &s = tile_state();
@@ -595,7 +608,8 @@ __device__ void build_tables(const Plan &p) {
         s.o_trip = o[1];
         s.o_box = o[2];
         s.o_hs = o[3];
-        s.o_r12 = o[4];
+        s.o_rows = o[4];
+        s.nhm = p.nhm;
         s.o_lst = o[5];
         s.o_pool = o[6];
         s.nG = p.nG;
@@ -627,9 +641,14 @@ __device__ void build_tables(const Plan &p) {
             for (int x = 0; x <= t; ++x)
                 for (int y = 0; y <= u; ++y)
                     for (int z = 0; z <= v; ++z) lst[at++] = (unsigned char)hidx(x, y, z);
-            r12row[h] = make_uint4(hidx(t + 2, u, v) | (hidx(t + 1, u + 1, v) << 16),
-                                     hidx(t + 1, u, v + 1) | (hidx(t, u + 2, v) << 16),
-                                     hidx(t, u + 1, v + 1) | (hidx(t, u, v + 2) << 16), 0u);
+            unsigned short *row = rows + h;
+            row[0] = (unsigned short)h;
+            row[p.nhm] = (unsigned short)hidx(t + 2, u, v);
+            row[2 * p.nhm] = (unsigned short)hidx(t + 1, u + 1, v);
+            row[3 * p.nhm] = (unsigned short)hidx(t + 1, u, v + 1);
+            row[4 * p.nhm] = (unsigned short)hidx(t, u + 2, v);
+            row[5 * p.nhm] = (unsigned short)hidx(t, u + 1, v + 1);
+            row[6 * p.nhm] = (unsigned short)hidx(t, u, v + 2);
         }
     }
     __syncthreads();
@@ -660,11 +679,15 @@ __host__ __device__ inline int y_stride(int ych) {
 // Entry stride of the tensors, in twos of primitive quartets: odd, so that 16-byte
 // loads of consecutive entries (the lanes of the ket pass) fall into different banks.
 __host__ __device__ inline int q_stride(int q) { return q | 1; }
-__host__ __device__ inline int cut_bytes(const Shape &s, int nk2, int nb, int xch, int ych, int nkc, int nij, int nijH) {
-    const int yp = y_stride(ych), qs = q_stride(nb * nij * nkc);
-    const int t = nb * nij * s.nT * yp * 8, o = s.nO * qs * 16;
-    return s.hs * nb * nijH * nkc * 16 + s.nE * qs * 16 + (nkc < nk2 ? t + o : (t > o ? t : o)) +
-           nb * s.NC * xch * yp * 8;
+// (64 bits: the sizes tried for dozens of kets of contractions of dozens of primitives
+// exceed 32.)
+__host__ __device__ inline long long cut_bytes(const Shape &s, int nk2, int nb, int xch, int ych, int nkc, int nij,
+                                               int nijH) {
+    const long long col = (long long)nb * nij, qs = (col * nkc) | 1;
+    const int yp = y_stride(ych);
+    const long long t = col * s.nT * yp * 8, o = s.nO * qs * 16;
+    return (long long)s.hs * nb * nijH * nkc * 16 + s.nE * qs * 16 + (nkc < nk2 ? t + o : (t > o ? t : o)) +
+           (long long)nb * s.NC * xch * yp * 8;
 }
 // The cut decides no rounding except where the inner primitive pairs are cut (nkc,
 // contractions of dozens of primitives), and that depends on the quartet alone:
@@ -691,11 +714,16 @@ __host__ __device__ inline Cut partition(const Shape &s, int nppx, int nfpx, int
     }
     const int np = nppx > 1 ? nppx : 1, items = s.nT * nchy, want = 4 * threads;
     if (c.nkc == nk2 && c.xch == nfpx && c.ych == nfpy) {
-                int nb = (want + items - 1) / items;
+        // kets until the ket pass has its four rounds with three outer primitive pairs each:
+        // a ket's columns, 3 x 5 twos of two uncontracted-by-three pairs, then sit together
+        // (kets first, one outer pair: 179 ms for the integrals of a 24-centre chain and
+        // 139 for 40 centres; two 174 and 135, three 172 and 132, all nine 177 and 140)
+        const int nij0 = np < 3 ? np : 3;
+        int nb = (want + items * nij0 - 1) / (items * nij0);
         const int nbh = (2 * threads + np * nppy - 1) / (np * (nppy > 1 ? nppy : 1));   // two header rounds
         if (nb < nbh) nb = nbh;
         if (nb > nkets) nb = nkets;
-        while (nb > 1 && cut_bytes(s, nk2, nb, c.xch, c.ych, c.nkc, 1, np) > pool) --nb;
+        while (nb > 1 && cut_bytes(s, nk2, nb, c.xch, c.ych, c.nkc, nij0, np) > pool) --nb;
         if (nb > 1) {
             const int groups = (nkets + nb - 1) / nb;
             c.nb = (nkets + groups - 1) / groups;
@@ -708,7 +736,7 @@ __host__ __device__ inline Cut partition(const Shape &s, int nppx, int nfpx, int
     c.nij = (np + groups - 1) / groups;
     c.nijH = c.nb > 1 ? np : c.nij;
     if (c.nb == 1 && c.nkc == nk2) {
-        const int rest = pool - cut_bytes(s, nk2, 1, c.xch, c.ych, c.nkc, c.nij, 0);
+        const int rest = pool - (int)cut_bytes(s, nk2, 1, c.xch, c.ych, c.nkc, c.nij, 0);
         int h = rest / (s.hs * c.nkc * 16);
         if (h > np) h = np;
         if (h < np) h = h / c.nij * c.nij;
@@ -877,13 +905,14 @@ __device__ __noinline__ void header_pass(const Group g) {
 }
 
 // Hermite recursion of a group, one auxiliary order per pass; order 0 ends in the
-// even tensors.  Items: (entry, ket, outer primitive pair, two of inner ones).
-template <bool GAUGE, int A>
-__device__ __noinline__ void recursion_pass(const Group g) {
-    typedef typename Arith<A>::Vec Vec;
-    typedef typename Arith<A == kF64 ? kF64 : kDF>::Vec HVec;
+// even tensors.  In FP64 the double-precision units bound it: items (entry, column) are
+// spread over all threads without a remainder (columns kept by a thread: 12.3 instead of
+// 11.5 ms for the integrals of a 7-centre chain).
+template <bool GAUGE>
+__device__ __forceinline__ void recursion_f64(const Group &g) {
+    typedef double2 Vec;
     const TileState &s = tile_state();
-    const HVec *H = at_byte<HVec>(s.o_pool);
+    const Vec *H = at_byte<Vec>(s.o_pool);
     Vec *Re = at_byte<Vec>(s.Re), *Ro = at_byte<Vec>(s.U);
     const int2 *stab = at_byte<int2>(s.o_src);
     const int L = s.L, Ltop = s.Ltop, nE_C = s.nE_C, nO_C = s.nO_C;
@@ -905,29 +934,108 @@ __device__ __noinline__ void recursion_pass(const Group g) {
             const int h = r12 ? e - cC : e;
             Vec r;
             if (h == 0) {
-                const HVec v = H[(r12 ? jR : jC) + hq];
-                if constexpr (A == kF32) r = v.x;
-                else r = v;
+                r = H[(r12 ? jR : jC) + hq];
             } else {
                 const int2 sw = stab[h];
                 const Vec *sp = src + (r12 ? sR : 0) + q;
-                const HVec xv = H[(sw.x & 3) * QH + hq];
+                const Vec xv = H[(sw.x & 3) * QH + hq];
                 const Vec a = sp[((sw.x >> 2) & 1023) * QS];
                 const Vec cc = sp[(sw.x >> 12) * QS];
-                const float cf = __int_as_float(sw.y);
-                if constexpr (A == kF64) {
-                    const double cd = (double)cf;
-                    r = make_double2(fma(cd, cc.x, xv.x * a.x), fma(cd, cc.y, xv.y * a.y));
-                } else if constexpr (A == kDF) {
-                    r = df_rec2(xv, a, pack2(cf, cf), cc);
-                } else {
-                    r = fma2(xv.x, a, mul2(pack2(cf, cf), cc));
-                }
+                const double cf = (double)__int_as_float(sw.y);
+                r = make_double2(fma(cf, cc.x, xv.x * a.x), fma(cf, cc.y, xv.y * a.y));
             }
             dst[((r12 ? dR : 0) + h) * QS + q] = r;
         }
         __syncthreads();
     }
+}
+
+template <int A>
+__device__ __forceinline__ typename Arith<A>::Vec rec_step(Arith<kDF>::Vec x, typename Arith<A>::Vec a, float cf,
+                                                           typename Arith<A>::Vec c) {
+    if constexpr (A == kDF) return df_rec2(x, a, pack2(cf, cf), c);
+    else return fma2(x.x, a, mul2(pack2(cf, cf), c));
+}
+
+// In FP32 (pairs) the shared-memory loads and the integer work around a step bound it: a
+// thread keeps one column (ket, outer primitive pair, two of inner ones) with the Q - P
+// that most entries step along, and takes two entries at a time, whose loads and about ten
+// dependent operations hide each other.  In the gauge kernel an entry of the Coulomb
+// tensor goes with the same entry of the r12 tensor: same sources, same Q - P.  Sources
+// whose coefficient is zero are not read.  Integrals of a 24-centre chain 172.6 ms, of an
+// 18-atom cluster 205; with items (entry, column) 178.6 and 214.5.
+template <bool GAUGE, int A>
+__device__ __forceinline__ void recursion_columns(const Group &g) {
+    typedef typename Arith<A>::Vec Vec;
+    typedef Arith<kDF>::Vec HVec;
+    const TileState &s = tile_state();
+    const int2 *stab = at_byte<int2>(s.o_src);
+    const int L = s.L, Ltop = s.Ltop;
+    const int Q2 = g.nb * g.nij * g.nk, QS = q_stride(Q2), QH = g.nb * g.nijH * g.nk;
+    // columns of the group in runs of at most the CTA's threads, W threads to a column
+    const int qn = min(Q2, (int)blockDim.x), W = (int)blockDim.x / qn;
+    const int e0 = (int)threadIdx.x / qn, qt = (int)threadIdx.x - e0 * qn;
+    const FastDiv db1(g.nij * g.nk);
+    const int dE = GAUGE ? s.nE_C * QS : 0, dO = GAUGE ? s.nO_C * QS : 0;       // the r12 tensor's parts
+    auto head = [](HVec v) -> Vec {
+        if constexpr (A == kF32) return v.x;
+        else return v;
+    };
+    for (int q0 = 0; q0 < Q2; q0 += qn) {
+        const int q = q0 + qt;
+        const bool mine = q < Q2 && e0 < W;
+        const HVec *Hq = at_byte<HVec>(s.o_pool) +
+                         (mine ? q + g.i0 * g.nk + (g.nb > 1 ? db1.div(q) * (g.nijH - g.nij) * g.nk : 0) : 0);
+        const HVec X0 = *Hq;                    // most entries step along x
+        for (int m = Ltop; m >= 0; --m) {
+            const int cC = m <= L ? nherm(L - m) : 0;                   // Coulomb tensor (with GAUGE: the second one)
+            const int cR = GAUGE ? nherm(Ltop - m) : cC;
+            Vec *dp = at_byte<Vec>((m & 1) ? s.U : s.Re) + q;
+            const Vec *sp = at_byte<Vec>((m & 1) ? s.Re : s.U) + q;
+            const int dR = (m & 1) ? dO : dE, sR = (m & 1) ? dE : dO;
+            if (m == Ltop) {            // one entry; there is no order above to read
+                if (mine && e0 == 0) dp[dR] = head(Hq[(GAUGE ? 4 + L + m : 3 + m) * QH]);
+            } else if (mine) {
+#pragma unroll 1
+                for (int h = e0; h < cR; h += 2 * W) {
+                    const int h2 = h + W;
+                    const bool two = h2 < cR;
+                    const int2 w1 = stab[h], w2 = stab[two ? h2 : h];
+                    const int a1 = ((w1.x >> 2) & 1023) * QS, b1 = (w1.x >> 12) * QS;
+                    const int a2 = ((w2.x >> 2) & 1023) * QS, b2 = (w2.x >> 12) * QS;
+                    HVec x1 = X0, x2 = X0;
+                    if (w1.x & 3) x1 = Hq[(w1.x & 3) * QH];
+                    if (w2.x & 3) x2 = Hq[(w2.x & 3) * QH];
+                    const float f1 = __int_as_float(w1.y), f2 = __int_as_float(w2.y);
+                    Vec r1 = sp[sR + a1], r2 = sp[sR + a2], c1 = r1, c2 = r2;     // coefficient 0: any value
+                    if (w1.y) c1 = sp[sR + b1];
+                    if (w2.y) c2 = sp[sR + b2];
+                    r1 = rec_step<A>(x1, r1, f1, c1);
+                    r2 = rec_step<A>(x2, r2, f2, c2);
+                    if (h == 0) r1 = head(Hq[(GAUGE ? 4 + L + m : 3 + m) * QH]);
+                    dp[dR + h * QS] = r1;
+                    if (two) dp[dR + h2 * QS] = r2;
+                    if (GAUGE && h < cC) {
+                        r1 = sp[a1], r2 = sp[a2], c1 = r1, c2 = r2;
+                        if (w1.y) c1 = sp[b1];
+                        if (w2.y) c2 = sp[b2];
+                        r1 = rec_step<A>(x1, r1, f1, c1);
+                        r2 = rec_step<A>(x2, r2, f2, c2);
+                        if (h == 0) r1 = head(Hq[(3 + m) * QH]);
+                        dp[h * QS] = r1;
+                        if (h2 < cC) dp[h2 * QS] = r2;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
+template <bool GAUGE, int A>
+__device__ __noinline__ void recursion_pass(const Group g) {
+    if constexpr (A == kF64) recursion_f64<GAUGE>(g);
+    else recursion_columns<GAUGE, A>(g);
 }
 
 // Ket pass of a group: T rows h < nhx from the Coulomb tensor, then (gauge) rows
@@ -947,6 +1055,7 @@ __device__ __noinline__ void ket_pass(const Group g) {
     const unsigned short *hs = at_byte<unsigned short>(s.o_hs);
     const unsigned char *lst = at_byte<unsigned char>(s.o_lst);
     const int nG = s.nG;
+    const bool swap = s.swap != 0;
     const FastDiv drow(nrows), dT(nT), dnij(g.nij);
     for (int it = threadIdx.x; it < nrows * (g.c1 - g.c0); it += blockDim.x) {
         const int ci = drow.div(it), row = it - ci * nrows;
@@ -959,7 +1068,7 @@ __device__ __noinline__ void ket_pass(const Group g) {
         const bool neg = ((tr ^ (tr >> 8) ^ (tr >> 16)) & 1) != 0;      // |gh| odd
         const int bx = box[k.box], cnt = bx >> 16;
         const Vec *R = Re + (r12 ? s.nE_C : 0) * QS + o * g.nk;
-        const long long ey = s.swap ? s.eAB : s.ket[g.ket0 + dnij.div(o)].eoff;
+        const long long ey = swap ? s.eAB : s.ket[g.ket0 + dnij.div(o)].eoff;
         const Vec *E = E0 + ey + (k.off * nk2y + g.k0);
         const int at = row * g.yp + k.k0 - g.y0;
         if (k.m == 2)
@@ -971,105 +1080,153 @@ __device__ __noinline__ void ket_pass(const Group g) {
     }
 }
 
-// Bra pass of a group, outer primitive pairs in order (the group size changes no rounding):
-// G[c][x][y] += sum_ij sum_{j in box x} E^{ij}_x[j] T[ij][row(c, h_j)][y];
-// a thread sums all components of one x and one y (FP64) or two (packed).
-template <bool GAUGE, int A>
-__device__ __noinline__ void bra_pass(const Group g) {
+// Bra pass of a group, outer primitive pairs in order (neither the group nor the tile
+// changes a rounding):
+//   G[c][x][y] += sum_ij sum_{j in box x} E^{ij}_x[j] T[ij][row(c, h_j)][y].
+// A thread sums one component of TX function pairs x of one box and TY twos of function
+// pairs y (FP64: TY function pairs).  With TX = TY = 2 every E and T value loaded serves
+// two sums; with 1 there are four times as many items, for quartets so small that the
+// larger tile leaves most of the CTA without work (bra_pass chooses).
+template <bool GAUGE, int A, int TX, int TY>
+__device__ __forceinline__ void bra_tiles(const Group &g) {
     typedef typename Arith<A>::Vec Vec;
-    constexpr int NC = GAUGE ? 7 : 1;
+    constexpr int NC = GAUGE ? 7 : 1, W = A == kF64 ? 1 : 2;            // function pairs y per step
     const TileState &s = tile_state();
-    const int nT = s.sh.nT, nk2x = s.nk2x, nij = g.nij, yp = g.yp;
-    const int tplane = g.nb * nij * nT * yp, r12off = (s.nhx - 4) * yp;
-    const int gc = g.xch * yp, gket = NC * gc, gplane = g.nb * gket;
-    const int ny = A == kF64 ? g.ych : (g.ych + 1) >> 1;
+    const int nT = s.sh.nT, nk2x = s.nk2x, nij = g.nij, yp = g.yp, nb = g.nb, xch = g.xch;
+    const int tplane = nb * nij * nT * yp, r12off = s.nhx - 4;
+    const int gc = xch * yp, gplane = nb * NC * gc;
+    const int ny = (g.ych + W * TY - 1) / (W * TY), nx = TX > 1 ? s.nchx : xch;
+    const Vec *E0 = e_entries<A>(s.tb);
+    const float2 *EX = s.tb.EX;
+    const int nboxx = s.nboxx;
+    const int4 *cx = reinterpret_cast<const int4 *>(s.cx);
+    const int2 *fx = reinterpret_cast<const int2 *>(s.fx) + g.x0;
+    const bool swap = s.swap != 0;
+    const long long eAB = s.eAB;
     const int *box = at_byte<int>(s.o_box);
     const unsigned char *lst0 = at_byte<unsigned char>(s.o_lst);
-    const uint4 *r12row = at_byte<uint4>(s.o_r12);
-    const FastDiv dy(ny), dx(g.xch);
-    for (int it = threadIdx.x; it < g.nb * g.xch * ny; it += blockDim.x) {
-        const int bx_ = dy.div(it), bk = dx.div(bx_), x = bx_ - bk * g.xch;
-        const int y = (it - bx_ * ny) * (A == kF64 ? 1 : 2);
-        const int2 fc = __ldg(reinterpret_cast<const int2 *>(s.fx + g.x0 + x));
-        const FuncPair f{fc.x, fc.y};
-        const int bx = box[f.fp >> 16], cnt = bx >> 16;
-        const unsigned char *lst = lst0 + (bx & 0xffff);
-        const Vec *ex = e_entries<A>(s.tb) + (s.swap ? s.ket[g.ket0 + bk].eoff : s.eAB) + f.off * nk2x;
-        const int gi = bk * gket + x * yp + y;
-        if constexpr (A == kF64) {
-            double sum[NC];
-            double *go = at_byte<double>(s.G) + gi;
-#pragma unroll
-            for (int cc = 0; cc < NC; ++cc) sum[cc] = go[cc * gc];
-            for (int i = 0; i < nij; ++i) {
-                const int ij = g.ih + g.i0 + i;
-                const double *e = reinterpret_cast<const double *>(ex + (ij >> 1)) + (ij & 1);
-                const double *t = at_byte<const double>(s.T) + (bk * nij + i) * nT * yp + y;
-                const double *tr12 = t + r12off;
-#pragma unroll 2
-                for (int j = 0; j < cnt; ++j) {
-                    const int h = lst[j];
-                    const double ev = __ldg(e + 2 * j * nk2x);
-                    sum[0] = fma(ev, t[h * yp], sum[0]);
-                    if constexpr (GAUGE) {
-                        const uint4 w = r12row[h];
-                        sum[1] = fma(ev, tr12[(w.x & 0xffff) * yp], sum[1]);
-                        sum[2] = fma(ev, tr12[(w.x >> 16) * yp], sum[2]);
-                        sum[3] = fma(ev, tr12[(w.y & 0xffff) * yp], sum[3]);
-                        sum[4] = fma(ev, tr12[(w.y >> 16) * yp], sum[4]);
-                        sum[5] = fma(ev, tr12[(w.z & 0xffff) * yp], sum[5]);
-                        sum[6] = fma(ev, tr12[(w.z >> 16) * yp], sum[6]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int cc = 0; cc < NC; ++cc) go[cc * gc] = sum[cc];
+    const unsigned short *rows = at_byte<unsigned short>(s.o_rows);
+    const int nhm = s.nhm, ij0 = g.ih + g.i0;
+    char *const Gp = at_byte<char>(s.G), *const Tp = at_byte<char>(s.T);
+    const FastDiv dy(ny), dx(nx), db(nb);
+#pragma unroll 1
+    for (int it = threadIdx.x; it < NC * nb * nx * ny; it += blockDim.x) {
+        const int r0 = dy.div(it), r1 = dx.div(r0), c = NC > 1 ? db.div(r1) : 0;
+        const int y = (it - r0 * ny) * W * TY, xi = r0 - r1 * nx, bk = r1 - c * nb;
+        int x, m, bx, off;
+        if (TX > 1) {
+            const int4 k = __ldg(cx + xi);
+            x = k.x;
+            m = k.y;
+            bx = k.z;
+            off = k.w;
         } else {
-            constexpr int es = A == kDF ? 4 : 2;        // floats per two of primitive pairs
-            f32x2 ah[NC], al[NC];
-            float *go = at_byte<float>(s.G) + gi;
+            const int2 f = __ldg(fx + xi);
+            x = xi;
+            m = 1;
+            bx = f.x >> 16;
+            off = f.y;
+        }
+        const int bb = box[bx], cnt = bb >> 16;
+        const unsigned char *lst = lst0 + (bb & 0xffff);
+        const unsigned short *row = rows + c * nhm;
+        const int rowoff = c ? r12off : 0;
+        const long long eoff = swap ? s.ket[g.ket0 + bk].eoff : eAB;
+        const int x1 = TX > 1 && m > 1 ? cnt : 0;                      // the second x's entries
+        const int y1 = TY > 1 ? min(W, yp - W - y) : 0;                // the second y, or one in the row
+        const int gi = (bk * NC + c) * gc + x * yp + y;
+        if constexpr (A == kF64) {
+            double sum[TX][TY];
+            double *go = reinterpret_cast<double *>(Gp) + gi;
 #pragma unroll
-            for (int cc = 0; cc < NC; ++cc) {
-                ah[cc] = *reinterpret_cast<const f32x2 *>(go + cc * gc);
-                al[cc] = A == kDF ? *reinterpret_cast<const f32x2 *>(go + gplane + cc * gc) : 0;
-            }
+            for (int p = 0; p < TX; ++p)
+#pragma unroll
+                for (int q = 0; q < TY; ++q) sum[p][q] = go[(p < m ? p : 0) * yp + (q ? y1 : 0)];
+#pragma unroll 1
             for (int i = 0; i < nij; ++i) {
-                const int ij = g.ih + g.i0 + i;
-                const float *e = reinterpret_cast<const float *>(ex + (ij >> 1)) + (ij & 1);
-                const float *t = at_byte<const float>(s.T) + (bk * nij + i) * nT * yp + y;
-                const float *tr12 = t + r12off;
+                const double *e =
+                    reinterpret_cast<const double *>(E0 + eoff + off * nk2x + ((ij0 + i) >> 1)) + ((ij0 + i) & 1);
+                const double *t = reinterpret_cast<const double *>(Tp) + ((bk * nij + i) * nT + rowoff) * yp + y;
 #pragma unroll 2
                 for (int j = 0; j < cnt; ++j) {
-                    const int h = lst[j];
-                    const float eh = __ldg(e + es * j * nk2x);
-                    const float el = A == kDF ? __ldg(e + es * j * nk2x + 2) : 0.f;
-                    const ulonglong2 ev = make_ulonglong2(pack2(eh, eh), pack2(el, el));
-                    auto term = [&](const float *tr, f32x2 &sh, f32x2 &sl) {
-                        const f32x2 th = *reinterpret_cast<const f32x2 *>(tr);
-                        if constexpr (A == kDF)
-                            df_madd2(ev, make_ulonglong2(th, *reinterpret_cast<const f32x2 *>(tr + tplane)), sh, sl);
-                        else
-                            sh = fma2(ev.x, th, sh);
-                    };
-                    term(t + h * yp, ah[0], al[0]);
-                    if constexpr (GAUGE) {
-                        const uint4 w = r12row[h];
-                        term(tr12 + (w.x & 0xffff) * yp, ah[1], al[1]);
-                        term(tr12 + (w.x >> 16) * yp, ah[2], al[2]);
-                        term(tr12 + (w.y & 0xffff) * yp, ah[3], al[3]);
-                        term(tr12 + (w.y >> 16) * yp, ah[4], al[4]);
-                        term(tr12 + (w.z & 0xffff) * yp, ah[5], al[5]);
-                        term(tr12 + (w.z >> 16) * yp, ah[6], al[6]);
+                    const double *tr = t + row[lst[j]] * yp;
+                    double tv[TY];
+#pragma unroll
+                    for (int q = 0; q < TY; ++q) tv[q] = tr[q ? y1 : 0];
+#pragma unroll
+                    for (int p = 0; p < TX; ++p) {
+                        const double ev = __ldg(e + 2 * (p ? x1 : 0) * nk2x);
+#pragma unroll
+                        for (int q = 0; q < TY; ++q) sum[p][q] = fma(ev, tv[q], sum[p][q]);
                     }
+                    e += 2 * nk2x;
                 }
             }
 #pragma unroll
-            for (int cc = 0; cc < NC; ++cc) {
-                *reinterpret_cast<f32x2 *>(go + cc * gc) = ah[cc];
-                if (A == kDF) *reinterpret_cast<f32x2 *>(go + gplane + cc * gc) = al[cc];
+            for (int p = 0; p < TX; ++p)
+#pragma unroll
+                for (int q = 0; q < TY; ++q)
+                    if (p < m && (q == 0 || y + 1 < g.ych)) go[p * yp + q] = sum[p][q];
+        } else {
+            f32x2 ah[TX][TY], al[TX][TY];
+            float *go = reinterpret_cast<float *>(Gp) + gi;
+#pragma unroll
+            for (int p = 0; p < TX; ++p)
+#pragma unroll
+                for (int q = 0; q < TY; ++q) {
+                    const float *v = go + (p < m ? p : 0) * yp + (q ? y1 : 0);
+                    ah[p][q] = *reinterpret_cast<const f32x2 *>(v);
+                    al[p][q] = A == kDF ? *reinterpret_cast<const f32x2 *>(v + gplane) : 0;
+                }
+#pragma unroll 1
+            for (int i = 0; i < nij; ++i) {
+                const float2 *e = EX + 2 * eoff + (ij0 + i) * nboxx + off;
+                const float *t = reinterpret_cast<const float *>(Tp) + ((bk * nij + i) * nT + rowoff) * yp + y;
+#pragma unroll 2
+                for (int j = 0; j < cnt; ++j) {
+                    const float *tr = t + row[lst[j]] * yp;
+                    f32x2 th[TY], tl[TY];
+#pragma unroll
+                    for (int q = 0; q < TY; ++q) {
+                        th[q] = *reinterpret_cast<const f32x2 *>(tr + (q ? y1 : 0));
+                        if (A == kDF) tl[q] = *reinterpret_cast<const f32x2 *>(tr + tplane + (q ? y1 : 0));
+                    }
+#pragma unroll
+                    for (int p = 0; p < TX; ++p) {
+                        const float2 ep = __ldg(e + (p ? x1 : 0));
+                        const ulonglong2 ev = make_ulonglong2(pack2(ep.x, ep.x), pack2(ep.y, ep.y));
+#pragma unroll
+                        for (int q = 0; q < TY; ++q) {
+                            if constexpr (A == kDF) df_madd2(ev, make_ulonglong2(th[q], tl[q]), ah[p][q], al[p][q]);
+                            else ah[p][q] = fma2(ev.x, th[q], ah[p][q]);
+                        }
+                    }
+                    ++e;
+                }
             }
+#pragma unroll
+            for (int p = 0; p < TX; ++p)
+#pragma unroll
+                for (int q = 0; q < TY; ++q)
+                    if (p < m && (q == 0 || y + 2 < g.ych)) {
+                        *reinterpret_cast<f32x2 *>(go + p * yp + 2 * q) = ah[p][q];
+                        if (A == kDF) *reinterpret_cast<f32x2 *>(go + gplane + p * yp + 2 * q) = al[p][q];
+                    }
         }
     }
+}
+
+template <bool GAUGE, int A>
+__device__ __noinline__ void bra_pass(const Group g) {
+    constexpr int NC = GAUGE ? 7 : 1, W = A == kF64 ? 1 : 2;
+    const TileState &s = tile_state();
+    // rounds of the CTA times instructions per term, about 72 against 26 in FP32 pairs (never
+    // the larger tile: integrals of a 40-centre chain 131 -> 134 ms, of a class with d shells
+    // 63 -> 66, of a 24-centre chain with the gauge term the same)
+    const int n1 = NC * g.nb * g.xch * ((g.ych + W - 1) / W), n2 = NC * g.nb * s.nchx * ((g.ych + 2 * W - 1) / (2 * W));
+    const int nt = blockDim.x, r1 = (n1 + nt - 1) / nt, r2 = (n2 + nt - 1) / nt;
+    if (g.xch == s.nfpx && 11 * r2 < 4 * r1) bra_tiles<GAUGE, A, 2, 2>(g);
+    else bra_tiles<GAUGE, A, 1, 1>(g);
 }
 
 // Describes the tile of bra pair AB and `nkets` ket pairs TileState::ket of CD's kind (X = CD
@@ -1082,6 +1239,9 @@ __device__ __noinline__ void set_tile(const PairTables &tb, const PairDev &AB, c
         s.tb = tb;
         s.fx = tb.fp + X.fpoff;
         s.cy = tb.ch + Y.choff;
+        s.cx = tb.ch + X.choff;
+        s.nchx = X.nch;
+        s.nboxx = X.nbox;
         s.eAB = AB.eoff;
         s.pAB = AB.ppoff;
         s.swap = swap;
@@ -1226,7 +1386,7 @@ __global__ void __launch_bounds__(256, 2) eri_rows_kernel(const EriParams *prms,
             const PairDev &CD = prm.pairs[s.ket[0].id];     // all kets of the tile are of its kind
             // contract the orientation with fewer multiply-adds; swapped -> the block is (CD|AB)
             const bool swap = orient_madds(CD, AB, GAUGE) < orient_madds(AB, CD, GAUGE);
-            set_tile(PairTables{prm.pp, prm.E, prm.E2, prm.E1, prm.fp, prm.ch, prm.boys}, AB, CD, swap, GAUGE, nkets,
+            set_tile(PairTables{prm.pp, prm.E, prm.E2, prm.E1, prm.EX, prm.fp, prm.ch, prm.boys}, AB, CD, swap, GAUGE, nkets,
                      pl.pool);
             auto emit = [&](const Group &g, auto value) {
                 const FuncPair *fpx = s.fx + g.x0;
@@ -1377,8 +1537,11 @@ void launch_ratio(const double *A, const double *B, long long rows, long long ld
     QDT_CHECK_LAUNCH();
 }
 
-void launch_split_pairs(const double2 *E, long long n, float4 *E2, float2 *E1, cudaStream_t s) {
+void launch_split_pairs(const PairDev *pairs, int nsp, const double2 *E, long long n, float4 *E2, float2 *E1,
+                        float2 *EX, cudaStream_t s) {
     if (n <= 0) return;
+    bra_entries_kernel<<<nsp, 128, 0, s>>>(pairs, E, EX);
+    QDT_CHECK_KERNEL("bra_entries_kernel");
     split_pairs_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(E, n, E2, E1);
     QDT_CHECK_KERNEL("split_pairs_kernel");
 }
@@ -1413,7 +1576,7 @@ void launch_schwarz(const PairClass &pc, const double *boys, double *Q, cudaStre
     const Plan pl = eri_plan(pc.maxnfp, pc.maxLab, pc.maxnpp, false);
     const size_t smem = plan_smem(pl);
     QDT_CUDA_TRY(cudaFuncSetAttribute(schwarz_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const PairTables tb{pc.d_pp, pc.d_E, nullptr, nullptr, pc.d_fp, pc.d_ch, boys};
+    const PairTables tb{pc.d_pp, pc.d_E, nullptr, nullptr, nullptr, pc.d_fp, pc.d_ch, boys};
     schwarz_kernel<<<pc.nsp, pl.threads, smem, s>>>(tb, pc.d_pairs, pl, Q);
     QDT_CHECK_LAUNCH();
 }

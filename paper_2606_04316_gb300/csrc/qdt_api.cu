@@ -128,7 +128,7 @@ T *dcopy_pinned(PinnedArena &a, DBuf &b, const std::vector<T> &v, cudaStream_t s
 }
 
 struct ClassBufs {
-    DBuf pairs, pp, E, E2, E1, fp, ch, Q, bra, brapos, pp_pair;
+    DBuf pairs, pp, E, E2, E1, EX, fp, ch, Q, bra, brapos, pp_pair;
 };
 
 // Instantiated graph of a batch round and the signature it was captured for.
@@ -619,8 +619,9 @@ void build_class(qdt_ctx *ctx, int c) {
                           (const double *)ctx->norms.p, pc.d_fp, pc.d_pp, pc.d_E, s);
     pc.d_E2 = (float4 *)b.E2.get(std::max<long long>(1, eoff) * sizeof(float4));
     pc.d_E1 = (float2 *)b.E1.get(std::max<long long>(1, eoff) * sizeof(float2));
-    launch_split_pairs(pc.d_E, eoff, pc.d_E2, pc.d_E1, s);
-    ctx->launches += 2;
+    pc.d_EX = (float2 *)b.EX.get(std::max<long long>(1, 2 * eoff) * sizeof(float2));
+    launch_split_pairs(pc.d_pairs, pc.nsp, pc.d_E, eoff, pc.d_E2, pc.d_E1, pc.d_EX, s);
+    ctx->launches += 3;
     // Schwarz diagonals, then the bra order (Q descending, ties by id)
     pc.d_Q = (double *)b.Q.get(std::max(1, pc.nsp) * sizeof(double));
     launch_schwarz(pc, (const double *)ctx->boys.p, pc.d_Q, s);
@@ -1096,6 +1097,7 @@ void batch_prepare(qdt_ctx *ctx, const ClassPlan &P, int b0, RowBatch &B) {
     prm.E = pc.d_E;
     prm.E2 = P.precision == QDT_SPLIT ? pc.d_E2 : nullptr;
     prm.E1 = P.precision == QDT_SPLIT ? pc.d_E1 : nullptr;
+    prm.EX = P.precision == QDT_SPLIT ? pc.d_EX : nullptr;
     prm.fp = pc.d_fp;
     prm.ch = pc.d_ch;
     prm.boys = (const double *)ctx->boys.p;
@@ -1878,7 +1880,7 @@ void qdt_destroy(qdt_ctx *c) {
                     &c->kpre1, &c->ksplit1, &c->kbpos, &c->kbfirst};
     for (DBuf *b : bufs) b->release();
     for (int k = 0; k < 2; ++k) {
-        c->cb[k].pairs.release(); c->cb[k].pp.release(); c->cb[k].E.release(); c->cb[k].E2.release(); c->cb[k].E1.release(); c->cb[k].fp.release(); c->cb[k].ch.release();
+        c->cb[k].pairs.release(); c->cb[k].pp.release(); c->cb[k].E.release(); c->cb[k].E2.release(); c->cb[k].E1.release(); c->cb[k].EX.release(); c->cb[k].fp.release(); c->cb[k].ch.release();
         c->cb[k].Q.release(); c->cb[k].bra.release(); c->cb[k].brapos.release(); c->cb[k].pp_pair.release();
     }
     split_release(c->split);

@@ -167,6 +167,9 @@ struct PairClass {
     double2 *d_E = nullptr;
     float4 *d_E2 = nullptr;     // E as FP32 pairs (hi0, hi1, lo0, lo1) for the split form's integrals
     float2 *d_E1 = nullptr;     // the high parts alone, for the quartets run in plain FP32
+    // E as FP32 pairs (hi, lo), [primitive pair][function pair][box entry] from 2 eoff: what
+    // the bra pass reads of one outer primitive pair lies together
+    float2 *d_EX = nullptr;
     FuncPair *d_fp = nullptr;
     PairChunk *d_ch = nullptr;
     double *d_Q = nullptr;
@@ -189,6 +192,7 @@ struct EriParams {
     const double2 *E;
     const float4 *E2;           // E as FP32 pairs: non-null selects the compensated FP32 contraction
     const float2 *E1;           // fl32(E), read by the tiles run in plain FP32
+    const float2 *EX;           // E by outer primitive pair (PairClass::d_EX)
     const FuncPair *fp;
     const PairChunk *ch;
     const double *boys;         // [kBoysGrid][kBoysCols], followed by the same as floats
@@ -268,8 +272,10 @@ void launch_eri(const EriParams *prms, const EriTask *tasks, int maxtasks, int *
 // max |A - B| / (Q_row Q_col) over integral rows (FP32 error model check).
 void launch_ratio(const double *A, const double *B, long long rows, long long ldw, int mult, const int *row_pair,
                   const int *col_pair, long long ncols, const double *Q, double *out, cudaStream_t s);
-// E2[i] = (hi, lo) of the two entries of E[i], hi = fl32(x), lo = fl32(x - hi); E1[i] the hi parts.
-void launch_split_pairs(const double2 *E, long long n, float4 *E2, float2 *E1, cudaStream_t s);
+// E2[i] = (hi, lo) of the two entries of E[i], hi = fl32(x), lo = fl32(x - hi); E1[i] the hi parts;
+// EX: PairClass::d_EX.
+void launch_split_pairs(const PairDev *pairs, int nsp, const double2 *E, long long n, float4 *E2, float2 *E1,
+                        float2 *EX, cudaStream_t s);
 int eri_default_threads(const EriShape &shape, bool gauge);
 void launch_schwarz(const PairClass &pc, const double *boys, double *Q, cudaStream_t s);
 
