@@ -9,55 +9,51 @@
 
 namespace qdt {
 
-constexpr int TM = 64, TN = 64, TK = 16;
+// The FP64 units bound both (about two multiply-adds per cycle and SM): a warp's DFMA
+// holds its scheduler for tens of cycles, so one output per thread keeps the units as busy as
+// sixteen would, and the loads, two shared values per multiply-add, hide behind it.
+// What is left is the balance over the SMs, which small tiles give.  16 x 16 instead of
+// 64 x 64: first half of a 7-centre chain (9.3 GFLOP) 16.9 -> 7.7 ms, 1.2 TFLOP/s; of an
+// 8-function molecule (0.16 GFLOP) 0.86 -> 0.15 ms; their second halves 1.86 -> 0.37 and 0.12 -> 0.04.
+// The sum of an output runs over k in order whatever the tile, so the tile decides no
+// bit.  Row extents of the screened prefix stay per 64 rows.
+constexpr int TM = 64;                   // rows of one prefix extent; the second half's upper tiles
+constexpr int TS = 16, TK = 16;          // tile of a CTA; k per step (32: 7.80 ms instead of 7.74 below)
+constexpr int kThreads = TS * TS;
 
 int gemm_fp64_tile_m() { return TM; }
 
-// 256 threads, 4x4 outputs each, register-blocked DFMA.
-__global__ void __launch_bounds__(256) dgemm_nn_ragged(const double *__restrict__ A, long long lda,
-                                                       const double *__restrict__ B, long long ldb,
-                                                       double *__restrict__ C, long long ldc,
-                                                       long long M, long long N,
-                                                       const long long *__restrict__ ktile, int accumulate) {
-    __shared__ double As[TK][TM + 1];
-    __shared__ double Bs[TK][TN];
-    const long long m0 = (long long)blockIdx.y * TM, n0 = (long long)blockIdx.x * TN;
-    const long long K = ktile[blockIdx.y];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[4][4] = {};
+__global__ void __launch_bounds__(kThreads) dgemm_nn_ragged(const double *__restrict__ A, long long lda,
+                                                            const double *__restrict__ B, long long ldb,
+                                                            double *__restrict__ C, long long ldc,
+                                                            long long M, long long N,
+                                                            const long long *__restrict__ ktile, int accumulate) {
+    __shared__ double As[TS][TK + 1];
+    __shared__ double Bs[TK][TS];
+    const unsigned nt = (unsigned)((N + TS - 1) / TS), mt = blockIdx.x / nt;
+    const long long m0 = (long long)mt * TS, n0 = (long long)(blockIdx.x - mt * nt) * TS;
+    const long long K = ktile[m0 / TM];
+    const int tx = threadIdx.x % TS, ty = threadIdx.x / TS;
+    const int ar = threadIdx.x / TK, ac = threadIdx.x % TK;
+    double acc = 0.0;
     for (long long k0 = 0; k0 < K; k0 += TK) {
-        for (int i = threadIdx.x; i < TM * TK; i += 256) {
-            int r = i / TK, c = i % TK;
-            long long gr = m0 + r, gc = k0 + c;
-            As[c][r] = (gr < M && gc < K) ? A[gr * lda + gc] : 0.0;
+#pragma unroll
+        for (int i = 0; i < TS; i += kThreads / TK) {
+            const long long gr = m0 + ar + i, gc = k0 + ac;
+            As[ar + i][ac] = (gr < M && gc < K) ? A[gr * lda + gc] : 0.0;
         }
-        for (int i = threadIdx.x; i < TK * TN; i += 256) {
-            int r = i / TN, c = i % TN;
-            long long gr = k0 + r, gc = n0 + c;
-            Bs[r][c] = (gr < K && gc < N) ? B[gr * ldb + gc] : 0.0;
+#pragma unroll
+        for (int i = 0; i < TK; i += kThreads / TS) {
+            const long long gr = k0 + ty + i, gc = n0 + tx;
+            Bs[ty + i][tx] = (gr < K && gc < N) ? B[gr * ldb + gc] : 0.0;
         }
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < TK; ++k) {
-            double a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[k][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[k][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
+        for (int k = 0; k < TK; ++k) acc = fma(As[ty][k], Bs[k][tx], acc);
         __syncthreads();
     }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            long long r = m0 + ty + 16 * i, c = n0 + tx + 16 * j;
-            if (r < M && c < N) C[r * ldc + c] = accumulate ? C[r * ldc + c] + acc[i][j] : acc[i][j];
-        }
+    const long long r = m0 + ty, c = n0 + tx;
+    if (r < M && c < N) C[r * ldc + c] = accumulate ? C[r * ldc + c] + acc : acc;
 }
 
 void gemm_fp64_nn_ragged(const double *A, long long lda, const double *B, long long ldb, double *C,
@@ -65,58 +61,47 @@ void gemm_fp64_nn_ragged(const double *A, long long lda, const double *B, long l
                          cudaStream_t s, bool accumulate) {
     if (M <= 0 || N <= 0) return;
     if (tileM != TM) throw Error{QDT_ERR_ARG, "ragged GEMM tile mismatch"};
-    dim3 grid((unsigned)((N + TN - 1) / TN), (unsigned)((M + TM - 1) / TM));
-    dgemm_nn_ragged<<<grid, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, ktile, accumulate ? 1 : 0);
+    const long long tiles = ((N + TS - 1) / TS) * ((M + TS - 1) / TS);
+    if (tiles > 0x7fffffffLL) throw Error{QDT_ERR_ARG, "FP64 GEMM: too many tiles"};
+    dgemm_nn_ragged<<<(unsigned)tiles, kThreads, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, ktile, accumulate ? 1 : 0);
     QDT_CHECK_LAUNCH();
 }
 
-// C (N x N) = A^T B over K rows; upper block tiles (bi <= bj); split-K slices
+// C (N x N) = A^T B over K rows; upper 64 x 64 tiles (bi <= bj; without `whole` only what
+// the packer reads of the diagonal ones), TS x TS of them per CTA; split-K slices
 // write partial[slice][N][N]; a second kernel sums slices in fixed order and
 // mirrors nothing (only the upper tiles are consumed by the packer).
-__global__ void __launch_bounds__(256) dgemm_tn_upper(const double *__restrict__ A, long long lda,
-                                                      const double *__restrict__ B, long long ldb,
-                                                      double *__restrict__ P, long long N, long long K,
-                                                      long long kchunk, int ntb) {
-    __shared__ double As[TK][TM];
-    __shared__ double Bs[TK][TN];
+__global__ void __launch_bounds__(kThreads) dgemm_tn_upper(const double *__restrict__ A, long long lda,
+                                                           const double *__restrict__ B, long long ldb,
+                                                           double *__restrict__ P, long long N, long long K,
+                                                           long long kchunk, int ntb, int whole) {
+    constexpr int kSub = TM / TS;
+    __shared__ double As[TK][TS];
+    __shared__ double Bs[TK][TS];
     // decode the upper tile index
-    int t = blockIdx.x, bi = 0;
+    const int sub = blockIdx.x % (kSub * kSub);
+    int t = blockIdx.x / (kSub * kSub), bi = 0;
     while (t >= ntb - bi) { t -= ntb - bi; ++bi; }
-    int bj = bi + t;
-    const long long m0 = (long long)bi * TM, n0 = (long long)bj * TN;
+    const int bj = bi + t;
+    const long long m0 = (long long)bi * TM + sub / kSub * TS, n0 = (long long)bj * TM + sub % kSub * TS;
+    if (m0 >= N || n0 >= N || (!whole && m0 > n0)) return;
     const long long kb = (long long)blockIdx.y * kchunk, ke = min(K, kb + kchunk);
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[4][4] = {};
+    const int tx = threadIdx.x % TS, ty = threadIdx.x / TS;
+    double acc = 0.0;
     for (long long k0 = kb; k0 < ke; k0 += TK) {
-        for (int i = threadIdx.x; i < TK * TM; i += 256) {
-            int r = i / TM, c = i % TM;
-            long long gk = k0 + r;
-            As[r][c] = (gk < ke && m0 + c < N) ? A[gk * lda + m0 + c] : 0.0;
-            Bs[r][c] = (gk < ke && n0 + c < N) ? B[gk * ldb + n0 + c] : 0.0;
+#pragma unroll
+        for (int i = 0; i < TK; i += kThreads / TS) {
+            const long long gk = k0 + ty + i;
+            As[ty + i][tx] = (gk < ke && m0 + tx < N) ? A[gk * lda + m0 + tx] : 0.0;
+            Bs[ty + i][tx] = (gk < ke && n0 + tx < N) ? B[gk * ldb + n0 + tx] : 0.0;
         }
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < TK; ++k) {
-            double a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[k][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[k][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
+        for (int k = 0; k < TK; ++k) acc = fma(As[k][ty], Bs[k][tx], acc);
         __syncthreads();
     }
-    double *Ps = P + (long long)blockIdx.y * N * N;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            long long r = m0 + ty + 16 * i, c = n0 + tx + 16 * j;
-            if (r < N && c < N) Ps[r * N + c] = acc[i][j];
-        }
+    const long long r = m0 + ty, c = n0 + tx;
+    if (r < N && c < N) P[(long long)blockIdx.y * N * N + r * N + c] = acc;
 }
 
 __global__ void reduce_slices(const double *P, int nslice, long long NN, double *C, int accumulate) {
@@ -132,7 +117,7 @@ __global__ void reduce_slices(const double *P, int nslice, long long NN, double 
 // nslice = partial_elems / (N*N) at most.
 void gemm_fp64_tn_sym(const double *A, long long lda, const double *B, long long ldb, double *C,
                       long long N, long long K, double *partial, size_t partial_elems,
-                      cudaStream_t s) {
+                      cudaStream_t s, bool whole) {
     if (N <= 0) return;
     int ntb = (int)((N + TM - 1) / TM);
     int ntiles = ntb * (ntb + 1) / 2;
@@ -147,9 +132,9 @@ void gemm_fp64_tn_sym(const double *A, long long lda, const double *B, long long
     if (kchunk < TK) kchunk = TK;
     int nslice = (int)((K + kchunk - 1) / kchunk);
     if (nslice < 1) nslice = 1;
-    dim3 grid(ntiles, nslice);
+    dim3 grid(ntiles * (TM / TS) * (TM / TS), nslice);
     if (K > 0) {
-        dgemm_tn_upper<<<grid, 256, 0, s>>>(A, lda, B, ldb, partial, N, K, kchunk, ntb);
+        dgemm_tn_upper<<<grid, kThreads, 0, s>>>(A, lda, B, ldb, partial, N, K, kchunk, ntb, whole);
         QDT_CHECK_LAUNCH();
     } else {
         launch_zero(partial, N * N, s);

@@ -735,7 +735,7 @@ void gemm_half1(SplitWorkspace &w, int precision, const double *A, long long lda
 void gemm_half2(SplitWorkspace &w, int precision, const double *A, long long lda, const double *B, long long ldb,
                 double *C, long long N, long long K, double *partial, size_t partial_elems, cudaStream_t s) {
     if (precision != QDT_SPLIT) {
-        gemm_fp64_tn_sym(A, lda, B, ldb, C, N, K, partial, partial_elems, s);
+        gemm_fp64_tn_sym(A, lda, B, ldb, C, N, K, partial, partial_elems, s, false);
         return;
     }
     if (N <= 0) return;

@@ -80,7 +80,7 @@ extern "C" int qdt_second_half_noalloc(const double *Dq, const double *V, long l
         // the reduction accumulates into O, so start from zero; the partial
         // sums of the previous call are overwritten slice by slice
         qdt::launch_zero(O, N * N, s);
-        qdt::gemm_fp64_tn_sym(Dq, N, V, N, O, N, K, scratch, (size_t)kNoAllocScratchDoubles, s);
+        qdt::gemm_fp64_tn_sym(Dq, N, V, N, O, N, K, scratch, (size_t)kNoAllocScratchDoubles, s, true);
     } catch (const qdt::Error &e) {
         put_msg(msg, msg_len, e.msg);
         return e.code;

@@ -324,7 +324,7 @@ void gemm_fp64_nn_ragged(const double *A, long long lda, const double *B, long l
                          const long long *ktile, int tileM, cudaStream_t s, bool accumulate = false);
 void gemm_fp64_tn_sym(const double *A, long long lda, const double *B, long long ldb, double *C,
                       long long N, long long K, double *partial, size_t partial_elems,
-                      cudaStream_t s);
+                      cudaStream_t s, bool whole);
 int gemm_fp64_tile_m();
 
 // packing
