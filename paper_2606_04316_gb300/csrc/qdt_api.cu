@@ -40,6 +40,8 @@ using namespace qdt;
 
 namespace {
 
+constexpr int kTimerEvents = 32;     // of a context: a call with a row batch per class needs at most 24
+
 // Device buffer that only grows; freed with the context.
 struct DBuf {
     void *p = nullptr;
@@ -180,7 +182,7 @@ struct qdt_ctx {
     int route = QDT_ROUTE_DENSITY;
     int mo_block = 0;           // outer MO indices per block of the MO-driven route
     DBuf qcols, qWL, qWS, qT1, qT, qVf, qCr1, qCr2, qkt[3];
-    cudaEvent_t ev[16];
+    cudaEvent_t ev[kTimerEvents];
     int launches = 0;
     // batches owned by this context (its stream carries the fused launches)
     DBuf bprms[4], btasks[4], bnext[4];      // per kernel kind: gauge x compensated FP32
@@ -648,21 +650,38 @@ void build_class(qdt_ctx *ctx, int c) {
     QDT_CUDA_TRY(cudaStreamSynchronize(s));
 }
 
+// The spans between events are read together once the stream is waited for (settle), so
+// that nothing waits for the GPU only to read a time.
 struct Timer {
+    struct Span { int a, b; double *to; };
     qdt_ctx *c;
     int n = 0;
     bool on = true;
+    std::vector<Span> spans;
     explicit Timer(qdt_ctx *cc, bool enabled = true) : c(cc), on(enabled) {}
-    void mark() {
-        if (on && n < 16) QDT_CUDA_TRY(cudaEventRecord(c->ev[n++], c->stream));
+    int mark() {
+        if (on) QDT_CUDA_TRY(cudaEventRecord(c->ev[n], c->stream));
+        return n++;
     }
-    double ms(int a, int b) {
-        float t = 0.f;
-        if (on && a < n && b < n && cudaEventElapsedTime(&t, c->ev[a], c->ev[b]) != cudaSuccess) {
-            cudaGetLastError();   // a timing failure must not surface as a later launch error
-            t = 0.f;
+    // Adds the milliseconds between two marks to *to at the next settle().
+    void span(int a, int b, double *to) { spans.push_back({a, b, to}); }
+    // Waits for the stream and reads the spans; events after the first may be used again.
+    void settle() {
+        QDT_CUDA_TRY(cudaStreamSynchronize(c->stream));
+        for (const Span &p : spans) {
+            float t = 0.f;
+            if (on && cudaEventElapsedTime(&t, c->ev[p.a], c->ev[p.b]) != cudaSuccess) {
+                cudaGetLastError();   // a timing failure must not surface as a later launch error
+                t = 0.f;
+            }
+            *p.to += t;
         }
-        return t;
+        spans.clear();
+        n = std::min(n, 1);
+    }
+    // Makes room for k more marks.
+    void room(int k) {
+        if (n + k > kTimerEvents) settle();
     }
 };
 
@@ -692,6 +711,9 @@ struct ClassPlan {
     int *d_split = nullptr;       // its device copy (split form)
     std::vector<double> h_Dmax;
     std::vector<long long> h_col, Krow;
+    long long *pin_col = nullptr;         // where the four above arrive (the context's pinned arena)
+    double *pin_Dmax = nullptr;
+    int *pin_prefix = nullptr, *pin_ketsp = nullptr;
     size_t wbudget = 0;
     KetBuckets kb;                // the ket list's positions by bucket, and on the device
     int *d_kbpos = nullptr, *d_kbfirst = nullptr;
@@ -711,14 +733,19 @@ void order_kets(qdt_ctx *ctx, ClassPlan &P, cudaStream_t s) {
     launch_ket_columns(pc.d_pairs, P.ketsp, pc.nsp, P.ketcol, s);
     launch_prefix_lengths(pc.d_Q, wsort, pc.nsp, tau, P.prefix, s);
     ctx->launches += 3;
-    P.h_prefix.resize(pc.nsp);
-    P.h_col.resize(pc.nsp + 1);
-    P.h_ketsp.resize(pc.nsp);
-    QDT_CUDA_TRY(cudaMemcpyAsync(P.h_prefix.data(), P.prefix, pc.nsp * sizeof(int), cudaMemcpyDeviceToHost, s));
-    QDT_CUDA_TRY(cudaMemcpyAsync(P.h_col.data(), P.ketcol, (pc.nsp + 1) * sizeof(long long), cudaMemcpyDeviceToHost, s));
-    QDT_CUDA_TRY(cudaMemcpyAsync(P.h_ketsp.data(), P.ketsp, pc.nsp * sizeof(int), cudaMemcpyDeviceToHost, s));
-    P.h_Dmax.resize(pc.nsp);
-    QDT_CUDA_TRY(cudaMemcpyAsync(P.h_Dmax.data(), P.Dmax, pc.nsp * sizeof(double), cudaMemcpyDeviceToHost, s));
+    // into pinned memory: class_finish waits once for all of it
+    const size_t n = pc.nsp;
+    if (!P.pin_col) {
+        char *q = (char *)ctx->pin.take((n + 1) * sizeof(long long) + n * (sizeof(double) + 2 * sizeof(int)));
+        P.pin_col = (long long *)q;
+        P.pin_Dmax = (double *)(P.pin_col + n + 1);
+        P.pin_prefix = (int *)(P.pin_Dmax + n);
+        P.pin_ketsp = P.pin_prefix + n;
+    }
+    QDT_CUDA_TRY(cudaMemcpyAsync(P.pin_prefix, P.prefix, n * sizeof(int), cudaMemcpyDeviceToHost, s));
+    QDT_CUDA_TRY(cudaMemcpyAsync(P.pin_col, P.ketcol, (n + 1) * sizeof(long long), cudaMemcpyDeviceToHost, s));
+    QDT_CUDA_TRY(cudaMemcpyAsync(P.pin_ketsp, P.ketsp, n * sizeof(int), cudaMemcpyDeviceToHost, s));
+    QDT_CUDA_TRY(cudaMemcpyAsync(P.pin_Dmax, P.Dmax, n * sizeof(double), cudaMemcpyDeviceToHost, s));
     // 3. ket-ordered density copy (density route) or the function indices of
     // the ket-ordered columns (quarter route)
     if (P.quarter) {
@@ -853,6 +880,10 @@ void class_finish(qdt_ctx *ctx, ClassPlan &P, qdt_stats *st) {
     PairClass &pc = ctx->cls[P.cr.c];
     cudaStream_t s = ctx->stream;
     QDT_CUDA_TRY(cudaStreamSynchronize(s));
+    P.h_prefix.assign(P.pin_prefix, P.pin_prefix + pc.nsp);
+    P.h_col.assign(P.pin_col, P.pin_col + pc.nsp + 1);
+    P.h_ketsp.assign(P.pin_ketsp, P.pin_ketsp + pc.nsp);
+    P.h_Dmax.assign(P.pin_Dmax, P.pin_Dmax + pc.nsp);
     long long kept = 0, f32 = 0;
     for (int i = 0; i < pc.nsp; ++i) kept += P.h_prefix[i];
     double bound = 0.0;
@@ -1405,7 +1436,7 @@ void half2_stats(const Half2 &H, qdt_stats *st) {
 // Step 4 for the current ket order: batches of bra rows, integral rows then
 // the first half over the density columns [c0, c1).
 void run_batches(qdt_ctx *ctx, ClassPlan &P, long long c0, long long c1, qdt_stats *st, Timer &tm,
-                 double &ms_eri, double &ms_h1) {
+                 double acc_ms[6]) {
     PairClass &pc = ctx->cls[P.cr.c];
     cudaStream_t s = ctx->stream;
     if (P.mirror) {     // every batch adds into V (its own rows and, transposed, the later ones)
@@ -1415,6 +1446,7 @@ void run_batches(qdt_ctx *ctx, ClassPlan &P, long long c0, long long c1, qdt_sta
     int b0 = 0;
     while (b0 < pc.nsp) {
         RowBatch B;
+        tm.room(3);
         batch_prepare(ctx, P, b0, B);
         const EriParams *d_prm = dcopy_pinned(ctx->pin, ctx->prms, std::vector<EriParams>{B.prm}, s);
         const EriShape shape{pc.maxnfp, pc.maxLab, pc.maxnpp};
@@ -1430,7 +1462,7 @@ void run_batches(qdt_ctx *ctx, ClassPlan &P, long long c0, long long c1, qdt_sta
                                               pc.d_pairs, P.mirror ? B.d_pre1 : P.prefix,
                                               df ? (P.mirror ? B.d_split1 : P.d_split) : nullptr, B.prm.ket_sp, B.d_kbpos,
                                               B.d_kbfirst, B.prm.gauge != 0, how, queue, d_tk, s);
-        int te = tm.n; tm.mark();
+        const int te = tm.mark();
         if (P.quarter) {    // the quarter route lays out whole rows
             launch_zero(B.W, B.rows * P.mult * B.ldw, s);
         } else {            // the rest reads each row tile only as far as its K extent
@@ -1442,18 +1474,16 @@ void run_batches(qdt_ctx *ctx, ClassPlan &P, long long c0, long long c1, qdt_sta
         launch_eri(d_prm, d_tk, ntiles, queue, shape, B.prm.gauge != 0, df, how, s);
         ctx->launches += 2 + (B.Wc ? 1 : 0);
         batch_stats(ctx, P, B, c1 - c0, st);
-        int th = tm.n; tm.mark();
+        const int th = tm.mark();
         if (P.quarter) {
             quarter_half1(ctx, P, B, st, s);
         } else {
             batch_half1(ctx, P, B, c0, c1, s);
             if (P.mirror) batch_half1_mirror(ctx, P, B, s);
         }
-        int tend = tm.n; tm.mark();
-        QDT_CUDA_TRY(cudaStreamSynchronize(s));
-        ms_eri += tm.ms(te, th);
-        ms_h1 += tm.ms(th, tend);
-        tm.n = te;   // reuse the batch's events
+        const int tend = tm.mark();
+        tm.span(te, th, &acc_ms[2]);
+        tm.span(th, tend, &acc_ms[3]);
         b0 = B.b1;
     }
 }
@@ -1464,14 +1494,16 @@ void run_class(qdt_ctx *ctx, const ClassRun &cr, int k0, int nKa, double tau, in
     PairClass &pc = ctx->cls[cr.c];
     cudaStream_t s = ctx->stream;
     ClassPlan P;
+    tm.room(3);
     const int t0 = tm.n;
     class_issue(ctx, cr, k0, nKa, tau, precision, P, tm);
-    double ms_eri = 0, ms_h1 = 0;
+    tm.span(t0, t0 + 1, &acc_ms[0]);
+    tm.span(t0 + 1, t0 + 2, &acc_ms[1]);
     const int parts = P.ku ? 2 : 4;
     const int nb = ctx->route == QDT_ROUTE_MO ? std::max(1, ctx->mo_block) : nKa;
     if (nb >= nKa) {
         class_finish(ctx, P, st);
-        run_batches(ctx, P, 0, P.N4, st, tm, ms_eri, ms_h1);
+        run_batches(ctx, P, 0, P.N4, st, tm, acc_ms);
     } else {
         // MO-driven: the outer MO index r runs in blocks; each block of density
         // columns (r, s >= r) is screened on its own Dmax and recomputes every
@@ -1486,29 +1518,24 @@ void run_class(qdt_ctx *ctx, const ClassRun &cr, int k0, int nKa, double tau, in
             split_invalidate(ctx->split);
             P.mo_blocks = true;
             class_finish(ctx, P, st);
-            run_batches(ctx, P, c0, c1, st, tm, ms_eri, ms_h1);
+            run_batches(ctx, P, c0, c1, st, tm, acc_ms);
         }
     }
-    acc_ms[2] += ms_eri;
-    acc_ms[3] += ms_h1;
     // 5. second half + packing, one block at a time
     Half2 H;
     half2_prepare(ctx, P, out_coul, out_gaunt, out_gauge, H);
     half2_stats(H, st);
     for (const Half2::Job &j : H.jobs) {
-        int t2 = tm.n; tm.mark();
+        tm.room(3);
+        const int t2 = tm.mark();
         half2_job(ctx, P, H, j, s);
-        int t3 = tm.n; tm.mark();
+        const int t3 = tm.mark();
         half2_pack(ctx, P, H, j, s);
-        int t4 = tm.n; tm.mark();
-        QDT_CUDA_TRY(cudaStreamSynchronize(s));
-        acc_ms[4] += tm.ms(t2, t3);
-        acc_ms[5] += tm.ms(t3, t4);
-        tm.n = t2;   // reuse events
+        const int t4 = tm.mark();
+        tm.span(t2, t3, &acc_ms[4]);
+        tm.span(t3, t4, &acc_ms[5]);
     }
-    acc_ms[0] += tm.ms(t0, t0 + 1);
-    acc_ms[1] += tm.ms(t0 + 1, t0 + 2);
-    tm.n = t0;
+    if (!tm.on) tm.settle();        // a batch's request: the caller goes on to other streams
 }
 
 // ------------------------------------------------------------------ batches
@@ -1848,7 +1875,7 @@ int qdt_create(qdt_ctx **out, int device, void *cuda_stream) {
             QDT_CUDA_TRY(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
             c->own_stream = true;
         }
-        for (int i = 0; i < 16; ++i) QDT_CUDA_TRY(cudaEventCreate(&c->ev[i]));
+        for (int i = 0; i < kTimerEvents; ++i) QDT_CUDA_TRY(cudaEventCreate(&c->ev[i]));
         QDT_CUDA_TRY(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
         QDT_CUDA_TRY(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
         // FP64 table [kBoysGrid][kBoysCols], then its FP32 and FP32-pair forms (boys_tables)
@@ -1887,7 +1914,7 @@ void qdt_destroy(qdt_ctx *c) {
     c->pin.release();
     for (GraphEntry &g : c->graph)
         if (g.exec) cudaGraphExecDestroy(g.exec);
-    for (int i = 0; i < 16; ++i) cudaEventDestroy(c->ev[i]);
+    for (int i = 0; i < kTimerEvents; ++i) cudaEventDestroy(c->ev[i]);
     if (c->fork_ev) cudaEventDestroy(c->fork_ev);
     if (c->join_ev) cudaEventDestroy(c->join_ev);
     if (c->own_stream) cudaStreamDestroy(c->stream);
@@ -2176,7 +2203,11 @@ int qdt_transform(qdt_ctx *c, unsigned blocks, int k_begin, int k_end, double ta
         if (S) { S->precision = precision; S->slices = split_slices(c->split); }
         c->launches = 0;
         Timer tm(c);
-        tm.mark();
+        const int first = tm.mark();
+        // one look at the contractions' status for the whole call; a contraction that gives
+        // up makes the later ones return at once
+        const bool split = precision == QDT_SPLIT;
+        if (split) split_begin_deferred(c->split, c->stream);
         double acc[6] = {0, 0, 0, 0, 0, 0};
         if (blocks & QDT_COULOMB) {
             ClassRun cr{0, true, false, false};
@@ -2186,17 +2217,26 @@ int qdt_transform(qdt_ctx *c, unsigned blocks, int k_begin, int k_end, double ta
             ClassRun cr{1, false, (blocks & QDT_GAUNT) != 0, (blocks & QDT_GAUGE) != 0};
             run_class(c, cr, k_begin, nKa, tau, precision, nullptr, o_g, o_b, S, tm, acc);
         }
-        if (!dev_out) QDT_CUDA_TRY(cudaMemcpyAsync(out, dst, need, cudaMemcpyDeviceToHost, c->stream));
-        tm.mark();
-        QDT_CUDA_TRY(cudaStreamSynchronize(c->stream));
+        if (!dev_out) {
+            if (split) split_end_deferred(c->split, c->stream);     // before the caller's memory is written
+            QDT_CUDA_TRY(cudaMemcpyAsync(out, dst, need, cudaMemcpyDeviceToHost, c->stream));
+        }
+        tm.room(1);
+        double ms_total = 0;
+        tm.span(first, tm.mark(), &ms_total);
+        if (split && dev_out) split_end_deferred(c->split, c->stream);
+        tm.settle();
         if (S) {
-            S->ms_total = tm.ms(0, 1);
+            S->ms_total = ms_total;
             S->ms_density = acc[0]; S->ms_screen = acc[1]; S->ms_eri = acc[2];
             S->ms_half1 = acc[3]; S->ms_half2 = acc[4]; S->ms_pack = acc[5];
             S->kernel_launches = c->launches;
             *st = local;
         }
     } catch (const Error &e) {
+        c->split.deferred = false;
+        cudaStreamSynchronize(c->stream);       // nothing of this call still writes to the caller's memory
+        cudaGetLastError();
         return fail(c, e);
     }
     c->err.clear();
