@@ -290,22 +290,25 @@ std::vector<int> tile_order(const PairClass &pc, std::vector<int> v, int order) 
 
 // Tiles of at most tile_kets() kets of one bucket per bra pair (list: shell pair at
 // each ket position); with `split`, positions
-// [0, split) and [split, prefix) are tiled apart, the second set in plain FP32.
+// [0, split) and [split, prefix) are tiled apart, the second set in plain FP32 and after
+// all tiles of the first.
 void build_tiles(const PairClass &pc, const std::vector<int> &bras, const std::vector<int> &prefix,
                  const KetBuckets &kb, const BucketCounts &below, const std::vector<int> &list, bool gauge,
                  const EriLaunch &how, int req, std::vector<EriTask> &out, const std::vector<int> *split = nullptr) {
-    for (int sp : bras)
-        for (int b = 0; b + 1 < (int)kb.first.size(); ++b) {
-            const PairDev &CD = pc.h_pairs[list[kb.pos[kb.first[b]]]];
-            const int kets = tile_kets(pc.h_pairs[sp], CD, gauge, how.budget, how.kets);
-            const int f = kb.first[b], pre = f + below(b, prefix[sp]), mid = split ? f + below(b, (*split)[sp]) : pre;
-            for (int q = f; q < mid; q += kets) out.push_back({sp, q, std::min(mid, q + kets), req, 0});
-            for (int q = mid; q < pre; q += kets) out.push_back({sp, q, std::min(pre, q + kets), req, 1});
-        }
+    for (int kind = 0; kind < (split ? 2 : 1); ++kind)
+        for (int sp : bras)
+            for (int b = 0; b + 1 < (int)kb.first.size(); ++b) {
+                const PairDev &CD = pc.h_pairs[list[kb.pos[kb.first[b]]]];
+                const int kets = tile_kets(pc.h_pairs[sp], CD, gauge, how.budget, how.kets);
+                const int f = kb.first[b], pre = f + below(b, prefix[sp]);
+                const int mid = split ? f + below(b, (*split)[sp]) : pre, end = kind ? pre : mid;
+                for (int q = kind ? mid : f; q < end; q += kets)
+                    out.push_back({sp, q, std::min(end, q + kets), req, kind});
+            }
 }
 
-// The same tiles written on the device, one warp per bra pair (tile order), lanes
-// over the buckets: the kets of a bucket below the kept prefix and the FP32 split
+// The same tiles written on the device, one warp per bra pair (tile order) and kind of
+// tile, lanes over the buckets: the kets of a bucket below the kept prefix and the FP32 split
 // point are found by bisection (split null: no FP32 tiles).  First pass (out null):
 // tiles of each bra pair into count; their exclusive sums are the second pass's
 // offsets, so only the bra list is uploaded, not the tiles.
@@ -321,30 +324,31 @@ __global__ void tiles_kernel(const PairDev *pairs, const int *bras, const int *p
                              EriLaunch how, const int *off, int *count, EriTask *out) {
     const int w = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
-    if (w >= n) return;
-    const int sp = bras[w], p_end = prefix[sp], p_mid = split ? split[sp] : p_end;
+    if (w >= (split ? 2 * n : n)) return;
+    const int kind = w >= n, sp = bras[w - kind * n], p_end = prefix[sp], p_mid = split ? split[sp] : p_end;
     const PairDev AB = pairs[sp];
     int done = out ? off[w] : 0;
     for (int b0 = 0; b0 < nbucket; b0 += 32) {
         const int b = b0 + lane;
-        int f = 0, mid = 0, pre = 0, kets = 1;
+        int f = 0, e = 0, kets = 1;
         if (b < nbucket) {
             f = first[b];
             kets = tile_kets(AB, pairs[list[pos[f]]], gauge, how.budget, how.kets);
-            pre = bucket_below(pos, f, first[b + 1], p_end);
-            mid = split ? bucket_below(pos, f, pre, p_mid) : pre;
+            e = bucket_below(pos, f, first[b + 1], p_end);
+            const int mid = split ? bucket_below(pos, f, e, p_mid) : e;
+            if (kind) f = mid;
+            else e = mid;
         }
-        const int n1 = (mid - f + kets - 1) / kets, n2 = (pre - mid + kets - 1) / kets;
-        int x = n1 + n2;                                    // inclusive scan over the lanes
+        const int nt = (e - f + kets - 1) / kets;
+        int x = nt;                                         // inclusive scan over the lanes
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
         if (out) {
-            EriTask *o = out + done + x - n1 - n2;
-            for (int q = f; q < mid; q += kets) *o++ = EriTask{sp, q, min(mid, q + kets), 0, 0};
-            for (int q = mid; q < pre; q += kets) *o++ = EriTask{sp, q, min(pre, q + kets), 0, 1};
+            EriTask *o = out + done + x - nt;
+            for (int q = f; q < e; q += kets) *o++ = EriTask{sp, q, min(e, q + kets), 0, kind};
         }
         done += __shfl_sync(0xffffffffu, x, 31);
     }
@@ -396,14 +400,14 @@ int launch_build_tiles(qdt_ctx *ctx, const std::vector<int> &bras, const std::ve
     if (most > 0x7fffffffLL) throw Error{QDT_ERR_ARG, "integral tiles: more than 2^31 tiles in one batch"};
     d_tiles = (EriTask *)ctx->tasks.get((size_t)std::max<long long>(1, most) * sizeof(EriTask));
     if (most == 0) return 0;
-    const int n = (int)bras.size();
+    const int n = (int)bras.size(), nw = d_split ? 2 * n : n;
     const int *d_bras = dcopy_pinned(ctx->pin, ctx->tbras, bras, s);
-    int *d_off = (int *)ctx->toff.get((size_t)n * sizeof(int));
-    const unsigned grid = (unsigned)((32LL * n + 255) / 256);
+    int *d_off = (int *)ctx->toff.get((size_t)nw * sizeof(int));
+    const unsigned grid = (unsigned)((32LL * nw + 255) / 256);
     tiles_kernel<<<grid, 256, 0, s>>>(d_pairs, d_bras, d_prefix, d_split, d_list, d_pos, d_first, nbucket, n, gauge, how,
                                       nullptr, d_off, nullptr);
     QDT_CHECK_KERNEL("tiles_kernel");
-    tile_scan_kernel<<<1, 1024, 0, s>>>(d_off, n, queue + 1);
+    tile_scan_kernel<<<1, 1024, 0, s>>>(d_off, nw, queue + 1);
     QDT_CHECK_KERNEL("tile_scan_kernel");
     tiles_kernel<<<grid, 256, 0, s>>>(d_pairs, d_bras, d_prefix, d_split, d_list, d_pos, d_first, nbucket, n, gauge, how,
                                       d_off, nullptr, d_tiles);
