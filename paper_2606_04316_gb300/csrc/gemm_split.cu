@@ -125,39 +125,63 @@ void split_forget(SplitWorkspace &w, const void *lo, const void *hi) {
 static inline long long rup(long long x, long long m) { return (x + m - 1) / m * m; }
 
 // ------------------------------------------------------------ digits
-__device__ inline int exp_of_max(double m) {
-    // smallest e with 2^e > m (m >= 0); 0 for m == 0
-    if (!(m > 0.0)) return 0;
-    long long bits = __double_as_longlong(m);
-    int ex = (int)((bits >> 52) & 0x7FF);
-    if (ex == 0) return -1022;
-    return ex - 1023 + 1;
+// The maximum is taken over the upper halves of |x| as integers (a double-precision
+// maximum would hold the FP64 pipe for longer than the rest of the slicing); NaNs are
+// passed over, and numbers below 2^-1022 count as zero, as they do in split_integer.
+__device__ inline unsigned top_half(double x) {
+    const unsigned h = (unsigned)__double2hiint(x) & 0x7FFFFFFFu;
+    return h > 0x7FF00000u ? 0u : h;
+}
+__device__ inline int exp_of_max(unsigned h) {
+    // smallest e with 2^e > m for every m of this upper half; 0 for m == 0
+    const int ex = (int)(h >> 20);
+    return ex ? ex - 1023 + 1 : 0;
 }
 
 // x 2^{42-e} rounded to the nearest integer X (|X| <= 2^42 when |x| < 2^e), by
-// integer operations on the bits, then its balanced digits: d_1 = round(X /
-// 2^35) in [-128, 128], X -= d_1 2^35, and so on down to d_6 = X in [-64, 63].
-__device__ inline void digits7(double x, int e, __nv_bfloat16 *d, size_t plane) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-    const int ex = (int)((bits >> 52) & 0x7FF);
-    long long X = 0;
-    if (ex != 0) {
-        const unsigned long long mant = (bits & ((1ULL << 52) - 1)) | (1ULL << 52);
-        const int sh = ex - 1075 + kFrac - e;         // |x| 2^{42-e} = mant 2^sh
-        unsigned long long M;
-        if (sh >= 0) M = 1ULL << kFrac;               // cannot happen when 2^e > |x|
-        else if (sh > -63) M = (mant + (1ULL << (-sh - 1))) >> (-sh);
-        else M = 0;
-        if (M > (1ULL << kFrac)) M = 1ULL << kFrac;
-        X = (bits >> 63) ? -(long long)M : (long long)M;
-    }
+// integer operations on the bits.
+__device__ inline long long split_integer(double x, int e) {
+    const unsigned h = (unsigned)__double2hiint(x);
+    const int ex = (int)(h >> 20) & 0x7FF, n = 1032 + e - ex;      // |x| 2^{42-e} = mant / 2^{n+1}, n >= 10 as 2^e > |x|
+    const unsigned long long mant =
+        ((unsigned long long)((h & 0xFFFFFu) | 0x100000u) << 32) | (unsigned)__double2loint(x);
+    unsigned long long M = ((mant >> min(max(n, 0), 63)) + 1) >> 1;
+    if (n < 10) M = 1ULL << kFrac;                    // an infinity or NaN
+    if (ex == 0) M = 0;
+    return (int)h < 0 ? -(long long)M : (long long)M;
+}
+// Its balanced digits: d_1 = round(X / 2^35) in [-128, 128], X -= d_1 2^35, and so on down to
+// d_6 = X in [-64, 63].  With U the part of X + 2^34 below 2^35, X - d_1 2^35 = U - 64 2^28, so
+// d_2 = floor((U + 2^27) / 2^28) - 64, and so on: after the second digit all in 32 bits.
+__device__ inline void balanced_digits(long long X, float (&d)[kSlices]) {
+    static_assert(kSlices == 6 && kBits == 7, "digits of 42 bits");
+    const long long Y = X + (1LL << 34);
+    // an integer 0 <= t <= 256 in the low mantissa bits of 2^23, less 2^23 and its bias
+    auto small = [](unsigned t, float bias) { return __uint_as_float(0x4B000000u + t) - (8388608.f + bias); };
+    d[0] = small((unsigned)(Y >> 35) + 128u, 128.f);
+    const unsigned long long Z = (unsigned long long)(Y & ((1LL << 35) - 1)) + (1ULL << 27);
+    d[1] = small((unsigned)(Z >> 28), 64.f);
+    unsigned z = ((unsigned)Z & ((1u << 28) - 1)) + (1u << 20);
+    d[2] = small(z >> 21, 64.f);
+    z = (z & ((1u << 21) - 1)) + (1u << 13);
+    d[3] = small(z >> 14, 64.f);
+    z = (z & ((1u << 14) - 1)) + (1u << 6);
+    d[4] = small(z >> 7, 64.f);
+    d[5] = small(z & 127u, 64.f);
+}
+// Digits of kRun neighbouring elements to neighbouring places of each plane, one store each.
+constexpr int kRun = 4;
+__device__ inline void store_digits(const double (&x)[kRun], int e, __nv_bfloat16 *out, size_t plane) {
+    float d[kRun][kSlices];
+#pragma unroll
+    for (int q = 0; q < kRun; ++q) balanced_digits(split_integer(x[q], e), d[q]);
 #pragma unroll
     for (int i = 0; i < kSlices; ++i) {
-        const int shift = kBits * (kSlices - 1 - i);
-        // floor((X + 2^{shift-1}) / 2^shift): arithmetic shift of a signed value
-        const long long di = shift ? (X + (1LL << (shift - 1))) >> shift : X;
-        X -= di * (1LL << shift);
-        d[i * plane] = __float2bfloat16_rn((float)di);
+        const __nv_bfloat162 a = __floats2bfloat162_rn(d[0][i], d[1][i]), b = __floats2bfloat162_rn(d[2][i], d[3][i]);
+        uint2 w;
+        w.x = *reinterpret_cast<const unsigned *>(&a);
+        w.y = *reinterpret_cast<const unsigned *>(&b);
+        *reinterpret_cast<uint2 *>(out + i * plane) = w;
     }
 }
 
@@ -165,54 +189,79 @@ __device__ inline void digits7(double x, int e, __nv_bfloat16 *d, size_t plane) 
 // r < Mpad, k < Kpad (zeros outside the matrix).  One CTA per row.  With the
 // K extents of the 128-row tiles (kt128), a row is sliced only as far as the
 // contraction reads it, its tile's extent rounded up to the 64-wide K
-// subtile (the digits past it are never loaded).
+// subtile (the digits past it are never loaded).  Memory bounds it on large matrices: 8 bytes
+// read twice and 12 written per element.  Four elements to a thread (32-byte loads where the
+// row allows, 8-byte stores), digits in 32 bits, the maximum in integers: 4096 rows of 3400 from
+// 179 to 56 us; an 18-atom cluster's four matrices 15 -> 6.6 ms (other block sizes, a row read
+// backwards the second time: the same).
 __global__ void slice_rows_kernel(const double *X, long long ld, long long M, long long K,
                                   long long Mpad, long long Kpad, __nv_bfloat16 *out, int *rowexp,
                                   const long long *kt128) {
-    long long r = blockIdx.x;
-    __shared__ double wm[32];
+    const long long r = blockIdx.x;
+    __shared__ unsigned wm[32];
     __shared__ int e_sh;
     const long long Kr = kt128 ? min(Kpad, (kt128[r / SBM] + SBK - 1) / SBK * SBK) : Kpad;
     const long long Kx = min(K, Kr);
-    double m = 0.0;
+    const double *row = X + r * ld;
+    const bool wide = ((uintptr_t)row & 15) == 0;
+    // kRun elements from k (a multiple of kRun), zeros from Kx on
+    auto load = [&](long long k, double (&x)[kRun]) {
+        if (wide && k + kRun <= Kx) {
+            const double2 a = *reinterpret_cast<const double2 *>(row + k), b = *reinterpret_cast<const double2 *>(row + k + 2);
+            x[0] = a.x;
+            x[1] = a.y;
+            x[2] = b.x;
+            x[3] = b.y;
+        } else {
+#pragma unroll
+            for (int q = 0; q < kRun; ++q) x[q] = k + q < Kx ? row[k + q] : 0.0;
+        }
+    };
+    unsigned m = 0;
     if (r < M)
-        for (long long k = threadIdx.x; k < Kx; k += blockDim.x) m = fmax(m, fabs(X[r * ld + k]));
+        for (long long k = threadIdx.x * kRun; k < Kx; k += blockDim.x * kRun) {
+            double x[kRun];
+            load(k, x);
+#pragma unroll
+            for (int q = 0; q < kRun; ++q) m = max(m, top_half(x[q]));
+        }
     // row maximum: warp shuffles, then the warps' maxima in the first warp
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
     __syncthreads();
     if (threadIdx.x < 32) {
-        m = threadIdx.x < (blockDim.x >> 5) ? wm[threadIdx.x] : 0.0;
+        m = threadIdx.x < (blockDim.x >> 5) ? wm[threadIdx.x] : 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (threadIdx.x == 0) e_sh = exp_of_max(m);
     }
     __syncthreads();
     const int e = e_sh;
     if (threadIdx.x == 0) rowexp[r] = e;
-    size_t plane = (size_t)Mpad * Kpad;
-    for (long long k = threadIdx.x; k < Kr; k += blockDim.x) {
-        double x = (r < M && k < Kx) ? X[r * ld + k] : 0.0;
-        digits7(x, e, out + (size_t)r * Kpad + k, plane);
+    const size_t plane = (size_t)Mpad * Kpad;
+    for (long long k = threadIdx.x * kRun; k < Kr; k += blockDim.x * kRun) {
+        double x[kRun] = {0.0, 0.0, 0.0, 0.0};
+        if (r < M) load(k, x);
+        store_digits(x, e, out + (size_t)r * Kpad + k, plane);
     }
 }
 
 // column maxima (as exponents) of X[rows][cols]
 __global__ void col_max_kernel(const double *X, long long ld, long long rows, long long cols,
-                               long long rows_per_block, unsigned long long *cmax) {
+                               long long rows_per_block, unsigned *cmax) {
     long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (c >= cols) return;
     long long r0 = blockIdx.y * rows_per_block, r1 = min(rows, r0 + rows_per_block);
-    double m = 0.0;
-    for (long long r = r0; r < r1; ++r) m = fmax(m, fabs(X[r * ld + c]));
-    atomicMax(cmax + c, (unsigned long long)__double_as_longlong(m));
+    unsigned m = 0;
+    for (long long r = r0; r < r1; ++r) m = max(m, top_half(X[r * ld + c]));
+    atomicMax(cmax + c, m);
 }
 
-__global__ void col_exp_kernel(const unsigned long long *cmax, long long cols, long long cols_pad, int *colexp) {
+__global__ void col_exp_kernel(const unsigned *cmax, long long cols, long long cols_pad, int *colexp) {
     long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (c >= cols_pad) return;
-    colexp[c] = (c < cols) ? exp_of_max(__longlong_as_double((long long)cmax[c])) : 0;
+    colexp[c] = (c < cols) ? exp_of_max(cmax[c]) : 0;
 }
 
 // B operand (or a transposed A): columns of X scaled per column, written
@@ -220,19 +269,23 @@ __global__ void col_exp_kernel(const unsigned long long *cmax, long long cols, l
 __global__ void slice_cols_t_kernel(const double *X, long long ld, long long rows, long long cols,
                                     long long Rpad, long long Cpad, const int *colexp,
                                     __nv_bfloat16 *out) {
-    __shared__ double t[64][33];
+    __shared__ double t[32][66];
     long long r0 = blockIdx.x * 64LL, c0 = blockIdx.y * 32LL;
     for (int i = threadIdx.x; i < 64 * 32; i += blockDim.x) {
         int rr = i / 32, cc = i % 32;
         long long r = r0 + rr, c = c0 + cc;
-        t[rr][cc] = (r < rows && c < cols) ? X[r * ld + c] : 0.0;
+        t[cc][rr] = (r < rows && c < cols) ? X[r * ld + c] : 0.0;
     }
     __syncthreads();
     size_t plane = (size_t)Cpad * Rpad;
-    for (int i = threadIdx.x; i < 64 * 32; i += blockDim.x) {
-        int cc = i / 64, rr = i % 64;
-        long long r = r0 + rr, c = c0 + cc;
-        if (r < Rpad && c < Cpad) digits7(t[rr][cc], colexp[c], out + (size_t)c * Rpad + r, plane);
+    for (int i = threadIdx.x; i < 64 / kRun * 32; i += blockDim.x) {
+        const int cc = i / (64 / kRun), rr = i % (64 / kRun) * kRun;
+        const long long r = r0 + rr, c = c0 + cc;
+        if (r < Rpad && c < Cpad) {            // Rpad is a multiple of 64
+                        const double2 a = *reinterpret_cast<const double2 *>(&t[cc][rr]), b = *reinterpret_cast<const double2 *>(&t[cc][rr + 2]);
+            const double x[kRun] = {a.x, a.y, b.x, b.y};
+            store_digits(x, colexp[c], out + (size_t)c * Rpad + r, plane);
+        }
     }
 }
 
@@ -598,8 +651,8 @@ static CUtensorMap make_map(void *ptr, long long rows, long long cols, int box_r
 // Column-scaled, transposed slices of X[rows][cols] into slot; returns (Cpad, Rpad).
 static void slice_cols(SplitWorkspace &w, int slot, const double *X, long long ld, long long rows, long long cols,
                        long long Rpad, long long Cpad, int *colexp, cudaStream_t s) {
-    unsigned long long *cmax = (unsigned long long *)ws_get(w, WS_ERR, std::max<size_t>(4096, (size_t)Cpad * 8 + 64));
-    QDT_CUDA_TRY(cudaMemsetAsync(cmax, 0, (size_t)Cpad * 8, s));
+    unsigned *cmax = (unsigned *)ws_get(w, WS_ERR, std::max<size_t>(4096, (size_t)Cpad * 4 + 64));
+    QDT_CUDA_TRY(cudaMemsetAsync(cmax, 0, (size_t)Cpad * sizeof(unsigned), s));
     long long rpb = std::max<long long>(64, (rows + 1023) / 1024);
     dim3 g1((unsigned)((cols + 255) / 256), (unsigned)((rows + rpb - 1) / rpb));
     if (rows > 0 && cols > 0) col_max_kernel<<<g1, 256, 0, s>>>(X, ld, rows, cols, rpb, cmax);
