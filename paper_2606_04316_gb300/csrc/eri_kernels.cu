@@ -14,18 +14,22 @@
 // The signs (-1)^{|h'|} are carried by the tensor: R~_g = (-1)^{|g|} R_g is the
 // tensor of Q - P, and (-1)^{|h'|} R_{h+h'} = (-1)^{|h|} R~_{h+h'}.
 //
-// Work layout: a CTA owns one bra shell pair and a run of ket shell pairs.
-// For every shell quartet the cheaper orientation is contracted: X outer, Y
-// inner.  Per outer primitive pair ij (several at once when the quartet is
-// small): the Hermite tensors of all inner primitive pairs by the recursion,
-// the ket pass T[h][y] = sum_kl sum_h' R~ E', and the bra pass G += E T.  The
-// headers (Boys values, prefactors) of the quartet's primitive quartets run
-// before that in one pass, because a header is one long dependent chain.
+// Work layout: a tile is one bra shell pair and up to 32 ket shell pairs of one kind
+// (function pairs and primitive pairs alike), so one orientation (the cheaper one; X
+// outer, Y inner) and one cut serve it all.  A CTA takes several kets and outer primitive
+// pairs ij at a time through four phases: the headers (Boys values, prefactors; one long dependent
+// chain each), the Hermite tensors of all inner primitive pairs by the recursion, the
+// ket pass T[h][y] = sum_kl sum_h' R~ E', and the bra pass G += E T.
 //
-// What bounds it: the multiply-adds of the two passes and the recursion, on the
-// FP32 pipe in the split form (12 operations per compensated multiply-add) and
-// on the FP64 pipe in the FP64 form.  Two things keep their number down and the
-// pipe busy:
+// What bounds it: in the split form no single unit.  The multiply-adds of the two passes
+// keep the FP32 pipe busy for a sixth to a quarter of the time, shared-memory loads
+// their unit for more than half; what is left is the latency of chains of table,
+// tensor and coefficient loads at 12 to 16 warps per SM (128 registers), and instruction
+// fetch: the phases of one form are about 75 KB of code.  Measured without gain: fewer
+// registers and more warps (80: 183 to 214 ms for the integrals of a 24-centre chain instead
+// of 179), tensor entries placed to avoid the ket pass's bank conflicts (172 for 169), four
+// function pairs per ket item (178 for 173).  In the FP64 form the FP64 pipe bounds it.
+// What keeps the work down:
 //  * Boxes.  The expansion of a function pair is a product of one-dimensional
 //    ones, so only the Hermite functions of its box (FuncPair) contribute, 27 to
 //    37 % of all for the pairs of p functions and derivatives.  Both passes
@@ -35,6 +39,10 @@
 //    instruction (fma.rn.f32x2) per operation: half the issue slots of the
 //    scalar form, and the two halves are independent chains.  The bra pass
 //    packs two function pairs y instead.
+//  * Several kets at a time: a small quartet alone leaves most lanes without work.
+// Integrals of a 24-centre chain (Coulomb, Gaunt, gauge) 477 -> 169 ms over these and the
+// choices at the phases below, 40-centre chain (Coulomb) 322 -> 125, an 18-atom cluster
+// 632 -> 205, a class with d shells 671 -> 64; FP64 form, 7-centre chain 39 -> 11.7.
 //
 // Split form (DF): recursion and both passes in compensated FP32 pairs (x = hi +
 // lo, ~48-bit significands): products by the exact-product FMA, sums by the

@@ -27,7 +27,8 @@
 //  kernel is the shared memory: a 128 x 80 MMA reads 6.5 KB of operands for 40
 //  cycles of the tensor pipe, a 128 x 240 one 11.5 KB for 120 (24-centre chain, all
 //  blocks, slicing included: first half 93.7 -> 72.1 ms, second 12.0 -> 9.8; 40-centre
-//  chain, Coulomb: 81.8 -> 60.5 and 21.1 -> 16.5, i.e. 1560 TF/s of digit products).
+//  chain, Coulomb: 81.8 -> 60.5 and 21.1 -> 16.5; with the faster slicing below 58.5 and 7.3,
+//  54.2 and 13.2, i.e. 1740 TF/s of digit products on the longer chain).
 //  Roles: one thread issues the TMA loads, one the MMAs (its loops
 //  unrolled over the digit planes, so A stage, barrier phase, accumulator and
 //  descriptors are compile-time constants), eight warps (two per TMEM lane
