@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "plan.h"
+#include "tiles.h"
 #include "qdt_internal.cuh"
 #include "split.cuh"
 
@@ -288,28 +289,7 @@ std::vector<int> tile_order(const PairClass &pc, std::vector<int> v, int order) 
     return v;
 }
 
-// Tiles of at most tile_kets() kets of one bucket per bra pair (list: shell pair at
-// each ket position); with `split`, positions
-// [0, split) and [split, prefix) are tiled apart, the second set in plain FP32 and after
-// all tiles of the first: the phases of both forms together are more code than the
-// instruction caches hold (interleaved, the integrals of a 40-centre chain took 131.1 ms
-// instead of 125.2, of a 24-centre chain 172.6 instead of 169.0).
-void build_tiles(const PairClass &pc, const std::vector<int> &bras, const std::vector<int> &prefix,
-                 const KetBuckets &kb, const BucketCounts &below, const std::vector<int> &list, bool gauge,
-                 const EriLaunch &how, int req, std::vector<EriTask> &out, const std::vector<int> *split = nullptr) {
-    for (int kind = 0; kind < (split ? 2 : 1); ++kind)
-        for (int sp : bras)
-            for (int b = 0; b + 1 < (int)kb.first.size(); ++b) {
-                const PairDev &CD = pc.h_pairs[list[kb.pos[kb.first[b]]]];
-                const int kets = tile_kets(pc.h_pairs[sp], CD, gauge, how.budget, how.kets);
-                const int f = kb.first[b], pre = f + below(b, prefix[sp]);
-                const int mid = split ? f + below(b, (*split)[sp]) : pre, end = kind ? pre : mid;
-                for (int q = kind ? mid : f; q < end; q += kets)
-                    out.push_back({sp, q, std::min(end, q + kets), req, kind});
-            }
-}
-
-// The same tiles written on the device, one warp per bra pair (tile order) and kind of
+// The tiles of build_tiles (tiles.h) written on the device, one warp per bra pair (tile order) and kind of
 // tile, lanes over the buckets: the kets of a bucket below the kept prefix and the FP32 split
 // point are found by bisection (split null: no FP32 tiles).  First pass (out null):
 // tiles of each bra pair into count; their exclusive sums are the second pass's
@@ -391,14 +371,12 @@ __global__ void __launch_bounds__(1024) tile_scan_kernel(int *count, int n, int 
 }
 
 // Host side: the uploads and launches; tiles into ctx->tasks, their number into
-// queue[1].  Returns a bound on it: full tiles of the smallest size and, for every
-// bucket of a bra pair, at most two part tiles.
-int launch_build_tiles(qdt_ctx *ctx, const std::vector<int> &bras, const std::vector<int> &prefix, int nbucket,
-                       const PairDev *d_pairs, const int *d_prefix, const int *d_split, const int *d_list,
-                       const int *d_pos, const int *d_first, bool gauge, const EriLaunch &how, int *queue,
-                       EriTask *&d_tiles, cudaStream_t s) {
-    long long most = 0;
-    for (int sp : bras) most += prefix[sp] / how.least + std::min<long long>(2LL * nbucket, prefix[sp]);
+// queue[1].  Returns a bound on it (tile_bound), which is also the list's room.
+int launch_build_tiles(qdt_ctx *ctx, const PairClass &pc, const std::vector<int> &bras, const std::vector<int> &prefix,
+                       int nbucket, const int *d_prefix, const int *d_split, const int *d_list, const int *d_pos,
+                       const int *d_first, bool gauge, const EriLaunch &how, int *queue, EriTask *&d_tiles,
+                       cudaStream_t s) {
+    const long long most = tile_bound(pc, bras, prefix, nbucket, gauge, how);
     if (most > 0x7fffffffLL) throw Error{QDT_ERR_ARG, "integral tiles: more than 2^31 tiles in one batch"};
     d_tiles = (EriTask *)ctx->tasks.get((size_t)std::max<long long>(1, most) * sizeof(EriTask));
     if (most == 0) return 0;
@@ -406,12 +384,12 @@ int launch_build_tiles(qdt_ctx *ctx, const std::vector<int> &bras, const std::ve
     const int *d_bras = dcopy_pinned(ctx->pin, ctx->tbras, bras, s);
     int *d_off = (int *)ctx->toff.get((size_t)nw * sizeof(int));
     const unsigned grid = (unsigned)((32LL * nw + 255) / 256);
-    tiles_kernel<<<grid, 256, 0, s>>>(d_pairs, d_bras, d_prefix, d_split, d_list, d_pos, d_first, nbucket, n, gauge, how,
+    tiles_kernel<<<grid, 256, 0, s>>>(pc.d_pairs, d_bras, d_prefix, d_split, d_list, d_pos, d_first, nbucket, n, gauge, how,
                                       nullptr, d_off, nullptr);
     QDT_CHECK_KERNEL("tiles_kernel");
     tile_scan_kernel<<<1, 1024, 0, s>>>(d_off, nw, queue + 1);
     QDT_CHECK_KERNEL("tile_scan_kernel");
-    tiles_kernel<<<grid, 256, 0, s>>>(d_pairs, d_bras, d_prefix, d_split, d_list, d_pos, d_first, nbucket, n, gauge, how,
+    tiles_kernel<<<grid, 256, 0, s>>>(pc.d_pairs, d_bras, d_prefix, d_split, d_list, d_pos, d_first, nbucket, n, gauge, how,
                                       d_off, nullptr, d_tiles);
     QDT_CHECK_KERNEL("tiles_kernel");
     ctx->launches += 3;
@@ -466,19 +444,13 @@ EriLaunch eri_launch_for(qdt_ctx *ctx, const PairClass &pc, const EriShape &shap
         }
     if (weight > 0.0) {
         def.budget = std::max<long long>(1, (long long)(mean / weight * 0.5 * (double)quartets / (4.0 * nsm * 32.0)));
-        def.least = def.kets;
-        for (int i : pc.bucket_rep)
-            for (int j : pc.bucket_rep)
-                def.least = std::min(def.least, tile_kets(pc.h_pairs[i], pc.h_pairs[j], gauge, def.budget, def.kets));
     }
     if (const char *pin = std::getenv("QDT_ERI_LAUNCH")) {
         EriLaunch p = def;
-        if (std::sscanf(pin, "%d,%d,%d", &p.threads, &p.kets, &p.order) == 3 && p.threads > 0 && p.kets > 0)
-            {
-                p.kets = std::min(p.kets, kMaxTileKets);
-                p.least = std::min(p.kets, p.least);
-                return p;
-            }
+        if (std::sscanf(pin, "%d,%d,%d", &p.threads, &p.kets, &p.order) == 3 && p.threads > 0 && p.kets > 0) {
+            p.kets = std::min(p.kets, kMaxTileKets);
+            return p;
+        }
         throw Error{QDT_ERR_ARG, "QDT_ERI_LAUNCH must read threads,kets,order"};
     }
     if (!env_flag("QDT_AUTOTUNE", true)) return def;
@@ -490,7 +462,6 @@ EriLaunch eri_launch_for(qdt_ctx *ctx, const PairClass &pc, const EriShape &shap
         if (it != g_tune.end()) {
             EriLaunch how = it->second;
             how.budget = def.budget;
-            how.least = std::min(how.kets, def.least);
             return how;
         }
     }
@@ -1464,8 +1435,8 @@ void run_batches(qdt_ctx *ctx, ClassPlan &P, long long c0, long long c1, qdt_sta
             eri_launch_for(ctx, pc, shape, B.prm.gauge != 0, df, d_prm, B.bras, pre, B.kb, B.list(P), quartets, s);
         EriTask *d_tk = nullptr;
         int *queue = (int *)ctx->next.get(2 * sizeof(int));
-        const int ntiles = launch_build_tiles(ctx, tile_order(pc, B.bras, how.order), pre, (int)B.kb.first.size() - 1,
-                                              pc.d_pairs, P.mirror ? B.d_pre1 : P.prefix,
+        const int ntiles = launch_build_tiles(ctx, pc, tile_order(pc, B.bras, how.order), pre, (int)B.kb.first.size() - 1,
+                                              P.mirror ? B.d_pre1 : P.prefix,
                                               df ? (P.mirror ? B.d_split1 : P.d_split) : nullptr, B.prm.ket_sp, B.d_kbpos,
                                               B.d_kbfirst, B.prm.gauge != 0, how, queue, d_tk, s);
         const int te = tm.mark();
@@ -1584,7 +1555,8 @@ uint64_t round_signature(const std::vector<BatchReq *> &fz, const std::vector<Er
     uint64_t h = 1469598103934665603ULL;
     for (int k = 0; k < kKinds; ++k) {
         h = fnv_v(h, tiles[k]);
-        h = fnv(h, &how[k], sizeof(EriLaunch));
+        const long long launch[] = {how[k].threads, how[k].kets, how[k].order, how[k].budget};
+        h = fnv(h, launch, sizeof launch);
         h = fnv(h, &shape[k], sizeof(EriShape));
     }
     for (BatchReq *r : fz) {

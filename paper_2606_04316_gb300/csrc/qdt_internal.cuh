@@ -255,7 +255,6 @@ struct EriLaunch {
     int threads = 0;            // 0: the plan's default
     int kets = kMaxTileKets;
     int order = 1;              // tile order: 0 bra pairs by Schwarz Q (bra order), 1 most expensive first
-    int least = 1;              // the smallest tile_kets() of the class under the budget
     long long budget = 0;       // quartet cost a tile may reach with more than one ket (0: no limit)
 };
 
