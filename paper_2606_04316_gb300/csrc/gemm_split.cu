@@ -78,14 +78,22 @@ static void *ws_get(SplitWorkspace &w, int slot, size_t bytes) {
     return w.buf[slot];
 }
 
-void split_release(SplitWorkspace &w) {
-    for (int i = 0; i < SplitWorkspace::kSlots; ++i) {
-        if (w.buf[i]) cudaFree(w.buf[i]);
-        w.buf[i] = nullptr;
-        w.bytes[i] = 0;
-    }
+static void ws_free(SplitWorkspace &w, int slot) {
+    if (w.buf[slot]) cudaFree(w.buf[slot]);
+    w.buf[slot] = nullptr;
+    w.bytes[slot] = 0;
+}
+
+void split_release_planes(SplitWorkspace &w) {
+    for (int i = 0; i < SplitWorkspace::kSlots; ++i)
+        if (i != WS_STAT) ws_free(w, i);
     w.bkey[0] = w.bkey[1] = SplitKey();
     w.bnext = 0;
+}
+
+void split_release(SplitWorkspace &w) {
+    split_release_planes(w);
+    ws_free(w, WS_STAT);
 }
 
 int split_slices(const SplitWorkspace &w) { return w.slices; }
@@ -98,6 +106,18 @@ size_t split_held_bytes(const SplitWorkspace &w) {
 
 void split_clear_status(SplitWorkspace &w, cudaStream_t s) {
     QDT_CUDA_TRY(cudaMemsetAsync(ws_get(w, WS_STAT, 256), 0, 256, s));
+    w.calls = 0;
+}
+
+// QDT_SPLIT_FAIL=n: the n-th contraction since the status was cleared finds a give-up already
+// recorded, as if a wait in it had run out (no wait does).  For tests of what follows a give-up.
+static bool inject_give_up(SplitWorkspace &w) {
+    ++w.calls;
+    const char *e = std::getenv("QDT_SPLIT_FAIL");
+    if (!e || !e[0]) return false;
+    const long long n = std::atoll(e);
+    if (n <= 0) throw Error{QDT_ERR_ARG, "QDT_SPLIT_FAIL must be a positive count"};
+    return n == w.calls;
 }
 
 void split_begin_deferred(SplitWorkspace &w, cudaStream_t s) {
@@ -673,6 +693,7 @@ static void run_umma(SplitWorkspace &w, void *Asl, long long Mpad, long long Kpa
     CUtensorMap tb = make_map(Bsl, kSlices * Npad, KpadB, SBN);
     int *status = (int *)ws_get(w, WS_STAT, 256);
     if (!w.deferred) QDT_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), s));
+    if (inject_give_up(w)) QDT_CUDA_TRY(cudaMemsetAsync(status, 1, sizeof(int), s));
     QDT_CUDA_TRY(cudaFuncSetAttribute(ozaki_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
     dim3 grid((unsigned)(Npad / SBN), (unsigned)(Mpad / SBM));
     ozaki_umma_kernel<<<grid, kThreads, kSmemBytes, s>>>(ta, tb, Mpad, Npad, d_kt128, rowexp, colexp, C, ldc, M, N,

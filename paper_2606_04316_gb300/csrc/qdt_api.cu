@@ -831,9 +831,9 @@ void f32_split(qdt_ctx *ctx, ClassPlan &P, double &bound_out) {
 }
 
 // QDT_W_BUDGET (bytes, > 0) replaces the device-memory test of the row-batch
-// decision: a class runs as one batch when its integral block fits the value,
-// else in batches of at most that many bytes (without bra-ket symmetry).
-// Small values exercise the batched path on small inputs.
+// decision: a class runs as one batch when its integral block fits the value
+// (the digit planes held are handed back first where both do not), else in batches
+// of at most that many bytes.  Small values exercise both on small inputs.
 size_t w_budget_override() {
     const char *e = std::getenv("QDT_W_BUDGET");
     if (!e || !e[0]) return 0;
@@ -894,7 +894,9 @@ void class_finish(qdt_ctx *ctx, ClassPlan &P, qdt_stats *st) {
     const size_t forced = w_budget_override();
     P.one_batch = forced ? (double)wall * wfac <= (double)forced : (double)wall * wfac + slices <= (double)usable;
     // what the decision counted as reusable is handed back first
-    if (P.one_batch && (double)wall * wfac + slices > 0.7 * (double)(fr + ctx->W.n + ctx->Wc.n)) split_release(ctx->split);
+    const bool tight = forced ? (double)wall * wfac + (double)split_held_bytes(ctx->split) > (double)forced
+                              : (double)wall * wfac + slices > 0.7 * (double)(fr + ctx->W.n + ctx->Wc.n);
+    if (P.one_batch && tight) split_release_planes(ctx->split);
     P.wbudget = P.one_batch ? wall : (forced ? forced : ((size_t)6 << 30));
     // row batches of the AO-driven density route keep bra-ket symmetry (each
     // kept pair of blocks computed once, the transpose contracted into the later

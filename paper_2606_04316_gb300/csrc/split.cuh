@@ -22,9 +22,13 @@ struct SplitWorkspace {
     SplitKey bkey[2];          // cached first-half B operands (density slices)
     int bnext = 0;
     bool deferred = false;     // status of the tensor-core waits read once at the end
+    long long calls = 0;       // contractions since the status was cleared
 };
 
 void split_release(SplitWorkspace &w);
+// Frees all but the status word, which belongs to the call in progress: a give-up that a
+// contraction of it recorded is read at its end, and nothing clears the word before then.
+void split_release_planes(SplitWorkspace &w);
 int split_slices(const SplitWorkspace &w);
 // Device bytes currently held by the workspace.
 size_t split_held_bytes(const SplitWorkspace &w);
