@@ -1670,6 +1670,13 @@ void batch_round(qdt_ctx *owner, std::vector<BatchReq> &R, int round, unsigned f
             }
         } catch (const Error &e) { item_fail(r, e); }
     }
+    // what the fused launches read of a request (ket lists, buckets, tile extents) is uploaded on
+    // the request's own stream
+    for (BatchReq *r : fz)
+        if (r->c->stream != s0) {
+            QDT_CUDA_TRY(cudaEventRecord(r->c->join_ev, r->c->stream));
+            QDT_CUDA_TRY(cudaStreamWaitEvent(s0, r->c->join_ev, 0));
+        }
     if (!fz.empty()) {
         // shared tile queues, one per kernel kind (Coulomb or gauge kernel, FP64 or
         // compensated FP32 contraction); tiles of all requests of the kind
