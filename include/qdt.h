@@ -236,6 +236,10 @@ size_t qdt_packed_size(const qdt_ctx *ctx, unsigned blocks, int k_begin, int k_e
  * batches that keep bra-ket symmetry (environment: QDT_W_BUDGET=bytes forces
  * batches of at most that size, QDT_BATCH_SYM=0 turns the symmetry across
  * batches off).  `stats` may be NULL.
+ * QDT_ERR_TIMEOUT: a contraction of the split form gave up waiting (the
+ * environment variable QDT_SPLIT_FAIL=n makes the n-th of a call report that).
+ * A device `out` then holds the blocks that were complete before it, the
+ * other blocks' parts are as they were; a host `out` is as it was.
  */
 int qdt_transform(qdt_ctx *ctx, unsigned blocks, int k_begin, int k_end, double schwarz_tau,
                   int precision, double *out, size_t out_bytes, qdt_stats *stats);

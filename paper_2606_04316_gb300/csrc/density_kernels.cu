@@ -532,8 +532,11 @@ void launch_zero_rows(double *W, long long ld, long long rows, const long long *
 // out[t][parts^2], t = pq nP - pq(pq-1)/2 + (rs - pq) for pq <= rs:
 // out[t][parts i + j] = O[parts pq + i][parts rs + j]  (parts 4: Kramers pairs,
 // parts 2: spinor pairs of Kramers-unrestricted input)
+// A non-zero status word (null: none) means that a contraction behind O gave up: then out keeps
+// what it holds.
 template <int PARTS>
-__global__ void pack_kernel(const double *O, long long ldo, int nP, double *out) {
+__global__ void pack_kernel(const double *O, long long ldo, int nP, double *out, const int *status) {
+    if (status && *status) return;
     int pq = blockIdx.y;
     for (int rs = pq + blockIdx.x * blockDim.x + threadIdx.x; rs < nP; rs += gridDim.x * blockDim.x) {
         long long t = (long long)pq * nP - (long long)pq * (pq - 1) / 2 + (rs - pq);
@@ -547,11 +550,11 @@ __global__ void pack_kernel(const double *O, long long ldo, int nP, double *out)
     }
 }
 
-void launch_pack(const double *O, long long ldo, int nP, int parts, double *out, cudaStream_t s) {
+void launch_pack(const double *O, long long ldo, int nP, int parts, double *out, const int *status, cudaStream_t s) {
     if (nP <= 0) return;
     dim3 grid((nP + 255) / 256, nP);
-    if (parts == 2) pack_kernel<2><<<grid, 256, 0, s>>>(O, ldo, nP, out);
-    else pack_kernel<4><<<grid, 256, 0, s>>>(O, ldo, nP, out);
+    if (parts == 2) pack_kernel<2><<<grid, 256, 0, s>>>(O, ldo, nP, out, status);
+    else pack_kernel<4><<<grid, 256, 0, s>>>(O, ldo, nP, out, status);
     QDT_CHECK_LAUNCH();
 }
 

@@ -120,6 +120,8 @@ static bool inject_give_up(SplitWorkspace &w) {
     return n == w.calls;
 }
 
+const int *split_status(SplitWorkspace &w) { return (const int *)ws_get(w, WS_STAT, 256); }
+
 void split_begin_deferred(SplitWorkspace &w, cudaStream_t s) {
     split_clear_status(w, s);
     w.deferred = true;

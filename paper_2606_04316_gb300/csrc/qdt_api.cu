@@ -1403,7 +1403,7 @@ void half2_job(qdt_ctx *ctx, const ClassPlan &P, const Half2 &H, const Half2::Jo
 }
 
 void half2_pack(qdt_ctx *ctx, const ClassPlan &P, const Half2 &H, const Half2::Job &j, cudaStream_t s) {
-    launch_pack(H.O, H.NO, P.nRS, P.ku ? 2 : 4, j.out, s);
+    launch_pack(H.O, H.NO, P.nRS, P.ku ? 2 : 4, j.out, P.precision == QDT_SPLIT ? split_status(ctx->split) : nullptr, s);
     ctx->launches++;
 }
 
@@ -2192,7 +2192,7 @@ int qdt_transform(qdt_ctx *c, unsigned blocks, int k_begin, int k_end, double ta
         Timer tm(c);
         const int first = tm.mark();
         // one look at the contractions' status for the whole call; a contraction that gives
-        // up makes the later ones return at once
+        // up makes the later ones return at once and their blocks' packing write nothing
         const bool split = precision == QDT_SPLIT;
         if (split) split_begin_deferred(c->split, c->stream);
         double acc[6] = {0, 0, 0, 0, 0, 0};

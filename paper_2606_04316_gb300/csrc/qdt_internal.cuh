@@ -328,7 +328,8 @@ int gemm_fp64_tile_m();
 
 // packing
 // parts: 4 (Kramers pairs) or 2 (spinor pairs, Kramers-unrestricted input); nP units
-void launch_pack(const double *O, long long ldo, int nP, int parts, double *out, cudaStream_t s);
+void launch_pack(const double *O, long long ldo, int nP, int parts, double *out, const int *status,
+                 cudaStream_t s);
 // n_units: Kramers pairs (ku false, 2 n spinors) or spinors (ku true)
 void launch_unpack(const double *packed, int n_units, int gaunt_like, bool ku, double *full, cudaStream_t s);
 void launch_zero(double *p, long long n, cudaStream_t s);

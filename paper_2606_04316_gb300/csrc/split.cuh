@@ -42,6 +42,8 @@ void split_invalidate(SplitWorkspace &w);
 void split_begin_deferred(SplitWorkspace &w, cudaStream_t s);
 void split_clear_status(SplitWorkspace &w, cudaStream_t s);
 void split_end_deferred(SplitWorkspace &w, cudaStream_t s);
+// The status word on the device, non-zero once a contraction gave up.
+const int *split_status(SplitWorkspace &w);
 // Runs one bounded wait on an mbarrier that nothing arrives at, with the
 // given limit; true when the wait gave up and reported it (the expected case).
 bool split_wait_probe(SplitWorkspace &w, double limit_s, cudaStream_t s);
