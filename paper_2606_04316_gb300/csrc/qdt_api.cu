@@ -434,17 +434,9 @@ EriLaunch eri_launch_for(qdt_ctx *ctx, const PairClass &pc, const EriShape &shap
     // a tile may cost a 32nd of a CTA slot's share of the work (4 slots per SM; about
     // half of the kept quartets are computed, the others are their transposes), so
     // that the queue ends evenly
-    double mean = 0.0, weight = 0.0;
-    for (int i = 0; i + 1 < (int)kb.first.size(); ++i)
-        for (int j = 0; j + 1 < (int)kb.first.size(); ++j) {
-            const double w = (double)(kb.first[i + 1] - kb.first[i]) * (kb.first[j + 1] - kb.first[j]);
-            mean += w * (double)quartet_cost(pc.h_pairs[list[kb.pos[kb.first[i]]]], pc.h_pairs[list[kb.pos[kb.first[j]]]],
-                                             gauge);
-            weight += w;
-        }
-    if (weight > 0.0) {
-        def.budget = std::max<long long>(1, (long long)(mean / weight * 0.5 * (double)quartets / (4.0 * nsm * 32.0)));
-    }
+    const double mean = mean_quartet_cost(pc, gauge);
+    if (mean > 0.0)
+        def.budget = std::max<long long>(1, (long long)(mean * 0.5 * (double)quartets / (4.0 * nsm * 32.0)));
     if (const char *pin = std::getenv("QDT_ERI_LAUNCH")) {
         EriLaunch p = def;
         if (std::sscanf(pin, "%d,%d,%d", &p.threads, &p.kets, &p.order) == 3 && p.threads > 0 && p.kets > 0) {
@@ -580,6 +572,7 @@ void build_class(qdt_ctx *ctx, int c) {
         pc.maxnfp = std::max(pc.maxnfp, pr.nfp);
         pc.maxLab = std::max(pc.maxLab, pr.Lab);
         pc.h_pairs.push_back(pr);
+        count_kind(pc, i);
     }
     pc.M = M;
     pc.npp_total = (long long)hpp.size();

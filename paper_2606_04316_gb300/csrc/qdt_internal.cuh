@@ -178,6 +178,13 @@ struct PairClass {
     // pairs, whose quartets with a bra pair are alike (ket_buckets in plan.h)
     std::vector<int> h_bucket;
     std::vector<int> bucket_rep;    // a shell pair of every bucket
+    // kinds of shell pairs (buckets that differ in primitive pairs only): how many pairs, their
+    // primitive pairs, and a pair with the most of them (count_kind in tiles.h)
+    struct Kind {
+        int pairs, most;
+        long long npp;
+    };
+    std::vector<Kind> kinds;
     std::vector<int> bra_pos;   // bra position of every shell pair (inverse of bra_order)
     int *d_bra_pos = nullptr;
     long long npp_total = 0, e_total = 0;
@@ -286,16 +293,24 @@ __host__ __device__ inline int t_rows(int Lx, bool gauge) { return nherm(Lx) + (
 // pass (T rows x the inner pair's box entries per primitive quartet) plus the
 // bra pass (components x the outer pair's box entries x inner function pairs
 // per outer primitive pair).
+// (px, py: primitive pairs of the two, also as means.)
+template <class T>
+__host__ __device__ inline T orient_madds_of(const PairDev &X, T px, const PairDev &Y, T py, bool gauge) {
+    return px * (py * t_rows(X.Lab, gauge) * Y.nbox + (T)X.nbox * Y.nfp * (gauge ? 7 : 1));
+}
 __host__ __device__ inline long long orient_madds(const PairDev &X, const PairDev &Y, bool gauge) {
-    return (long long)X.npp * ((long long)Y.npp * t_rows(X.Lab, gauge) * Y.nbox +
-                               (long long)X.nbox * Y.nfp * (gauge ? 7 : 1));
+    return orient_madds_of<long long>(X, X.npp, Y, Y.npp, gauge);
 }
 // Cost of a shell quartet in multiply-adds: its contraction, and the Hermite
 // recursion as four per entry of its order-0 tensors.
-__host__ __device__ inline long long quartet_cost(const PairDev &A, const PairDev &C, bool gauge) {
+template <class T>
+__host__ __device__ inline T quartet_cost_of(const PairDev &A, T pa, const PairDev &C, T pc, bool gauge) {
     const int L = A.Lab + C.Lab;
-    const long long a = orient_madds(A, C, gauge), c = orient_madds(C, A, gauge);
-    return (a < c ? a : c) + 4LL * A.npp * C.npp * (nherm(L) + (gauge ? nherm(L + 2) : 0));
+    const T a = orient_madds_of<T>(A, pa, C, pc, gauge), c = orient_madds_of<T>(C, pc, A, pa, gauge);
+    return (a < c ? a : c) + (T)4 * pa * pc * (nherm(L) + (gauge ? nherm(L + 2) : 0));
+}
+__host__ __device__ inline long long quartet_cost(const PairDev &A, const PairDev &C, bool gauge) {
+    return quartet_cost_of<long long>(A, A.npp, C, C.npp, gauge);
 }
 // Kets per tile of a bra pair and a bucket: a tile's kets share its CTA one group
 // after another, so expensive quartets come in small tiles and cheap ones, which

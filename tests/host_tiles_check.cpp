@@ -2,7 +2,9 @@
 // classes, from bases of cheap quartets (few kinds, long prefixes: the largest tiles) to
 // mixed ones: the buckets group a ket list, the tiles of a bra pair cover each of its kept
 // kets once, within one bucket and the launch shape's sizes, and the list's room
-// (tile_bound) holds them for every shape a launch may take.
+// (tile_bound) holds them for every shape a launch may take; the mean cost and the smallest
+// tile of a class, taken over its kinds, agree with those over all its buckets.
+#include <algorithm>
 #include <cstdio>
 #include <random>
 
@@ -18,9 +20,16 @@ int main() {
         const bool gauge = rng() % 2 != 0;
         PairClass pc;
         pc.nsp = nsp;
-        std::vector<PairDev> kind(nbk);
-        for (PairDev &k : kind) {
+        std::vector<PairDev> kind(nbk);           // bucket by bucket; every third starts a kind
+        for (int b = 0; b < nbk; ++b) {
+            PairDev &k = kind[b];
+            if (b % 3) {
+                k = kind[b - 1];
+                k.npp = k.npp % 12 + 1;
+                continue;
+            }
             k = PairDev{};
+            k.fpoff = b;
             k.Lab = seed % 4 == 1 ? 0 : (int)(rng() % 5);
             k.npp = seed % 4 == 1 ? 1 : 1 + (int)(rng() % 9);
             k.nfp = 1 + (int)(rng() % (seed % 4 == 1 ? 2 : 18));
@@ -35,6 +44,7 @@ int main() {
             }
             pc.h_pairs.push_back(kind[k]);
             pc.h_bucket.push_back(of[k]);
+            count_kind(pc, i);
         }
         const int nbucket = (int)pc.bucket_rep.size();
         // a ket list: the class in random order, or (row batches) part of it
@@ -63,6 +73,28 @@ int main() {
         for (int i : pc.bucket_rep)
             for (int j : pc.bucket_rep) mean += quartet_cost(pc.h_pairs[i], pc.h_pairs[j], gauge);
         mean /= (long long)nbucket * nbucket;
+        // the sums over kinds against all pairs of buckets: the mean is exact but for the choice of
+        // the orientation, for which a mean takes one and every bucket its own
+        double sum = 0.0;
+        for (int i = 0; i < nsp; ++i)
+            for (int j : pc.bucket_rep)
+                sum += (double)quartet_cost(pc.h_pairs[i], pc.h_pairs[j], gauge) *
+                       (double)std::count(pc.h_bucket.begin(), pc.h_bucket.end(), pc.h_bucket[j]);
+        sum /= (double)nsp * nsp;
+        const double by_kind = mean_quartet_cost(pc, gauge);
+        if (by_kind < sum * (1.0 - 1e-9) || by_kind > 2.0 * sum) {
+            std::printf("seed %d: mean cost %.6e by kinds, %.6e\n", seed, by_kind, sum);
+            ++fails;
+        }
+        for (long long budget : {0LL, 1LL, mean, 12 * mean, 200 * mean}) {
+            EriLaunch how;
+            how.budget = budget;
+            int least = how.kets;
+            for (int i : pc.bucket_rep)
+                for (int j : pc.bucket_rep)
+                    least = std::min(least, tile_kets(pc.h_pairs[i], pc.h_pairs[j], gauge, budget, how.kets));
+            if (smallest_tile(pc, gauge, how) != least) { std::printf("seed %d: smallest tile\n", seed); ++fails; }
+        }
         for (int kets : {1, 8, 16, kMaxTileKets})
             for (long long budget : {0LL, 1LL, mean, 3 * mean, 12 * mean, 200 * mean})
                 for (int form = 0; form < 2; ++form) {
