@@ -25,8 +25,8 @@
 // keep the FP32 pipe busy for a sixth to a quarter of the time, shared-memory loads
 // their unit for more than half; what is left is the latency of chains of table,
 // tensor and coefficient loads at 12 to 16 warps per SM (128 registers), and instruction
-// fetch: the phases of one form are about 75 KB of code.  Measured without gain: fewer
-// registers and more warps (80: 183 to 214 ms for the integrals of a 24-centre chain instead
+// fetch: tiles of both forms interleaved take 131 ms where apart they take 125 (build_tiles).
+// Measured without gain: fewer registers and more warps (80: 183 to 214 ms for the integrals of a 24-centre chain instead
 // of 179), tensor entries placed to avoid the ket pass's bank conflicts (172 for 169), four
 // function pairs per ket item (178 for 173).  In the FP64 form the FP64 pipe bounds it.
 // What keeps the work down:
@@ -40,9 +40,9 @@
 //    scalar form, and the two halves are independent chains.  The bra pass
 //    packs two function pairs y instead.
 //  * Several kets at a time: a small quartet alone leaves most lanes without work.
-// Integrals of a 24-centre chain (Coulomb, Gaunt, gauge) 477 -> 169 ms over these and the
-// choices at the phases below, 40-centre chain (Coulomb) 322 -> 125, an 18-atom cluster
-// 632 -> 205, a class with d shells 671 -> 64; FP64 form, 7-centre chain 39 -> 11.7.
+// Integrals of a 24-centre chain (Coulomb, Gaunt, gauge) 477 -> 171 ms over these and the
+// choices at the phases below, 40-centre chain (Coulomb) 322 -> 128, an 18-atom cluster
+// 632 -> 208, a class with d shells 671 -> 65; FP64 form, 7-centre chain 39 -> 11.7.
 //
 // Split form (DF): recursion and both passes in compensated FP32 pairs (x = hi +
 // lo, ~48-bit significands): products by the exact-product FMA, sums by the

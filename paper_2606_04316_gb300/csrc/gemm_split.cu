@@ -57,7 +57,7 @@ constexpr size_t kPlaneBudget = (size_t)16 << 30;   // digit planes of one secon
 constexpr int kATile = SBM * SBK * 2;         // 16 KB: one A digit plane of a K subtile
 constexpr int kBTile = SBN * SBK * 2;         // 10 KB: one B digit plane
 constexpr int kBPanel = kSlices * kBTile;     // 60 KB: the six B planes of a K subtile
-// shared memory: one stage per A plane (6 x 16 KB) and two B panels (2 x 48 KB)
+// shared memory: one stage per A plane (6 x 16 KB) and two B panels (2 x 60 KB)
 constexpr int kSmemBytes = kSlices * kATile + 2 * kBPanel + 1024 + 256;
 constexpr long long kWaitNs = 2000000000LL;   // 2 s bound on every wait
 
@@ -305,7 +305,8 @@ __global__ void slice_cols_t_kernel(const double *X, long long ld, long long row
         const int cc = i / (64 / kRun), rr = i % (64 / kRun) * kRun;
         const long long r = r0 + rr, c = c0 + cc;
         if (r < Rpad && c < Cpad) {            // Rpad is a multiple of 64
-                        const double2 a = *reinterpret_cast<const double2 *>(&t[cc][rr]), b = *reinterpret_cast<const double2 *>(&t[cc][rr + 2]);
+            const double2 a = *reinterpret_cast<const double2 *>(&t[cc][rr]);
+            const double2 b = *reinterpret_cast<const double2 *>(&t[cc][rr + 2]);
             const double x[kRun] = {a.x, a.y, b.x, b.y};
             store_digits(x, colexp[c], out + (size_t)c * Rpad + r, plane);
         }

@@ -459,7 +459,8 @@ EriLaunch eri_launch_for(qdt_ctx *ctx, const PairClass &pc, const EriShape &shap
     }
     long long total = 0;
     for (int sp : bras) total += prefix[sp];
-    // too little work to tell the candidates apart: fewer than ~64 tiles per CTA slot in the sample
+    // too little work to tell the candidates apart: fewer than 512 quartets per CTA slot in the
+    // sample, 64 tiles of 8 kets or 16 of 32
     if (total / 8 < 64LL * 8 * 4 * nsm) return def;
     std::vector<int> sample;
     for (size_t i = 0; i < bras.size(); i += 8) sample.push_back(bras[i]);
@@ -1548,6 +1549,7 @@ inline int kind_of(const EriParams &p) { return (p.gauge ? 2 : 0) + (p.E2 ? 1 : 
 uint64_t round_signature(const std::vector<BatchReq *> &fz, const std::vector<EriTask> tiles[kKinds],
                          const EriLaunch how[kKinds], const EriShape shape[kKinds]) {
     uint64_t h = 1469598103934665603ULL;
+    if (const char *e = std::getenv("QDT_SPLIT_FAIL")) h = fnv(h, e, std::strlen(e));     // captured with the contractions
     for (int k = 0; k < kKinds; ++k) {
         h = fnv_v(h, tiles[k]);
         const long long launch[] = {how[k].threads, how[k].kets, how[k].order, how[k].budget};
@@ -1704,7 +1706,8 @@ void batch_round(qdt_ctx *owner, std::vector<BatchReq> &R, int round, unsigned f
                                     (k & 1) != 0, d_prms[k], fz[first]->B.bras, fz[first]->P.h_prefix,
                                     fz[first]->B.kb, fz[first]->P.h_ketsp, quartets, s0);
             // tile order across requests: request by request in bra order, or
-            // all bra pairs most expensive first
+            // all bra pairs most expensive first; a bra pair's plain-FP32 tiles follow its
+            // own compensated ones (build_tiles is called pair by pair)
             struct Key { double cost; int i; int sp; };
             std::vector<Key> order;
             for (size_t i = 0; i < fz.size(); ++i) {

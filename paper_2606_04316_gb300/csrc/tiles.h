@@ -12,9 +12,8 @@
 namespace qdt {
 
 // Tiles of at most tile_kets() kets of one bucket per bra pair (list: shell pair at
-// each ket position); with `split`, positions
-// [0, split) and [split, prefix) are tiled apart, the second set in plain FP32 and after
-// all tiles of the first: the phases of both forms together are more code than the
+// each ket position); with `split`, positions [0, split) and [split, prefix) are tiled
+// apart, the second set in plain FP32 and after all tiles of the first for these bra pairs: the phases of both forms together are more code than the
 // instruction caches hold (interleaved, the integrals of a 40-centre chain took 131.1 ms
 // instead of 125.2, of a 24-centre chain 172.6 instead of 169.0).
 inline void build_tiles(const PairClass &pc, const std::vector<int> &bras, const std::vector<int> &prefix,
